@@ -1372,7 +1372,7 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
     const int64_t nb = (n + kBlockB - 1) / kBlockB;
     CKF(dalloc(&h->x, h->n_alloc));
     CKF(dalloc(&h->x_sub, h->n_alloc / kProxyStride + kProxyTile));
-    CKF(dalloc(&h->pf, 4 * n));
+    CKF(dalloc(&h->pf, 4 * prefix_stride(n)));
     CKF(dalloc(&h->bf, 5 * nb));
     CKF(dalloc(&h->pok, nb));
     CKF(dalloc(&h->pscale, 2));
@@ -1380,11 +1380,17 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
     CKF(dalloc(&h->envst, 2 * (size_t)kEnvLevels * h->nblk));
     CKF(dalloc(&h->status, 1));
     CKF(dalloc(&h->absmax, 1));
-    CKF(cudaMemsetAsync(h->x, 0, h->n_alloc * 4, s));
+    // the pads past the series are zero (tile readers read whole tiles)
+    const int64_t sub_n = h->n_alloc / kProxyStride + kProxyTile, sub_written = prefix_stride(n) / kProxyStride;
+    CKF(cudaMemsetAsync(h->x + n, 0, (size_t)(h->n_alloc - n) * 4, s));
     CKF(cudaMemcpyAsync(h->x, series, n * 4, cudaMemcpyDefault, s));
     CKF(cudaMemsetAsync(h->status, 0, 4, s));
     CKF(cudaMemsetAsync(h->absmax, 0, 4, s));
-    CKF(launch_check_finite(h->x, n, h->status, h->absmax, s));
+    CKF(cudaMemsetAsync(h->x_sub + sub_written, 0, (size_t)(sub_n - sub_written) * 4, s));
+    unsigned *excursion = reinterpret_cast<unsigned *>(h->pscale + 1);
+    CKF(launch_series_first(h->x, n, h->status, h->absmax, excursion, h->x_sub, h->envst, h->nblk, s));
+    CKF(launch_prefix(h->x, n, h->pf, h->bf, h->pok, excursion, h->pscale, s));
+    CKF(launch_block_envelope(h->envst, h->nblk, s));
     int flag = 0;
     unsigned amax = 0;
     CKF(cudaMemcpyAsync(&flag, h->status, 4, cudaMemcpyDeviceToHost, s));
@@ -1395,10 +1401,6 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
         set_err("series contains NaN or Inf");
         return fail(DTWS_ENONFINITE);
     }
-    CKF(cudaMemsetAsync(h->x_sub, 0, (h->n_alloc / kProxyStride + kProxyTile) * 4, s));
-    CKF(launch_subsample(h->x, h->n_alloc / kProxyStride, h->x_sub, h->num_sms, s));
-    CKF(launch_prefix(h->x, n, h->pf, h->bf, h->pok, reinterpret_cast<unsigned *>(h->pscale + 1), h->pscale, s));
-    CKF(launch_block_envelope(h->x, n, h->envst, h->nblk, s));
     CKF(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
     CKF(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     CKF(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
@@ -1409,7 +1411,6 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
             break;
         } else
             h->ev_ok = true;
-    CKF(cudaStreamSynchronize(s));
 #undef CKF
     *out = h;
     return DTWS_OK;

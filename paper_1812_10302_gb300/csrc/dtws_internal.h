@@ -14,21 +14,28 @@ namespace dtws {
 void set_error_detail(const char *fmt, ...);
 
 // ---- series level (series_kernels.cu)
-cudaError_t launch_check_finite(const float *x, int64_t n, int *flag, unsigned *absmax, cudaStream_t s);
+// one pass over the padded series (whole blocks readable): *flag |= 1 when a
+// value is not finite, *absmax = max |x| bits, *excursion = bits of the largest
+// |x - x[block start]|, x_sub[j] = x[kProxyStride j] (whole blocks written),
+// st: level 0 of the block envelope
+cudaError_t launch_series_first(const float *x, int64_t n, int *flag, unsigned *absmax, unsigned *excursion,
+                                float *x_sub, float *st, int64_t nblk, cudaStream_t s);
 cudaError_t launch_fill(float *p, int64_t count, float v, int num_sms, cudaStream_t s);
-// xe[j] = x[2j], j < count
-cudaError_t launch_subsample(const float *x, int64_t count, float *xs, int num_sms, cudaStream_t s);
-// pf: 4*n floats (P1 hi, P1 lo, P2 hi, P2 lo); bf: 5*nb floats (T1 hi, lo,
-// T2 hi, lo, anchors); ok: nb flags; nb = ceil(n / kBlockB); maxabs: one
-// word of scratch; scale: one float (the series' power-of-two scale)
-cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *ok, unsigned *maxabs,
+// pf: 4 * prefix_stride(n) floats (P1 hi, P1 lo, P2 hi, P2 lo); bf: 5*nb
+// floats (T1 hi, lo, T2 hi, lo, anchors); ok: nb flags; nb = ceil(n /
+// kBlockB); excursion: from launch_series_first; scale: one float (the
+// series' power-of-two scale).  The prefix arrays hold whole blocks, so that
+// every block is stored in 16-byte pieces.
+inline int64_t prefix_stride(int64_t n) { return (n + kBlockB - 1) / kBlockB * kBlockB; }
+cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *ok, const unsigned *excursion,
                           float *scale, cudaStream_t s);
 cudaError_t launch_window_stats(const float *x, int64_t n, int m, const float *pf, const float *bf,
                                 const int *ok, const float *scale, float *mu_hi, float *mu_lo, float *inv_sigma,
                                 float *smu_hi, float *sinv_sigma, int num_sms, cudaStream_t s);
 cudaError_t launch_envelope(const float *x, int64_t n, int r, float *U, float *L, cudaStream_t s);
-// block envelope: st = [max levels 0..kEnvLevels-1 | min levels], nblk floats each
-cudaError_t launch_block_envelope(const float *x, int64_t n, float *st, int64_t nblk, cudaStream_t s);
+// block envelope: st = [max levels 0..kEnvLevels-1 | min levels], nblk floats
+// each; levels 1.. from level 0
+cudaError_t launch_block_envelope(float *st, int64_t nblk, cudaStream_t s);
 
 // ---- query level (query_kernels.cu)
 struct QueryBufs {

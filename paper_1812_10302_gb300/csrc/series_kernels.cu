@@ -1,7 +1,8 @@
 // series_kernels.cu -- per-series and per-(series, m | r) kernels:
-//   * finiteness check of the series;
-//   * anchored, compensated FP64 prefix sums of the series (once per
-//     series), stored as FP32 pairs;
+//   * one pass over the series: finiteness check, largest |x| and in-block
+//     excursion, its every fourth sample, level 0 of the block envelope;
+//   * anchored, compensated prefix sums of the series (once per series),
+//     stored as FP32 pairs;
 //   * window statistics for a query length m (Sec. 2.2, Eq. 5, population
 //     sigma) from those sums;
 //   * the raw sliding envelope of the series for a band half-width r
@@ -12,28 +13,80 @@
 
 namespace dtws {
 
-// ------------------------------------------------------------------ finite
-// Also the largest |x| (as its FP32 bit pattern, which orders like the value
-// for non-negative floats; meaningful when no value is NaN or Inf).
-__global__ void k_check_finite(const float *__restrict__ x, int64_t n, int *flag, unsigned *absmax) {
+// ------------------------------------------------------------------ first pass
+// One CTA per block of kBlockB samples reads the series once and takes from
+// it everything that needs no other block: the finiteness flag, the largest
+// |x| (as its FP32 bit pattern, which orders like the value for non-negative
+// floats; meaningful when no value is NaN or Inf), the largest in-block
+// excursion |x - x[block start]| (the scale of the prefix sums), the series'
+// every kProxyStride-th sample (x_sub[j] = x[kProxyStride j]) and level 0 of
+// the block envelope (max and min of kEnvG samples).  Bound by memory: 4 B
+// read and 1.5 B written per sample.  (As four kernels, each reading the
+// series again, the same work took 85 us per 1e7 samples.)
+// x is the padded series, so whole float4s are read past n; those samples
+// count for nothing.
+constexpr int kFirstThreads = 256;
+__global__ void __launch_bounds__(kFirstThreads)
+k_series_first(const float *__restrict__ x, int64_t n, int *__restrict__ flag, unsigned *__restrict__ absmax,
+               unsigned *__restrict__ excursion, float *__restrict__ x_sub, float *__restrict__ mx0,
+               float *__restrict__ mn0, int64_t nblk) {
+    static_assert(kProxyStride == 4 && kEnvG == 16, "one float4 per kept sample, four per envelope block");
+    const int64_t t0 = (int64_t)blockIdx.x * kBlockB;
+    const float inf = __int_as_float(0x7f800000);
+    const float a = x[t0];
+    const float4 *x4 = reinterpret_cast<const float4 *>(x + t0);
     bool bad = false;
-    unsigned amax = 0u;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const float v = x[t];
-        bad |= !isfinite(v);
-        amax = max(amax, __float_as_uint(fabsf(v)));
-    }
-    if (__any_sync(0xffffffffu, bad) && lane_id() == 0) atomicOr(flag, 1);
+    float amax = 0.0f, emax = 0.0f;
+    // (a block's float4s: kBlockB / 4 = 8 per thread)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane_id() == 0 && amax) atomicMax(absmax, amax);
+    for (int q = 0; q < kBlockB / 4 / kFirstThreads; ++q) {
+        const int i = q * kFirstThreads + (int)threadIdx.x;
+        const int64_t t = t0 + 4 * (int64_t)i;
+        const float4 v = x4[i];
+        const float w[4] = {v.x, v.y, v.z, v.w};
+        float hi = -inf, lo = inf;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (t + e < n) {
+                bad |= !isfinite(w[e]);
+                amax = fmaxf(amax, fabsf(w[e]));
+                emax = fmaxf(emax, fabsf(w[e] - a));
+                hi = fmaxf(hi, w[e]);
+                lo = fminf(lo, w[e]);
+            }
+        x_sub[t >> 2] = v.x;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        }
+        const int64_t j = t / kEnvG;
+        if ((threadIdx.x & 3) == 0 && j < nblk) {
+            mx0[j] = hi;
+            mn0[j] = lo;
+        }
+    }
+    unsigned ua = __float_as_uint(amax), ue = __float_as_uint(emax);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ua = max(ua, __shfl_xor_sync(0xffffffffu, ua, o));
+        ue = max(ue, __shfl_xor_sync(0xffffffffu, ue, o));
+    }
+    const bool anybad = __any_sync(0xffffffffu, bad);
+    if (lane_id() == 0) {
+        if (anybad) atomicOr(flag, 1);
+        if (ua) atomicMax(absmax, ua);
+        if (ue) atomicMax(excursion, ue);
+    }
 }
 
-cudaError_t launch_check_finite(const float *x, int64_t n, int *flag, unsigned *absmax, cudaStream_t s) {
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
-    k_check_finite<<<blocks, 256, 0, s>>>(x, n, flag, absmax);
+cudaError_t launch_series_first(const float *x, int64_t n, int *flag, unsigned *absmax, unsigned *excursion,
+                                float *x_sub, float *st, int64_t nblk, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(excursion, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+    const int64_t nb = (n + kBlockB - 1) / kBlockB;
+    k_series_first<<<(unsigned)nb, kFirstThreads, 0, s>>>(x, n, flag, absmax, excursion, x_sub, st,
+                                                          st + (size_t)kEnvLevels * nblk, nblk);
     return cudaGetLastError();
 }
 
@@ -48,111 +101,6 @@ cudaError_t launch_fill(float *p, int64_t count, float v, int num_sms, cudaStrea
     int64_t blocks = (count + 255) / 256;
     if (blocks > 8LL * num_sms) blocks = 8LL * num_sms;
     k_fill<<<(int)blocks, 256, 0, s>>>(p, count, v);
-    return cudaGetLastError();
-}
-
-// The series' every kProxyStride-th sample, xs[j] = x[kProxyStride j] for
-// j < count (the proxy scan scores every kProxyStride-th window at term
-// positions that are multiples of kProxyStride, so it reads only these).
-__global__ void k_subsample(const float *__restrict__ x, int64_t count, float *__restrict__ xs) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count; j += (int64_t)gridDim.x * blockDim.x)
-        xs[j] = x[kProxyStride * j];
-}
-
-cudaError_t launch_subsample(const float *x, int64_t count, float *xs, int num_sms, cudaStream_t s) {
-    if (count <= 0) return cudaSuccess;
-    int64_t blocks = (count + 255) / 256;
-    if (blocks > 8LL * num_sms) blocks = 8LL * num_sms;
-    k_subsample<<<(int)blocks, 256, 0, s>>>(x, count, xs);
-    return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------ prefix
-// One thread per block b of kBlockB samples.  The anchor a_b = x[b*B]; every
-// sum inside the block runs over d = x - a_b, in FP64, so no sum grows with
-// the series.  The running sums are compensated (Neumaier's variant of Kahan
-// summation), so each prefix is within about one FP64 ulp of the exact sum of
-// the (rounded) terms, whatever the block length -- plain sequential sums
-// could drift by up to B/2 ulps.  Each FP64 prefix is stored as the exact
-// pair hi = fl32(v), lo = fl32(v - hi) (|v - hi - lo| <= 2^-48 |v|), so the
-// per-window arithmetic runs in FP32 pairs instead of FP64 (GB300 issues
-// FP64 at a small fraction of its FP32 rate).  Outputs, for t in block b:
-//   P1[t] = sum_{bB <= u < t} d_u,  P2[t] = sum d_u^2   (exclusive prefix)
-//   T1[b], T2[b] = block totals, A[b] = a_b,
-//   ok[b] = 1 when every nonzero |d| in the block lies in [2^-40, 2^40], so
-//   that no pair over- or underflows FP32 (else windows touching the block
-//   take the two-pass FP64 path).
-// All of it in units scaled by one power of two per series, 2^s with s such
-// that the largest in-block excursion max|x - a_b| lies in [1, 2) (exact
-// scaling; it keeps the pairs away from FP32 over- and underflow whatever the
-// series' units).  Layout: pf = [P1h | P1l | P2h | P2l] (n floats each),
-// bf = [T1h | T1l | T2h | T2l | A] (nb floats each, A scaled), scale[0] = 2^s.
-__device__ __forceinline__ void neumaier_add(double &s, double &c, double v) {
-    const double t = s + v;
-    c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
-    s = t;
-}
-
-__device__ __forceinline__ void split_store(double v, float *hi, float *lo, int64_t t) {
-    const float h = (float)v;
-    hi[t] = h;
-    lo[t] = (float)(v - (double)h);
-}
-
-// largest |x[t] - x[block start]| of the series, as float bits (non-negative
-// floats order like their bits)
-__global__ void k_block_maxabs(const float *__restrict__ x, int64_t n, unsigned *out) {
-    float mx = 0.0f;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const float d = (float)fabs((double)x[t] - (double)x[t / kBlockB * kBlockB]);
-        mx = fmaxf(mx, d);
-    }
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane_id() == 0) atomicMax(out, __float_as_uint(mx));
-}
-
-__global__ void k_prefix(const float *__restrict__ x, int64_t n, float *__restrict__ pf,
-                         float *__restrict__ bf, int *__restrict__ ok, int64_t nb,
-                         const unsigned *__restrict__ maxabs, float *__restrict__ scale_out) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const float mx = __uint_as_float(*maxabs);
-    // 2^s with mx * 2^s in [1, 2); 1 for a constant series
-    const double sc = mx > 0.0f ? ldexp(1.0, -ilogbf(mx)) : 1.0;
-    if (b == 0) scale_out[0] = (float)sc;
-    if (b >= nb) return;
-    const int64_t t0 = b * kBlockB;
-    const int64_t t1 = t0 + kBlockB < n ? t0 + kBlockB : n;
-    float *p1h = pf, *p1l = pf + n, *p2h = pf + 2 * n, *p2l = pf + 3 * n;
-    const float af = x[t0];
-    const double a = (double)af;
-    double s1 = 0.0, c1 = 0.0, s2 = 0.0, c2 = 0.0;
-    bool good = true;
-    for (int64_t t = t0; t < t1; ++t) {
-        split_store(s1 + c1, p1h, p1l, t);
-        split_store(s2 + c2, p2h, p2l, t);
-        const double d = ((double)x[t] - a) * sc;
-        const double ad = fabs(d);
-        good &= d == 0.0 || (ad >= 9.094947017729282e-13 && ad <= 1099511627776.0);  // 2^-40, 2^40
-        neumaier_add(s1, c1, d);
-        neumaier_add(s2, c2, d * d);
-    }
-    split_store(s1 + c1, bf, bf + nb, b);
-    split_store(s2 + c2, bf + 2 * nb, bf + 3 * nb, b);
-    const double as = a * sc;
-    bf[4 * nb + b] = (float)as;
-    ok[b] = good && (double)(float)as == as && fabs(as) < 1e30 ? 1 : 0;
-}
-
-cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *ok, unsigned *maxabs,
-                          float *scale, cudaStream_t s) {
-    int64_t nb = (n + kBlockB - 1) / kBlockB;
-    cudaError_t e = cudaMemsetAsync(maxabs, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    k_block_maxabs<<<(unsigned)blocks, 256, 0, s>>>(x, n, maxabs);
-    k_prefix<<<(unsigned)((nb + 63) / 64), 64, 0, s>>>(x, n, pf, bf, ok, nb, maxabs, scale);
     return cudaGetLastError();
 }
 
@@ -192,6 +140,199 @@ __device__ __forceinline__ f2 f2_mul_f(f2 x, float f) {
 }
 __device__ __forceinline__ f2 ld2(const float *h, const float *l, int64_t t) { return {h[t], l[t]}; }
 
+// ------------------------------------------------------------------ prefix
+// One CTA per block b of kBlockB samples.  The anchor a_b = x[b*B]; every sum
+// inside the block runs over d = x - a_b, so no sum grows with the series.
+// Outputs, for t in block b:
+//   P1[t] = sum_{bB <= u < t} d_u,  P2[t] = sum d_u^2   (exclusive prefix)
+//   T1[b], T2[b] = block totals, A[b] = a_b,
+//   ok[b] = 1 when every nonzero |d| in the block lies in [2^-40, 2^40], so
+//   that no pair over- or underflows FP32 (else windows touching the block
+//   take the two-pass FP64 path).
+// Each prefix is stored as the pair hi = fl32(v), lo = fl32(v - hi)
+// (|v - hi - lo| <= 2^-48 |v|), so the per-window arithmetic runs in FP32
+// pairs.  All of it in units scaled by one power of two per series, 2^s with
+// s such that the largest in-block excursion max|x - a_b| lies in [1, 2)
+// (exact scaling; it keeps the pairs away from FP32 over- and underflow
+// whatever the series' units).  Layout: pf = [P1h | P1l | P2h | P2l]
+// (prefix_stride(n) floats each), bf = [T1h | T1l | T2h | T2l | A] (nb floats
+// each, A scaled), scale[0] = 2^s.
+//
+// Arithmetic: FP32 with error-free transformations, no FP64 (this part issues
+// it at 1/64 of the FP32 rate).  d is the exact pair TwoSum(x, -a); d^2 the
+// exact sum of dh^2 (product and FMA residual), 2 dh dl (likewise) and dl^2;
+// a running sum is three floats A + B + C, A and B updated by TwoSum, so only
+// C rounds (second-order compensated summation, Klein 2006): a sum of B terms
+// is exact to about B^2 2^-72 of its largest partial sum, well inside the
+// pair that stores it.  A thread owns kPfPer consecutive samples: it sums
+// them, the CTA scans the threads' sums (warp shuffles, then across warps),
+// and the thread sums them again from its carry and stores every prefix.
+// Bound by FP32 issue (~160 instructions per sample; 4 B read and 16 B
+// written).  Measured per 1e7 samples: 0.10 ms, against 8.97 ms (9.9 ms per 1e8)
+// with one thread per block and FP64 Neumaier sums -- a serial chain of 8192
+// samples whatever the series' length.
+struct f3 {
+    float a, b, c;
+};
+struct exact2 {
+    float s, e;
+};
+__device__ __forceinline__ exact2 two_sum_rn(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+// t += h + l
+__device__ __forceinline__ void f3_add(f3 &t, float h, float l) {
+    const exact2 p = two_sum_rn(t.a, h), q = two_sum_rn(t.b, l), r = two_sum_rn(q.s, p.e);
+    t.a = p.s;
+    t.b = r.s;
+    t.c = __fadd_rn(t.c, __fadd_rn(q.e, r.e));
+}
+// t += (h + l)^2
+__device__ __forceinline__ void f3_add_sq(f3 &t, float h, float l) {
+    const float p = __fmul_rn(h, h), pe = __fmaf_rn(h, h, -p);
+    const float h2 = __fadd_rn(h, h), q = __fmul_rn(h2, l), qe = __fmaf_rn(h2, l, -q);
+    f3_add(t, p, pe);
+    const exact2 r = two_sum_rn(t.b, q);
+    t.b = r.s;
+    t.c = __fadd_rn(t.c, __fadd_rn(r.e, __fmaf_rn(l, l, qe)));
+}
+__device__ __forceinline__ f3 f3_sum(f3 x, f3 y) {
+    f3_add(x, y.a, y.b);
+    x.c = __fadd_rn(x.c, y.c);
+    return x;
+}
+__device__ __forceinline__ f3 f3_shfl_up(f3 v, int o) {
+    return {__shfl_up_sync(0xffffffffu, v.a, o), __shfl_up_sync(0xffffffffu, v.b, o),
+            __shfl_up_sync(0xffffffffu, v.c, o)};
+}
+// the pair that stores a sum: hi = fl32 of it, lo the rest
+__device__ __forceinline__ f2 f3_pair(const f3 &t) {
+    const exact2 p = two_sum_rn(t.a, t.b);
+    const float l = __fadd_rn(p.e, t.c), hi = __fadd_rn(p.s, l);
+    return {hi, __fsub_rn(l, __fsub_rn(hi, p.s))};
+}
+
+constexpr int kPfThreads = 512, kPfPer = kBlockB / kPfThreads, kPfWarps = kPfThreads / 32;
+__global__ void __launch_bounds__(kPfThreads)
+k_prefix(const float *__restrict__ x, int64_t n, float *__restrict__ pf, float *__restrict__ bf,
+         int *__restrict__ ok, int64_t nb, int64_t stride, const unsigned *__restrict__ excursion,
+         float *__restrict__ scale_out) {
+    static_assert(kPfPer % 4 == 0 && kPfWarps <= 32, "whole float4s per thread, one scan across warps");
+    __shared__ f3 w1[kPfWarps], w2[kPfWarps];
+    const int64_t b = blockIdx.x, t0 = b * kBlockB + (int64_t)threadIdx.x * kPfPer;
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const float mx = __uint_as_float(*excursion);
+    // 2^s with mx * 2^s in [1, 2); 1 for a constant series
+    const float sc = mx > 0.0f ? (float)ldexp(1.0, -ilogbf(mx)) : 1.0f;
+    if (b == 0 && threadIdx.x == 0) scale_out[0] = sc;
+    const float a = x[b * kBlockB];
+    float xv[kPfPer];
+#pragma unroll
+    for (int q = 0; q < kPfPer / 4; ++q) {
+        const float4 v = reinterpret_cast<const float4 *>(x + t0)[q];
+        xv[4 * q] = v.x;
+        xv[4 * q + 1] = v.y;
+        xv[4 * q + 2] = v.z;
+        xv[4 * q + 3] = v.w;
+    }
+    // d = x - a, scaled; samples past the series add nothing
+    auto diff = [&](int e) {
+        exact2 d = two_sum_rn(t0 + e < n ? xv[e] : a, -a);
+        d.s = __fmul_rn(d.s, sc);
+        d.e = __fmul_rn(d.e, sc);
+        return d;
+    };
+    f3 s1{0.0f, 0.0f, 0.0f}, s2{0.0f, 0.0f, 0.0f};
+    bool good = true;
+#pragma unroll
+    for (int e = 0; e < kPfPer; ++e) {
+        const exact2 d = diff(e);
+        const float ad = fabsf(d.s);
+        good &= d.s == 0.0f || (ad >= 0x1p-40f && ad <= 0x1p40f);  // (NaN: not good)
+        f3_add(s1, d.s, d.e);
+        f3_add_sq(s2, d.s, d.e);
+    }
+    // inclusive scan of the threads' sums within the warp, then of the warps'
+    f3 i1 = s1, i2 = s2;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const f3 u1 = f3_shfl_up(i1, o), u2 = f3_shfl_up(i2, o);
+        if (lane >= o) {
+            i1 = f3_sum(u1, i1);
+            i2 = f3_sum(u2, i2);
+        }
+    }
+    if (lane == 31) {
+        w1[warp] = i1;
+        w2[warp] = i2;
+    }
+    const bool all_good = __syncthreads_and(good);
+    if (warp == 0) {
+        f3 v1{0.0f, 0.0f, 0.0f}, v2{0.0f, 0.0f, 0.0f};
+        if (lane < kPfWarps) {
+            v1 = w1[lane];
+            v2 = w2[lane];
+        }
+#pragma unroll
+        for (int o = 1; o < kPfWarps; o <<= 1) {
+            const f3 u1 = f3_shfl_up(v1, o), u2 = f3_shfl_up(v2, o);
+            if (lane >= o) {
+                v1 = f3_sum(u1, v1);
+                v2 = f3_sum(u2, v2);
+            }
+        }
+        if (lane < kPfWarps) {
+            w1[lane] = v1;
+            w2[lane] = v2;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const f2 p1 = f3_pair(w1[kPfWarps - 1]), p2 = f3_pair(w2[kPfWarps - 1]);
+        bf[b] = p1.hi;
+        bf[nb + b] = p1.lo;
+        bf[2 * nb + b] = p2.hi;
+        bf[3 * nb + b] = p2.lo;
+        const float as = __fmul_rn(a, sc);
+        bf[4 * nb + b] = as;
+        // (the scaled anchor must be exact, so that scaling it back gives a)
+        ok[b] = all_good && (double)as == (double)a * (double)sc && fabsf(as) < 1e30f ? 1 : 0;
+    }
+    // this thread's carry: the warps before, then the lanes before
+    f3 c1 = f3_shfl_up(i1, 1), c2 = f3_shfl_up(i2, 1);
+    if (lane == 0) c1 = c2 = f3{0.0f, 0.0f, 0.0f};
+    if (warp > 0) {
+        c1 = f3_sum(w1[warp - 1], c1);
+        c2 = f3_sum(w2[warp - 1], c2);
+    }
+#pragma unroll
+    for (int q = 0; q < kPfPer / 4; ++q) {
+        f2 o1[4], o2[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            o1[e] = f3_pair(c1);
+            o2[e] = f3_pair(c2);
+            const exact2 d = diff(4 * q + e);
+            f3_add(c1, d.s, d.e);
+            f3_add_sq(c2, d.s, d.e);
+        }
+        // (the arrays hold whole blocks: prefix_stride)
+        const int64_t t = t0 + 4 * q;
+        *reinterpret_cast<float4 *>(pf + t) = make_float4(o1[0].hi, o1[1].hi, o1[2].hi, o1[3].hi);
+        *reinterpret_cast<float4 *>(pf + stride + t) = make_float4(o1[0].lo, o1[1].lo, o1[2].lo, o1[3].lo);
+        *reinterpret_cast<float4 *>(pf + 2 * stride + t) = make_float4(o2[0].hi, o2[1].hi, o2[2].hi, o2[3].hi);
+        *reinterpret_cast<float4 *>(pf + 3 * stride + t) = make_float4(o2[0].lo, o2[1].lo, o2[2].lo, o2[3].lo);
+    }
+}
+
+cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *ok, const unsigned *excursion,
+                          float *scale, cudaStream_t s) {
+    const int64_t nb = (n + kBlockB - 1) / kBlockB;
+    k_prefix<<<(unsigned)nb, kPfThreads, 0, s>>>(x, n, pf, bf, ok, nb, prefix_stride(n), excursion, scale);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ window stats
 // Eq. 5 statistics of window i = [i, i+m) from the anchored sums.  A window
 // spans at most two blocks (m <= kBlockB); the second block's sums are moved
@@ -211,13 +352,13 @@ __device__ __forceinline__ f2 ld2(const float *h, const float *l, int64_t t) { r
 // window normalises to all zeros).
 __global__ void k_window_stats(const float *__restrict__ x, int64_t n, int m, const float *__restrict__ pf,
                                const float *__restrict__ bf, const int *__restrict__ ok,
-                               const float *__restrict__ scale, int64_t nb,
+                               const float *__restrict__ scale, int64_t nb, int64_t stride,
                                float *__restrict__ mu_hi, float *__restrict__ mu_lo,
                                float *__restrict__ inv_sigma, float *__restrict__ smu_hi,
                                float *__restrict__ sinv_sigma) {
     const int64_t N = n - m + 1;
     const float sc = scale[0], isc = 1.0f / sc;  // powers of two
-    const float *p1h = pf, *p1l = pf + n, *p2h = pf + 2 * n, *p2l = pf + 3 * n;
+    const float *p1h = pf, *p1l = pf + stride, *p2h = pf + 2 * stride, *p2l = pf + 3 * stride;
     const float *t1h = bf, *t1l = bf + nb, *t2h = bf + 2 * nb, *t2l = bf + 3 * nb, *A = bf + 4 * nb;
     // 1/m as a pair: hi = fl(1/m), lo = (1 - hi*m)/m (the FMA residual is exact)
     const float ih = 1.0f / (float)m;
@@ -302,8 +443,8 @@ cudaError_t launch_window_stats(const float *x, int64_t n, int m, const float *p
     const int64_t N = n - m + 1, nb = (n + kBlockB - 1) / kBlockB;
     int64_t blocks = (N + 255) / 256;
     if (blocks > (int64_t)num_sms * 16) blocks = (int64_t)num_sms * 16;
-    k_window_stats<<<(unsigned)blocks, 256, 0, s>>>(x, n, m, pf, bf, ok, scale, nb, mu_hi, mu_lo, inv_sigma, smu_hi,
-                                                    sinv_sigma);
+    k_window_stats<<<(unsigned)blocks, 256, 0, s>>>(x, n, m, pf, bf, ok, scale, nb, prefix_stride(n), mu_hi, mu_lo,
+                                                    inv_sigma, smu_hi, sinv_sigma);
     return cudaGetLastError();
 }
 
@@ -381,41 +522,58 @@ cudaError_t launch_envelope(const float *x, int64_t n, int r, float *U, float *L
 
 // ------------------------------------------------------------------ block envelope
 // Sparse table over blocks of kEnvG samples: level 0 holds each block's max
-// (min), level k the max (min) of blocks [j, j + 2^k); entries whose range
-// passes the last block are left unset and never read.
-__global__ void k_env_level0(const float *__restrict__ x, int64_t n, float *__restrict__ mx,
-                             float *__restrict__ mn, int64_t nblk) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nblk;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t0 = j * kEnvG, t1 = t0 + kEnvG < n ? t0 + kEnvG : n;
-        float u = x[t0], l = u;
-        for (int64_t t = t0 + 1; t < t1; ++t) {
-            u = fmaxf(u, x[t]);
-            l = fminf(l, x[t]);
+// (min; written by k_series_first), level k the max (min) of blocks
+// [j, j + 2^k); entries whose range passes the last block are left unset and
+// never read.  A CTA makes every level of kLvTile blocks from those blocks
+// and the 2^(kEnvLevels-1) - 1 after them, doubling in shared memory: level 0
+// is read twice and each level written once (one launch per level read the
+// previous level from L2 twice and took 6.6 us each at 1e7 samples).
+constexpr int kLvTile = 1024, kLvSpan = kLvTile + (1 << (kEnvLevels - 1)), kLvThreads = 512;
+__global__ void __launch_bounds__(kLvThreads) k_env_levels(float *__restrict__ mx, float *__restrict__ mn,
+                                                           int64_t nblk) {
+    __shared__ float u[kLvSpan], l[kLvSpan];
+    constexpr int kPer = (kLvSpan + kLvThreads - 1) / kLvThreads;
+    const int64_t j0 = (int64_t)blockIdx.x * kLvTile;
+    const float inf = __int_as_float(0x7f800000);
+    for (int i = threadIdx.x; i < kLvSpan; i += kLvThreads) {
+        const bool in = j0 + i < nblk;
+        u[i] = in ? mx[j0 + i] : -inf;
+        l[i] = in ? mn[j0 + i] : inf;
+    }
+    __syncthreads();
+    for (int k = 1; k < kEnvLevels; ++k) {
+        const int h = 1 << (k - 1);
+        const int64_t last = nblk - (1ll << k);
+        float a[kPer], c[kPer];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int i = q * kLvThreads + (int)threadIdx.x;
+            // (past the span's end the run is not needed by any output)
+            const int v = i + h < kLvSpan ? i + h : kLvSpan - 1;
+            a[q] = i < kLvSpan ? fmaxf(u[i], u[v]) : 0.0f;
+            c[q] = i < kLvSpan ? fminf(l[i], l[v]) : 0.0f;
         }
-        mx[j] = u;
-        mn[j] = l;
+        __syncthreads();
+        float *qm = mx + (size_t)k * nblk, *qn = mn + (size_t)k * nblk;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int i = q * kLvThreads + (int)threadIdx.x;
+            if (i < kLvSpan) {
+                u[i] = a[q];
+                l[i] = c[q];
+            }
+            if (i < kLvTile && j0 + i <= last) {
+                qm[j0 + i] = a[q];
+                qn[j0 + i] = c[q];
+            }
+        }
+        __syncthreads();
     }
 }
 
-__global__ void k_env_level(float *__restrict__ mx, float *__restrict__ mn, int64_t nblk, int k) {
-    const int64_t h = 1ll << (k - 1), last = nblk - (1ll << k);
-    const float *pm = mx + (size_t)(k - 1) * nblk, *pn = mn + (size_t)(k - 1) * nblk;
-    float *qm = mx + (size_t)k * nblk, *qn = mn + (size_t)k * nblk;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j <= last;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        qm[j] = fmaxf(pm[j], pm[j + h]);
-        qn[j] = fminf(pn[j], pn[j + h]);
-    }
-}
-
-cudaError_t launch_block_envelope(const float *x, int64_t n, float *st, int64_t nblk, cudaStream_t s) {
-    float *mx = st, *mn = st + (size_t)kEnvLevels * nblk;
-    int64_t blocks = (nblk + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    k_env_level0<<<(unsigned)blocks, 256, 0, s>>>(x, n, mx, mn, nblk);
-    for (int k = 1; k < kEnvLevels && (1ll << k) <= nblk; ++k)
-        k_env_level<<<(unsigned)blocks, 256, 0, s>>>(mx, mn, nblk, k);
+cudaError_t launch_block_envelope(float *st, int64_t nblk, cudaStream_t s) {
+    k_env_levels<<<(unsigned)((nblk + kLvTile - 1) / kLvTile), kLvThreads, 0, s>>>(
+        st, st + (size_t)kEnvLevels * nblk, nblk);
     return cudaGetLastError();
 }
 
