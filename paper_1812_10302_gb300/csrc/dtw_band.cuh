@@ -660,7 +660,7 @@ __device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restri
 // Knuth's error-free transformations (TwoSum, FastTwoSum, FMA-based
 // products).  It runs on the FP32 pipes, which on this part issue far more
 // than its FP64 units; accumulated relative error over a DTW is ~1e-14.
-struct dfloat {
+struct alignas(8) dfloat {  // (one 8-byte shared-memory access)
     float hi, lo;
 };
 __device__ __forceinline__ dfloat df_from(double v) {

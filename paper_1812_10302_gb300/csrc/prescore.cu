@@ -1,4 +1,5 @@
 // prescore.cu -- the side-stream pre-score of the best Euclidean seed.
+#include "dtw_fx.cuh"
 #include "dtw_kernels.cuh"
 
 namespace dtws {
@@ -6,7 +7,67 @@ namespace dtws {
 // Pre-score of the best Euclidean seed, run on a side stream while the
 // lower-bound scan streams: its FP32 DTW enters the result list (the survivor
 // pass skips it) and its extended-precision re-score waits for the final
-// stage.  Paired mode (when both copies fit in shared memory): warp 0 runs
+// stage.  One CTA: the last warp runs the FP32 walk, the others the
+// fixed-point re-score beside it (dtw_fx).  When the scan is short the search
+// waits for this kernel, so its latency counts: 172 us at m = 1024, r = 102,
+// against 289 us with the double-float walk on one warp.
+template <int K>
+__global__ void __launch_bounds__(kFxThreads + 32) k_prescore_fx(QueryBufs b, QueryArgs a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ FxShared sh;
+    QueryState *st = b.st;
+    if (!st->valid) return;
+    const unsigned idx = prescored_window(st, a);
+    if (idx == 0xffffffffu) return;
+    const int m = a.m, r = a.r, t = threadIdx.x;
+    const float *xw = b.x + idx;
+    // the fixed-point walk's memory first, then the FP32 walk's padded copies
+    if (t >= kFxThreads) {
+        const int lane = t & 31, pad = diag_pad(r, 32, K);
+        float *q32 = (float *)(smraw + fx_bytes(m, r, K)), *c32 = q32 + (size_t)((m + 2 * pad + 3) & ~3);
+        const float INF = __int_as_float(0x7f800000);
+        fill_pads(q32, m, pad, INF, lane, 32);
+        fill_pads(c32, m, pad, -INF, lane, 32);
+        const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
+        for (int j = lane; j < m; j += 32) {
+            q32[pad + j] = b.qh32[j];
+            c32[pad + j] = fmaf(xw[j] - mh, is, -ls);
+        }
+        __syncwarp();
+        int cells = 0;
+        const float d32 = dtw_diag<float, 32, K, false>(q32 + pad, c32 + pad, nullptr, m, r, INF, 0xffffffffu, lane,
+                                                         cells);
+        if (lane == 0) {
+            const unsigned long long key = make_key(key_quantize(d32, a.qgrid), idx);
+            list_insert(st->res_keys, a.list_cap, key);
+            if (a.xz_z > 0 && d32 < DINF) xz_offer(b, a, key, true);
+            atomicAdd(&st->ctr[kCtrDtwStarted], 1ull);
+            atomicAdd(&st->ctr[kCtrCells], (unsigned long long)cells);
+        }
+        return;
+    }
+    dfloat *qd, *cd;
+    fx_setup<K>(smraw, b.qh64, m, r, t, &qd, &cd);
+    fx_window(xw, m, a.raw != 0, cd, sh, t, 1);
+    const double d64 = dtw_fx<K>(qd, cd, m, r, 0.0f, t, sh, (unsigned long long *)smraw, 1);
+    if (t == 0) {
+        st->pre_d64 = d64;
+        __threadfence();
+        st->pre_done = 1;
+    }
+}
+
+template <int K>
+static cudaError_t prescore_fx_launch(const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
+    const size_t smem = fx_bytes(a.m, a.r, K) + pre_span(a.m, a.r, 32, K) * 8;
+    cudaError_t e = cudaFuncSetAttribute(k_prescore_fx<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_prescore_fx<K><<<1, kFxThreads + 32, smem, s>>>(b, a);
+    return cudaGetLastError();
+}
+
+// The pre-score where dtw_fx does not apply (fx_used: bands past r = 254, or
+// copies that do not fit).  Paired mode (when both copies fit in shared memory): warp 0 runs
 // the FP32 DTW while warps 1..DfW run the re-score beside it, DfW warps wide
 // (the double-float walk's latency per anti-diagonal is what bounds the
 // stage).  Otherwise one warp runs both in turn.
@@ -129,6 +190,16 @@ __global__ void k_prescore(QueryBufs b, QueryArgs a) {
 
 cudaError_t launch_prescore(const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
     if (!a.prescore) return cudaSuccess;
+    if (fx_used(a.m, a.r)) {
+        switch (fx_cells(a.r)) {
+        case 1: return prescore_fx_launch<1>(b, a, s);
+        case 2: return prescore_fx_launch<2>(b, a, s);
+        case 3: return prescore_fx_launch<3>(b, a, s);
+        case 4: return prescore_fx_launch<4>(b, a, s);
+        case 6: return prescore_fx_launch<6>(b, a, s);
+        default: return prescore_fx_launch<8>(b, a, s);
+        }
+    }
     int L, K;
     diag_shape(a.r, &L, &K);
     if (a.r > kDiagRMax) {  // the FP32 walk's wide shapes (one warp, 24 or 32 cells)

@@ -1,0 +1,72 @@
+"""The fixed-point re-score walk (up to two offsets per SM of dtws_dtw_at_f64,
+the pre-score and the final stage of a search) against the FP64 oracle, at the
+edges of its shapes: 32 K >= r + 2 cells for K = 1, 2, 3, 4, 6, 8, whole and
+ragged chunks of 16 anti-diagonals, its widest band and the first past it.
+
+Tolerance: costs carry the double-float normalisation (2^-48 of |z| <= sqrt(m)
+against differences of ~0.05 sigma and more: ~2^-40 per term at worst) and the
+oracle's own FP64 sums; 1e-10 relative covers both with room."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1812_10302_gb300 import dtws, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def series():
+    x = synth.random_walk(40_000, 15)
+    x[3000:3600] = 7.25  # constant windows
+    return x
+
+
+@pytest.mark.parametrize("m,r", [(2, 0), (2, 1), (3, 2), (8, 7), (9, 3), (31, 30), (32, 31), (64, 31), (65, 62), (100, 63),
+                                 (128, 94), (129, 95), (300, 126), (301, 127), (400, 190), (401, 191), (600, 254),
+                                 (600, 255), (1000, 100), (5000, 30), (8192, 20), (8192, 254)])
+def test_at_the_edges_of_its_shapes(series, m, r):
+    q, o = synth.noisy_copy(series, m, m + r, m + 2 * r, noise=0.1)
+    offs = np.random.default_rng(m + r).integers(0, series.size - m + 1, 24)
+    offs[:3] = [o, 0, series.size - m]
+    if m <= 600:
+        offs[3] = 3000
+    with dtws.Index(series) as ix:
+        got = ix.dtw_at_f64(q, r, offs)
+        assert ix.sync_status() == dtws.DTWS_OK
+    want = oracle.dtw_at(series, q, r, offs)
+    np.testing.assert_allclose(got, want, rtol=1e-10, atol=1e-18 * m)
+
+
+@pytest.mark.parametrize("unnormalised,scale", [(0, 1.0), (1, 1.0), (1, 2.0 ** -30), (1, 2.0 ** 20)])
+def test_far_below_the_euclidean_distance(unnormalised, scale):
+    """Shifted copies of a smooth window: warping absorbs the shift, so the DTW
+    lies orders of magnitude below the bound that first scales the walk, which
+    is then repeated on a finer scale."""
+    t = np.arange(6000)
+    x = ((np.sin(t / 40.0) + 0.3 * np.sin(t / 17.0 + 1.0)) * 100.0 * scale).astype(np.float32)
+    m, r = 512, 60
+    q = x[1000:1000 + m].copy()
+    offs = np.array([1000, 1001, 1003, 1010, 1030, 1055, 900, 2500])
+    with dtws.Index(x, options=dict(unnormalised=unnormalised)) as ix:
+        got = ix.dtw_at_f64(q, r, offs)
+        assert ix.sync_status() == dtws.DTWS_OK
+    want = (np.array([oracle.dtw(q, x[o:o + m], r) for o in offs]) if unnormalised
+            else oracle.dtw_at(x, q, r, offs))
+    assert got[0] <= 1e-20 * want[-1]
+    np.testing.assert_allclose(got[1:], want[1:], rtol=1e-8)
+
+
+def test_a_match_and_its_exact_copies_keep_their_order():
+    """The pre-scored window and later bit-identical copies of it come back in
+    offset order: compared windows are walked with one bound."""
+    x = synth.random_walk(30_000, 77)
+    m = 200
+    for at in (20_000, 9_000, 25_000):
+        x[at:at + m] = x[4_000:4_000 + m]
+    q = x[4_000:4_000 + m] + np.random.default_rng(5).normal(0, 0.05, m).astype(np.float32)
+    with dtws.Index(x) as ix:
+        for k in (1, 4):
+            idx, dist = ix.query(q, 20, k)
+            np.testing.assert_array_equal(idx, [4_000, 9_000, 20_000, 25_000][:k])
+            assert np.all(dist == dist[0])
