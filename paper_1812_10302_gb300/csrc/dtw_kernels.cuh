@@ -130,7 +130,7 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                                        (lay.tail ? lay.tail_bytes() : 0))
                            : nullptr;
     // survivor pass: the seeds' offsets (already evaluated by the seed pass)
-    // and the first 128 query positions in |q_hat| order with q_hat and the
+    // and the query's ordered terms (positions) with q_hat and the
     // query envelope there (the pre-check reads them for every candidate)
     __shared__ unsigned seeds_s[kSeedMax];
     __shared__ int n_seeds_s;
@@ -140,7 +140,7 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
         if (threadIdx.x == 0) n_seeds_s = st->n_seeds;
         for (int t = threadIdx.x; t < st->n_seeds; t += blockDim.x) seeds_s[t] = st->seed_off[t];
         for (int t = threadIdx.x; t < 128; t += blockDim.x) {
-            const bool in = t < m;
+            const bool in = t < terms_of(m);
             ord_s[t] = in ? (int)b.ord[t] : 0;
             sq_s[t] = in ? b.sq[t] : 0.0f;
             su_s[t] = in ? b.sU[t] : 0.0f;
@@ -214,13 +214,13 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                 }
                 if (pass && has_env) {
                     // Eq. 10 (q_hat against the window's envelope) and Eq. 8
-                    // (the window against the query's envelope; the scan took
-                    // only its first terms) with early abandon, terms in
-                    // |q_hat| descending order until either partial sum passes
-                    // thr -- each is a lower bound on its own (rows and
-                    // columns of the same warping path).  Past 128 terms the
-                    // full Eq. 10 below (row order, with the suffix sums the
-                    // DTW needs) takes over.
+                    // (the window against the query's envelope: the scan took
+                    // its first kScanTerms terms, which with LB_KimFL make up
+                    // the survivor's bound) with early abandon, until either
+                    // partial sum passes thr -- each is a lower bound on its
+                    // own (rows and columns of the same warping path).  Past
+                    // the ordered terms the full Eq. 10 below (row order, with
+                    // the suffix sums the DTW needs) takes over.
                     TailCtx pc;
                     pc.Uw = b.U ? b.U + id : nullptr;
                     pc.Lw = b.L ? b.L + id : nullptr;
@@ -231,18 +231,19 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                     pc.t0 = id;
                     pc.r = r;
                     const float *xp = b.x + id;
-                    const int budget = m < 128 ? m : 128;
-                    float acc = 0.0f, acc8 = 0.0f;
+                    const int budget = terms_of(m);
+                    float acc = 0.0f, acc8 = lbv;
                     // 8 terms per step: their loads are issued together, the
                     // abandon test runs once per step
                     constexpr int kB = 8;
                     for (int j0 = 0; j0 < budget; j0 += kB) {
                         float xv[kB], uv[kB], lv[kB];
+                        const bool eq8 = j0 >= kScanTerms;
 #pragma unroll
                         for (int t = 0; t < kB; ++t) {
                             const int j = j0 + t < budget ? j0 + t : budget - 1;
                             const int pos = ord_s[j];
-                            xv[t] = xp[pos];
+                            if (eq8) xv[t] = xp[pos];
                             env_at(pc, pos, uv[t], lv[t]);
                         }
 #pragma unroll
@@ -252,10 +253,12 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                             const float u = fmaf(uv[t] - pmh, pis, -pls), l = fmaf(lv[t] - pmh, pis, -pls);
                             const float q = sq_s[j];
                             const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
-                            const float cv = fmaf(xv[t] - pmh, pis, -pls);
-                            const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
                             acc = fmaf(dq, dq, acc);
-                            acc8 = fmaf(e, e, acc8);
+                            if (eq8) {
+                                const float cv = fmaf(xv[t] - pmh, pis, -pls);
+                                const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
+                                acc8 = fmaf(e, e, acc8);
+                            }
                         }
                         if (acc > th || acc8 > th) {
                             pass = false;
@@ -347,31 +350,35 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
             // the same pre-check as the batch schedule's, L terms per step
             // over the group (the sums are reduced, so every lane takes the
             // same exit)
-            float acc = 0.0f, acc8 = 0.0f;
+            float acc = 0.0f, acc8 = lb;
             bool pruned = false;
-            const int budget = m < 128 ? m : 128;
+            const int budget = terms_of(m);
             for (int c0 = 0; c0 < budget; c0 += L) {
                 const int j = c0 + lane;
+                const bool eq8 = c0 >= kScanTerms;
                 float v = 0.0f, v8 = 0.0f;
                 if (j < budget) {
                     const int pos = ord_s[j];
-                    const float x = xw[pos];
+                    const float x = eq8 ? xw[pos] : 0.0f;
                     float U, Lo;
                     env_at(tc, pos, U, Lo);
                     const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
                     const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
                     v = dq * dq;
-                    const float cv = fmaf(x - mh, is, -ls);
-                    const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                    v8 = e * e;
+                    if (eq8) {
+                        const float cv = fmaf(x - mh, is, -ls);
+                        const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
+                        v8 = e * e;
+                    }
                 }
 #pragma unroll
-                for (int o = L / 2; o > 0; o >>= 1) {
-                    v += __shfl_xor_sync(gmask, v, o, L);
-                    v8 += __shfl_xor_sync(gmask, v8, o, L);
-                }
+                for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask, v, o, L);
                 acc += v;
-                acc8 += v8;
+                if (eq8) {
+#pragma unroll
+                    for (int o = L / 2; o > 0; o >>= 1) v8 += __shfl_xor_sync(gmask, v8, o, L);
+                    acc8 += v8;
+                }
                 if (acc > thr || acc8 > thr) {
                     pruned = true;
                     break;
@@ -700,7 +707,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
         if (threadIdx.x == 0) n_seeds_s = st->n_seeds;
         for (int i = threadIdx.x; i < st->n_seeds; i += blockDim.x) seeds_s[i] = st->seed_off[i];
         for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-            const bool in = i < m;
+            const bool in = i < terms_of(m);
             ord_s[i] = in ? (int)b.ord[i] : 0;
             sq_s[i] = in ? b.sq[i] : 0.0f;
             su_s[i] = in ? b.sU[i] : 0.0f;
@@ -737,6 +744,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
         if (c >= count) break;
         const float thr = thr_s[g][it];
         unsigned idx = 0;
+        float lb = 0.0f;
         if (MODE == kModeSeed) {
             idx = st->seed_off[c];
         } else if (MODE == kModeOut) {
@@ -748,7 +756,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
             idx = (unsigned)o;
         } else {
             idx = b.sort_idx[c];
-            const float lb = b.sort_lb[c];
+            lb = b.sort_lb[c];
             if (lb > thr) {
                 // survivors are in ascending bins and thr only shrinks
                 if (bin_floor(bin_of(lb, thr_scan), thr_scan) > thr) break;
@@ -774,9 +782,9 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
         tc.is = is;
         tc.ls = ls;
         if (has_env) {
-            // Eq. 10 and Eq. 8 over the 128 largest-|q_hat| rows (one pass:
+            // Eq. 10 and Eq. 8 over the ordered terms (one pass:
             // 128 threads, one term each), reduced over the group
-            const int budget = m < 128 ? m : 128;
+            const int budget = terms_of(m);
             float v = 0.0f, v8 = 0.0f;
             for (int j = t; j < budget; j += nthr) {
                 const int pos = ord_s[j];
@@ -785,9 +793,11 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
                 const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
                 const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
                 v = fmaf(dq, dq, v);
-                const float cv = fmaf(xw[pos] - mh, is, -ls);
-                const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                v8 = fmaf(e, e, v8);
+                if (j >= kScanTerms) {  // (the scan took the others)
+                    const float cv = fmaf(xw[pos] - mh, is, -ls);
+                    const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
+                    v8 = fmaf(e, e, v8);
+                }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -799,7 +809,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
                 xch[g].red[1][w] = v8;
             }
             group_bar(bar, nthr);
-            float acc = 0.0f, acc8 = 0.0f;
+            float acc = 0.0f, acc8 = lb;
 #pragma unroll
             for (int u = 0; u < W; ++u) {
                 acc += xch[g].red[0][u];

@@ -688,15 +688,15 @@ dtws_status enqueue_search(dtws_t h, const Exec &e, const QueryArgs &a, const fl
         half = learn_half(m);
         launches += 3;
     }
-    if (P > 0 && !e.le) {  // (the proxy scan merges its proposals and gathers the seeds itself)
-        int c0 = 0;
-        CK(launch_seed_scan(b, a, P, h->opt.proxy_terms, R, half, h->opt.rng_seed, &c0, s));
+    int ctas = 0;
+    if (P > 0 && !e.le) {  // (the proxy scan's windows are seeds as they stand)
+        CK(launch_seed_scan(b, a, P, h->opt.proxy_terms, R, h->opt.rng_seed, &ctas, s));
         ++launches;
     } else {
         CK(launch_seed_gather(b, a, R, P, half, h->opt.rng_seed, s));
         ++launches;
     }
-    CK(launch_seed_ed(b, a, R + P * (2 * half + 1), s));
+    CK(launch_seed_ed(b, a, ctas, R, h->opt.rng_seed, R + P * (2 * half + 1), s));
     if (k > 1 && a.xz_z == 0) {  // exact DTW seeds tighten a k-th bound the Euclidean seeds leave loose
         // (the neighbours of one match, which is all these seeds are, bound
         // nothing with an exclusion zone)

@@ -34,6 +34,7 @@ constexpr int kListMax = 128;       // result list capacity (k + near-tie margin
 constexpr int kSeedMax = 128;       // random seeds + proxy proposals
 constexpr int kPropMax = 64;
 constexpr int kCtaSlots = 1024;     // per-CTA best windows of one proposal scan (at most this many CTAs)
+constexpr int kScanConsumers = 8;   // consumer warps of a scan's CTA
 constexpr int kProxyStride = 4;     // the proxy scan looks at every fourth window
 // Euclidean seeds around each proxy proposal: offsets within +-kProxyHalf.
 // A match off the proxy's grid is never scored by the proxy itself; on a
@@ -60,6 +61,11 @@ constexpr int kTile = 1024;         // windows per lower-bound tile
 constexpr int kProxyTile = 4096;    // windows per proxy-scan tile (a multiple of kTile)
 constexpr int kStages = 4;          // shared-memory stages of the scan pipeline
 constexpr int kBins = 1024;         // survivor ordering bins
+// terms of the early-abandoning bounds: at most kTerms of the query's inner
+// positions (see k_qprep)
+constexpr int kTerms = 128;
+constexpr int kScanTerms = 64;  // of them the lower-bound scan takes for every window that it keeps
+__host__ __device__ inline int terms_of(int m) { return m - 2 < kTerms ? m - 2 : kTerms; }
 constexpr int kDiagRMax = 511;      // widest band of the anti-diagonal DTW kernels (all shapes)
 constexpr int kDiagRMaxF32 = 1023;  // widest band of the FP32 anti-diagonal kernels (24, 32 cells per lane)
 constexpr uint64_t kEmptyKey = ~0ull;
@@ -121,6 +127,8 @@ struct QueryState {
     // CTAs of the proxy scan and of the survivor histogram that have
     // finished: the last one of each takes the step that needs all of them
     unsigned int prop_done, bin_done, final_done;
+    // (last: the words above that the scans' atomics meet on stay where they were)
+    unsigned long long warp_best[kCtaSlots * kScanConsumers];  // each proxy-scan warp's best window
 };
 
 // Scalars of one query, passed by value to every kernel.

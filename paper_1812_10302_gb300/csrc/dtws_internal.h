@@ -159,15 +159,18 @@ cudaError_t launch_query_reset(const QueryBufs &b, const QueryArgs &a, cudaStrea
 cudaError_t launch_qprep(const float *Q, const QueryBufs &b, const QueryArgs &a, cudaStream_t s);
 // proposal scans: each CTA writes its best window to cta_best[slot * kCtaSlots + cta];
 // *ctas receives the grid size; launch_prop_merge then keeps the best `proposals`.
-// The proxy scan does that merge itself, and the seed lists (launch_seed_gather
-// with n_random, H and rng), in the last of its CTAs to finish.
-cudaError_t launch_seed_scan(const QueryBufs &b, const QueryArgs &a, int proposals, int terms, int n_random, int H,
+// For k > 1 the proxy scan does that merge itself, and the list of exact-DTW
+// seeds, in the last of its CTAs to finish.
+cudaError_t launch_seed_scan(const QueryBufs &b, const QueryArgs &a, int proposals, int terms, int n_random,
                              unsigned long long rng, int *ctas, cudaStream_t s);
 // half: Euclidean seeds cover the proposals' offsets +-half
 cudaError_t launch_seed_gather(const QueryBufs &b, const QueryArgs &a, int n_random,
                                int proposals, int half, unsigned long long rng, cudaStream_t s);
-// max_seeds: an upper bound on the Euclidean seed list's length (grid size)
-cudaError_t launch_seed_ed(const QueryBufs &b, const QueryArgs &a, int max_seeds, cudaStream_t s);
+// Euclidean seeds: after the proxy scan (ctas > 0, its grid) the neighbourhood
+// of every scan warp's best window and n_random random windows; else the list of
+// launch_seed_gather, max_seeds an upper bound of its length
+cudaError_t launch_seed_ed(const QueryBufs &b, const QueryArgs &a, int ctas, int n_random, unsigned long long rng,
+                           int max_seeds, cudaStream_t s);
 // k > 1: offsets within +-k of the two best Euclidean seeds join the DTW seeds
 cudaError_t launch_seed_expand(const QueryBufs &b, const QueryArgs &a, cudaStream_t s);
 cudaError_t launch_dtw_seeds(const QueryBufs &b, const QueryArgs &a, cudaStream_t s);

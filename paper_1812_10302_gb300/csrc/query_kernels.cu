@@ -3,8 +3,8 @@
 //   k_query_reset   clear the device query state
 //   k_qprep         z-normalise Q (Sec. 2.2, Eq. 5; FP64 two-pass; taken as
 //                   it is for unnormalised DTW), its envelope (Eq. 9) and the
-//                   order of |q_hat| (largest first)
-//   k_seed_scan     proxy scan: each CTA's window with the smallest squared
+//                   ordered terms of the early-abandoning bounds
+//   k_seed_scan     proxy scan: each warp's window with the smallest squared
 //                   distance on evenly spaced query positions, to its slot
 //   k_prop_merge    the P best of the per-CTA slots (rank selection)
 //   k_seed_gather   seed offsets = seeded random windows (the paper's random
@@ -85,27 +85,43 @@ cudaError_t launch_query_reset(const QueryBufs &b, const QueryArgs &, cudaStream
 }
 
 // ------------------------------------------------------------------ query prep
-// One CTA of 128, 256 or 512 threads.  Dynamic smem: one row of kQBins
-// 16-bit counters per warp (the ordering's counting sort), then q_hat, its
-// upper and its lower envelope, FP32 [m] each.
-constexpr int kQBins = 1024;  // |q_hat| quantised to 1/256, up to 4
+// One CTA of 128, 256 or 512 threads: latency, every later kernel waits for it.
+// Dynamic smem: q_hat and two pairs of envelope buffers, FP32 [m] each.
+//
+// The terms of the early-abandoning bounds (ord, sq, sU, sL; terms_of(m) of
+// them): the query's positions 1 .. m-2 (its ends belong to LB_KimFL) are cut
+// into at most kTerms equal segments, each represented by its position of
+// largest |q_hat|, and the segments are taken in golden-ratio steps, so that
+// any prefix -- 8 terms, 32, 64 -- covers the whole query evenly.
+// Neighbouring samples of a series say the same thing: in |q_hat|-descending
+// order the first 64 terms sat in one or two excursions of the query (on 1e8
+// windows, m = 512, five queries: 0.13 to 2.1e6 windows passed 64 of them,
+// 0.02 to 0.45e6 pass 64 spread ones with LB_KimFL added).  Any choice of terms is admissible.
+__device__ __forceinline__ int gcd_of(int a, int b) {
+    while (b) {
+        const int t = a % b;
+        a = b;
+        b = t;
+    }
+    return a;
+}
 __global__ void __launch_bounds__(512) k_qprep(const float *__restrict__ Q, QueryBufs b, QueryArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int bad;
-    __shared__ unsigned wsum[16];
     const int m = a.m, r = a.r;
-    const int nw = (int)(blockDim.x >> 5), wid = (int)(threadIdx.x >> 5), lane = lane_id();
-    unsigned short *tab = reinterpret_cast<unsigned short *>(smraw);
-    float *qs = reinterpret_cast<float *>(tab + nw * kQBins);
-    float *us = qs + m, *ls = us + m;
+    float *qs = reinterpret_cast<float *>(smraw);
+    float *up = qs + m, *dn = up + m, *up2 = dn + m, *dn2 = up2 + m;
 
     // the query's state starts clear (this kernel opens every query)
     reset_state(b.st);
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
     bool nf = false;
-    for (int j = threadIdx.x; j < m; j += blockDim.x)
-        nf |= !isfinite(Q[j]) || (a.raw && fabsf(Q[j]) > kRawAbsMax);
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const float v = Q[j];
+        qs[j] = v;
+        nf |= !isfinite(v) || (a.raw && fabsf(v) > kRawAbsMax);
+    }
     if (nf) atomicOr(&bad, 1);
     __syncthreads();
     if (bad) {
@@ -116,19 +132,14 @@ __global__ void __launch_bounds__(512) k_qprep(const float *__restrict__ Q, Quer
         return;
     }
     // Eq. 5, two-pass in FP64: mu, then sum (x - mu)^2 / m (population).
-    // One warp does the FP64 work: this part's FP64 units retire about one
+    // One warp does the FP64 sums: this part's FP64 units retire about one
     // lane operation per cycle per SM, so FP64 shuffle reductions in every
     // warp of the block would cost far more than the sums themselves.
     // Unnormalised DTW takes the query as it is.
     __shared__ double mu_s, isg_s;
-    if (threadIdx.x < 32 && a.raw) {
-        for (int j = threadIdx.x; j < m; j += 32) {
-            b.qh64[j] = (double)Q[j];
-            qs[j] = Q[j];
-        }
-    } else if (threadIdx.x < 32) {
+    if (threadIdx.x < 32) {
         double s = 0.0;
-        for (int j = threadIdx.x; j < m; j += 32) s += (double)Q[j];
+        for (int j = threadIdx.x; j < m; j += 32) s += (double)qs[j];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) mu_s = s / (double)m;  // one division
@@ -136,7 +147,7 @@ __global__ void __launch_bounds__(512) k_qprep(const float *__restrict__ Q, Quer
         const double mu = mu_s;
         double v = 0.0;
         for (int j = threadIdx.x; j < m; j += 32) {
-            const double d = (double)Q[j] - mu;
+            const double d = (double)qs[j] - mu;
             v = fma(d, d, v);
         }
 #pragma unroll
@@ -145,104 +156,78 @@ __global__ void __launch_bounds__(512) k_qprep(const float *__restrict__ Q, Quer
             const double var = v / (double)m, mm = mu * mu;
             // one square root and reciprocal
             isg_s = var <= 1e-24 * (mm > 1.0 ? mm : 1.0) ? 0.0 : 1.0 / sqrt(var);
+            if (a.raw) {
+                mu_s = 0.0;
+                isg_s = 1.0;
+            }
         }
-        __syncwarp();
-        const double isg = isg_s;
-        for (int j = threadIdx.x; j < m; j += 32) {
-            const double qh = ((double)Q[j] - mu) * isg;
-            b.qh64[j] = qh;
-            qs[j] = (float)qh;
-        }
-    }
-    __syncthreads();
-    // envelope of q_hat, half-width r, clipped (Eq. 9)
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        int lo = j - r > 0 ? j - r : 0, hi = j + r < m - 1 ? j + r : m - 1;
-        float u = qs[lo], l = qs[lo];
-        for (int t = lo + 1; t <= hi; ++t) {
-            u = fmaxf(u, qs[t]);
-            l = fminf(l, qs[t]);
-        }
-        b.Uq[j] = u;
-        b.Lq[j] = l;
-        us[j] = u;
-        ls[j] = l;
-        b.qh32[j] = qs[j];
-    }
-    // order by |q_hat| descending, quantised to 1/256 (the order only decides
-    // which terms the early-abandoning bounds take first: any order is
-    // admissible), ties by position ascending: a stable counting sort over
-    // the warps.  Warp w owns positions [w C, (w + 1) C) and a row of
-    // counters: (1) each warp counts its keys, 32 positions at a time (equal
-    // keys found by a match, counted once by their lowest lane); (2) per key,
-    // from the largest |q_hat| down, the rows' counts become each row's first
-    // slot (a scan over the keys of the rows' totals, then down the rows);
-    // (3) each warp places its positions in order, ranking equal keys within
-    // 32 positions by lane.
-    for (int t = threadIdx.x; t < nw * kQBins; t += blockDim.x) tab[t] = 0;
-    __syncthreads();
-    auto qkey = [&](int j) {
-        const int v = (int)(fabsf(qs[j]) * 256.0f);
-        return (kQBins - 1) - (v < kQBins - 1 ? v : kQBins - 1);  // 0 = the largest |q_hat|
-    };
-    const int C = ((m + nw - 1) / nw + 31) & ~31;
-    const int j0 = wid * C < m ? wid * C : m, j1 = j0 + C < m ? j0 + C : m;
-    unsigned short *row = tab + wid * kQBins;
-    for (int c0 = j0; c0 < j1; c0 += 32) {
-        const int j = c0 + lane;
-        const bool in = j < j1;
-        const int kk = in ? qkey(j) : -1 - lane;  // (out-of-range lanes match nobody)
-        const unsigned peers = __match_any_sync(0xffffffffu, kk);
-        if (in && (peers & ((1u << lane) - 1u)) == 0u) row[kk] = (unsigned short)(row[kk] + __popc(peers));
-        __syncwarp();
     }
     __syncthreads();
     {
-        const int per = kQBins / (int)blockDim.x;  // 8, 4 or 2 keys per thread
-        const int k0 = (int)threadIdx.x * per;
-        unsigned run = 0;
-        for (int u = 0; u < per; ++u)
-            for (int w = 0; w < nw; ++w) run += tab[w * kQBins + k0 + u];
-        unsigned incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
+        const double mu = mu_s, isg = isg_s;
+        for (int j = threadIdx.x; j < m; j += blockDim.x) {
+            const double qh = ((double)qs[j] - mu) * isg;
+            const float q = (float)qh;
+            b.qh64[j] = qh;
+            b.qh32[j] = q;
+            qs[j] = q;
+            up[j] = q;
+            dn[j] = q;
         }
-        if (lane == 31) wsum[wid] = incl;
-        __syncthreads();
-        unsigned start = incl - run;
-        for (int w = 0; w < wid; ++w) start += wsum[w];
-        for (int u = 0; u < per; ++u)
-            for (int w = 0; w < nw; ++w) {
-                const unsigned v = tab[w * kQBins + k0 + u];
-                tab[w * kQBins + k0 + u] = (unsigned short)start;
-                start += v;
-            }
     }
     __syncthreads();
-    for (int c0 = j0; c0 < j1; c0 += 32) {
-        const int j = c0 + lane;
-        const bool in = j < j1;
-        const int kk = in ? qkey(j) : -1 - lane;
-        const unsigned peers = __match_any_sync(0xffffffffu, kk);
-        const unsigned rank = __popc(peers & ((1u << lane) - 1u));
-        const unsigned slot = in ? row[kk] + rank : 0u;
-        __syncwarp();
-        if (in && rank == 0) row[kk] = (unsigned short)(row[kk] + __popc(peers));
-        if (in) {
-            b.ord[slot] = (unsigned short)j;
-            b.sq[slot] = qs[j];
-            b.sU[slot] = us[j];
-            b.sL[slot] = ls[j];
+    // envelope of q_hat, half-width r, clipped (Eq. 9), by doubling: after
+    // each pass up[u] (dn[u]) is the max (min) over [u, u + span) clipped to
+    // the query.  With span the largest power of two <= r + 1, which every
+    // clipped window holds, four runs inside [lo, hi] cover it.  (A loop over
+    // each position's window took 40 us at m = 1024, r = 921.)
+    int span = 1;
+    for (; 2 * span <= r + 1; span *= 2) {
+        for (int j = threadIdx.x; j < m; j += blockDim.x) {
+            const int v = j + span < m ? j + span : m - 1;
+            up2[j] = fmaxf(up[j], up[v]);
+            dn2[j] = fminf(dn[j], dn[v]);
         }
-        __syncwarp();
+        __syncthreads();
+        float *t = up;
+        up = up2;
+        up2 = t;
+        t = dn;
+        dn = dn2;
+        dn2 = t;
+    }
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const int lo = j - r > 0 ? j - r : 0, hi = j + r < m - 1 ? j + r : m - 1, e = hi - span + 1;
+        const int c = lo + span < e ? lo + span : e, d = e - span > lo ? e - span : lo;
+        const float u = fmaxf(fmaxf(up[lo], up[c]), fmaxf(up[d], up[e]));
+        const float l = fminf(fminf(dn[lo], dn[c]), fminf(dn[d], dn[e]));
+        b.Uq[j] = u;
+        b.Lq[j] = l;
+        up2[j] = u;
+        dn2[j] = l;
+    }
+    __syncthreads();
+    // the ordered terms
+    const int T = terms_of(m);
+    if ((int)threadIdx.x < T) {
+        int g = (T * 5 + 4) / 8;  // near the golden ratio's share, then coprime to T
+        while (gcd_of(T, g) != 1) --g;
+        const int seg = ((int)threadIdx.x + 1) * g % T;  // (the segments next to the ends not first)
+        const int j0 = 1 + seg * (m - 2) / T, j1 = 1 + (seg + 1) * (m - 2) / T;
+        int pos = j0;
+        for (int j = j0 + 1; j < j1; ++j)
+            if (fabsf(qs[j]) > fabsf(qs[pos])) pos = j;
+        b.ord[threadIdx.x] = (unsigned short)pos;
+        b.sq[threadIdx.x] = qs[pos];
+        b.sU[threadIdx.x] = up2[pos];
+        b.sL[threadIdx.x] = dn2[pos];
     }
 }
 
 cudaError_t launch_qprep(const float *Q, const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
+    static_assert(kTerms <= 128, "one thread per term");
     const int threads = a.m < 256 ? 128 : (a.m < 1024 ? 256 : 512);
-    const size_t smem = (size_t)(threads / 32) * kQBins * 2 + (size_t)a.m * 12;
+    const size_t smem = (size_t)a.m * 20;
     cudaError_t e = cudaFuncSetAttribute(k_qprep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_qprep<<<1, threads, smem, s>>>(Q, b, a);
@@ -332,8 +317,6 @@ __device__ __forceinline__ void issue_tile(const Tile &t, const QueryBufs &b, in
     bulk_g2s(t.is, LY::is(b) + s0, sb, t.full);
 }
 
-constexpr int kScanConsumers = 8;                       // consumer warps
-constexpr int kLaneEqMin = 20;  // LB_KimFL passers in a row of 32 above which each lane takes its own Eq. 8
 constexpr int kScanThreads = (kScanConsumers + 1) * 32;  // + one producer warp
 
 // Runs process(tile, i0) in every consumer warp for each tile this CTA takes
@@ -502,15 +485,20 @@ __device__ __forceinline__ unsigned long long lds64_at(unsigned addr) {
 
 __device__ void prop_rank_select(QueryState *st, const unsigned long long *keys, int n, int first, int stride,
                                  int proposals);
+// exact-DTW seeds only pay off for k > 1, and not with a wide exclusion zone
+// (no seed pass runs then, so the survivor pass must not skip them)
+__device__ __forceinline__ bool exact_seeds(const QueryArgs &a) { return a.k > 1 && a.xz_z == 0; }
 __device__ void seed_lists(const QueryBufs &b, const QueryArgs &a, int n_random, int proposals, int H,
                            unsigned long long rng, unsigned *cand, int *wcnt, int *total);
 
-// The last CTA of the scan to finish (a completion count; nothing waits)
-// then merges every CTA's best into the proposals and builds the seed
-// lists, the work of k_prop_merge and k_seed_gather without their launches.
+// Every warp's best window is a Euclidean seed (k_seed_ed reads the slots).
+// For exact-DTW seeds (k > 1) the last CTA of the scan to finish (a completion
+// count; nothing waits) then ranks the CTAs' bests into the proposals and
+// builds the seed list, the work of k_prop_merge and k_seed_gather without their
+// launches.
 template <int TERMS>
 __global__ void __launch_bounds__(kScanThreads) k_seed_scan(QueryBufs b, QueryArgs a, int proposals, int stages,
-                                                            int n_random, int H, unsigned long long rng) {
+                                                            int n_random, unsigned long long rng) {
     constexpr int kPer = kScanConsumers * 64;           // scored windows per pass of the CTA (two per lane)
     constexpr int kIt = ProxyLayout::S / kPer;          // passes per tile
     static_assert(ProxyLayout::S % kPer == 0 && kIt % 2 == 0, "whole pairs of passes per tile");
@@ -622,16 +610,24 @@ __global__ void __launch_bounds__(kScanThreads) k_seed_scan(QueryBufs b, QueryAr
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
         best = v < best ? v : best;
     }
-    if (lane_id() == 0) wbest[threadIdx.x >> 5] = best;
+    if (lane_id() == 0) {
+        wbest[threadIdx.x >> 5] = best;
+        if ((threadIdx.x >> 5) < kScanConsumers)
+            b.st->warp_best[blockIdx.x * kScanConsumers + (threadIdx.x >> 5)] = best;
+    }
     __shared__ int last, wcnt[kScanConsumers + 2], total;
     // (every copy into the stages has landed unless a wait ran out)
     const bool all_ok = __syncthreads_and(piped);
+    const bool lists = exact_seeds(a);
     if (threadIdx.x == 0) {
         for (int w = 1; w < (int)(blockDim.x >> 5); ++w) best = wbest[w] < best ? wbest[w] : best;
-        b.st->cta_best[blockIdx.x] = best;
-        __threadfence();
-        last = atomicAdd(&b.st->prop_done, 1u) == gridDim.x - 1;
+        if (lists) {
+            b.st->cta_best[blockIdx.x] = best;
+            __threadfence();
+            last = atomicAdd(&b.st->prop_done, 1u) == gridDim.x - 1;
+        }
     }
+    if (!lists) return;
     __syncthreads();
     if (!last || !all_ok) return;  // (a timed-out query ends with an error)
     __threadfence();
@@ -644,41 +640,38 @@ __global__ void __launch_bounds__(kScanThreads) k_seed_scan(QueryBufs b, QueryAr
     __syncthreads();
     prop_rank_select(b.st, keys, n, threadIdx.x, blockDim.x, proposals);
     __syncthreads();
-    seed_lists(b, a, n_random, proposals, H, rng, reinterpret_cast<unsigned *>(spare), wcnt, &total);
+    seed_lists(b, a, n_random, proposals, -1, rng, reinterpret_cast<unsigned *>(spare), wcnt, &total);
 }
 
 template <int TERMS>
-static cudaError_t launch_seed_scan_t(const QueryBufs &b, const QueryArgs &a, int proposals, int n_random, int H,
+static cudaError_t launch_seed_scan_t(const QueryBufs &b, const QueryArgs &a, int proposals, int n_random,
                                       unsigned long long rng, int *ctas, cudaStream_t s) {
     size_t smem = 0;
     const int stages = scan_stages((const void *)k_seed_scan<TERMS>, stage_bytes<ProxyLayout>(a.m), 2, &smem);
     // the last CTA's keys and candidates fit in the data part of stage 0
-    const size_t tail = (size_t)(kCtaSlots + 8) * 8 > (size_t)(n_random + proposals * (2 * H + 1)) * 4
-                            ? (size_t)(kCtaSlots + 8) * 8
-                            : (size_t)(n_random + proposals * (2 * H + 1)) * 4;
+    const size_t tail = (size_t)(kCtaSlots + 8) * 8;  // (more than n_random + proposals offsets)
     if (stage_bytes<ProxyLayout>(a.m) < kStageHeader + tail) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k_seed_scan<TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (a.N + ProxyLayout::W - 1) / ProxyLayout::W;
     int grid = scan_grid((const void *)k_seed_scan<TERMS>, kScanThreads, smem, b.num_sms, tiles);
     if (grid > kCtaSlots) grid = kCtaSlots;
-    k_seed_scan<TERMS><<<grid, kScanThreads, smem, s>>>(b, a, proposals, stages, n_random, H, rng);
+    k_seed_scan<TERMS><<<grid, kScanThreads, smem, s>>>(b, a, proposals, stages, n_random, rng);
     *ctas = grid;
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_scan(const QueryBufs &b, const QueryArgs &a, int proposals, int terms, int n_random, int H,
+cudaError_t launch_seed_scan(const QueryBufs &b, const QueryArgs &a, int proposals, int terms, int n_random,
                              unsigned long long rng, int *ctas, cudaStream_t s) {
     *ctas = 0;
-    if (proposals <= 0 || proposals > kPropMax || n_random + proposals * (2 * H + 1) > kEdMax)
-        return cudaErrorInvalidValue;
+    if (proposals <= 0 || proposals > kPropMax || n_random > kKMax) return cudaErrorInvalidValue;
     // evenly spaced positions at multiples of 2 * kProxyStride, so at most
     // m / (2 * kProxyStride) distinct terms
     constexpr int g = 2 * kProxyStride;
-    if (terms >= 16 && a.m >= 16 * g) return launch_seed_scan_t<16>(b, a, proposals, n_random, H, rng, ctas, s);
-    if (terms >= 8 && a.m >= 8 * g) return launch_seed_scan_t<8>(b, a, proposals, n_random, H, rng, ctas, s);
-    if (terms >= 4 && a.m >= 4 * g) return launch_seed_scan_t<4>(b, a, proposals, n_random, H, rng, ctas, s);
-    return launch_seed_scan_t<2>(b, a, proposals, n_random, H, rng, ctas, s);
+    if (terms >= 16 && a.m >= 16 * g) return launch_seed_scan_t<16>(b, a, proposals, n_random, rng, ctas, s);
+    if (terms >= 8 && a.m >= 8 * g) return launch_seed_scan_t<8>(b, a, proposals, n_random, rng, ctas, s);
+    if (terms >= 4 && a.m >= 4 * g) return launch_seed_scan_t<4>(b, a, proposals, n_random, rng, ctas, s);
+    return launch_seed_scan_t<2>(b, a, proposals, n_random, rng, ctas, s);
 }
 
 // The proposals: the `proposals` smallest of the per-CTA best windows of one
@@ -744,10 +737,10 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
 
 // Seed windows.  seed_off (exact DTW seeds, used when k > 1): the random
 // windows (the paper's random first bsf, Algorithm 1) and the proposals.
-// ed_off (Euclidean seeds): the random windows and, for each proposal, the
-// 2 * kProxyHalf + 1 windows centred on it, since the proxy scan looked at
-// every kProxyStride-th window only.  Both lists hold distinct offsets: a repeated seed
-// would fill two of the k slots with one window.
+// ed_off (Euclidean seeds of the learned scan, H >= 0): the random windows
+// and, for each proposal, the 2H + 1 windows centred on it.  Both lists hold
+// distinct offsets: a repeated seed would fill two of the k slots with one
+// window.
 // Append the distinct values of src[0..n) (0xffffffff: none) to dst after
 // its first `start` entries, in first-occurrence order, up to cap entries in
 // all; returns the count.  Every thread of
@@ -799,7 +792,7 @@ __device__ int distinct_append(unsigned *dst, int cap, const unsigned *src, int 
     return *total < cap ? *total : cap;
 }
 
-// cand: room for n_random + proposals * (2H + 1) offsets (16-byte aligned);
+// cand: room for n_random + proposals * max(2H + 1, 1) offsets (16-byte aligned);
 // wcnt: one int per warp of the block and one more.
 __device__ void seed_lists(const QueryBufs &b, const QueryArgs &a, int n_random, int proposals, int H,
                            unsigned long long rng, unsigned *cand, int *wcnt, int *total_p) {
@@ -813,24 +806,25 @@ __device__ void seed_lists(const QueryBufs &b, const QueryArgs &a, int n_random,
     }
     __syncthreads();
     const int ns = distinct_append(b.st->seed_off, kSeedMax, cand, n_random + proposals, 0, wcnt, &total);
-    // Euclidean seeds: random windows + neighbourhoods of the proposals
-    const int span = 2 * H + 1;
-    for (int e = threadIdx.x; e < proposals * span; e += blockDim.x) {
-        const int p = e / span, d = e - p * span - H;
-        const unsigned long long key = b.st->prop_keys[p];
-        unsigned o = 0xffffffffu;
-        if (key != kEmptyKey) {
-            const long long v = (long long)key_idx(key) + d;
-            if (v >= 0 && v < a.N) o = (unsigned)v;
+    int ne = 0;
+    if (H >= 0) {
+        // Euclidean seeds: random windows + neighbourhoods of the proposals
+        const int span = 2 * H + 1;
+        for (int e = threadIdx.x; e < proposals * span; e += blockDim.x) {
+            const int p = e / span, d = e - p * span - H;
+            const unsigned long long key = b.st->prop_keys[p];
+            unsigned o = 0xffffffffu;
+            if (key != kEmptyKey) {
+                const long long v = (long long)key_idx(key) + d;
+                if (v >= 0 && v < a.N) o = (unsigned)v;
+            }
+            cand[n_random + e] = o;
         }
-        cand[n_random + e] = o;
+        __syncthreads();
+        ne = distinct_append(b.st->ed_off, kEdMax, cand, n_random + proposals * span, 0, wcnt, &total);
     }
-    __syncthreads();
-    const int ne = distinct_append(b.st->ed_off, kEdMax, cand, n_random + proposals * span, 0, wcnt, &total);
     if (threadIdx.x == 0) {
-        // exact seeds only pay off for k > 1, and not with a wide exclusion
-        // zone (no seed pass runs then, so the survivor pass must not skip them)
-        b.st->n_seeds = (a.k > 1 && a.xz_z == 0) ? ns : 0;
+        b.st->n_seeds = exact_seeds(a) ? ns : 0;
         b.st->n_ed = ne;
         b.st->work = 0;
     }
@@ -844,30 +838,113 @@ __global__ void __launch_bounds__(1024) k_seed_gather(QueryBufs b, QueryArgs a, 
     seed_lists(b, a, n_random, proposals, H, rng, cand, wcnt, &total);
 }
 
-// Squared Euclidean distance of the normalised query and window (the
-// diagonal warping path, so an upper bound of the banded DTW, Eq. 4) for
-// every Euclidean seed, one warp each; the k smallest go to ed_keys.
-__global__ void k_seed_ed(QueryBufs b, QueryArgs a) {
+// Squared Euclidean distances of the normalised query and windows (the
+// diagonal warping path, so upper bounds of the banded DTW, Eq. 4); the k
+// smallest go to ed_keys.  Without lists (slots > 0), after the proxy scan: one
+// warp per warp of that scan takes the 2 * kProxyHalf + 1 windows centred on
+// that warp's best (the scan looked at every kProxyStride-th window only), one
+// more warp each random window.  Every warp's best, not the 16 best CTAs': a
+// match that the proxy ranks below a few lucky random windows is then still
+// found, as long as it is the best of its own warp's share -- on 1e6 windows,
+// m = 128, the 16 best missed it for two queries of six, which left 1.6e5 to
+// 3.3e5 survivors and took 250 us instead of 75, and on 1e8 windows, m = 512,
+// one query in six met it in 3 % of its runs -- and no list has to be made; the
+// windows of a warp share their samples.  With lists (the learned scan) one
+// warp per entry of ed_off.  An offset scored twice has the same key and
+// occupies one slot.
+__device__ __forceinline__ unsigned long long splitmix64(unsigned long long z);
+constexpr int kEdWarps = 16;  // warps of a block
+__global__ void __launch_bounds__(kEdWarps * 32) k_seed_ed(QueryBufs b, QueryArgs a, int slots, int n_random,
+                                                           unsigned long long rng) {
+    __shared__ unsigned long long wkey[kEdWarps];
     QueryState *st = b.st;
     if (!st->valid) return;
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = lane_id();
-    if (w >= st->n_ed) return;
-    const unsigned idx = st->ed_off[w];
-    const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
-    const float *xw = b.x + idx;
-    float acc = 0.0f;
-    for (int j = lane; j < a.m; j += 32) {
-        const float d = b.qh32[j] - fmaf(xw[j] - mh, is, -ls);
-        acc = fmaf(d, d, acc);
+    constexpr int kW = 2 * kProxyHalf + 1;
+    const int lane = lane_id(), warp = threadIdx.x >> 5, w = blockIdx.x * kEdWarps + warp;
+    long long first = -1;  // the warp's windows: first .. first + nw - 1
+    int nw = 0;
+    if (slots > 0) {
+        if (w < slots) {
+            const unsigned long long key = st->warp_best[w];
+            if (key != kEmptyKey) {
+                const long long c = key_idx(key), lo = c - kProxyHalf > 0 ? c - kProxyHalf : 0;
+                const long long hi = c + kProxyHalf < a.N - 1 ? c + kProxyHalf : a.N - 1;
+                first = lo;
+                nw = (int)(hi - lo) + 1;
+            }
+        } else if (w < slots + n_random) {
+            first = (long long)(splitmix64(rng + (unsigned long long)(w - slots)) % (unsigned long long)a.N);
+            nw = 1;
+        }
+    } else if (w < st->n_ed) {
+        first = st->ed_off[w];
+        nw = 1;
     }
+    unsigned long long key = kEmptyKey;  // lane d: window first + d
+    if (nw > 0) {
+        float acc[kW], mh[kW], is[kW], ls[kW];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-        const unsigned long long key = make_key(key_quantize(acc, a.qgrid), idx);
-        list_insert(st->ed_keys, a.k, key);
-        // the Euclidean distance bounds the window's DTW from above, so it
-        // may stand for the window in a bucket list (never in the buffer)
-        if (a.xz_z > 0) xz_offer(b, a, key, false);
+        for (int d = 0; d < kW; ++d) {
+            const long long i = first + (d < nw ? d : 0);
+            mh[d] = b.mu_hi[i];
+            is[d] = b.inv_sigma[i];
+            ls[d] = b.mu_lo[i] * is[d];
+            acc[d] = 0.0f;
+        }
+        const float *xw = b.x + first;  // (reads stay inside the padded series)
+        if (nw == 1) {
+            for (int j = lane; j < a.m; j += 32) {
+                const float d = b.qh32[j] - fmaf(xw[j] - mh[0], is[0], -ls[0]);
+                acc[0] = fmaf(d, d, acc[0]);
+            }
+        } else {
+            for (int j = lane; j < a.m; j += 32) {
+                const float q = b.qh32[j];
+#pragma unroll
+                for (int d = 0; d < kW; ++d) {
+                    const float v = q - fmaf(xw[j + d] - mh[d], is[d], -ls[d]);
+                    acc[d] = fmaf(v, v, acc[d]);
+                }
+            }
+        }
+        float mine = 0.0f;
+#pragma unroll
+        for (int d = 0; d < kW; ++d) {
+            if (d > 0 && nw == 1) break;
+            float v = acc[d];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == d) mine = v;
+        }
+        if (lane < nw) key = make_key(key_quantize(mine, a.qgrid), (unsigned)first + lane);
+    }
+    if (slots <= 0) {  // a list: every entry counts
+        if (lane == 0 && nw > 0) {
+            list_insert(st->ed_keys, a.k, key);
+            // the Euclidean distance bounds the window's DTW from above, so
+            // it may stand for the window in a bucket list (never in the
+            // buffer)
+            if (a.xz_z > 0) xz_offer(b, a, key, false);
+        }
+        return;
+    }
+    // thousands of scan warps: the block's best alone is inserted, and for k > 1
+    // only the two best matter (their neighbours join as exact-DTW seeds,
+    // k_seed_expand, which bound the k-th distance).  (Inserting every window
+    // queued on the list's words: 56 us more at k = 10.)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, key, o);
+        key = v < key ? v : key;
+    }
+    if (lane == 0) wkey[warp] = key;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int u = 1; u < kEdWarps; ++u) key = wkey[u] < key ? wkey[u] : key;
+        if (key != kEmptyKey) {
+            list_insert(st->ed_keys, exact_seeds(a) ? 2 : a.k, key);
+            if (a.xz_z > 0) xz_offer(b, a, key, false);
+        }
     }
 }
 
@@ -908,11 +985,15 @@ cudaError_t launch_seed_expand(const QueryBufs &b, const QueryArgs &a, cudaStrea
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_ed(const QueryBufs &b, const QueryArgs &a, int max_seeds, cudaStream_t s) {
-    // one warp per seed, for at most max_seeds seeds (the lists' bound)
-    if (max_seeds < 1) max_seeds = 1;
-    if (max_seeds > kEdMax) max_seeds = kEdMax;
-    k_seed_ed<<<(max_seeds * 32 + 255) / 256, 256, 0, s>>>(b, a);
+cudaError_t launch_seed_ed(const QueryBufs &b, const QueryArgs &a, int ctas, int n_random, unsigned long long rng,
+                           int max_seeds, cudaStream_t s) {
+    // one warp per warp of the proxy scan and random window, or per list entry
+    // (for at most max_seeds, the list's bound)
+    const int slots = ctas * kScanConsumers;
+    int warps = slots > 0 ? slots + n_random : max_seeds;
+    if (warps < 1) warps = 1;
+    if (slots <= 0 && warps > kEdMax) warps = kEdMax;
+    k_seed_ed<<<(warps + kEdWarps - 1) / kEdWarps, kEdWarps * 32, 0, s>>>(b, a, slots, n_random, rng);
     return cudaGetLastError();
 }
 
@@ -1371,13 +1452,10 @@ cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int6
 // normalised with the window's statistics: looser than the window-clipped
 // envelope, still admissible), is evaluated for each survivor by the DTW
 // kernel, whose tail bound consists of exactly its per-row terms.
-// LB_Keogh (Eq. 8) chunks of 32 terms the scan takes at most per window; the
-// first kEqSmem of them come from shared memory, any further ones through L1
-// (the same few values for every window).  Measured: 8 chunks moved work
-// from the survivor stage into the scan (whose warp holds all 32 lanes per
-// passing window) and slowed the m = 512 workload by 7 %, so the scan stops
-// after 2 and the survivor stage's pre-check takes over.
-constexpr int kEqChunks = 2, kEqSmem = 2;
+static_assert(kScanTerms == 64 && kScanTerms <= kTerms, "two of the scan's terms per lane in registers");
+constexpr int kLaneRow = 4;     // passers in a row of 32 from which each lane first takes kLaneFirst terms
+constexpr int kLaneFirst = 8;
+constexpr int kLaneEqMin = 16;  // windows left after them from which the lanes go on
 
 // The lower-bound scan normalises with the mean's high part alone: the
 // window's values then sit shifted by mu_lo / sigma, and |mu_lo| <= ulp(mu_hi)
@@ -1402,80 +1480,83 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// The ordered query terms the scan takes: in shared memory for the lane-wise
+// form, and each lane's own first two (terms lane and 32 + lane) in registers
+// for the warp-wise one.  nt of them; past nt an envelope that every value
+// lies in.
+struct EqTerms {
+    const int *o;
+    const float *u, *l;
+    int nt, o0, o1;
+    float u0, l0, u1, l1;
+};
+
 // Each warp scans 32 windows at a time with LB_KimFL (one window per lane);
-// the rare windows that pass are then bounded by the whole warp, one at a
-// time: lanes take 32 consecutive terms of the |q_hat|-ordered LB_Keogh sums
-// and the warp abandons as soon as a chunk's running total exceeds thr.  No
-// thread waits on another warp's survivors.
-// The rare part of a row of 32 windows (entered only when some window
-// passed LB_KimFL): the windows that passed (bal) are bounded by
-// LB_Keogh of the window against the query envelope (Eq. 8) over the
-// kEqChunks * 32 largest-|q_hat| terms, and the survivors are appended as
-// (bound, offset) by one warp-aggregated atomic.  A dense row (a loose
-// bound) gives each passing lane its own window's terms; otherwise the warp
-// takes one window at a time, 32 terms per step.  Returns the survivors.
-// (Eq. 10's first 32 terms here as well, for each window past Eq. 8, halved
-// the survivors on 1e8 windows, m = 512 -- 38,000 to 21,000, the survivor
-// pass 55 -> 43 us -- but slowed the scan 278 -> 300 us: the random loads of
-// the series envelope stall the warps that feed the ring.)
-__device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, QueryState *st, const int *o_s,
-                                         const float *u_s, const float *l_s, int m, float thr, unsigned bal,
-                                         int wrow, int lane, float kim, float mh, float is, float sd, int64_t i0) {
+// this is the rare part of such a row, entered only when some window passed
+// (bal): LB_KimFL plus the LB_Keogh terms of the window against the query
+// envelope (Eq. 8) at the first kScanTerms ordered positions.  The sum is
+// a lower bound: LB_KimFL is the cost of the path's first and last cells, in
+// columns 0 and m-1, the terms bound the cells of other columns.  Survivors
+// are appended as (bound, offset) by one warp-aggregated atomic; their number
+// is returned.  A row with several passers first gives each lane kLaneFirst
+// terms of its own window; what is left is taken one window at a time, 32
+// terms per step, where a single term above what is left of thr already
+// prunes (a vote), or lane by lane to the end where most of the row is left
+// (a loose bound).  No thread waits on another warp's survivors.
+// Measured (1e8 windows, m = 512, five queries, 0.2 to 5.8e6 past LB_KimFL):
+// 231 to 384 us, 0.29 ms on average; one 32-term shuffle sum per window in
+// |q_hat| order 233 to 641 us, 0.44 ms.
+// (Eq. 10's first 32 terms here as well, for each window past Eq. 8, slowed
+// the scan more than it saved: the random loads of the series envelope stall
+// the warps that feed the ring.  128 terms instead of 64: scan +90 us,
+// survivor pass -37 us.)
+__device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, QueryState *st, const EqTerms &e,
+                                            float thr, unsigned bal, int wrow, int lane, float kim, int64_t i0) {
     const int w = wrow + lane;
-    unsigned keep = 0;   // windows of this row that survive Eq. 8
-    float my_lb = 0.0f;  // lane t holds window t's bound when it survives
-    if (__popc(bal) >= kLaneEqMin) {
-        // the same terms in the same |q_hat| order, each lane abandoning once
-        // its sum exceeds thr (checked every 8 terms): 32 windows per step
-        // instead of one window and a shuffle reduction per chunk
-        const int nt = m < kEqChunks * 32 ? m : kEqChunks * 32;
-        float s2 = 0.0f;
+    unsigned keep = 0;  // windows of this row that survive Eq. 8
+    float my_lb = kim;  // the lane's window: its bound so far
+    if (__popc(bal) >= kLaneRow) {
+        const float mh = t.mh[w], is = t.is[w], sd = shift_bound(mh, is);
         bool alive = (bal >> lane) & 1u;
-        for (int j0 = 0; j0 < nt; j0 += 8) {
-            if (!__any_sync(0xffffffffu, alive)) break;
-            if (alive) {
+        float s2 = kim;
 #pragma unroll
-                for (int v = 0; v < 8; ++v) {
-                    const int j = j0 + v;
-                    if (j < nt) {
-                        const bool sm = j < kEqSmem * 32;
-                        const int o = sm ? o_s[j] : (int)__ldg(b.ord + j);
-                        const float uq = sm ? u_s[j] : __ldg(b.sU + j), lq = sm ? l_s[j] : __ldg(b.sL + j);
-                        s2 += keogh_term((t.xs[w + o] - mh) * is, uq + sd, lq - sd);
-                    }
+        for (int j = 0; j < kLaneFirst; ++j)
+            s2 += keogh_term((t.xs[w + e.o[j]] - mh) * is, e.u[j] + sd, e.l[j] - sd);
+        alive = alive && !(s2 > thr);
+        bal = __ballot_sync(0xffffffffu, alive);
+        if (__popc(bal) >= kLaneEqMin) {
+            for (int j0 = kLaneFirst; j0 < e.nt; j0 += kLaneFirst) {
+                if (!__any_sync(0xffffffffu, alive)) break;
+                if (alive) {
+#pragma unroll
+                    for (int v = 0; v < kLaneFirst; ++v)
+                        s2 += keogh_term((t.xs[w + e.o[j0 + v]] - mh) * is, e.u[j0 + v] + sd, e.l[j0 + v] - sd);
+                    alive = !(s2 > thr);
                 }
-                alive = !(s2 > thr);
             }
+            keep = __ballot_sync(0xffffffffu, alive);
+            my_lb = s2;
+            bal = 0;
         }
-        keep = __ballot_sync(0xffffffffu, alive);
-        my_lb = fmaxf(kim, s2);
-    } else {
-        while (bal) {
-            const int src = __ffs(bal) - 1;
-            bal &= bal - 1;
-            const int ws = wrow + src;
-            const float smh = t.mh[ws], sis = t.is[ws], ssd = shift_bound(smh, sis);
-            const float *xw = t.xs + ws;
-            // a window that survives these chunks (the neighbourhood of a
-            // match) goes to the DTW stage with the partial sum, itself a
-            // lower bound, rather than holding this warp for the full sum
-            float s2 = 0.0f;
-            for (int base = 0; base < m && base < kEqChunks * 32; base += 32) {
-                const int j = base + lane;
-                float term = 0.0f;
-                if (j < m) {
-                    const bool sm = base < kEqSmem * 32;
-                    const int o = sm ? o_s[j] : (int)__ldg(b.ord + j);
-                    const float uq = sm ? u_s[j] : __ldg(b.sU + j), lq = sm ? l_s[j] : __ldg(b.sL + j);
-                    term = keogh_term((xw[o] - smh) * sis, uq + ssd, lq - ssd);
-                }
-                s2 += warp_sum(term);
-                if (s2 > thr) break;
-            }
-            if (s2 > thr) continue;
-            keep |= 1u << src;
-            if (lane == src) my_lb = fmaxf(kim, s2);
-        }
+    }
+    while (bal) {
+        const int src = __ffs(bal) - 1;
+        bal &= bal - 1;
+        const int ws = wrow + src;
+        const float smh = t.mh[ws], sis = t.is[ws], ssd = shift_bound(smh, sis);
+        const float left = thr - __shfl_sync(0xffffffffu, kim, src);
+        const float *xw = t.xs + ws;
+        // a window that survives these steps (the neighbourhood of a match)
+        // goes to the DTW stage with the partial sum, itself a lower bound,
+        // rather than holding this warp for the full sum
+        const float t0 = keogh_term((xw[e.o0] - smh) * sis, e.u0 + ssd, e.l0 - ssd);
+        if (__any_sync(0xffffffffu, t0 > left)) continue;
+        const float t1 = keogh_term((xw[e.o1] - smh) * sis, e.u1 + ssd, e.l1 - ssd);
+        if (__any_sync(0xffffffffu, t0 + t1 > left)) continue;
+        const float s2 = warp_sum(t0 + t1);
+        if (s2 > left) continue;
+        keep |= 1u << src;
+        if (lane == src) my_lb = kim + s2;
     }
     // one append per row of 32 windows: a warp-aggregated atomic
     if (keep) {
@@ -1503,13 +1584,16 @@ __global__ void __launch_bounds__(kScanThreads, 5) k_lb_scan(QueryBufs b, QueryA
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     constexpr int kPerWarp = TW / kScanConsumers;
     // the ordered query terms the scan uses, in shared memory
-    __shared__ int o_s[kEqSmem * 32];
-    __shared__ float u_s[kEqSmem * 32], l_s[kEqSmem * 32];
-    for (int j = threadIdx.x; j < kEqSmem * 32; j += blockDim.x) {
-        o_s[j] = j < m ? (int)b.ord[j] : 0;
-        u_s[j] = j < m ? b.sU[j] : 0.0f;
-        l_s[j] = j < m ? b.sL[j] : 0.0f;
+    __shared__ int o_s[kScanTerms];
+    __shared__ float u_s[kScanTerms], l_s[kScanTerms];
+    const int nt = terms_of(m) < kScanTerms ? terms_of(m) : kScanTerms;
+    for (int j = threadIdx.x; j < kScanTerms; j += blockDim.x) {
+        o_s[j] = j < nt ? (int)b.ord[j] : 0;
+        u_s[j] = j < nt ? b.sU[j] : DINF;
+        l_s[j] = j < nt ? b.sL[j] : -DINF;
     }
+    __syncthreads();
+    const EqTerms eq{o_s, u_s, l_s, nt, o_s[lane], o_s[32 + lane], u_s[lane], l_s[lane], u_s[32 + lane], l_s[32 + lane]};
     unsigned c1 = 0, c2 = 0;  // (per lane: at most the windows its warp scans)
     const int64_t ntiles = (a.N + TW - 1) / TW;
     tile_pipeline<LbLayout<TW>>(smraw, b, m, ntiles, &st->tile_ctr[1], stages, [&](const Tile &t, int64_t i0) {
@@ -1561,9 +1645,7 @@ __global__ void __launch_bounds__(kScanThreads, 5) k_lb_scan(QueryBufs b, QueryA
                 });
                 if (!bu) continue;
                 const int w = (int)w0 + u * 32;
-                const float mh = t.mh[w], is = t.is[w];
-                c2 += lb_row_keogh(t, b, st, o_s, u_s, l_s, m, thr, bu, w - lane, lane, ku, mh, is,
-                                   shift_bound(mh, is), i0);
+                c2 += lb_row_keogh(t, b, st, eq, thr, bu, w - lane, lane, ku, i0);
             }
         }
     });
