@@ -360,17 +360,65 @@ __device__ __forceinline__ float diag_result(const float (&p1)[K], int lane, int
     return res;
 }
 
+// ------------------------------------------------------------------ corner bound
+// A lower bound of the banded DTW from its two corners: every path crosses
+// anti-diagonal kCorner-2 or kCorner-1, so the smallest d over their cells
+// bounds the cost of the path's cells up to there, and the same from the far
+// end; the two corners share no cell when m > kCorner.  One warp, lane i row i
+// (and row m-1-i) of the corner, both corners side by side: 32 steps of two
+// exchanges each, ~0.6 us, with no staging, no envelope and no barrier.  It is
+// what tells windows apart where the band is so wide that LB_Keogh is flat:
+// at m = 1024, r = 921 the full walk of a survivor ended after ~36
+// anti-diagonals but cost 10 us per candidate and group to set up.
+// qs: q_hat; xw: the window's raw samples.  Every lane returns the bound;
+// *back (if given) is the far corner's share.
+constexpr int kCorner = 32;
+__device__ __forceinline__ bool corner_applies(int m) { return m > 2 * kCorner; }
+__device__ __forceinline__ float corner_bound(const float *__restrict__ qs, const float *__restrict__ xw, float mh,
+                                              float is, float ls, int m, int r, int lane, float *back) {
+    const float INF = __int_as_float(0x7f800000);
+    const float qf = qs[lane], qb = qs[m - 1 - lane];
+    const float cf = fmaf(xw[lane] - mh, is, -ls), cb = fmaf(xw[m - 1 - lane] - mh, is, -ls);
+    // own cells of the previous anti-diagonal, and the row above's of the two
+    // before (base: the cell before the corner costs nothing)
+    float pf = INF, pb = INF, df = lane == 0 ? 0.0f : INF, db = df, lf = INF, lb = INF;
+#pragma unroll
+    for (int a = 0; a < kCorner; ++a) {
+        const int src = (a - lane) & 31, e = 2 * lane - a;
+        const float xf = __shfl_sync(0xffffffffu, cf, src), xb = __shfl_sync(0xffffffffu, cb, src);
+        float uf = __shfl_up_sync(0xffffffffu, pf, 1), ub = __shfl_up_sync(0xffffffffu, pb, 1);
+        if (lane == 0) uf = ub = INF;
+        const bool in = lane <= a && e <= r && -e <= r;
+        const float vf = fmaf(qf - xf, qf - xf, fminf(fminf(pf, df), uf));
+        const float vb = fmaf(qb - xb, qb - xb, fminf(fminf(pb, db), ub));
+        df = uf;
+        db = ub;
+        pf = in ? vf : INF;
+        pb = in ? vb : INF;
+        if (a >= kCorner - 2) {
+            lf = fminf(lf, pf);
+            lb = fminf(lb, pb);
+        }
+    }
+    // (costs are not negative: their bit patterns order like their values)
+    const float f = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lf)));
+    const float g = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lb)));
+    if (back) *back = g;
+    return f + g;
+}
+
 // qp, cp: the query and the group's normalised window, each padded by
 // diag_pad(r, L, K) elements (+inf / -inf) on both sides, pointing at
 // element 0.  cbs: the rows' coarse tail bound for ABANDON (or nullptr):
 // cbs[g] bounds the cost of the rows kTailG*g .. m-1 from below, so the
 // rows after row i are bounded by cbs[ceil((i+1)/kTailG)] (fewer rows, a
-// smaller sum).  cells: lane 0 accumulates the cells evaluated (in the band
-// and the matrix).  The walk takes diag_unroll(K) anti-diagonal pairs per
+// smaller sum).  back: a lower bound of the cost of the path's cells on the
+// last kCorner anti-diagonals (corner_bound), 0 if unknown.  cells: lane 0
+// accumulates the cells evaluated (in the band and the matrix).  The walk takes diag_unroll(K) anti-diagonal pairs per
 // iteration; the abandon test runs once per iteration.
 template <typename T, int L, int K, bool ABANDON>
-__device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const float *cbs, int m, int r, T thr,
-                      unsigned gmask, int lane, int &cells) {
+__device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const float *cbs, float back, int m, int r,
+                      T thr, unsigned gmask, int lane, int &cells) {
     static_assert(sizeof(T) == 4, "the FP32 walk");
     constexpr int U = diag_unroll(K);
     const float INF = __int_as_float(0x7f800000);
@@ -422,12 +470,14 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
         bj += U;
         if (ABANDON) {
             // p1: anti-diagonal a-1, p2: a-2, both on rows bi - 1 - p
+            // (the cells still ahead include the far corner's)
+            const float rest = a <= last - kCorner ? back : 0.0f;
             float low = INF;
 #pragma unroll
             for (int t = 0; t < K; ++t) {
                 const int i = bi - 1 - (lane * K + t);
                 const float tail = (cbs && i >= 0 && i < m) ? cbs[(i + kTailG) / kTailG] : 0.0f;
-                low = fminf(low, fminf(p1[t], p2[t]) + tail);
+                low = fminf(low, fminf(p1[t], p2[t]) + fmaxf(tail, rest));
             }
 #pragma unroll
             for (int o = L / 2; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(gmask, low, o, L));
@@ -549,13 +599,13 @@ __device__ __forceinline__ void shift_q_mw(float (&qv)[K], const float *qp, int 
 
 // qp, cp: element 0 of the query / the group's normalised window, padded by
 // diag_pad(r, 32*W, K) on both sides (+inf / -inf); cbs: the coarse tail
-// bound (as dtw_diag) or nullptr.  Called by all 32 W threads of warps
+// bound and back (as dtw_diag) or nullptr and 0.  Called by all 32 W threads of warps
 // w = 0..W-1 of the group; bar: the group's named barrier.  Every thread
 // returns the distance (+inf when abandoned); thread 0 of the group adds the
 // cells evaluated to `cells`.
 template <int W, int K, bool ABANDON>
-__device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restrict__ cp, const float *cbs, int m,
-                             int r, float thr, int w, int lane, MwXchg &x, int bar, int &cells) {
+__device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restrict__ cp, const float *cbs, float back,
+                             int m, int r, float thr, int w, int lane, MwXchg &x, int bar, int &cells) {
     static_assert(W >= 2 && W <= 8, "two to eight warps");
     constexpr int U = diag_unroll(K);
     const float INF = __int_as_float(0x7f800000);
@@ -607,12 +657,13 @@ __device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restri
         bi += U;
         bj += U;
         if (ABANDON) {
+            const float rest = a <= last - kCorner ? back : 0.0f;  // (as in dtw_diag)
             float low = INF;
 #pragma unroll
             for (int t = 0; t < K; ++t) {
                 const int i = bi - 1 - (gl * K + t);
                 const float tail = (cbs && i >= 0 && i < m) ? cbs[(i + kTailG) / kTailG] : 0.0f;
-                low = fminf(low, fminf(p1[t], p2[t]) + tail);
+                low = fminf(low, fminf(p1[t], p2[t]) + fmaxf(tail, rest));
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));

@@ -386,6 +386,11 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
             }
             if (pruned) continue;
         }
+        float back = 0.0f;
+        if constexpr (MODE == kModeSurv && L == 32 && K > 0) {
+            // the corners' bound, before the window is staged
+            if (corner_applies(m) && corner_bound(qs, xw, mh, is, ls, m, r, lane, &back) > thr) continue;
+        }
         if (cbuf) {  // the group's normalised copy of the window
             for (int j = lane; j < m; j += L) cbuf[j] = fmaf(xw[j] - mh, is, -ls);
         }
@@ -409,9 +414,9 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                                              gmask, lane, cells);
         } else {
             if (MODE == kModeOut)
-                d = dtw_diag<float, L, K, false>(qs, cbuf, nullptr, m, r, thr, gmask, lane, cells);
+                d = dtw_diag<float, L, K, false>(qs, cbuf, nullptr, 0.0f, m, r, thr, gmask, lane, cells);
             else
-                d = dtw_diag<float, L, K, true>(qs, cbuf, cbs, m, r, thr, gmask, lane, cells);
+                d = dtw_diag<float, L, K, true>(qs, cbuf, cbs, back, m, r, thr, gmask, lane, cells);
         }
         cells_acc += cells;
         if (lane == 0) {
@@ -674,6 +679,56 @@ __host__ __device__ inline size_t wide_span(int m, int r, int K) {
 }
 __host__ __device__ inline size_t wide_tail(int m) { return (size_t)((tail_entries(m) + 3) & ~3); }
 
+// One warp's bounds of a survivor that need no staging: Eq. 10 and Eq. 8 over
+// the ordered terms (32 per step; the scan took the first kScanTerms of Eq. 8,
+// which are in lb), then the corners.  True: the window is out.
+constexpr int kWideTries = 8;  // candidates a warp looks at before the group meets
+__device__ __forceinline__ bool wide_prune(const QueryBufs &b, const float *qs, unsigned idx, float lb, float thr, int m,
+                                           int r, int lane, const int *ord_s, const float *sq_s, const float *su_s,
+                                           const float *sl_s, bool has_env, float *back) {
+    const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
+    const float *xw = b.x + idx;
+    if (corner_applies(m) && corner_bound(qs, xw, mh, is, ls, m, r, lane, back) > thr) return true;
+    if (!has_env) return false;
+    TailCtx tc;
+    tc.Uw = b.U ? b.U + idx : nullptr;
+    tc.Lw = b.L ? b.L + idx : nullptr;
+    tc.stmax = b.stmax;
+    tc.stmin = b.stmin;
+    tc.nblk = b.nblk;
+    tc.n = b.n;
+    tc.t0 = idx;
+    tc.r = r;
+    float acc = 0.0f, acc8 = lb;
+    for (int c0 = 0; c0 < terms_of(m); c0 += 32) {
+        const int j = c0 + lane;
+        const bool eq8 = c0 >= kScanTerms;
+        float v = 0.0f, v8 = 0.0f;
+        if (j < terms_of(m)) {
+            const int pos = ord_s[j];
+            float U, Lo;
+            env_at(tc, pos, U, Lo);
+            const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
+            const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
+            v = dq * dq;
+            if (eq8) {
+                const float cv = fmaf(xw[pos] - mh, is, -ls);
+                const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
+                v8 = e * e;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (eq8) v8 += __shfl_xor_sync(0xffffffffu, v8, o);
+        }
+        acc += v;
+        acc8 += v8;
+        if (acc > thr || acc8 > thr) return true;
+    }
+    return false;
+}
+
 template <int W, int K, int MODE>
 __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, const int64_t *offsets,
                                                    int64_t count_host, float *out) {
@@ -682,6 +737,9 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
     __shared__ MwXchg xch[GMAX];
     __shared__ int cur_s[GMAX][2];
     __shared__ float thr_s[GMAX][2];
+    __shared__ unsigned found_s[GMAX][W];
+    __shared__ float fback_s[GMAX][W];
+    __shared__ bool dry_s[GMAX][W];
     __shared__ unsigned seeds_s[kSeedMax];
     __shared__ int n_seeds_s;
     __shared__ int ord_s[128];
@@ -724,47 +782,107 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
     long long cells_acc = 0;
     int started = 0, abandoned = 0, passed_s = 0;
     int cells = 0;
+    bool dry = false;  // survivor mode: this warp found the end of the list
+    int slot = W;      // ... and the slot of found_s the group takes next (W: all taken)
     for (int it = 0;; it ^= 1) {
-        // cur_s / thr_s alternate between two slots: a slot is written again
-        // only after the next iteration's barrier, which every thread of the
-        // group reaches after reading it
-        if (t == 0) {
-            cur_s[g][it] = atomicAdd(cursor, 1);
-            float th = DINF;
-            if (MODE == kModeSeed) {
-                const float kth = list_kth(st->seed_keys, a.k);
-                th = kth < DINF ? fmaf(kth, 1.0f + a.delta, a.alpha) : DINF;
-            } else if (MODE == kModeSurv) {
-                th = current_thr(st, a);
-            }
-            thr_s[g][it] = th;
-        }
-        group_bar(bar, nthr);
-        const int c = cur_s[g][it];
-        if (c >= count) break;
-        const float thr = thr_s[g][it];
         unsigned idx = 0;
-        float lb = 0.0f;
-        if (MODE == kModeSeed) {
-            idx = st->seed_off[c];
-        } else if (MODE == kModeOut) {
-            const int64_t o = offsets[c];
-            if (o < 0 || o >= a.N) {
-                if (t == 0) out[c] = __int_as_float(0x7fc00000);
+        int c = 0;
+        float thr, back = 0.0f;
+        if (MODE == kModeSurv) {
+            // Each warp looks for a candidate of its own that passes every
+            // bound that needs no staging (found_s); the group then walks
+            // them one after another.
+            if (slot == W) {
+                unsigned found = 0xffffffffu;
+                float fback = 0.0f;
+                for (int tries = 0; tries < kWideTries && !dry; ++tries) {
+                    int cc = 0;
+                    float th = 0.0f;
+                    if (lane == 0) {
+                        cc = atomicAdd(cursor, 1);
+                        th = current_thr(st, a);
+                    }
+                    cc = __shfl_sync(0xffffffffu, cc, 0);
+                    th = __shfl_sync(0xffffffffu, th, 0);
+                    if (cc >= count) {
+                        dry = true;
+                        break;
+                    }
+                    const unsigned id = b.sort_idx[cc];
+                    const float lb = b.sort_lb[cc];
+                    if (lb > th) {
+                        // survivors are in ascending bins and thr only shrinks
+                        dry = bin_floor(bin_of(lb, thr_scan), thr_scan) > th;
+                        continue;
+                    }
+                    bool seen = id == pre;  // scored already: by the seed pass or on the side stream
+                    for (int i = lane; i < n_seeds_s; i += 32) seen |= seeds_s[i] == id;
+                    if (__any_sync(0xffffffffu, seen)) continue;
+                    if (wide_prune(b, qs, id, lb, th, m, r, lane, ord_s, sq_s, su_s, sl_s, has_env, &fback)) continue;
+                    found = id;
+                    break;
+                }
+                // (the slots' last readers have passed the group's barriers
+                // of the walks since)
+                if (lane == 0) {
+                    found_s[g][w] = found;
+                    fback_s[g][w] = fback;
+                    dry_s[g][w] = dry;
+                }
+                slot = 0;
+                group_bar(bar, nthr);
+                bool all = true, any = false;
+#pragma unroll
+                for (int u = 0; u < W; ++u) {
+                    all = all && dry_s[g][u];
+                    any = any || found_s[g][u] != 0xffffffffu;
+                }
+                if (!any) {
+                    if (all) break;
+                    slot = W;
+                    group_bar(bar, nthr);  // (the slots are read before they are written again)
+                    continue;
+                }
+            }
+            while (slot < W && found_s[g][slot] == 0xffffffffu) ++slot;
+            if (slot == W) {
+                group_bar(bar, nthr);
                 continue;
             }
-            idx = (unsigned)o;
+            idx = found_s[g][slot];
+            back = fback_s[g][slot];
+            ++slot;
+            // the threshold may have fallen since: read once for the group
+            if (t == 0) thr_s[g][it] = current_thr(st, a);
+            group_bar(bar, nthr);
+            thr = thr_s[g][it];
         } else {
-            idx = b.sort_idx[c];
-            lb = b.sort_lb[c];
-            if (lb > thr) {
-                // survivors are in ascending bins and thr only shrinks
-                if (bin_floor(bin_of(lb, thr_scan), thr_scan) > thr) break;
-                continue;
+            // cur_s / thr_s alternate between two slots: a slot is written again
+            // only after the next iteration's barrier, which every thread of the
+            // group reaches after reading it
+            if (t == 0) {
+                cur_s[g][it] = atomicAdd(cursor, 1);
+                float th = DINF;
+                if (MODE == kModeSeed) {
+                    const float kth = list_kth(st->seed_keys, a.k);
+                    th = kth < DINF ? fmaf(kth, 1.0f + a.delta, a.alpha) : DINF;
+                }
+                thr_s[g][it] = th;
             }
-            bool seen = idx == pre;  // scored already: by the seed pass or on the side stream
-            for (int i = 0; i < n_seeds_s; ++i) seen |= seeds_s[i] == idx;
-            if (seen) continue;
+            group_bar(bar, nthr);
+            c = cur_s[g][it];
+            if (c >= count) break;
+            thr = thr_s[g][it];
+            if (MODE == kModeSeed) {
+                idx = st->seed_off[c];
+            } else {
+                const int64_t o = offsets[c];
+                if (o < 0 || o >= a.N) {
+                    if (t == 0) out[c] = __int_as_float(0x7fc00000);
+                    continue;
+                }
+                idx = (unsigned)o;
+            }
         }
         const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
         const float *xw = b.x + idx;
@@ -781,42 +899,6 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
         tc.mh = mh;
         tc.is = is;
         tc.ls = ls;
-        if (has_env) {
-            // Eq. 10 and Eq. 8 over the ordered terms (one pass:
-            // 128 threads, one term each), reduced over the group
-            const int budget = terms_of(m);
-            float v = 0.0f, v8 = 0.0f;
-            for (int j = t; j < budget; j += nthr) {
-                const int pos = ord_s[j];
-                float U, Lo;
-                env_at(tc, pos, U, Lo);
-                const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
-                const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
-                v = fmaf(dq, dq, v);
-                if (j >= kScanTerms) {  // (the scan took the others)
-                    const float cv = fmaf(xw[pos] - mh, is, -ls);
-                    const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                    v8 = fmaf(e, e, v8);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                v += __shfl_xor_sync(0xffffffffu, v, o);
-                v8 += __shfl_xor_sync(0xffffffffu, v8, o);
-            }
-            if (lane == 0) {
-                xch[g].red[0][w] = v;
-                xch[g].red[1][w] = v8;
-            }
-            group_bar(bar, nthr);
-            float acc = 0.0f, acc8 = lb;
-#pragma unroll
-            for (int u = 0; u < W; ++u) {
-                acc += xch[g].red[0][u];
-                acc8 += xch[g].red[1][u];
-            }
-            if (acc > thr || acc8 > thr) continue;
-        }
         for (int j = t; j < m; j += nthr) cd[j] = fmaf(xw[j] - mh, is, -ls);
         if (has_env) {
             // the coarse tail bound: kTailG-row sums, then a suffix scan by
@@ -853,7 +935,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
             if (cbs[0] > thr) continue;  // Eq. 10 over every row
             if (t == 0) ++passed_s;
         }
-        const float d = dtw_diag_mw<W, K, MODE != kModeOut>(qs, cd, has_env ? cbs : nullptr, m, r, thr, w, lane,
+        const float d = dtw_diag_mw<W, K, MODE != kModeOut>(qs, cd, has_env ? cbs : nullptr, back, m, r, thr, w, lane,
                                                             xch[g], bar, cells);
         if (t == 0) {
             ++started;

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(kFxThreads + 32) k_prescore_fx(QueryBufs b, Qu
         }
         __syncwarp();
         int cells = 0;
-        const float d32 = dtw_diag<float, 32, K, false>(q32 + pad, c32 + pad, nullptr, m, r, INF, 0xffffffffu, lane,
+        const float d32 = dtw_diag<float, 32, K, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, 0xffffffffu, lane,
                                                          cells);
         if (lane == 0) {
             const unsigned long long key = make_key(key_quantize(d32, a.qgrid), idx);
@@ -103,7 +103,7 @@ __global__ void k_prescore(QueryBufs b, QueryArgs a) {
         __syncwarp(gmask);
         int cells = 0;
         const float d32 =
-            dtw_diag<float, L, K, false>(q32 + pad, c32 + pad, nullptr, m, r, INF, gmask, lane, cells);
+            dtw_diag<float, L, K, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, gmask, lane, cells);
         if (lane == 0) {
             const unsigned long long key = make_key(key_quantize(d32, a.qgrid), idx);
             list_insert(st->res_keys, a.list_cap, key);

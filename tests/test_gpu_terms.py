@@ -62,3 +62,21 @@ def test_seeds_from_few_and_ragged_tiles(n, m):
         assert idx[0] == o
         np.testing.assert_allclose(dist, d, rtol=1e-4, atol=1e-6 * m)
         assert bsf >= d * (1 - 1e-3) - 1e-6 * m  # a Euclidean distance: an upper bound
+
+
+@pytest.mark.parametrize("m,r", [(64, 40), (65, 33), (65, 64), (66, 50), (97, 96), (300, 31), (300, 35), (513, 512),
+                                 (600, 520), (1025, 1000), (1100, 1099)])
+@pytest.mark.parametrize("k", [1, 6])
+def test_corner_bound_keeps_every_answer(series, m, r, k):
+    """Bands from the narrowest that one warp walks (32 lanes) to the whole
+    query, query lengths around twice the corner, with and without a tight
+    first bound."""
+    x = series[:9000]
+    q, _ = synth.noisy_copy(x, m, 5 * m + r, m + 3, noise=0.4)
+    oi, od = oracle.search_cascade(x, q, r, k)
+    for proposals in (16, 0):
+        with dtws.Index(x, options=dict(seed_proposals=proposals)) as ix:
+            idx, dist = ix.query(q, r, k)
+            assert ix.sync_status() == dtws.DTWS_OK
+        np.testing.assert_array_equal(idx, oi)
+        np.testing.assert_allclose(dist, od, rtol=1e-4, atol=1e-6 * m)
