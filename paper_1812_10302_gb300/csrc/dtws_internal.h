@@ -221,12 +221,18 @@ cudaError_t launch_lock_selftest(const QueryBufs &b, const QueryArgs &a, cudaStr
 cudaError_t launch_enc_pack(float *params, const float *grad, float *m1, float *v1, uint8_t *blob, bool adam,
                             float lr, float beta1, float beta2, float eps, float c1, float c2, cudaStream_t s);
 cudaError_t launch_enc_prep(const float *X, const int64_t *off, int rows, int m, float *u, cudaStream_t s);
-// ws == nullptr: embeddings to e; else the training workspace receives activations
-cudaError_t launch_enc_forward(const uint8_t *blob, const float *u, int rows, float *e, uint8_t *ws, int num_sms,
-                               cudaStream_t s);
-// loss (accumulated into *loss), data and weight gradients of B triples
-cudaError_t launch_enc_backward(const uint8_t *blob, const float *y, int B, float *loss, float *grad,
+// u: the first `split` sequences' inputs, u2: the others'; ws == nullptr:
+// embeddings to e; else the training workspace receives activations
+cudaError_t launch_enc_forward(const uint8_t *blob, const float *u, const float *u2, int split, int rows, float *e,
+                               uint8_t *ws, int num_sms, cudaStream_t s);
+// loss (accumulated into *loss), data and weight gradients (accumulated into
+// grad) of B triples of a batch of `total`
+cudaError_t launch_enc_backward(const uint8_t *blob, const float *y, int B, int total, float *loss, float *grad,
                                 uint8_t *ws, int num_sms, cudaStream_t s);
+// triples of a batch that is worked through in parts: nine whole rounds of the
+// per-sequence kernels' groups (measured for 10,000 triples: 1.54 ms in parts
+// of three rounds, 1.44 of six, 1.38 of nine)
+int enc_chunk_pairs(int num_sms);
 size_t enc_workspace_bytes(int rows);
 cudaError_t launch_enc_series(const uint8_t *blob, const float *x, int64_t n, int b, const float *inv_sigma,
                               int64_t Nw, void *E, int num_sms, cudaStream_t s);

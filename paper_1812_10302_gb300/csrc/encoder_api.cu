@@ -47,6 +47,15 @@ cudaError_t pack_params(const float *params, float *pbuf, uint8_t *blob, cudaStr
     return launch_enc_pack(pbuf, nullptr, nullptr, nullptr, blob, false, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, s);
 }
 
+bool on_device(const void *p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
 bool finite_all(const float *v, int64_t n) {
     for (int64_t i = 0; i < n; ++i)
         if (!(v[i] - v[i] == 0.0f)) return false;
@@ -104,7 +113,7 @@ dtws_status dtws_enc_forward(const float *params, const float *u, int32_t rows, 
     EK(ed.alloc((size_t)rows * DTWS_ENC_DIM * 4));
     EK(pack_params(params, pb.as<float>(), blob.as<uint8_t>(), s));
     EK(cudaMemcpyAsync(ud.p, u, (size_t)rows * DTWS_ENC_U * 4, cudaMemcpyDefault, s));
-    EK(launch_enc_forward(blob.as<uint8_t>(), ud.as<float>(), rows, ed.as<float>(), nullptr, num_sms(), s));
+    EK(launch_enc_forward(blob.as<uint8_t>(), ud.as<float>(), nullptr, rows, rows, ed.as<float>(), nullptr, num_sms(), s));
     EK(cudaMemcpyAsync(e, ed.p, (size_t)rows * DTWS_ENC_DIM * 4, cudaMemcpyDefault, s));
     EK(cudaStreamSynchronize(s));
     return DTWS_OK;
@@ -118,25 +127,49 @@ dtws_status dtws_enc_loss_grad(const float *params, const float *uq, const float
     }
     cudaStream_t s = (cudaStream_t)stream;
     const size_t urow = (size_t)DTWS_ENC_U * 4;
-    DevMem pb, blob, ud, yd, ld, gd, ws;
-    EK(pb.alloc((size_t)kEncParams * 4));
-    EK(blob.alloc(kEncBlobBytes));
-    EK(ud.alloc(2 * (size_t)batch * urow));
-    EK(yd.alloc((size_t)batch * 4));
-    EK(ld.alloc(4));
-    EK(gd.alloc((size_t)kEncParams * 4));
-    EK(ws.alloc(enc_workspace_bytes(2 * batch)));
-    EK(pack_params(params, pb.as<float>(), blob.as<uint8_t>(), s));
-    EK(cudaMemcpyAsync(ud.p, uq, (size_t)batch * urow, cudaMemcpyDefault, s));
-    EK(cudaMemcpyAsync(ud.as<uint8_t>() + (size_t)batch * urow, uc, (size_t)batch * urow, cudaMemcpyDefault, s));
-    EK(cudaMemcpyAsync(yd.p, y, (size_t)batch * 4, cudaMemcpyDefault, s));
-    EK(cudaMemsetAsync(ld.p, 0, 4, s));
     const int sms = num_sms();
-    EK(launch_enc_forward(blob.as<uint8_t>(), ud.as<float>(), 2 * batch, nullptr, ws.as<uint8_t>(), sms, s));
-    EK(launch_enc_backward(blob.as<uint8_t>(), yd.as<float>(), batch, ld.as<float>(), gd.as<float>(),
-                           ws.as<uint8_t>(), sms, s));
-    EK(cudaMemcpyAsync(grad, gd.p, (size_t)kEncParams * 4, cudaMemcpyDefault, s));
-    EK(cudaMemcpyAsync(loss, ld.p, 4, cudaMemcpyDeviceToHost, s));
+    // The batch is worked through in parts (30 KB of activations per sequence:
+    // 210 MB instead of 610 at 10,000 triples); one allocation holds everything
+    // (seven, of that size, took 0.9 ms per call).  Inputs already on the
+    // device are read where they are.
+    const int part = batch < enc_chunk_pairs(sms) ? batch : enc_chunk_pairs(sms);
+    const bool qdev = on_device(uq), cdev = on_device(uc), ydev = on_device(y);
+    size_t bytes = 0;
+    auto take = [&](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_pb = take((size_t)kEncParams * 4), o_blob = take(kEncBlobBytes), o_grad = take((size_t)kEncParams * 4);
+    const size_t o_loss = take(4), o_q = take(qdev ? 0 : (size_t)batch * urow), o_c = take(cdev ? 0 : (size_t)batch * urow);
+    const size_t o_y = take(ydev ? 0 : (size_t)batch * 4), o_ws = take(enc_workspace_bytes(2 * part));
+    DevMem mem;
+    EK(mem.alloc(bytes));
+    uint8_t *base = mem.as<uint8_t>(), *blob = base + o_blob, *ws = base + o_ws;
+    float *grad_d = (float *)(base + o_grad), *loss_d = (float *)(base + o_loss);
+    const float *q_d = uq, *c_d = uc, *y_d = y;
+    EK(pack_params(params, (float *)(base + o_pb), blob, s));
+    if (!qdev) {
+        EK(cudaMemcpyAsync(base + o_q, uq, (size_t)batch * urow, cudaMemcpyDefault, s));
+        q_d = (const float *)(base + o_q);
+    }
+    if (!cdev) {
+        EK(cudaMemcpyAsync(base + o_c, uc, (size_t)batch * urow, cudaMemcpyDefault, s));
+        c_d = (const float *)(base + o_c);
+    }
+    if (!ydev) {
+        EK(cudaMemcpyAsync(base + o_y, y, (size_t)batch * 4, cudaMemcpyDefault, s));
+        y_d = (const float *)(base + o_y);
+    }
+    EK(cudaMemsetAsync(grad_d, 0, o_loss + 4 - o_grad, s));  // the gradient and the loss behind it
+    for (int b0 = 0; b0 < batch; b0 += part) {
+        const int B = batch - b0 < part ? batch - b0 : part;
+        EK(launch_enc_forward(blob, q_d + (size_t)b0 * DTWS_ENC_U, c_d + (size_t)b0 * DTWS_ENC_U, B, 2 * B, nullptr, ws,
+                              sms, s));
+        EK(launch_enc_backward(blob, y_d + b0, B, batch, loss_d, grad_d, ws, sms, s));
+    }
+    EK(cudaMemcpyAsync(grad, grad_d, (size_t)kEncParams * 4, cudaMemcpyDefault, s));
+    EK(cudaMemcpyAsync(loss, loss_d, 4, cudaMemcpyDeviceToHost, s));
     EK(cudaStreamSynchronize(s));
     return DTWS_OK;
 }
@@ -221,8 +254,9 @@ dtws_status dtws_trainer_step(dtws_trainer_t t, const float *xq, const float *xc
     EK(launch_enc_prep(xq, t->off, batch, m, t->u, s));
     EK(launch_enc_prep(xc, t->off + batch, batch, m, t->u + (size_t)batch * DTWS_ENC_U, s));
     EK(cudaMemsetAsync(t->loss, 0, 4, s));
-    EK(launch_enc_forward(t->blob, t->u, 2 * batch, nullptr, t->ws, t->sms, s));
-    EK(launch_enc_backward(t->blob, t->y, batch, t->loss, t->grad, t->ws, t->sms, s));
+    EK(cudaMemsetAsync(t->grad, 0, (size_t)kEncParams * 4, s));
+    EK(launch_enc_forward(t->blob, t->u, t->u + (size_t)batch * DTWS_ENC_U, batch, 2 * batch, nullptr, t->ws, t->sms, s));
+    EK(launch_enc_backward(t->blob, t->y, batch, batch, t->loss, t->grad, t->ws, t->sms, s));
     ++t->t;
     const double c1 = 1.0 - pow((double)t->hp.beta1, (double)t->t);
     const double c2 = 1.0 - pow((double)t->hp.beta2, (double)t->t);
