@@ -281,13 +281,17 @@ __host__ __device__ inline int tail_entries(int m) { return (m + kTailG - 1) / k
 // cells p > r as well; the odd step's cell p = r alone has a neighbour in
 // the band (its left, cell r of the even anti-diagonal), so only that cell
 // is forced to +inf, by the per-lane penalty pen (K <= 8) or a compare.
-template <int L, int K, int ODD, int QP, int CP>
+// SPARE: L K >= r + 2, so the group's last cell lies past the band on every
+// anti-diagonal.  It is +inf where lane 0 would see it (even steps), and where
+// it would see lane 0's cell (odd steps) the penalty, which then covers every
+// p >= r, makes it +inf: the exchange may wrap around without a select.
+template <int L, int K, int ODD, int QP, int CP, bool SPARE = false>
 __device__ __forceinline__ void diag_step(const float (&qv)[K], const float (&cv)[K], float (&p1)[K],
                                           float (&p2)[K], const float (&pen)[K], int lane, int r, unsigned gmask) {
     const float INF = __int_as_float(0x7f800000);
     // the one neighbour held by the adjacent lane: p-1 (even) / p+1 (odd)
     float nb = __shfl_sync(gmask, ODD ? p1[0] : p1[K - 1], ODD ? ((lane + 1) & (L - 1)) : ((lane - 1) & (L - 1)), L);
-    if (ODD ? (lane == L - 1) : (lane == 0)) nb = INF;
+    if (!SPARE && (ODD ? (lane == L - 1) : (lane == 0))) nb = INF;
     float cur[K];
 #pragma unroll
     for (int t = 0; t < K; ++t) {
@@ -316,9 +320,17 @@ __device__ __forceinline__ void diag_step(const float (&qv)[K], const float (&cv
 // an odd step qbase grows by one (the query values move one cell up, lane 0
 // loads the new one).  The move is a rotation: the slot whose value leaves
 // the lane takes the arriving one, and the phase (CP, QP) advances.
+// With an odd K every lane loads its arriving value from the padded array
+// itself (stride K: no bank conflict within a group), which needs no shuffle,
+// no select, and nothing from another lane; with an even K the lanes' loads
+// would meet in the banks, and the value comes from the adjacent lane.
 template <int L, int K, int CP>
 __device__ __forceinline__ void rot_c(float (&cv)[K], const float *cp, int cbase_new, int lane, unsigned gmask) {
     constexpr int s = CP % K;  // logical 0: leaves downwards, becomes logical K-1
+    if constexpr (K & 1) {
+        cv[s] = cp[cbase_new + (lane + 1) * K - 1];
+        return;
+    }
     const float from_next = __shfl_down_sync(gmask, cv[s], 1, L);
     const float fresh = cp[cbase_new + L * K - 1];
     cv[s] = lane == L - 1 ? fresh : from_next;
@@ -326,6 +338,10 @@ __device__ __forceinline__ void rot_c(float (&cv)[K], const float *cp, int cbase
 template <int L, int K, int QP>
 __device__ __forceinline__ void rot_q(float (&qv)[K], const float *qp, int qbase_new, int lane, unsigned gmask) {
     constexpr int s = ((K - 1 - QP) % K + K) % K;  // logical K-1: leaves upwards, becomes logical 0
+    if constexpr (K & 1) {
+        qv[s] = qp[qbase_new - lane * K];
+        return;
+    }
     const float from_prev = __shfl_up_sync(gmask, qv[s], 1, L);
     const float fresh = qp[qbase_new];
     qv[s] = lane == 0 ? fresh : from_prev;
@@ -416,10 +432,11 @@ __device__ __forceinline__ float corner_bound(const float *__restrict__ qs, cons
 // last kCorner anti-diagonals (corner_bound), 0 if unknown.  cells: lane 0
 // accumulates the cells evaluated (in the band and the matrix).  The walk takes diag_unroll(K) anti-diagonal pairs per
 // iteration; the abandon test runs once per iteration.
-template <typename T, int L, int K, bool ABANDON>
+template <typename T, int L, int K, bool ABANDON, bool SPARE = false>
 __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const float *cbs, float back, int m, int r,
                       T thr, unsigned gmask, int lane, int &cells) {
     static_assert(sizeof(T) == 4, "the FP32 walk");
+    static_assert(!SPARE || K <= 8, "the penalty is a register per cell");
     constexpr int U = diag_unroll(K);
     const float INF = __int_as_float(0x7f800000);
     const int p0 = (r - (r & 1)) >> 1;
@@ -428,7 +445,7 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
     for (int t = 0; t < K; ++t) {
         p1[t] = INF;
         p2[t] = (lane * K + t == p0) ? 0.0f : INF;
-        pen[t] = (lane * K + t == r) ? INF : 0.0f;
+        pen[t] = (SPARE ? lane * K + t >= r : lane * K + t == r) ? INF : 0.0f;
     }
     const int last = 2 * m - 2;
     const int pe_even = r >> 1, pe_odd = (r - 1) >> 1;  // cell e = 0 by the parity of (last + r)
@@ -443,7 +460,7 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
             qv[t] = qp[qb - (lane * K + t)];
             cv[t] = cp[cb + (lane * K + t)];
         }
-        diag_step<L, K, 1, 0, 0>(qv, cv, p1, p2, pen, lane, r, gmask);
+        diag_step<L, K, 1, 0, 0, SPARE>(qv, cv, p1, p2, pen, lane, r, gmask);
         a = 1;
         shift_q<L, K>(qv, qp, qb + 1, lane, gmask);
     } else {
@@ -460,9 +477,9 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
     while (a + 2 * U - 1 < last) {
         static_for<U>([&](auto uc) {
             constexpr int u = decltype(uc)::value;
-            diag_step<L, K, 0, u % K, u % K>(qv, cv, p1, p2, pen, lane, r, gmask);
+            diag_step<L, K, 0, u % K, u % K, SPARE>(qv, cv, p1, p2, pen, lane, r, gmask);
             rot_c<L, K, u % K>(cv, cp, bj + u + 1, lane, gmask);
-            diag_step<L, K, 1, u % K, (u + 1) % K>(qv, cv, p1, p2, pen, lane, r, gmask);
+            diag_step<L, K, 1, u % K, (u + 1) % K, SPARE>(qv, cv, p1, p2, pen, lane, r, gmask);
             rot_q<L, K, u % K>(qv, qp, bi + u + 1, lane, gmask);
         });
         a += 2 * U;
@@ -491,13 +508,13 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
     // is 0 here (the loop above took whole multiples of K pairs), so the
     // windows shift by register moves and keep that phase
     for (;; a += 2, ++bi, ++bj) {
-        diag_step<L, K, 0, 0, 0>(qv, cv, p1, p2, pen, lane, r, gmask);
+        diag_step<L, K, 0, 0, 0, SPARE>(qv, cv, p1, p2, pen, lane, r, gmask);
         if (a == last) {
             res = diag_result<K>(p1, lane, pe_even);
             break;
         }
         shift_c<L, K>(cv, cp, bj + 1, lane, gmask);
-        diag_step<L, K, 1, 0, 0>(qv, cv, p1, p2, pen, lane, r, gmask);
+        diag_step<L, K, 1, 0, 0, SPARE>(qv, cv, p1, p2, pen, lane, r, gmask);
         if (a + 1 == last) {
             res = diag_result<K>(p1, lane, pe_odd);
             break;

@@ -10,6 +10,12 @@ __global__ void k_reset_cursor(QueryState *st) { st->work = 0; }
 
 cudaError_t launch_dtw_at(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                           int64_t count, float *out, cudaStream_t s) {
+    // every walk runs to its end, so the grid's throughput counts, not one
+    // walk's latency: the shapes of dtw_at.cuh where one fits
+    if (a.tune_l == 0) {
+        const cudaError_t e = launch_dtw_at_many(b, a, offsets, count, out, s);
+        if (e != cudaErrorNotSupported) return e;
+    }
     k_reset_cursor<<<1, 1, 0, s>>>(b.st);
     return dtw_dispatch<kModeOut>(b, a, offsets, count, out, count, s);
 }

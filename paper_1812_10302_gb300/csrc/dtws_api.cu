@@ -1659,7 +1659,6 @@ dtws_status dtws_autotune(dtws_t h, const int32_t *m_arr, const int32_t *r_arr, 
         const int64_t N = h->n - m + 1;
         for (int t = 0; t < samples; ++t) offs[t] = (int64_t)((double)t * (double)(N - 1) / samples);
         CK(cudaMemcpyAsync(off_d, offs.data(), ob, cudaMemcpyHostToDevice, s));
-        CK(launch_query_reset(b, a, s));
         CK(launch_qprep(h->x + N / 2, b, a, s));
         auto timed = [&](int L, int K, int W, float *out, float *ms) -> cudaError_t {
             float best = 1e30f;
@@ -1860,7 +1859,6 @@ static dtws_status at_prepare(dtws_t h, const float *Q, int32_t m, int32_t r, co
     *b = make_bufs(h, se, ee);
     *a = make_args(h, m, r, 1);
     a->prescore = 0;
-    CK(launch_query_reset(*b, *a, s));
     CK(launch_qprep(Qd, *b, *a, s));
     return DTWS_OK;
 }

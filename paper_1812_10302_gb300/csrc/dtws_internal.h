@@ -155,7 +155,6 @@ struct SurvPool {
     long long cap;
 };
 
-cudaError_t launch_query_reset(const QueryBufs &b, const QueryArgs &a, cudaStream_t s);
 cudaError_t launch_qprep(const float *Q, const QueryBufs &b, const QueryArgs &a, cudaStream_t s);
 // proposal scans: each CTA writes its best window to cta_best[slot * kCtaSlots + cta];
 // *ctas receives the grid size; launch_prop_merge then keeps the best `proposals`.
@@ -199,6 +198,10 @@ cudaError_t launch_xz_finalize(const QueryBufs &b, const QueryArgs &a, int64_t *
 // element-wise building blocks
 cudaError_t launch_dtw_at(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                           int64_t count, float *out, cudaStream_t s);
+// the same in the shapes that suit many windows (dtw_at.cuh);
+// cudaErrorNotSupported where none fits
+cudaError_t launch_dtw_at_many(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets, int64_t count, float *out,
+                               cudaStream_t s);
 // the autotuner's probes: a shape (see plan_shape) and DTW at offsets with it;
 // the survivor pass's default shape for (m, r) (false: the multi-warp or
 // row-systolic kernel, not a plan_shape shape)

@@ -23,9 +23,10 @@
 #include <mutex>
 
 #include "../../include/dtws.h"
-#include "dtw_band.cuh"
+#include "dtw_at.cuh"
 #include "dtws_common.cuh"
 #include "dtws_internal.h"
+#include "fp_sum.cuh"
 
 namespace {
 
@@ -46,19 +47,36 @@ static __device__ __align__(256) float g_noalloc_scratch[kNoAllocFloats];
 namespace dtws {
 namespace {
 
-// z-normalise Q into scratch[0, m) (Sec. 2.2, Eq. 5, FP64 two-pass, same
+// Mean (FP64) and deviation of n samples y over `threads` threads' shares
+// (start t, stride `threads`): each thread's part is summed in FP32 expansions
+// (fp_sum.cuh), the parts in FP64 by `reduce` -- two-pass, no less exact than
+// FP64 sums throughout and not bound by this part's FP64 rate.
+template <typename Reduce>
+__device__ __forceinline__ void mean_and_variance(const float *__restrict__ y, int n, int t, int threads, Reduce &&reduce,
+                                                  double &mu, double &var) {
+    f3 s{0.0f, 0.0f, 0.0f};
+    for (int j = t; j < n; j += threads) f3_add(s, y[j], 0.0f);
+    mu = reduce(f3_value(s)) / (double)n;
+    const float mh = (float)mu, ml = (float)(mu - (double)mh);
+    f3 v{0.0f, 0.0f, 0.0f};
+    for (int j = t; j < n; j += threads) {
+        exact2 d = two_sum_rn(y[j], -mh);
+        d = two_sum_rn(d.s, __fsub_rn(d.e, ml));
+        f3_add_sq(v, d.s, d.e);
+    }
+    var = reduce(f3_value(v)) / (double)n;
+}
+
+// z-normalise Q into scratch[0, m) (Sec. 2.2, Eq. 5, two-pass, same
 // zero-variance rule as the search) and reset the work cursor.  A
 // non-finite query leaves a NaN in scratch[0] so the DTW kernel writes NaN.
-__global__ void __launch_bounds__(1024) k_noalloc_prep(const float *__restrict__ Q, int m,
-                                                       float *scratch) {
-    __shared__ double red[32];
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
+constexpr int kPrepThreads = 256;
+__global__ void __launch_bounds__(kPrepThreads) k_noalloc_prep(const float *__restrict__ Q, int m,
+                                                               float *scratch) {
+    __shared__ double red[kPrepThreads / 32];
     bool nf = false;
     for (int j = threadIdx.x; j < m; j += blockDim.x) nf |= !isfinite(Q[j]);
-    if (nf) atomicOr(&bad, 1);
-    __syncthreads();
+    const bool bad = __syncthreads_or(nf);
     if (threadIdx.x == 0) *(unsigned long long *)(scratch + kNoAllocCursor) = 0ull;
     if (bad) {
         if (threadIdx.x == 0) scratch[0] = __int_as_float(0x7fc00000);
@@ -70,24 +88,48 @@ __global__ void __launch_bounds__(1024) k_noalloc_prep(const float *__restrict__
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
         __syncthreads();
         double s = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
+        for (int i = 0; i < kPrepThreads / 32; ++i) s += red[i];
         return s;
     };
-    double s = 0.0;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) s += (double)Q[j];
-    const double mu = bsum(s) / (double)m;
-    double v = 0.0;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        const double d = (double)Q[j] - mu;
-        v = fma(d, d, v);
-    }
-    const double var = bsum(v) / (double)m, mm = mu * mu;
+    double mu, var;
+    mean_and_variance(Q, m, threadIdx.x, blockDim.x, bsum, mu, var);
+    const double mm = mu * mu;
     const bool zero = var <= 1e-24 * (mm > 1.0 ? mm : 1.0);
-    const double sg = zero ? 0.0 : sqrt(var);
+    const double inv = zero ? 0.0 : 1.0 / sqrt(var);
     for (int j = threadIdx.x; j < m; j += blockDim.x)
-        scratch[j] = zero ? 0.0f : (float)(((double)Q[j] - mu) / sg);
+        scratch[j] = zero ? 0.0f : (float)(((double)Q[j] - mu) * inv);
 }
 
+// The throughput shapes (dtw_at.cuh) with each window's Eq. 5 statistics
+// formed by its lane group.  Measured (20,000 windows, m = 256, r = 25): 75 us
+// and 9 us for the query, against 512 with the row-systolic walk below and 32.
+template <int L, int K>
+__global__ void __launch_bounds__(kAtThreads, at_min_blocks(K))
+k_noalloc_at(const float *__restrict__ x, int64_t n, int m, int r, const int64_t *__restrict__ offsets, int64_t count,
+             float *__restrict__ out, const float *__restrict__ scratch) {
+    if (!(scratch[0] == scratch[0])) {  // a non-finite query
+        for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count; c += (int64_t)gridDim.x * blockDim.x)
+            out[c] = __int_as_float(0x7fc00000);
+        return;
+    }
+    at_body<L, K>(scratch, x, n - m + 1, m, r, offsets, count, out,
+                  [&](int64_t o, int lane, unsigned gmask, float &mh, float &is, float &ls) {
+                      auto gsum = [&](double v) {
+#pragma unroll
+                          for (int q = L / 2; q > 0; q >>= 1) v += __shfl_xor_sync(gmask, v, q, L);
+                          return v;
+                      };
+                      double mu, var;
+                      mean_and_variance(x + o, m, lane, L, gsum, mu, var);
+                      const double mm = mu * mu;
+                      const double inv = var <= 1e-24 * (mm > 1.0 ? mm : 1.0) ? 0.0 : 1.0 / sqrt(var);
+                      mh = (float)mu;
+                      is = (float)inv;
+                      ls = (float)(mu - (double)mh) * is;
+                  });
+}
+
+// Bands that the shapes above do not take (fewer than 5 cells, more than 256):
 // FP32 banded DTW of the normalised query (scratch) against the windows at
 // offsets; each window's Eq. 5 statistics are computed two-pass in FP64 by
 // its lane group.  Groups of L lanes pull offsets from the scratch cursor.
@@ -191,6 +233,15 @@ inline size_t noalloc_smem(int m, int r, int L, int warps) {
     return qbytes + (size_t)warps * per_warp;
 }
 
+template <int L, int K>
+cudaError_t launch_noalloc_at(const float *x, int64_t n, int m, int r, const int64_t *offsets, int64_t count, float *out,
+                              const float *scratch, const AtPlan &p, int sms, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_noalloc_at<L, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    if (e != cudaSuccess) return e;
+    k_noalloc_at<L, K><<<at_grid(p, count, sms), p.warps * 32, p.smem, s>>>(x, n, m, r, offsets, count, out, scratch);
+    return cudaGetLastError();
+}
+
 template <int L>
 cudaError_t launch_noalloc_dtw(const float *x, int64_t n, int m, int r, const int64_t *offsets,
                                int64_t count, float *out, float *scratch, cudaStream_t s) {
@@ -245,9 +296,11 @@ extern "C" dtws_status dtws_dtw_at_noalloc(const float *series, int64_t n, const
     if (st != DTWS_OK) return st;
     if (count == 0) return DTWS_OK;
     const int rr = r > m - 1 ? m - 1 : r;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     {  // one warp's shared memory must fit the device's per-block limit
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
+        int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         const size_t need = noalloc_smem(m, rr, lanes_for(rr), 1);
         if (optin > 0 && need > (size_t)optin) {
@@ -257,9 +310,16 @@ extern "C" dtws_status dtws_dtw_at_noalloc(const float *series, int64_t n, const
         }
     }
     cudaStream_t s = (cudaStream_t)stream;
-    k_noalloc_prep<<<1, 1024, 0, s>>>(Q, m, scratch);
+    k_noalloc_prep<<<1, kPrepThreads, 0, s>>>(Q, m, scratch);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) {
+    AtPlan p{};
+    if (e == cudaSuccess && at_plan(m, rr, &p)) {
+        e = cudaErrorInvalidValue;
+#define DTWS_CASE(LL, KK) \
+    if (p.L == LL && p.K == KK) e = launch_noalloc_at<LL, KK>(series, n, m, rr, offsets, count, out, scratch, p, sms, s);
+        DTWS_AT_SHAPES(DTWS_CASE)
+#undef DTWS_CASE
+    } else if (e == cudaSuccess) {
         switch (lanes_for(rr)) {
         case 1: e = launch_noalloc_dtw<1>(series, n, m, rr, offsets, count, out, scratch, s); break;
         case 2: e = launch_noalloc_dtw<2>(series, n, m, rr, offsets, count, out, scratch, s); break;

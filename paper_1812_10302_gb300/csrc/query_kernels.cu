@@ -1,7 +1,6 @@
 // query_kernels.cu -- per-query kernels of the search (arxiv 1812.10302):
 //
-//   k_query_reset   clear the device query state
-//   k_qprep         z-normalise Q (Sec. 2.2, Eq. 5; FP64 two-pass; taken as
+//   k_qprep         clear the device query state, z-normalise Q (Sec. 2.2, Eq. 5; FP64 two-pass; taken as
 //                   it is for unnormalised DTW), its envelope (Eq. 9) and the
 //                   ordered terms of the early-abandoning bounds
 //   k_seed_scan     proxy scan: each warp's window with the smallest squared
@@ -75,13 +74,6 @@ __device__ __forceinline__ void reset_state(QueryState *st) {
         st->pre_done = 0;
         st->margin_skip = 0;
     }
-}
-
-__global__ void k_query_reset(QueryState *st) { reset_state(st); }
-
-cudaError_t launch_query_reset(const QueryBufs &b, const QueryArgs &, cudaStream_t s) {
-    k_query_reset<<<1, 1024, 0, s>>>(b.st);
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ query prep
