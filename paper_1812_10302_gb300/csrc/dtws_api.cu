@@ -40,15 +40,37 @@ cudaError_t dalloc(T **p, size_t count) {
 
 int64_t round_up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
+// Several arrays in one device allocation: take() lays them out, alloc() makes
+// the block, at() gives an array.  (An allocation costs ~45 us and its release
+// 20 to 80, whatever their size up to 100 MB; indexing a series, searching it
+// once and letting it go made thirty of each.)
+struct Arena {
+    size_t bytes = 0;
+    char *base = nullptr;
+    template <typename T>
+    size_t take(size_t count) {
+        const size_t at = bytes;
+        bytes += (count * sizeof(T) + 256 + 255) / 256 * 256;  // (as dalloc: a little room past each array)
+        return at;
+    }
+    cudaError_t alloc() { return dalloc(&base, bytes); }
+    template <typename T>
+    T *at(size_t offset) const {
+        return reinterpret_cast<T *>(base + offset);
+    }
+};
+
 struct StatsEntry {
     int m = 0;
     int64_t used = 0;
+    char *block = nullptr;  // the allocation the arrays lie in
     float *mu_hi = nullptr, *mu_lo = nullptr, *inv_sigma = nullptr;
     float *smu_hi = nullptr, *sinv_sigma = nullptr;  // every kProxyStride-th window (proxy scan)
 };
 struct EnvEntry {
     int r = 0;
     int64_t used = 0;
+    char *block = nullptr;
     float *U = nullptr, *L = nullptr;
 };
 
@@ -73,14 +95,10 @@ constexpr int kLearnSlots = 2;
 // window-statistics slot, and its own streams, so that queries on different
 // lanes overlap on the GPU.
 struct Lane {
-    QueryState *st = nullptr;
-    float *qh32 = nullptr, *Uq = nullptr, *Lq = nullptr, *sq = nullptr, *sU = nullptr, *sL = nullptr;
-    double *qh64 = nullptr;
-    unsigned short *ord = nullptr;
+    char *block = nullptr;  // the allocation its arrays lie in
     float *cand_lb = nullptr, *sort_lb = nullptr;
     unsigned *cand_idx = nullptr, *sort_idx = nullptr;
-    StatsEntry stats;  // slot sized for the batch's smallest m
-    int64_t stats_cap = 0;
+    StatsEntry stats;  // slot that serves every m (in the lane's block)
     cudaStream_t stream = nullptr, side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_done = nullptr;
 };
@@ -97,6 +115,7 @@ void dtws::set_error_detail(const char *fmt, ...) {
 struct dtws_ctx {
     int device = 0, num_sms = 0;
     int64_t n = 0, n_alloc = 0;
+    char *block = nullptr;               // the allocation of the per-series arrays below
     float *x = nullptr;
     float *x_sub = nullptr;              // x[kProxyStride j] for j < n_alloc/kProxyStride, plus a zero tail
     float *pf = nullptr, *bf = nullptr;  // prefix sums as FP32 pairs, block totals and anchors
@@ -110,6 +129,11 @@ struct dtws_ctx {
     StatsEntry ident;                    // unnormalised DTW: mean 0, 1/sigma 1 for every window
     std::vector<EnvEntry> env;
     int64_t clock = 0;
+    // the stream whose order every queued reader of the caches is in (several
+    // since the last device-wide wait: a slot that is reused waits for all)
+    cudaStream_t cache_stream = nullptr;
+    bool cache_used = false, cache_mixed = false;
+    char *work_block = nullptr, *cand_block = nullptr;
     QueryState *st = nullptr;
     int *status = nullptr;
     float *qh32 = nullptr, *Uq = nullptr, *Lq = nullptr, *sq = nullptr, *sU = nullptr, *sL = nullptr;
@@ -123,6 +147,7 @@ struct dtws_ctx {
     size_t stage_cap = 0;
     void *hstage = nullptr;
     size_t hstage_cap = 0;
+    int64_t reads = 0;  // results read back
     dtws_options opt;
     cudaStream_t last_stream = nullptr;
     QueryState *last_st = nullptr;  // the state the last query's counters are in
@@ -145,6 +170,7 @@ struct dtws_ctx {
     std::vector<int64_t> graph_sig;  // what the cached graph was captured for
     cudaGraphExec_t qgraph_exec = nullptr;  // the same for single queries
     std::vector<int64_t> qgraph_sig;
+    std::vector<int64_t> qseen_sig;  // the last query's, launched without a graph
     int64_t qgraph_launches = 0;
     // learned proposal encoder
     uint8_t *enc_blob = nullptr;
@@ -152,6 +178,7 @@ struct dtws_ctx {
     std::vector<LearnEntry> learn;
     // batch: per-query states and query buffers, the survivor pool of the
     // persistent stage, its query table and shape lists
+    char *bq_block = nullptr, *bqf_block = nullptr, *pool_block = nullptr;
     QueryState *bq_st = nullptr;
     int bq_cap = 0;
     float *bq_f = nullptr;           // qh32, Uq, Lq, sq, sU, sL: 6 runs of bq_fcap
@@ -218,6 +245,15 @@ dtws_status read_back(dtws_t h, cudaStream_t s, const int64_t *idx_d, const floa
     const char *lo = !idev ? (const char *)idx_d : (const char *)dist_d;
     const char *hi = !ddev ? (const char *)dist_d + db : (const char *)idx_d + ib;
     const size_t span = (size_t)(hi - lo);
+    char local[1024];
+    if (h->reads++ == 0 && span <= sizeof local) {
+        // a handle's first result: not worth pinned memory of its own
+        CK(cudaMemcpyAsync(local, lo, span, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (!idev) memcpy(out_idx, local + ((const char *)idx_d - lo), ib);
+        if (!ddev) memcpy(out_dist, local + ((const char *)dist_d - lo), db);
+        return DTWS_OK;
+    }
     if (h->hstage_cap < span) {
         if (h->hstage) cudaFreeHost(h->hstage);
         h->hstage = nullptr;
@@ -239,17 +275,61 @@ dtws_status read_back(dtws_t h, cudaStream_t s, const int64_t *idx_d, const floa
 }
 
 void free_stats(StatsEntry &e) {
-    cudaFree(e.mu_hi);
-    cudaFree(e.mu_lo);
-    cudaFree(e.inv_sigma);
-    cudaFree(e.smu_hi);
-    cudaFree(e.sinv_sigma);
+    if (e.block) cudaFree(e.block);
     e = StatsEntry();
 }
 void free_env(EnvEntry &e) {
-    cudaFree(e.U);
-    cudaFree(e.L);
+    if (e.block) cudaFree(e.block);
     e = EnvEntry();
+}
+
+// A stream is about to read or write the caches.
+void use_caches(dtws_t h, cudaStream_t s) {
+    h->cache_mixed = h->cache_mixed || (h->cache_used && h->cache_stream != s);
+    h->cache_used = true;
+    h->cache_stream = s;
+}
+// A cache slot's arrays are about to be rewritten in the order of `s`: no
+// kernel queued elsewhere may still read them.
+cudaError_t settle_caches(dtws_t h, cudaStream_t s) {
+    if (!h->cache_used || (!h->cache_mixed && h->cache_stream == s)) return cudaSuccess;
+    const cudaError_t e = cudaDeviceSynchronize();
+    h->cache_used = h->cache_mixed = false;
+    return e;
+}
+
+// Window statistics arrays that serve every m (room for the windows of m = 2):
+// a slot of another length is reused as it is.  Past the windows of the
+// longest query they hold zeros until written: bulk copies read whole tiles.
+int64_t stats_cap(dtws_t h) { return round_up(h->n - 1, kProxyTile) + kProxyTile; }
+struct StatsLayout {
+    size_t mh, ml, is, smh, sis;
+};
+StatsLayout take_stats(Arena &a, int64_t cap) {
+    StatsLayout l;
+    l.mh = a.take<float>(cap);
+    l.ml = a.take<float>(cap);
+    l.is = a.take<float>(cap);
+    l.smh = a.take<float>(cap / kProxyStride);
+    l.sis = a.take<float>(cap / kProxyStride);
+    return l;
+}
+void place_stats(StatsEntry *e, const Arena &a, const StatsLayout &l) {
+    e->mu_hi = a.at<float>(l.mh);
+    e->mu_lo = a.at<float>(l.ml);
+    e->inv_sigma = a.at<float>(l.is);
+    e->smu_hi = a.at<float>(l.smh);
+    e->sinv_sigma = a.at<float>(l.sis);
+}
+cudaError_t clear_stats_tail(dtws_t h, const StatsEntry &e, cudaStream_t s) {
+    const int64_t cap = stats_cap(h), from = h->n > kMMax ? round_up(h->n - kMMax, 4) - 4 : 0;
+    const int64_t sfrom = from / kProxyStride, scap = cap / kProxyStride;
+    cudaError_t ce = cudaMemsetAsync(e.mu_hi + from, 0, (cap - from) * 4, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.mu_lo + from, 0, (cap - from) * 4, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.inv_sigma + from, 0, (cap - from) * 4, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.smu_hi + sfrom, 0, (scap - sfrom) * 4, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.sinv_sigma + sfrom, 0, (scap - sfrom) * 4, s);
+    return ce;
 }
 
 dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *computed) {
@@ -257,39 +337,39 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
     for (auto &e : h->stats)
         if (e.m == m) {
             e.used = ++h->clock;
+            use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
-    if ((int)h->stats.size() >= kCacheSlots) {
+    StatsEntry e;
+    if ((int)h->stats.size() >= kCacheSlots) {  // the least recently used slot's arrays
         size_t lru = 0;
         for (size_t i = 1; i < h->stats.size(); ++i)
             if (h->stats[i].used < h->stats[lru].used) lru = i;
-        CK(cudaDeviceSynchronize());  // no queued kernel may still read it
-        free_stats(h->stats[lru]);
+        CK(settle_caches(h, s));
+        e = h->stats[lru];
         h->stats.erase(h->stats.begin() + lru);
+    } else {
+        Arena a;
+        const StatsLayout l = take_stats(a, stats_cap(h));
+        if (a.alloc() != cudaSuccess) {
+            cudaGetLastError();
+            set_err("window statistics for m=%d: out of device memory", m);
+            return DTWS_ENOMEM;
+        }
+        e.block = a.base;
+        place_stats(&e, a, l);
+        const cudaError_t ce = clear_stats_tail(h, e, s);
+        if (ce != cudaSuccess) {
+            free_stats(e);
+            cudaGetLastError();
+            set_err("window statistics for m=%d: %s", m, cudaGetErrorString(ce));
+            return DTWS_ECUDA;
+        }
     }
-    StatsEntry e;
     e.m = m;
-    const int64_t N = h->n - m + 1;
-    const int64_t cap = round_up(N, kProxyTile) + kProxyTile;
-    const int64_t scap = cap / kProxyStride;
-    cudaError_t a1 = dalloc(&e.mu_hi, cap), a2 = dalloc(&e.mu_lo, cap), a3 = dalloc(&e.inv_sigma, cap);
-    cudaError_t a4 = dalloc(&e.smu_hi, scap), a6 = dalloc(&e.sinv_sigma, scap);
-    if (a1 != cudaSuccess || a2 != cudaSuccess || a3 != cudaSuccess || a4 != cudaSuccess ||
-        a6 != cudaSuccess) {
-        free_stats(e);
-        cudaGetLastError();
-        set_err("window statistics for m=%d: out of device memory", m);
-        return DTWS_ENOMEM;
-    }
-    cudaError_t ce = cudaMemsetAsync(e.mu_hi, 0, cap * 4, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.mu_lo, 0, cap * 4, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.inv_sigma, 0, cap * 4, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.smu_hi, 0, scap * 4, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.sinv_sigma, 0, scap * 4, s);
-    if (ce == cudaSuccess)
-        ce = launch_window_stats(h->x, h->n, m, h->pf, h->bf, h->pok, h->pscale, e.mu_hi, e.mu_lo, e.inv_sigma,
-                                 e.smu_hi, e.sinv_sigma, h->num_sms, s);
+    const cudaError_t ce = launch_window_stats(h->x, h->n, m, h->pf, h->bf, h->pok, h->pscale, e.mu_hi, e.mu_lo,
+                                               e.inv_sigma, e.smu_hi, e.sinv_sigma, h->num_sms, s);
     if (ce != cudaSuccess) {  // nothing half-initialised stays in the cache
         free_stats(e);
         cudaGetLastError();
@@ -297,6 +377,7 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
         return DTWS_ECUDA;
     }
     e.used = ++h->clock;
+    use_caches(h, s);
     h->stats.push_back(e);
     *out = &h->stats.back();
     *computed = true;
@@ -310,18 +391,16 @@ dtws_status get_ident(dtws_t h, cudaStream_t s, StatsEntry **out, bool *computed
     *computed = false;
     if (!h->ident.mu_hi) {
         StatsEntry e;
-        const int64_t N = h->n - 1;
-        const int64_t cap = round_up(N, kProxyTile) + kProxyTile;
-        const int64_t scap = cap / kProxyStride;
-        cudaError_t a1 = dalloc(&e.mu_hi, cap), a2 = dalloc(&e.mu_lo, cap), a3 = dalloc(&e.inv_sigma, cap);
-        cudaError_t a4 = dalloc(&e.smu_hi, scap), a6 = dalloc(&e.sinv_sigma, scap);
-        if (a1 != cudaSuccess || a2 != cudaSuccess || a3 != cudaSuccess || a4 != cudaSuccess ||
-            a6 != cudaSuccess) {
-            free_stats(e);
+        Arena a;
+        const int64_t cap = stats_cap(h), scap = cap / kProxyStride;
+        const StatsLayout l = take_stats(a, cap);
+        if (a.alloc() != cudaSuccess) {
             cudaGetLastError();
             set_err("unnormalised statistics: out of device memory");
             return DTWS_ENOMEM;
         }
+        e.block = a.base;
+        place_stats(&e, a, l);
         cudaError_t ce = cudaMemsetAsync(e.mu_hi, 0, cap * 4, s);
         if (ce == cudaSuccess) ce = cudaMemsetAsync(e.mu_lo, 0, cap * 4, s);
         if (ce == cudaSuccess) ce = cudaMemsetAsync(e.smu_hi, 0, scap * 4, s);
@@ -336,6 +415,7 @@ dtws_status get_ident(dtws_t h, cudaStream_t s, StatsEntry **out, bool *computed
         h->ident = e;
         *computed = true;
     }
+    use_caches(h, s);
     *out = &h->ident;
     return DTWS_OK;
 }
@@ -351,29 +431,40 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
     for (auto &e : h->env)
         if (e.r == r) {
             e.used = ++h->clock;
+            use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
-    if ((int)h->env.size() >= kCacheSlots) {
+    EnvEntry e;
+    if ((int)h->env.size() >= kCacheSlots) {  // the least recently used slot's arrays
         size_t lru = 0;
         for (size_t i = 1; i < h->env.size(); ++i)
             if (h->env[i].used < h->env[lru].used) lru = i;
-        CK(cudaDeviceSynchronize());  // no queued kernel may still read it
-        free_env(h->env[lru]);
+        CK(settle_caches(h, s));
+        e = h->env[lru];
         h->env.erase(h->env.begin() + lru);
+    } else {
+        Arena a;
+        const size_t u = a.take<float>(h->n_alloc), l = a.take<float>(h->n_alloc);
+        if (a.alloc() != cudaSuccess) {
+            cudaGetLastError();
+            set_err("series envelope for r=%d: out of device memory", r);
+            return DTWS_ENOMEM;
+        }
+        e.block = a.base;
+        e.U = a.at<float>(u);
+        e.L = a.at<float>(l);
+        cudaError_t ce = cudaMemsetAsync(e.U + h->n, 0, (h->n_alloc - h->n) * 4, s);
+        if (ce == cudaSuccess) ce = cudaMemsetAsync(e.L + h->n, 0, (h->n_alloc - h->n) * 4, s);
+        if (ce != cudaSuccess) {
+            free_env(e);
+            cudaGetLastError();
+            set_err("series envelope for r=%d: %s", r, cudaGetErrorString(ce));
+            return DTWS_ECUDA;
+        }
     }
-    EnvEntry e;
     e.r = r;
-    cudaError_t a1 = dalloc(&e.U, h->n_alloc), a2 = dalloc(&e.L, h->n_alloc);
-    if (a1 != cudaSuccess || a2 != cudaSuccess) {
-        free_env(e);
-        cudaGetLastError();
-        set_err("series envelope for r=%d: out of device memory", r);
-        return DTWS_ENOMEM;
-    }
-    cudaError_t ce = cudaMemsetAsync(e.U, 0, h->n_alloc * 4, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(e.L, 0, h->n_alloc * 4, s);
-    if (ce == cudaSuccess) ce = launch_envelope(h->x, h->n, r, e.U, e.L, s);
+    const cudaError_t ce = launch_envelope(h->x, h->n, r, e.U, e.L, s);
     if (ce != cudaSuccess) {
         free_env(e);
         cudaGetLastError();
@@ -381,17 +472,11 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
         return DTWS_ECUDA;
     }
     e.used = ++h->clock;
+    use_caches(h, s);
     h->env.push_back(e);
     *out = &h->env.back();
     *computed = true;
     return DTWS_OK;
-}
-
-// Allocate whatever is still missing, so a call that failed half way (out
-// of memory) leaves a handle that the next call completes or destroy frees.
-template <typename T>
-cudaError_t need(T **p, size_t count) {
-    return *p ? cudaSuccess : dalloc(p, count);
 }
 
 void free_learn(LearnEntry &e) {
@@ -488,24 +573,36 @@ dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, Lea
 }
 
 dtws_status ensure_workspace(dtws_t h) {
-    CK(need(&h->st, 1));
-    CK(need(&h->qh32, kMMax));
-    CK(need(&h->Uq, kMMax));
-    CK(need(&h->Lq, kMMax));
-    CK(need(&h->sq, kMMax));
-    CK(need(&h->sU, kMMax));
-    CK(need(&h->sL, kMMax));
-    CK(need(&h->qh64, kMMax));
-    CK(need(&h->ord, kMMax));
+    if (h->work_block) return DTWS_OK;
+    Arena a;
+    const size_t st = a.take<QueryState>(1), qh32 = a.take<float>(kMMax), Uq = a.take<float>(kMMax),
+                 Lq = a.take<float>(kMMax), sq = a.take<float>(kMMax), sU = a.take<float>(kMMax),
+                 sL = a.take<float>(kMMax), qh64 = a.take<double>(kMMax), ord = a.take<unsigned short>(kMMax);
+    CK(a.alloc());
+    h->work_block = a.base;
+    h->st = a.at<QueryState>(st);
+    h->qh32 = a.at<float>(qh32);
+    h->Uq = a.at<float>(Uq);
+    h->Lq = a.at<float>(Lq);
+    h->sq = a.at<float>(sq);
+    h->sU = a.at<float>(sU);
+    h->sL = a.at<float>(sL);
+    h->qh64 = a.at<double>(qh64);
+    h->ord = a.at<unsigned short>(ord);
     return DTWS_OK;
 }
 
 dtws_status ensure_candidates(dtws_t h) {
+    if (h->cand_block) return DTWS_OK;
     const int64_t cap = h->n;  // at most N <= n survivors
-    CK(need(&h->cand_lb, cap));
-    CK(need(&h->sort_lb, cap));
-    CK(need(&h->cand_idx, cap));
-    CK(need(&h->sort_idx, cap));
+    Arena a;
+    const size_t cl = a.take<float>(cap), sl = a.take<float>(cap), ci = a.take<unsigned>(cap), si = a.take<unsigned>(cap);
+    CK(a.alloc());
+    h->cand_block = a.base;
+    h->cand_lb = a.at<float>(cl);
+    h->sort_lb = a.at<float>(sl);
+    h->cand_idx = a.at<unsigned>(ci);
+    h->sort_idx = a.at<unsigned>(si);
     h->cand_cap = cap;
     return DTWS_OK;
 }
@@ -738,6 +835,15 @@ dtws_status enqueue_search(dtws_t h, const Exec &e, const QueryArgs &a, const fl
     return DTWS_OK;
 }
 
+bool stream_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
 // One query on the handle's own buffers (dtws_query).
 dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *idx_d, float *dist_d,
                       cudaStream_t s, int xz_z = 0) {
@@ -769,7 +875,7 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
     a.xz_z = xz_z;
     int64_t launches = 0;
     // Repeated queries with the same arguments replay one CUDA graph of the
-    // search (the caches above are resolved first, on the caller's stream;
+    // search, captured when they repeat (the caches above are resolved first, on the caller's stream;
     // no phase events are recorded in a graph).  The signature holds every
     // value the captured kernels' arguments depend on.
     const bool graph = h->opt.batch_graph && !h->opt.timing;
@@ -783,6 +889,17 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
         if (h->qgraph_exec && sig == h->qgraph_sig) {
             CK(cudaGraphLaunch(h->qgraph_exec, s));
             launches = h->qgraph_launches;
+        } else if (sig != h->qseen_sig || stream_capturing(s)) {
+            // a query seen for the first time is launched as it is: capturing
+            // and instantiating a graph costs more than one replay saves (and
+            // a stream that is being captured by the caller cannot be forked
+            // into a capture of its own)
+            if (stream_capturing(s) && sig != h->qseen_sig) {
+                set_err("dtws_query: a stream under capture takes a query that has run once before");
+                return DTWS_ECUDA;
+            }
+            h->qseen_sig = sig;
+            if ((st = enqueue_search(h, e, a, Qd, idx_d, dist_d, &launches)) != DTWS_OK) return st;
         } else {
             if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
             if (!h->batch_fork) CK(cudaEventCreateWithFlags(&h->batch_fork, cudaEventDisableTiming));
@@ -827,11 +944,7 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
 }
 
 void free_lane(Lane &l) {
-    void *ptrs[] = {l.st, l.qh32, l.Uq, l.Lq, l.sq, l.sU, l.sL, l.qh64, l.ord, l.cand_lb, l.sort_lb, l.cand_idx,
-                    l.sort_idx};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    free_stats(l.stats);
+    if (l.block) cudaFree(l.block);  // (its statistics lie in it)
     if (l.stream) cudaStreamDestroy(l.stream);
     if (l.side) cudaStreamDestroy(l.side);
     if (l.ev_fork) cudaEventDestroy(l.ev_fork);
@@ -850,51 +963,38 @@ void drop_graph(dtws_t h) {
 }
 
 
-// Lanes with statistics slots for windows of at least m_min samples.
-dtws_status ensure_lanes(dtws_t h, int count, int m_min) {
-    const int64_t need_cap = round_up(h->n - m_min + 1, kProxyTile) + kProxyTile;
-    for (auto &l : h->lanes)
-        if (l.stats_cap < need_cap) {  // too small: rebuild all (rare)
-            CK(cudaDeviceSynchronize());
-            drop_graph(h);
-            for (auto &x : h->lanes) free_lane(x);
-            h->lanes.clear();
-            break;
-        }
+// Lanes for `count` queries in flight.
+dtws_status ensure_lanes(dtws_t h, int count) {
     if (!h->batch_fork) CK(cudaEventCreateWithFlags(&h->batch_fork, cudaEventDisableTiming));
     if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     while ((int)h->lanes.size() < count) {
         h->lanes.emplace_back();
         Lane &l = h->lanes.back();
-        const int64_t cap = h->n, scap = need_cap / kProxyStride;
-        cudaError_t e = cudaSuccess;
+        const int64_t cap = h->n;
+        Arena a;
+        const size_t cl = a.take<float>(cap), sl = a.take<float>(cap), ci = a.take<unsigned>(cap),
+                     si = a.take<unsigned>(cap);
+        const StatsLayout sl_ = take_stats(a, stats_cap(h));
+        cudaError_t e = a.alloc();
         auto al = [&](cudaError_t r) {
             if (e == cudaSuccess) e = r;
         };
-        al(dalloc(&l.st, 1));
-        al(dalloc(&l.qh32, kMMax));
-        al(dalloc(&l.Uq, kMMax));
-        al(dalloc(&l.Lq, kMMax));
-        al(dalloc(&l.sq, kMMax));
-        al(dalloc(&l.sU, kMMax));
-        al(dalloc(&l.sL, kMMax));
-        al(dalloc(&l.qh64, kMMax));
-        al(dalloc(&l.ord, kMMax));
-        al(dalloc(&l.cand_lb, cap));
-        al(dalloc(&l.sort_lb, cap));
-        al(dalloc(&l.cand_idx, cap));
-        al(dalloc(&l.sort_idx, cap));
-        al(dalloc(&l.stats.mu_hi, need_cap));
-        al(dalloc(&l.stats.mu_lo, need_cap));
-        al(dalloc(&l.stats.inv_sigma, need_cap));
-        al(dalloc(&l.stats.smu_hi, scap));
-        al(dalloc(&l.stats.sinv_sigma, scap));
+        if (e == cudaSuccess) {
+            l.block = a.base;
+            l.cand_lb = a.at<float>(cl);
+            l.sort_lb = a.at<float>(sl);
+            l.cand_idx = a.at<unsigned>(ci);
+            l.sort_idx = a.at<unsigned>(si);
+            place_stats(&l.stats, a, sl_);
+        }
         al(cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking));
         al(cudaStreamCreateWithFlags(&l.side, cudaStreamNonBlocking));
         al(cudaEventCreateWithFlags(&l.ev_fork, cudaEventDisableTiming));
         al(cudaEventCreateWithFlags(&l.ev_join, cudaEventDisableTiming));
         al(cudaEventCreateWithFlags(&l.ev_done, cudaEventDisableTiming));
-        l.stats_cap = need_cap;
+        // statistics slots must hold finite values beyond N (bulk copies read whole tiles)
+        if (e == cudaSuccess) al(clear_stats_tail(h, l.stats, l.stream));
+        if (e == cudaSuccess) al(cudaStreamSynchronize(l.stream));
         if (e != cudaSuccess) {
             free_lane(l);
             h->lanes.pop_back();
@@ -905,27 +1005,12 @@ dtws_status ensure_lanes(dtws_t h, int count, int m_min) {
             }
             break;  // fewer lanes than asked: use what fits
         }
-        // statistics slots must hold finite values beyond N (bulk copies read whole tiles)
-        CK(cudaMemset(l.stats.mu_hi, 0, need_cap * 4));
-        CK(cudaMemset(l.stats.mu_lo, 0, need_cap * 4));
-        CK(cudaMemset(l.stats.inv_sigma, 0, need_cap * 4));
-        CK(cudaMemset(l.stats.smu_hi, 0, scap * 4));
-        CK(cudaMemset(l.stats.sinv_sigma, 0, scap * 4));
     }
     return DTWS_OK;
 }
 
 QueryBufs lane_bufs(dtws_t h, const Lane &l, const EnvEntry *ee) {
-    QueryBufs b = make_bufs(h, &l.stats, ee);
-    b.st = l.st;
-    b.qh32 = l.qh32;
-    b.qh64 = l.qh64;
-    b.Uq = l.Uq;
-    b.Lq = l.Lq;
-    b.ord = l.ord;
-    b.sq = l.sq;
-    b.sU = l.sU;
-    b.sL = l.sL;
+    QueryBufs b = make_bufs(h, &l.stats, ee);  // (the caller sets the query's own state and buffers)
     b.cand_lb = l.cand_lb;
     b.sort_lb = l.sort_lb;
     b.cand_idx = l.cand_idx;
@@ -940,63 +1025,66 @@ dtws_status ensure_batch(dtws_t h, int nq, int64_t sum_m, long long pool_cap) {
         if (h->bq_st) {
             CK(cudaDeviceSynchronize());
             drop_graph(h);
-            cudaFree(h->bq_st);
-            cudaFree(h->pq_dev);
-            cudaFree(h->plist_dev);
+            cudaFree(h->bq_block);
+            h->bq_block = nullptr;
             h->bq_st = nullptr;
             h->pq_dev = nullptr;
             h->plist_dev = nullptr;
             h->bq_cap = h->pq_cap = 0;
         }
-        CK(dalloc(&h->bq_st, (size_t)nq));
-        CK(dalloc(&h->pq_dev, (size_t)nq));
-        CK(dalloc(&h->plist_dev, (size_t)nq));
+        Arena a;
+        const size_t st = a.take<QueryState>(nq), pq = a.take<PoolQuery>(nq), pl = a.take<int>(nq);
+        CK(a.alloc());
+        h->bq_block = a.base;
+        h->bq_st = a.at<QueryState>(st);
+        h->pq_dev = a.at<PoolQuery>(pq);
+        h->plist_dev = a.at<int>(pl);
         h->bq_cap = h->pq_cap = nq;
     }
     if (h->bq_fcap < sum_m) {
         if (h->bq_f) {
             CK(cudaDeviceSynchronize());
             drop_graph(h);
-            cudaFree(h->bq_f);
-            cudaFree(h->bq_d);
-            cudaFree(h->bq_o);
+            cudaFree(h->bqf_block);
+            h->bqf_block = nullptr;
             h->bq_f = nullptr;
             h->bq_d = nullptr;
             h->bq_o = nullptr;
             h->bq_fcap = 0;
         }
-        CK(dalloc(&h->bq_f, (size_t)sum_m * 6));
-        CK(dalloc(&h->bq_d, (size_t)sum_m));
-        CK(dalloc(&h->bq_o, (size_t)sum_m));
+        Arena a;
+        const size_t f = a.take<float>((size_t)sum_m * 6), d = a.take<double>(sum_m), o = a.take<unsigned short>(sum_m);
+        CK(a.alloc());
+        h->bqf_block = a.base;
+        h->bq_f = a.at<float>(f);
+        h->bq_d = a.at<double>(d);
+        h->bq_o = a.at<unsigned short>(o);
         h->bq_fcap = sum_m;
     }
     if (h->pool.cap != pool_cap && (h->pool.cap < pool_cap || h->pool_limit >= 0)) {
         if (h->pool.idx || h->pool.cap) {
             CK(cudaDeviceSynchronize());
             drop_graph(h);
-            void *ptrs[] = {h->pool.idx, h->pool.lb, h->pool.mh, h->pool.is, h->pool.ls, h->pool.cursor};
-            for (void *p : ptrs) cudaFree(p);
+            cudaFree(h->pool_block);
+            h->pool_block = nullptr;
             h->pool = SurvPool{};
         }
         if (pool_cap <= 0) return DTWS_OK;  // no pool: every query keeps its survivors
         SurvPool p{};
-        cudaError_t e = cudaSuccess;
-        auto al = [&](cudaError_t r) {
-            if (e == cudaSuccess) e = r;
-        };
-        al(dalloc(&p.idx, (size_t)pool_cap));
-        al(dalloc(&p.lb, (size_t)pool_cap));
-        al(dalloc(&p.mh, (size_t)pool_cap));
-        al(dalloc(&p.is, (size_t)pool_cap));
-        al(dalloc(&p.ls, (size_t)pool_cap));
-        al(dalloc(&p.cursor, 1));
-        if (e != cudaSuccess) {
-            void *ptrs[] = {p.idx, p.lb, p.mh, p.is, p.ls, p.cursor};
-            for (void *q : ptrs)
-                if (q) cudaFree(q);
+        Arena a;
+        const size_t idx = a.take<unsigned>(pool_cap), lb = a.take<float>(pool_cap), mh = a.take<float>(pool_cap),
+                     is = a.take<float>(pool_cap), ls = a.take<float>(pool_cap), cu = a.take<unsigned long long>(1);
+        if (a.alloc() != cudaSuccess) {
             cudaGetLastError();
             return DTWS_OK;  // no pool: every query keeps its survivors (h->pool.cap stays 0)
         }
+        h->pool_block = a.base;
+        p.idx = a.at<unsigned>(idx);
+        p.lb = a.at<float>(lb);
+        p.mh = a.at<float>(mh);
+        p.is = a.at<float>(is);
+        p.ls = a.at<float>(ls);
+        p.cursor = a.at<unsigned long long>(cu);
         p.cap = pool_cap;
         h->pool = p;
     }
@@ -1023,14 +1111,13 @@ dtws_status run_batch(dtws_t h, const float *Qd, const int64_t *q_off, const int
     dtws_status st;
     const bool learned = h->opt.seed_proposals > 0 && h->opt.ordering == DTWS_ORDER_LEARNED;
     const int nl = std::max(1, std::min<int>(h->opt.batch_lanes, nq));
-    int m_min = m_arr[0];
     int64_t sum_m = 0, sum_N = 0;
     for (int q = 0; q < nq; ++q) {
-        m_min = std::min<int>(m_min, m_arr[q]);
         sum_m += m_arr[q];
         sum_N += h->n - m_arr[q] + 1;
     }
-    if ((st = ensure_lanes(h, nl, m_min)) != DTWS_OK) return st;
+    use_caches(h, s);  // (the lanes fork from s and join into it)
+    if ((st = ensure_lanes(h, nl)) != DTWS_OK) return st;
     long long pool_want = std::min<long long>(1ll << 27, std::max<long long>(1, sum_N));
     if (h->pool_limit >= 0) pool_want = h->pool_limit;
     if ((st = ensure_batch(h, nq, sum_m, pool_want)) != DTWS_OK) return st;
@@ -1325,10 +1412,8 @@ dtws_status dtws_destroy(dtws_t h) {
     for (auto &l : h->lanes) free_lane(l);
     if (h->batch_fork) cudaEventDestroy(h->batch_fork);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-    void *ptrs[] = {h->x, h->x_sub, h->pf, h->bf, h->pok, h->pscale, h->envst, h->absmax, h->st, h->status, h->qh32, h->Uq,
-                    h->Lq, h->sq, h->sU, h->sL, h->qh64, h->ord, h->cand_lb, h->sort_lb,
-                    h->cand_idx, h->sort_idx, h->stage, h->xz_buf, h->xz_sel, h->xz_d64, h->bq_st, h->bq_f, h->bq_d, h->bq_o, h->pool.idx,
-                    h->pool.lb, h->pool.mh, h->pool.is, h->pool.ls, h->pool.cursor, h->pq_dev, h->plist_dev};
+    void *ptrs[] = {h->block, h->work_block, h->cand_block, h->stage, h->xz_buf, h->xz_sel, h->xz_d64, h->bq_block,
+                    h->bqf_block, h->pool_block};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->hstage) cudaFreeHost(h->hstage);
@@ -1370,16 +1455,25 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
     h->n = n;
     h->n_alloc = round_up(n, kProxyTile) + kMMax + 64;
     const int64_t nb = (n + kBlockB - 1) / kBlockB;
-    CKF(dalloc(&h->x, h->n_alloc));
-    CKF(dalloc(&h->x_sub, h->n_alloc / kProxyStride + kProxyTile));
-    CKF(dalloc(&h->pf, 4 * prefix_stride(n)));
-    CKF(dalloc(&h->bf, 5 * nb));
-    CKF(dalloc(&h->pok, nb));
-    CKF(dalloc(&h->pscale, 2));
     h->nblk = (n + kEnvG - 1) / kEnvG;
-    CKF(dalloc(&h->envst, 2 * (size_t)kEnvLevels * h->nblk));
-    CKF(dalloc(&h->status, 1));
-    CKF(dalloc(&h->absmax, 1));
+    {
+        Arena ar;
+        const size_t x = ar.take<float>(h->n_alloc), xs = ar.take<float>(h->n_alloc / kProxyStride + kProxyTile),
+                     pf = ar.take<float>(4 * prefix_stride(n)), bf = ar.take<float>(5 * nb), ok = ar.take<int>(nb),
+                     sc = ar.take<float>(2), es = ar.take<float>(2 * (size_t)kEnvLevels * h->nblk), st = ar.take<int>(1),
+                     am = ar.take<unsigned>(1);
+        CKF(ar.alloc());
+        h->block = ar.base;
+        h->x = ar.at<float>(x);
+        h->x_sub = ar.at<float>(xs);
+        h->pf = ar.at<float>(pf);
+        h->bf = ar.at<float>(bf);
+        h->pok = ar.at<int>(ok);
+        h->pscale = ar.at<float>(sc);
+        h->envst = ar.at<float>(es);
+        h->status = ar.at<int>(st);
+        h->absmax = ar.at<unsigned>(am);
+    }
     // the pads past the series are zero (tile readers read whole tiles)
     const int64_t sub_n = h->n_alloc / kProxyStride + kProxyTile, sub_written = prefix_stride(n) / kProxyStride;
     CKF(cudaMemsetAsync(h->x + n, 0, (size_t)(h->n_alloc - n) * 4, s));
