@@ -39,4 +39,33 @@ __device__ __forceinline__ void f3_add_sq(f3 &t, float h, float l) {
 }
 __device__ __forceinline__ double f3_value(const f3 &t) { return ((double)t.c + (double)t.b) + (double)t.a; }
 
+// Mean (FP64) and variance of n samples y over `threads` threads' shares
+// (start t, stride `threads`): each thread's part is summed in FP32 expansions,
+// the parts in FP64 by `reduce` (the same result in every thread) -- two-pass,
+// no less exact than FP64 sums throughout and not bound by this part's FP64
+// rate.  Sums that overflow FP32 are taken again on samples scaled by 2^-80.
+// (None underflows that matters: a variance below 1e-24 counts as none.)
+template <typename Reduce>
+__device__ __forceinline__ void mean_and_variance(const float *__restrict__ y, int n, int t, int threads, Reduce &&reduce,
+                                                  double &mu, double &var) {
+    float f = 1.0f;
+    for (;;) {
+        f3 s{0.0f, 0.0f, 0.0f};
+        for (int j = t; j < n; j += threads) f3_add(s, __fmul_rn(y[j], f), 0.0f);
+        mu = reduce(f3_value(s)) / (double)n;
+        const float mh = (float)mu, ml = (float)(mu - (double)mh);
+        f3 v{0.0f, 0.0f, 0.0f};
+        for (int j = t; j < n; j += threads) {
+            exact2 d = two_sum_rn(__fmul_rn(y[j], f), -mh);
+            d = two_sum_rn(d.s, __fsub_rn(d.e, ml));
+            f3_add_sq(v, d.s, d.e);
+        }
+        var = reduce(f3_value(v)) / (double)n;
+        if (isfinite(var) || f < 1.0f) break;
+        f = 0x1p-80f;
+    }
+    mu *= f < 1.0f ? 0x1p80 : 1.0;
+    var *= f < 1.0f ? 0x1p160 : 1.0;
+}
+
 }  // namespace dtws

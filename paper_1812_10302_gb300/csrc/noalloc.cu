@@ -47,26 +47,6 @@ static __device__ __align__(256) float g_noalloc_scratch[kNoAllocFloats];
 namespace dtws {
 namespace {
 
-// Mean (FP64) and deviation of n samples y over `threads` threads' shares
-// (start t, stride `threads`): each thread's part is summed in FP32 expansions
-// (fp_sum.cuh), the parts in FP64 by `reduce` -- two-pass, no less exact than
-// FP64 sums throughout and not bound by this part's FP64 rate.
-template <typename Reduce>
-__device__ __forceinline__ void mean_and_variance(const float *__restrict__ y, int n, int t, int threads, Reduce &&reduce,
-                                                  double &mu, double &var) {
-    f3 s{0.0f, 0.0f, 0.0f};
-    for (int j = t; j < n; j += threads) f3_add(s, y[j], 0.0f);
-    mu = reduce(f3_value(s)) / (double)n;
-    const float mh = (float)mu, ml = (float)(mu - (double)mh);
-    f3 v{0.0f, 0.0f, 0.0f};
-    for (int j = t; j < n; j += threads) {
-        exact2 d = two_sum_rn(y[j], -mh);
-        d = two_sum_rn(d.s, __fsub_rn(d.e, ml));
-        f3_add_sq(v, d.s, d.e);
-    }
-    var = reduce(f3_value(v)) / (double)n;
-}
-
 // z-normalise Q into scratch[0, m) (Sec. 2.2, Eq. 5, two-pass, same
 // zero-variance rule as the search) and reset the work cursor.  A
 // non-finite query leaves a NaN in scratch[0] so the DTW kernel writes NaN.

@@ -53,3 +53,24 @@ def test_bad_device_offsets_give_nan(series):
         for r in (2, 12, 100):
             got = ix.dtw_at(q, r, offs)
             np.testing.assert_array_equal(np.isnan(got), [False, True, True, False, True])
+
+
+@pytest.mark.parametrize("scale", [1e-8, 1e30, 3e35])
+def test_without_allocations_in_any_units(series, scale):
+    """Values whose squares, and sums, leave FP32's range: normalisation takes
+    the units off, so the distances are those of the series in plain units
+    (each value off by an ulp of itself, as in the 1e-4 above)."""
+    import torch
+    q, _ = synth.noisy_copy(series, 128, 9, 11, noise=0.3)
+    offs = np.random.default_rng(3).integers(0, series.size - 127, 40)
+    xs = (series.astype(np.float64) * scale).astype(np.float32)
+    qs = (q.astype(np.float64) * scale).astype(np.float32)
+    assert np.isfinite(xs).all()
+    for r in (3, 12):
+        want = oracle.dtw_at(xs.astype(np.float64) / scale, qs.astype(np.float64) / scale, r, offs)
+        xd, qd, od = (torch.from_numpy(a).cuda() for a in (xs, qs, offs))
+        out = torch.empty(offs.size, device="cuda")
+        st = dtws.load().dtws_dtw_at_noalloc(xd.data_ptr(), series.size, qd.data_ptr(), 128, r, od.data_ptr(),
+                                             offs.size, out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert st == dtws.DTWS_OK
+        np.testing.assert_allclose(out.cpu().numpy(), want, rtol=1e-4, atol=1e-6 * 128)
