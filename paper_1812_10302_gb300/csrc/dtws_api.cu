@@ -369,7 +369,7 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
     }
     e.m = m;
     const cudaError_t ce = launch_window_stats(h->x, h->n, m, h->pf, h->bf, h->pok, h->pscale, e.mu_hi, e.mu_lo,
-                                               e.inv_sigma, e.smu_hi, e.sinv_sigma, h->num_sms, s);
+                                               e.inv_sigma, e.smu_hi, e.sinv_sigma, s);
     if (ce != cudaSuccess) {  // nothing half-initialised stays in the cache
         free_stats(e);
         cudaGetLastError();
@@ -1261,8 +1261,7 @@ dtws_status run_batch(dtws_t h, const float *Qd, const int64_t *q_off, const int
         const int m = m_arr[q];
         if (lane_m[li] != m) {
             CKB(launch_window_stats(h->x, h->n, m, h->pf, h->bf, h->pok, h->pscale, l.stats.mu_hi, l.stats.mu_lo,
-                                    l.stats.inv_sigma, l.stats.smu_hi, l.stats.sinv_sigma,
-                                    h->num_sms, l.stream));
+                                    l.stats.inv_sigma, l.stats.smu_hi, l.stats.sinv_sigma, l.stream));
             lane_m[li] = m;
             ++launches;
         }

@@ -31,7 +31,7 @@ cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *
                           float *scale, cudaStream_t s);
 cudaError_t launch_window_stats(const float *x, int64_t n, int m, const float *pf, const float *bf,
                                 const int *ok, const float *scale, float *mu_hi, float *mu_lo, float *inv_sigma,
-                                float *smu_hi, float *sinv_sigma, int num_sms, cudaStream_t s);
+                                float *smu_hi, float *sinv_sigma, cudaStream_t s);
 cudaError_t launch_envelope(const float *x, int64_t n, int r, float *U, float *L, cudaStream_t s);
 // block envelope: st = [max levels 0..kEnvLevels-1 | min levels], nblk floats
 // each; levels 1.. from level 0

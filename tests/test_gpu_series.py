@@ -51,3 +51,31 @@ def test_non_finite_sample_is_refused_wherever_it_is(n, at):
     with pytest.raises(dtws.DtwsError) as e:
         dtws.Index(x)
     assert e.value.status == dtws.DTWS_ENONFINITE
+
+
+@pytest.mark.parametrize("n", [1024, 8192, 8197, 20001])
+@pytest.mark.parametrize("m", [2, 3, 5, 6, 511, 1022, 1024])
+def test_statistics_of_every_remainder(n, m):
+    """Two windows a thread, every fourth window kept: every remainder of m and of
+    the window count by four, windows that end with a block and with the series."""
+    x = synth.random_walk(n, 80 + n + m)
+    with dtws.Index(x) as ix:
+        mh, ml, inv = ix.window_stats(m)
+    mu, sg = oracle.window_stats(x, m, "twopass")
+    got = mh.astype(np.float64) + ml.astype(np.float64)
+    nz = sg > 0.0
+    np.testing.assert_array_equal(inv == 0.0, ~nz)
+    assert np.all(np.abs(got[nz] - mu[nz]) <= 1e-7 * sg[nz] + 1e-12 * np.abs(mu[nz]))
+    assert np.abs(inv[nz].astype(np.float64) * sg[nz] - 1.0).max() <= 2.0 ** -22
+
+
+@pytest.mark.parametrize("n", [2, 4095, 4097, 20_003])
+@pytest.mark.parametrize("r", [0, 1, 2, 3, 4, 5, 6, 7, 9, 16, 31, 100, 1023, 4096, 8191])
+def test_envelope_of_every_remainder(n, r):
+    """The group split at every remainder of r, tiles past the series' end."""
+    x = synth.random_walk(n, 90 + n)
+    with dtws.Index(x) as ix:
+        U, L = ix.series_envelope(r)
+    Uo, Lo = oracle.series_envelope(x, r)
+    np.testing.assert_array_equal(U, Uo)
+    np.testing.assert_array_equal(L, Lo)
