@@ -9,12 +9,21 @@ namespace dtws {
 // One window's re-score is pure latency: 2m - 1 dependent anti-diagonals.  In
 // double-float (dtw_diag_df) a step costs ~41 instructions per cell, most of
 // them the cell's cost, and one warp issued them all: 262 cycles per step at
-// r = 51.  Here the CTA splits the work.  Eleven producer warps form the costs
-// (q_hat_i - c_j)^2 of the coming anti-diagonals in double-float, as before,
-// turn each into a 64-bit integer and leave it in a shared-memory ring; one
-// consumer warp walks: per cell two integer minima and one addition (10
-// instructions), per step one neighbour exchange by shuffle.  The two
-// halves meet at a named barrier every kFxSteps anti-diagonals.
+// r = 51.  Three things split the work.
+//   * Producer warps form the costs (q_hat_i - c_j)^2 of the coming
+//     anti-diagonals in double-float, as before, turn each into a 64-bit
+//     integer and leave it in a shared-memory ring; consumer warps walk: per
+//     cell two integer minima and one addition (10 instructions), per step one
+//     neighbour exchange by shuffle.  The two halves meet at a named barrier
+//     every chunk of anti-diagonals.
+//   * Integer sums do not depend on their order, so the matrix is walked from
+//     both ends at once, by the two CTAs of a cluster (the second one on the
+//     reversed sequences), and the best path is the best way of joining the
+//     two middle anti-diagonals: half the steps, the same result to the bit.
+//   * Bands past one warp's cells (four a lane: r > 126) take W consumer warps
+//     whose cells overlap by one lane on each side.  In kFxUnit = 8 steps an
+//     error at a warp's edge travels four cells, one lane; then the overlap is
+//     taken anew from the neighbours (one exchange per chunk).
 //
 // The fixed point: with an upper bound U of the DTW (the caller's, or the
 // diagonal path's cost) no partial sum above U lies on the best path.
@@ -29,45 +38,86 @@ namespace dtws {
 // with the same bound (or with the diagonal's) score identically when their
 // values are identical.
 //
-// Measured, dtws_dtw_at_f64 of one window, whole call: 105 us at m = 512,
-// r = 51 (164 us before), 210 us at m = 1024, r = 102 (412 us); bound by the
-// consumer's ALU issue (25 cycles per cell of a lane) past two cells per lane.
-constexpr int kFxThreads = 384, kFxWarps = kFxThreads / 32, kFxSteps = 16, kFxUnit = 8;
+// Measured, dtws_dtw_at_f64 of one window, whole call: 76 us at m = 512,
+// r = 51 (105 us walked from one end, 164 us in double-float), 132 us at
+// m = 1024, r = 102 (210, 412), 170 us at r = 200 (311, 513); bound by the
+// consumers' ALU issue (25 cycles per cell of a lane) past two cells per lane,
+// and on several warps by the producers' beside it.
+constexpr int kFxUnit = 8, kFxRMax = 1023, kFxClusterCtas = 2;
 // a saturated cost; the value saturated sums are set back to every kFxUnit
 // steps (kFxInf + kFxUnit * kFxCost < 2^64, so no sum wraps in between)
 constexpr unsigned long long kFxCost = 1ull << 60, kFxInf = 1ull << 61, kFxRedo = 1ull << 51;
 
-// Cells per lane: 32 K >= r + 2, so the last cell of every anti-diagonal lies
-// past the band and is always saturated; the neighbour exchange may then wrap
-// around the warp without a special case.
-__host__ __device__ inline int fx_cells(int r) {
-    const int need = (r + 2 + 31) / 32;
-    return need <= 4 ? need : need <= 6 ? 6 : 8;
+// A walk's shape: K cells per lane, W consumer warps.
+template <int K_, int W_>
+struct Fx {
+    static constexpr int K = K_, W = W_;
+    static constexpr int kThreads = W == 1 ? 384 : 768, kWarps = kThreads / 32;
+    static constexpr int kSteps = W == 1 ? 16 : kFxUnit;   // anti-diagonals of a chunk
+    static constexpr int kLanes = W == 1 ? 32 : 30 * W + 2;  // lanes without the overlaps
+    static constexpr int kCells = K * kLanes;
+    static constexpr int kStep = ((K + 1) / 2) * kLanes * 2;  // words of a step in the ring
+    static constexpr size_t kRing = (size_t)2 * kSteps * kStep * 8;
+    static_assert(W == 1 || K == 4, "an overlap is one lane and lasts kFxUnit steps");
+};
+
+// kCells >= r + 2, so the last cell of every anti-diagonal lies past the band
+// and is always saturated: the neighbour exchange may then wrap around the
+// warp without a special case at the upper end.
+#define DTWS_FX_SHAPES(X) X(1, 1) X(2, 1) X(3, 1) X(4, 1) X(4, 2) X(4, 3) X(4, 4) X(4, 6) X(4, 9)
+struct FxPlan {
+    int K, W, threads;
+    size_t ring;
+};
+__host__ __device__ inline FxPlan fx_plan(int r) {
+#define DTWS_FX_TRY(KK, WW) \
+    if (Fx<KK, WW>::kCells >= r + 2) return FxPlan{KK, WW, Fx<KK, WW>::kThreads, Fx<KK, WW>::kRing};
+    DTWS_FX_SHAPES(DTWS_FX_TRY)
+#undef DTWS_FX_TRY
+    return FxPlan{0, 0, 0, 0};
 }
-constexpr int kFxRMax = 254;  // 32 * 8 - 2
-__host__ __device__ constexpr size_t fx_ring_bytes(int K) {
-    return (size_t)2 * kFxSteps * ((K + 1) / 2) * 32 * 16;
-}
-// Padding on each side of the query's and the window's double-floats: the
-// producers' positions run to r/2 + 32 K + kFxSteps past either end.
-__host__ __device__ inline int fx_pad(int r, int K) { return ((r >> 1) + 32 * K + kFxSteps + 4) & ~1; }
-__host__ __device__ inline size_t fx_span(int m, int r, int K) { return (size_t)((m + 2 * fx_pad(r, K) + 1) & ~1); }
+// Padding on each side of the query's and the window's double-floats: a
+// producer's positions run to r/2 + 1 before either start and, on the last
+// chunk's steps past the middle, at most 12 past either end.
+__host__ __device__ inline int fx_pad(int r) { return ((r >> 1) + 20) & ~1; }
+__host__ __device__ inline size_t fx_span(int m, int r) { return (size_t)((m + 2 * fx_pad(r) + 1) & ~1); }
 // shared memory of one window: the ring, the query's and the window's padded double-floats
-__host__ __device__ inline size_t fx_bytes(int m, int r, int K) { return fx_ring_bytes(K) + fx_span(m, r, K) * 16; }
-// whether a search re-scores with this walk (the pre-score needs its FP32
-// walk's padded copies beside it): one rule for the pre-score and the final
-// stage, so that equal windows are compared on equal terms
+__host__ __device__ inline size_t fx_bytes(int m, int r) { return fx_plan(r).ring + fx_span(m, r) * 16; }
+// whether a search re-scores with this walk: one rule for the pre-score and
+// the final stage, so that equal windows are compared on equal terms
 __host__ __device__ inline bool fx_used(int m, int r) {
-    if (r > kFxRMax) return false;
-    const int K = fx_cells(r);
-    return fx_bytes(m, r, K) + (size_t)((m + 2 * diag_pad(r, 32, K) + 3) & ~3) * 8 <= (size_t)216 * 1024;
+    return r <= kFxRMax && fx_bytes(m, r) <= (size_t)216 * 1024;
 }
 
 struct FxShared {
-    float red[kFxWarps];
+    float red[24];
     unsigned long long res;
+    ulonglong2 edge[2][9][2][4];  // [chunk parity][warp][lower, upper edge][p1's two pairs, p2's two pairs]
     double mu, inv;
 };
+
+// The cluster's barrier and its peer's shared memory.
+__device__ __forceinline__ int cluster_rank() {
+    int v;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
+    return v;
+}
+__device__ __forceinline__ void cluster_bar() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ unsigned peer_addr(const void *p, int rank) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), v;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(v) : "r"(a), "r"(rank));
+    return v;
+}
+__device__ __forceinline__ unsigned long long peer_load(unsigned a) {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void peer_store(unsigned a, unsigned long long v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
 
 __device__ __forceinline__ unsigned long long fx_min(unsigned long long x, unsigned long long y) {
     return x < y ? x : y;
@@ -104,14 +154,15 @@ __device__ __forceinline__ unsigned long long fx_round(float hi, float lo) {
 // -1e15): a cell outside [0, m)^2 comes out far above 2^59, as do sums that
 // overflow, and everything not below 2^59 becomes kFxCost.  dst: the steps'
 // ring slots.
-template <int K>
+template <typename S>
 __device__ __forceinline__ void fx_produce(const dfloat *qd, const dfloat *cd, int r, float f, int v0, int blk,
                                            unsigned long long *dst, int lane) {
-    constexpr int kStep = ((K + 1) / 2) * 64;  // words of a step
     const int p = blk * 32 + lane, a = v0 - (r & 1);
-    const dfloat *qp = qd + (((a + r) >> 1) - p), *cp = cd + (((a - r) >> 1) + p);
-    const int pl = p / K, pt = p - pl * K;
-    unsigned long long *o = dst + ((pt >> 1) * 32 + pl) * 2 + (pt & 1);
+    if (S::kCells % 32 && p >= S::kCells) return;
+    const int pc = p < r ? p : r;  // (past the band no cost counts, and no address either)
+    const dfloat *qp = qd + (((a + r) >> 1) - pc), *cp = cd + (((a - r) >> 1) + pc);
+    const int pl = p / S::K, pt = p - pl * S::K;
+    unsigned long long *o = dst + ((pt >> 1) * S::kLanes + pl) * 2 + (pt & 1);
     const bool in0 = p <= r, in1 = p < r;  // cells of an even, of an odd step
     dfloat c = cp[0];
 #pragma unroll
@@ -126,24 +177,27 @@ __device__ __forceinline__ void fx_produce(const dfloat *qd, const dfloat *cd, i
             const float er = fmaf(h + h, l, fmaf(h, h, -sq));
             const bool fine = (e ? in1 : in0) && sq < 0x1p59f;
             const unsigned long long w = fx_round(sq, er);
-            o[(s + e) * kStep] = fine ? w : kFxCost;
+            o[(s + e) * S::kStep] = fine ? w : kFxCost;
         }
     }
 }
 
-// One anti-diagonal of the walk: cell t of the lane (as diag_step).
-template <int K, int ODD>
-__device__ __forceinline__ void fx_step(const unsigned long long *buf, unsigned long long (&p1)[K],
-                                        unsigned long long (&p2)[K], int lane) {
+// One anti-diagonal of the walk: cell t of the lane (as diag_step).  vl: the
+// lane's place on the anti-diagonal.
+template <typename S, int ODD>
+__device__ __forceinline__ void fx_step(const unsigned long long *buf, unsigned long long (&p1)[S::K],
+                                        unsigned long long (&p2)[S::K], int lane, int vl) {
+    constexpr int K = S::K;
     unsigned long long cost[((K + 1) / 2) * 2];
 #pragma unroll
     for (int t = 0; t < (K + 1) / 2; ++t) {
-        const ulonglong2 c = reinterpret_cast<const ulonglong2 *>(buf)[t * 32 + lane];
+        const ulonglong2 c = reinterpret_cast<const ulonglong2 *>(buf)[t * S::kLanes + vl];
         cost[2 * t] = c.x;
         cost[2 * t + 1] = c.y;
     }
-    const unsigned long long nb =
+    unsigned long long nb =
         __shfl_sync(0xffffffffu, ODD ? p1[0] : p1[K - 1], ODD ? ((lane + 1) & 31) : ((lane - 1) & 31));
+    if (S::W > 1 && !ODD) nb = vl == 0 ? kFxInf : nb;  // (the first warp's last lane is not the band's end)
     unsigned long long cur[K];
 #pragma unroll
     for (int t = 0; t < K; ++t) {
@@ -170,140 +224,214 @@ __device__ __forceinline__ void fx_clamp(unsigned long long (&v)[K]) {
     }
 }
 
-// The walk by the kFxThreads threads t = 0.. of a group that owns named
-// barrier `bar`.  qd, cd: element 0 of q_hat and of the normalised window as
-// double-floats, padded by fx_pad(r, K) elements of +1e15 and -1e15 on both
+// The walk by the S::kThreads threads of each of a cluster's two CTAs (all
+// of them).  dir: the CTA's rank, 1 for the reversed sequences.  qd, cd:
+// element 0 of q_hat and of the normalised window as double-floats (reversed
+// when dir is 1), padded by fx_pad(r) elements of +1e15 and -1e15 on both
 // sides; bound: an upper bound of the DTW, 0 for the diagonal path's cost;
-// ring: fx_ring_bytes(K), 16-byte aligned.  Every thread returns
+// ring: S::kRing bytes, 16-byte aligned.  Every thread of both CTAs returns
 // the distance.
-template <int K>
+template <typename S>
 __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict__ cd, int m, int r, float bound,
-                         int t, FxShared &sh, unsigned long long *ring, int bar) {
-    const int lane = t & 31, warp = t >> 5;
-    constexpr int kStep = ((K + 1) / 2) * 64;  // words of a step
-    // the diagonal path's cost, an upper bound of the DTW (the same sum in every thread)
+                         int dir, FxShared &sh, unsigned long long *ring) {
+    constexpr int K = S::K, W = S::W;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // the diagonal path's cost, an upper bound of the DTW (the same sum, in
+    // the same order, in every thread of both CTAs)
     auto euclid = [&]() {
         float ed = 0.0f;
-        for (int j = t; j < m; j += kFxThreads) {
-            const float d = df_sub(qd[j], cd[j]).hi;
+        for (int j = t; j < m; j += S::kThreads) {
+            const int i = dir ? m - 1 - j : j;
+            const float d = df_sub(qd[i], cd[i]).hi;
             ed = fmaf(d, d, ed);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ed += __shfl_xor_sync(0xffffffffu, ed, o);
         if (lane == 0) sh.red[warp] = ed;
-        group_bar(bar, kFxThreads);
+        __syncthreads();
         ed = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kFxWarps; ++w) ed += sh.red[w];
-        group_bar(bar, kFxThreads);  // (sh.red is read before it is written again)
+        for (int w = 0; w < S::kWarps; ++w) ed += sh.red[w];
+        __syncthreads();  // (sh.red is read before it is written again)
         return ed;
     };
     auto scale_of = [](float bound) { return (58 - (ilogbf(bound * 1.001f) + 1)) >> 1; };
     if (!(bound > 0.0f && bound < 1e30f)) bound = euclid();
     if (!(bound > 0.0f)) return 0.0;  // (the Euclidean distance is 0)
     int h = scale_of(bound);          // the scale is 2^(2h)
-    const int V = 2 * m - 1 + (r & 1), chunks = (V + kFxSteps - 1) / kFxSteps;
-    const int p0 = (r - (r & 1)) >> 1, last = 2 * m - 2, pe = (r - ((last + r) & 1)) >> 1;
+    // the forward walk ends on anti-diagonal m - 1, the reversed one on the
+    // next (its own m - 2)
+    const int V = m - dir + (r & 1), chunks = (V + S::kSteps - 1) / S::kSteps;
+    const int p0 = (r - (r & 1)) >> 1;
+    const int vl = W == 1 ? lane : warp * 30 + lane;
+    // the lanes whose cells are this warp's own
+    const bool own = warp < W && (warp == 0 || lane > 0) && (warp == W - 1 || lane < 31);
     for (int pass = 0;; ++pass) {
         const float f = ldexpf(1.0f, h);
         // a chunk's units: kFxUnit steps of one block of 32 cells each
+        constexpr int kBlks = (S::kCells + 31) / 32;
         auto produce = [&](int c, int w, int nw) {
-            unsigned long long *buf = ring + (size_t)(c & 1) * kFxSteps * kStep;
-            for (int u = w; u < K * (kFxSteps / kFxUnit); u += nw) {
-                const int blk = u % K, s0 = u / K * kFxUnit;
-                fx_produce<K>(qd, cd, r, f, c * kFxSteps + s0, blk, buf + s0 * kStep, lane);
+            unsigned long long *buf = ring + (size_t)(c & 1) * S::kSteps * S::kStep;
+            for (int u = w; u < kBlks * (S::kSteps / kFxUnit); u += nw) {
+                const int blk = u % kBlks, s0 = u / kBlks * kFxUnit;
+                fx_produce<S>(qd, cd, r, f, c * S::kSteps + s0, blk, buf + s0 * S::kStep, lane);
             }
         };
-        produce(0, warp, kFxWarps);
-        group_bar(bar, kFxThreads);
+        produce(0, warp, S::kWarps);
+        __syncthreads();
         unsigned long long p1[K], p2[K];
 #pragma unroll
         for (int u = 0; u < K; ++u) {
             // the base cell lies on anti-diagonal -2: two steps before v = 0
             // when r is even, one before when r is odd
-            const unsigned long long base = lane * K + u == p0 ? 0ull : kFxInf;
+            const unsigned long long base = vl * K + u == p0 ? 0ull : kFxInf;
             p1[u] = (r & 1) ? base : kFxInf;
             p2[u] = (r & 1) ? kFxInf : base;
         }
         for (int c = 0; c < chunks; ++c) {
-            const unsigned long long *buf = ring + (size_t)(c & 1) * kFxSteps * kStep;
-            if (warp == 0) {
-                const int steps = V - c * kFxSteps < kFxSteps ? V - c * kFxSteps : kFxSteps;
-                if (steps == kFxSteps) {
+            const unsigned long long *buf = ring + (size_t)(c & 1) * S::kSteps * S::kStep;
+            if (warp < W) {
+                const int steps = V - c * S::kSteps < S::kSteps ? V - c * S::kSteps : S::kSteps;
+                if (steps == S::kSteps) {
 #pragma unroll 1
-                    for (int s0 = 0; s0 < kFxSteps; s0 += kFxUnit) {
+                    for (int s0 = 0; s0 < S::kSteps; s0 += kFxUnit) {
 #pragma unroll
                         for (int s = s0; s < s0 + kFxUnit; s += 2) {
-                            fx_step<K, 0>(buf + s * kStep, p1, p2, lane);
-                            fx_step<K, 1>(buf + (s + 1) * kStep, p1, p2, lane);
+                            fx_step<S, 0>(buf + s * S::kStep, p1, p2, lane, vl);
+                            fx_step<S, 1>(buf + (s + 1) * S::kStep, p1, p2, lane, vl);
                         }
                         fx_clamp<K>(p1);
                         fx_clamp<K>(p2);
                     }
                 } else {
                     for (int s = 0; s < steps; s += 2) {
-                        fx_step<K, 0>(buf + s * kStep, p1, p2, lane);
-                        if (s + 1 < steps) fx_step<K, 1>(buf + (s + 1) * kStep, p1, p2, lane);
+                        fx_step<S, 0>(buf + s * S::kStep, p1, p2, lane, vl);
+                        if (s + 1 < steps) fx_step<S, 1>(buf + (s + 1) * S::kStep, p1, p2, lane, vl);
                         if ((s + 2) % kFxUnit == 0) {
                             fx_clamp<K>(p1);
                             fx_clamp<K>(p2);
                         }
                     }
                 }
+                if constexpr (W > 1) {  // the own cells beside each overlap
+                    if (lane == 1 || lane == 30) {
+                        ulonglong2 *e = sh.edge[c & 1][warp][lane == 30];
+                        e[0] = make_ulonglong2(p1[0], p1[1]);
+                        e[1] = make_ulonglong2(p1[2], p1[3]);
+                        e[2] = make_ulonglong2(p2[0], p2[1]);
+                        e[3] = make_ulonglong2(p2[2], p2[3]);
+                    }
+                }
             } else if (c + 1 < chunks) {
-                produce(c + 1, warp - 1, kFxWarps - 1);
+                produce(c + 1, warp - W, S::kWarps - W);
             }
-            group_bar(bar, kFxThreads);
+            __syncthreads();
+            if constexpr (W > 1) {
+                if ((lane == 0 && warp > 0 && warp < W) || (lane == 31 && warp < W - 1)) {
+                    const ulonglong2 *e = lane == 0 ? sh.edge[c & 1][warp - 1][1] : sh.edge[c & 1][warp + 1][0];
+                    const ulonglong2 a0 = e[0], a1 = e[1], b0 = e[2], b1 = e[3];
+                    p1[0] = a0.x;
+                    p1[1] = a0.y;
+                    p1[2] = a1.x;
+                    p1[3] = a1.y;
+                    p2[0] = b0.x;
+                    p2[1] = b0.y;
+                    p2[2] = b1.x;
+                    p2[3] = b1.y;
+                }
+                __syncwarp();
+            }
         }
-        if (warp == 0) {
+        // The join.  The reversed walk's cell p' of an even (odd) step is the
+        // forward one's r - p' (r - 1 - p').  A path goes through
+        // anti-diagonal m - 1 (p1) and then m or, diagonally, m + 1, or from
+        // m - 2 (p2) diagonally to m.
+        fx_clamp<K>(p1);
+        fx_clamp<K>(p2);
+        unsigned long long *last1 = ring, *last2 = ring + S::kCells;
+        if (t == 0) sh.res = ~0ull;
+        if (dir && own) {
 #pragma unroll
-            for (int u = 0; u < K; ++u)
-                if (lane * K + u == pe) sh.res = p1[u];
+            for (int u = 0; u < K; ++u) {
+                last1[vl * K + u] = p1[u];
+                last2[vl * K + u] = p2[u];
+            }
         }
-        group_bar(bar, kFxThreads);
+        cluster_bar();
+        if (!dir && warp < W) {
+            const bool even = ((m - 1 + r) & 1) == 0;  // anti-diagonal m - 1 is an even step
+            const unsigned a1 = peer_addr(last1, 1), a2 = peer_addr(last2, 1);
+            auto at = [](unsigned a, int j) { return j >= 0 ? peer_load(a + (unsigned)j * 8) : kFxInf; };
+            const int j1 = (even ? r - 1 : r) - vl * K, j2 = (even ? r : r - 1) - vl * K;
+            unsigned long long best = ~0ull;
+            if (own) {
+                // anti-diagonal m: the cells beside cell u are u - 1 and u
+                // when m - 1 is an even step, u and u + 1 when it is odd
+                unsigned long long n[K + 1];
+#pragma unroll
+                for (int u = 0; u <= K; ++u) {
+                    const int p = vl * K + u - (even ? 1 : 0);
+                    n[u] = p >= 0 ? at(a1, j1 - (p - vl * K)) : kFxInf;
+                }
+#pragma unroll
+                for (int u = 0; u < K; ++u) {
+                    const unsigned long long d = even ? n[u + 1] : n[u];
+                    best = fx_min(best, p1[u] + fx_min(fx_min(n[u], n[u + 1]), at(a2, j2 - u)));
+                    best = fx_min(best, p2[u] + d);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) best = fx_min(best, __shfl_xor_sync(0xffffffffu, best, o));
+            if (lane == 0) atomicMin(&sh.res, best);
+        }
+        __syncthreads();
+        if (!dir && t == 0) peer_store(peer_addr(&sh.res, 1), sh.res);
+        cluster_bar();
         const unsigned long long res = sh.res;
-        group_bar(bar, kFxThreads);  // (sh.res is read before it is written again)
-        if (res > (1ull << 59)) {  // `bound` did not hold: the Euclidean distance does
+        __syncthreads();  // (sh.res is read before it is written again)
+        if (res > (1ull << 59) && pass < 3) {  // `bound` did not hold: the Euclidean distance does
             bound = euclid();
             h = scale_of(bound);
             continue;
         }
         if (res >= kFxRedo || pass >= 3) return ldexp((double)res, -2 * h);
-        // a DTW far below the bound: again on its own scale (its
-        // V roundings allowed for), which puts it below 2^57; never past what
+        // a DTW far below the bound: again on its own scale (its 2 m - 1
+        // roundings allowed for), which puts it below 2^57; never past what
         // FP32 scales by (2^(2 * 120))
-        const int up = (56 - (63 - __clzll((long long)(res + V)))) >> 1;
+        const int up = (56 - (63 - __clzll((long long)(res + 2 * m)))) >> 1;
         if (h + up > 120) return ldexp((double)res, -2 * h);
         h += up;
     }
 }
 
-__device__ __forceinline__ void fill_pads_fx(dfloat *base, int m, int pad, dfloat v, int t) {
-    for (int u = t; u < 2 * pad; u += kFxThreads) base[u < pad ? u : m + u] = v;
+template <typename S>
+__device__ __forceinline__ void fill_pads_fx(dfloat *base, int m, int pad, dfloat v) {
+    for (int u = threadIdx.x; u < 2 * pad; u += S::kThreads) base[u < pad ? u : m + u] = v;
 }
 
 // The padded query and window copies behind the ring, their pads poisoned and
-// the query filled, by the group's threads (the caller's next barrier, in
-// fx_window, makes them visible).
-template <int K>
-__device__ __forceinline__ void fx_setup(unsigned char *sm, const double *__restrict__ qh64, int m, int r, int t,
+// the query filled (reversed when dir is 1), by the CTA's threads (the next
+// barrier, in fx_window, makes them visible).
+template <typename S>
+__device__ __forceinline__ void fx_setup(unsigned char *sm, const double *__restrict__ qh64, int m, int r, int dir,
                                          dfloat **qd, dfloat **cd) {
-    const int pad = fx_pad(r, K);
-    dfloat *q = (dfloat *)(sm + fx_ring_bytes(K)), *c = q + fx_span(m, r, K);
-    fill_pads_fx(q, m, pad, dfloat{1e15f, 0.0f}, t);
-    fill_pads_fx(c, m, pad, dfloat{-1e15f, 0.0f}, t);
-    for (int j = t; j < m; j += kFxThreads) q[pad + j] = df_from(qh64[j]);
+    const int pad = fx_pad(r);
+    dfloat *q = (dfloat *)(sm + S::kRing), *c = q + fx_span(m, r);
+    fill_pads_fx<S>(q, m, pad, dfloat{1e15f, 0.0f});
+    fill_pads_fx<S>(c, m, pad, dfloat{-1e15f, 0.0f});
+    for (int j = threadIdx.x; j < m; j += S::kThreads) q[pad + (dir ? m - 1 - j : j)] = df_from(qh64[j]);
     *qd = q + pad;
     *cd = c + pad;
 }
 
-// Two-pass FP64 statistics (Eq. 5) of the window xw by the group's first warp
+// Two-pass FP64 statistics (Eq. 5) of the window xw by the CTA's first warp
 // into sh.mu, sh.inv (0 under the zero-variance rule; 0 and 1 for raw
-// values), then its normalised values as double-floats.  All kFxThreads
-// threads of the group call it; they have met at the barrier on return.
-__device__ __forceinline__ void fx_window(const float *__restrict__ xw, int m, bool raw, dfloat *cd, FxShared &sh,
-                                          int t, int bar) {
-    const int lane = t & 31;
+// values), then its normalised values as double-floats (reversed when dir is
+// 1).  All threads of the CTA call it; they have met at the barrier on return.
+template <typename S>
+__device__ __forceinline__ void fx_window(const float *__restrict__ xw, int m, bool raw, int dir, dfloat *cd,
+                                          FxShared &sh) {
+    const int t = threadIdx.x, lane = t & 31;
     if (t < 32) {
         double s = 0.0;
         for (int j = lane; j < m; j += 32) s += (double)xw[j];
@@ -323,10 +451,10 @@ __device__ __forceinline__ void fx_window(const float *__restrict__ xw, int m, b
             sh.inv = raw ? 1.0 : var <= 1e-24 * (mm > 1.0 ? mm : 1.0) ? 0.0 : 1.0 / sqrt(var);
         }
     }
-    group_bar(bar, kFxThreads);
+    __syncthreads();
     const double mu = sh.mu, inv = sh.inv;
-    for (int j = t; j < m; j += kFxThreads) cd[j] = df_from(((double)xw[j] - mu) * inv);
-    group_bar(bar, kFxThreads);
+    for (int j = t; j < m; j += S::kThreads) cd[dir ? m - 1 - j : j] = df_from(((double)xw[j] - mu) * inv);
+    __syncthreads();
 }
 
 }  // namespace dtws

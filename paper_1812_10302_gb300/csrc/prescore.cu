@@ -7,12 +7,18 @@ namespace dtws {
 // Pre-score of the best Euclidean seed, run on a side stream while the
 // lower-bound scan streams: its FP32 DTW enters the result list (the survivor
 // pass skips it) and its extended-precision re-score waits for the final
-// stage.  One CTA: the last warp runs the FP32 walk, the others the
-// fixed-point re-score beside it (dtw_fx).  When the scan is short the search
-// waits for this kernel, so its latency counts: 172 us at m = 1024, r = 102,
-// against 289 us with the double-float walk on one warp.
-template <int K>
-__global__ void __launch_bounds__(kFxThreads + 32) k_prescore_fx(QueryBufs b, QueryArgs a) {
+// stage.  Two clusters of two CTAs: the first walks the fixed-point re-score
+// (dtw_fx), the second's first CTA the FP32 DTW (one warp, or several past
+// one warp's four cells per lane).  When the scan is short the search waits
+// for this kernel, so its latency counts: at m = 1001, r = 400 the final stage
+// waits 0.17 ms for it, against 0.47 ms with the double-float walk on four
+// warps.
+__host__ __device__ constexpr int fx_f32_warps(int W) { return W == 1 ? 1 : W == 2 ? 4 : 8; }
+__host__ __device__ constexpr int fx_f32_cells(int K, int W) { return W == 1 ? K : W <= 4 ? 2 : 4; }
+template <int K, int W>
+__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+k_prescore_fx(QueryBufs b, QueryArgs a) {
+    using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ FxShared sh;
     QueryState *st = b.st;
@@ -21,23 +27,33 @@ __global__ void __launch_bounds__(kFxThreads + 32) k_prescore_fx(QueryBufs b, Qu
     if (idx == 0xffffffffu) return;
     const int m = a.m, r = a.r, t = threadIdx.x;
     const float *xw = b.x + idx;
-    // the fixed-point walk's memory first, then the FP32 walk's padded copies
-    if (t >= kFxThreads) {
-        const int lane = t & 31, pad = diag_pad(r, 32, K);
-        float *q32 = (float *)(smraw + fx_bytes(m, r, K)), *c32 = q32 + (size_t)((m + 2 * pad + 3) & ~3);
+    if (blockIdx.x >= kFxClusterCtas) {  // the FP32 DTW, as the survivor pass would compute it
+        constexpr int W32 = fx_f32_warps(W), K32 = fx_f32_cells(K, W), kThr = 32 * W32;
+        static_assert(kThr * K32 + 2 >= S::kCells || kThr * K32 > kFxRMax, "a cell per offset of the band");
+        if (blockIdx.x > kFxClusterCtas || t >= kThr) return;
+        const int lane = t & 31, pad = diag_pad(r, kThr, K32);
+        float *q32 = (float *)smraw, *c32 = q32 + pre_span(m, r, kThr, K32);
         const float INF = __int_as_float(0x7f800000);
-        fill_pads(q32, m, pad, INF, lane, 32);
-        fill_pads(c32, m, pad, -INF, lane, 32);
+        fill_pads(q32, m, pad, INF, t, kThr);
+        fill_pads(c32, m, pad, -INF, t, kThr);
         const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
-        for (int j = lane; j < m; j += 32) {
+        for (int j = t; j < m; j += kThr) {
             q32[pad + j] = b.qh32[j];
             c32[pad + j] = fmaf(xw[j] - mh, is, -ls);
         }
-        __syncwarp();
         int cells = 0;
-        const float d32 = dtw_diag<float, 32, K, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, 0xffffffffu, lane,
-                                                         cells);
-        if (lane == 0) {
+        float d32;
+        if constexpr (W32 == 1) {
+            __syncwarp();
+            d32 = dtw_diag<float, 32, K32, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, 0xffffffffu, lane,
+                                                  cells);
+        } else {
+            __shared__ MwXchg xchg;
+            group_bar(1, kThr);
+            d32 = dtw_diag_mw<W32, K32, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, t >> 5, lane, xchg, 1,
+                                               cells);
+        }
+        if (t == 0) {
             const unsigned long long key = make_key(key_quantize(d32, a.qgrid), idx);
             list_insert(st->res_keys, a.list_cap, key);
             if (a.xz_z > 0 && d32 < DINF) xz_offer(b, a, key, true);
@@ -46,28 +62,31 @@ __global__ void __launch_bounds__(kFxThreads + 32) k_prescore_fx(QueryBufs b, Qu
         }
         return;
     }
+    const int dir = cluster_rank();
     dfloat *qd, *cd;
-    fx_setup<K>(smraw, b.qh64, m, r, t, &qd, &cd);
-    fx_window(xw, m, a.raw != 0, cd, sh, t, 1);
-    const double d64 = dtw_fx<K>(qd, cd, m, r, 0.0f, t, sh, (unsigned long long *)smraw, 1);
-    if (t == 0) {
+    fx_setup<S>(smraw, b.qh64, m, r, dir, &qd, &cd);
+    fx_window<S>(xw, m, a.raw != 0, dir, cd, sh);
+    const double d64 = dtw_fx<S>(qd, cd, m, r, 0.0f, dir, sh, (unsigned long long *)smraw);
+    if (t == 0 && dir == 0) {
         st->pre_d64 = d64;
         __threadfence();
         st->pre_done = 1;
     }
 }
 
-template <int K>
+template <int K, int W>
 static cudaError_t prescore_fx_launch(const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
-    const size_t smem = fx_bytes(a.m, a.r, K) + pre_span(a.m, a.r, 32, K) * 8;
-    cudaError_t e = cudaFuncSetAttribute(k_prescore_fx<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t fx = fx_bytes(a.m, a.r), f32 = pre_span(a.m, a.r, 32 * fx_f32_warps(W), fx_f32_cells(K, W)) * 8;
+    const size_t smem = fx > f32 ? fx : f32;
+    cudaError_t e =
+        cudaFuncSetAttribute(k_prescore_fx<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_prescore_fx<K><<<1, kFxThreads + 32, smem, s>>>(b, a);
+    k_prescore_fx<K, W><<<2 * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a);
     return cudaGetLastError();
 }
 
-// The pre-score where dtw_fx does not apply (fx_used: bands past r = 254, or
-// copies that do not fit).  Paired mode (when both copies fit in shared memory): warp 0 runs
+// The pre-score where dtw_fx does not apply (fx_used: bands of 487 to 1023
+// cells on queries whose copies do not fit beside the ring).  Paired mode (when both copies fit in shared memory): warp 0 runs
 // the FP32 DTW while warps 1..DfW run the re-score beside it, DfW warps wide
 // (the double-float walk's latency per anti-diagonal is what bounds the
 // stage).  Otherwise one warp runs both in turn.
@@ -191,14 +210,11 @@ __global__ void k_prescore(QueryBufs b, QueryArgs a) {
 cudaError_t launch_prescore(const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
     if (!a.prescore) return cudaSuccess;
     if (fx_used(a.m, a.r)) {
-        switch (fx_cells(a.r)) {
-        case 1: return prescore_fx_launch<1>(b, a, s);
-        case 2: return prescore_fx_launch<2>(b, a, s);
-        case 3: return prescore_fx_launch<3>(b, a, s);
-        case 4: return prescore_fx_launch<4>(b, a, s);
-        case 6: return prescore_fx_launch<6>(b, a, s);
-        default: return prescore_fx_launch<8>(b, a, s);
-        }
+        const FxPlan p = fx_plan(a.r);
+#define DTWS_FX_CASE(KK, WW) \
+    if (p.K == KK && p.W == WW) return prescore_fx_launch<KK, WW>(b, a, s);
+        DTWS_FX_SHAPES(DTWS_FX_CASE)
+#undef DTWS_FX_CASE
     }
     int L, K;
     diag_shape(a.r, &L, &K);
@@ -222,9 +238,7 @@ cudaError_t launch_prescore(const QueryBufs &b, const QueryArgs &a, cudaStream_t
         k_prescore<LL, KK><<<1, threads, smem, s>>>(b, a);                                          \
         return cudaGetLastError();                                                                  \
     }
-    DTWS_CASE(1, 1) DTWS_CASE(2, 1) DTWS_CASE(4, 1) DTWS_CASE(8, 1) DTWS_CASE(16, 1)
-    DTWS_CASE(32, 1) DTWS_CASE(32, 2) DTWS_CASE(32, 3) DTWS_CASE(32, 4) DTWS_CASE(32, 6) DTWS_CASE(32, 8) \
-    DTWS_CASE(32, 10) DTWS_CASE(32, 12) DTWS_CASE(32, 16) DTWS_CASE(32, 24) DTWS_CASE(32, 32)
+    DTWS_CASE(32, 16) DTWS_CASE(32, 24) DTWS_CASE(32, 32)
 #undef DTWS_CASE
     return cudaErrorInvalidValue;
 }

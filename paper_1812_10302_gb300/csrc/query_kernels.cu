@@ -1374,61 +1374,57 @@ static cudaError_t dtw64_dispatch(const QueryBufs &b, const QueryArgs &a, const 
 namespace {
 __global__ void k_reset_cursor(QueryState *st) { st->work = 0; }
 
-// The fixed-point walk at given offsets, a CTA per window.
-template <int K>
-__global__ void __launch_bounds__(kFxThreads) k_dtw_fx_at(QueryBufs b, QueryArgs a, const int64_t *offsets,
-                                                          int64_t count, double *out) {
+// The fixed-point walk at given offsets, a cluster of two CTAs per window.
+template <int K, int W>
+__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+k_dtw_fx_at(QueryBufs b, QueryArgs a, const int64_t *offsets, int64_t count, double *out) {
+    using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ FxShared sh;
     if (!b.st->valid) return;
-    const int m = a.m, t = threadIdx.x;
+    const int m = a.m, t = threadIdx.x, dir = cluster_rank();
     dfloat *qd, *cd;
-    fx_setup<K>(smraw, b.qh64, m, a.r, t, &qd, &cd);
-    for (int64_t c = blockIdx.x; c < count; c += gridDim.x) {
+    fx_setup<S>(smraw, b.qh64, m, a.r, dir, &qd, &cd);
+    for (int64_t c = blockIdx.x / kFxClusterCtas; c < count; c += gridDim.x / kFxClusterCtas) {
         const int64_t o = offsets[c];
         if (o < 0 || o >= a.N) {
-            if (t == 0) out[c] = __longlong_as_double(0x7ff8000000000000ll);
+            if (t == 0 && dir == 0) out[c] = __longlong_as_double(0x7ff8000000000000ll);
             continue;
         }
-        fx_window(b.x + o, m, a.raw != 0, cd, sh, t, 1);
-        const double d = dtw_fx<K>(qd, cd, m, a.r, 0.0f, t, sh, (unsigned long long *)smraw, 1);
-        if (t == 0) out[c] = d;
+        fx_window<S>(b.x + o, m, a.raw != 0, dir, cd, sh);
+        const double d = dtw_fx<S>(qd, cd, m, a.r, 0.0f, dir, sh, (unsigned long long *)smraw);
+        if (t == 0 && dir == 0) out[c] = d;
     }
 }
 
-template <int K>
+template <int K, int W>
 cudaError_t dtw_fx_at_launch(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets, int64_t count,
                              double *out, cudaStream_t s) {
-    const size_t smem = fx_bytes(a.m, a.r, K);
-    cudaError_t e = cudaFuncSetAttribute(k_dtw_fx_at<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = fx_bytes(a.m, a.r);
+    cudaError_t e = cudaFuncSetAttribute(k_dtw_fx_at<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dtw_fx_at<K>, kFxThreads, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t cap = (int64_t)b.num_sms * (per_sm > 0 ? per_sm : 1);
-    k_dtw_fx_at<K><<<(unsigned)(count < cap ? count : cap), kFxThreads, smem, s>>>(b, a, offsets, count, out);
+    k_dtw_fx_at<K, W><<<(unsigned)count * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, offsets, count, out);
     return cudaGetLastError();
 }
 
-// Up to two offsets per SM each window gets a CTA's fixed-point walk (latency);
-// past that the double-float walks, a group of warps per window (throughput).
-// Measured for 64 / 600 windows, fixed-point against double-float:
-// m = 512, r = 51 103 / 190 us against 210 / 213; m = 1024, r = 102 210 / 599
-// against 598 / 609; m = 1024, r = 200 311 / 920 against 513 / 721.
+// Few offsets get the fixed-point walk (latency), a cluster each: up to two
+// per SM where one warp walks, up to one cluster per two SMs where several do
+// (a CTA then fills an SM).  Past that the double-float walks, a group of warps
+// per window (throughput).  Measured for 64 / 600 windows, fixed-point (from
+// one end) against double-float: m = 512, r = 51 103 / 190 us against 210 /
+// 213; m = 1024, r = 102 210 / 599 against 598 / 609; from both ends 64 take
+// 78 and 132 us, and at m = 1024, r = 921 428 us.
 constexpr int kFxAtPerSm = 2;
 }  // namespace
 
 cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                               int64_t count, double *out, cudaStream_t s) {
-    if (fx_used(a.m, a.r) && count > 0 && count <= (int64_t)kFxAtPerSm * b.num_sms) {
-        switch (fx_cells(a.r)) {
-        case 1: return dtw_fx_at_launch<1>(b, a, offsets, count, out, s);
-        case 2: return dtw_fx_at_launch<2>(b, a, offsets, count, out, s);
-        case 3: return dtw_fx_at_launch<3>(b, a, offsets, count, out, s);
-        case 4: return dtw_fx_at_launch<4>(b, a, offsets, count, out, s);
-        case 6: return dtw_fx_at_launch<6>(b, a, offsets, count, out, s);
-        default: return dtw_fx_at_launch<8>(b, a, offsets, count, out, s);
-        }
+    const FxPlan p = fx_plan(a.r);
+    if (fx_used(a.m, a.r) && count > 0 && count <= (int64_t)(p.W == 1 ? kFxAtPerSm * b.num_sms : b.num_sms / 2)) {
+#define DTWS_FX_CASE(KK, WW) \
+    if (p.K == KK && p.W == WW) return dtw_fx_at_launch<KK, WW>(b, a, offsets, count, out, s);
+        DTWS_FX_SHAPES(DTWS_FX_CASE)
+#undef DTWS_FX_CASE
     }
     k_reset_cursor<<<1, 1, 0, s>>>(b.st);
     return dtw64_dispatch(b, a, offsets, count, out, count, s, FinalOut{});
@@ -1891,13 +1887,15 @@ __global__ void k_final_sort(QueryBufs b, QueryArgs a, int64_t *out_idx, float *
 
 // The whole final stage with the fixed-point walk (fx_used): every CTA makes
 // the margin list itself from the result list (the same list in every CTA),
-// CTA c re-scores its windows skip + c, skip + c + grid, ..., and the last CTA
-// to finish (a completion count; nothing waits) orders the list and writes
-// the output.  A window's walk is latency, so each has a CTA to itself.  A
-// top-10 search re-scores ten windows here: 0.16 ms, against 0.53 ms on one
-// double-float warp each (m = 999, r = 99).
-template <int K>
-__global__ void __launch_bounds__(kFxThreads) k_final_fx(QueryBufs b, QueryArgs a, FinalOut fin) {
+// cluster c re-scores its windows skip + c, skip + c + clusters, ..., and the
+// last cluster to finish (a completion count; nothing waits) orders the list
+// and writes the output.  A window's walk is latency, so each has a cluster to
+// itself.  A top-10 search re-scores ten windows here: 0.1 ms, against 0.53 ms
+// on one double-float warp each (m = 999, r = 99).
+template <int K, int W>
+__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+k_final_fx(QueryBufs b, QueryArgs a, FinalOut fin) {
+    using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ FxShared sh;
     __shared__ unsigned long long ms_keys[kListMax];
@@ -1906,9 +1904,10 @@ __global__ void __launch_bounds__(kFxThreads) k_final_fx(QueryBufs b, QueryArgs 
     __shared__ int ms_n, ms_skip, last;
     __shared__ float ms_bound;
     QueryState *st = b.st;
-    const int m = a.m, t = threadIdx.x;
+    const int m = a.m, t = threadIdx.x, dir = cluster_rank();
+    const int first = (int)(blockIdx.x / kFxClusterCtas), clusters = (int)(gridDim.x / kFxClusterCtas);
     const bool valid = st->valid != 0;
-    for (int j = t; j < a.list_cap; j += kFxThreads) ms_keys[j] = valid ? st->res_keys[j] : kEmptyKey;
+    for (int j = t; j < a.list_cap; j += S::kThreads) ms_keys[j] = valid ? st->res_keys[j] : kEmptyKey;
     __syncthreads();
     if (t == 0) {
         int skip = 0;
@@ -1937,34 +1936,35 @@ __global__ void __launch_bounds__(kFxThreads) k_final_fx(QueryBufs b, QueryArgs 
     dfloat *qd = nullptr, *cd = nullptr;
     // (a CTA with no window to re-score skips the query's copy: usually all of
     // them for k = 1, the best window being pre-scored)
-    if (ms_skip + (int)blockIdx.x < ms_n) fx_setup<K>(smraw, b.qh64, m, a.r, t, &qd, &cd);
-    for (int c = ms_skip + (int)blockIdx.x; c < ms_n; c += (int)gridDim.x) {
-        fx_window(b.x + ms_idx[c], m, a.raw != 0, cd, sh, t, 1);
-        const double d = dtw_fx<K>(qd, cd, m, a.r, ms_bound, t, sh, (unsigned long long *)smraw, 1);
-        if (t == 0) {
+    if (ms_skip + first < ms_n) fx_setup<S>(smraw, b.qh64, m, a.r, dir, &qd, &cd);
+    for (int c = ms_skip + first; c < ms_n; c += clusters) {
+        fx_window<S>(b.x + ms_idx[c], m, a.raw != 0, dir, cd, sh);
+        const double d = dtw_fx<S>(qd, cd, m, a.r, ms_bound, dir, sh, (unsigned long long *)smraw);
+        if (t == 0 && dir == 0) {
             st->margin_d64[c] = d;
             __threadfence();  // (before this CTA counts itself done)
         }
     }
+    if (dir != 0) return;
     __syncthreads();
     if (t == 0) {
         __threadfence();
-        last = atomicAdd(&st->final_done, 1u) == gridDim.x - 1;
+        last = atomicAdd(&st->final_done, 1u) == (unsigned)clusters - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int j = t; j < ms_n; j += kFxThreads) ms_d[j] = j < ms_skip ? st->pre_d64 : __ldcg(&st->margin_d64[j]);
+    for (int j = t; j < ms_n; j += S::kThreads) ms_d[j] = j < ms_skip ? st->pre_d64 : __ldcg(&st->margin_d64[j]);
     __syncthreads();
-    final_order(ms_idx, ms_d, ms_n, a, fin.idx, fin.dist, t, kFxThreads);
+    final_order(ms_idx, ms_d, ms_n, a, fin.idx, fin.dist, t, S::kThreads);
 }
 
-template <int K>
+template <int K, int W>
 static cudaError_t final_fx_launch(const QueryBufs &b, const QueryArgs &a, FinalOut fin, cudaStream_t s) {
-    const size_t smem = fx_bytes(a.m, a.r, K);
-    cudaError_t e = cudaFuncSetAttribute(k_final_fx<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = fx_bytes(a.m, a.r);
+    cudaError_t e = cudaFuncSetAttribute(k_final_fx<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_final_fx<K><<<a.list_cap, kFxThreads, smem, s>>>(b, a, fin);
+    k_final_fx<K, W><<<a.list_cap * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, fin);
     return cudaGetLastError();
 }
 
@@ -1976,14 +1976,11 @@ cudaError_t launch_finalize(const QueryBufs &b, const QueryArgs &a, int64_t *out
     *launches = 1;
     if (fx_used(a.m, a.r)) {
         const FinalOut fin{out_idx, out_dist};
-        switch (fx_cells(a.r)) {
-        case 1: return final_fx_launch<1>(b, a, fin, s);
-        case 2: return final_fx_launch<2>(b, a, fin, s);
-        case 3: return final_fx_launch<3>(b, a, fin, s);
-        case 4: return final_fx_launch<4>(b, a, fin, s);
-        case 6: return final_fx_launch<6>(b, a, fin, s);
-        default: return final_fx_launch<8>(b, a, fin, s);
-        }
+        const FxPlan p = fx_plan(a.r);
+#define DTWS_FX_CASE(KK, WW) \
+    if (p.K == KK && p.W == WW) return final_fx_launch<KK, WW>(b, a, fin, s);
+        DTWS_FX_SHAPES(DTWS_FX_CASE)
+#undef DTWS_FX_CASE
     }
     cudaError_t e = dtw64_dispatch(b, a, nullptr, 0, nullptr, kListMax, s, FinalOut{out_idx, out_dist});
     if (e != cudaErrorNotSupported) return e;

@@ -1,7 +1,8 @@
 """The fixed-point re-score walk (up to two offsets per SM of dtws_dtw_at_f64,
 the pre-score and the final stage of a search) against the FP64 oracle, at the
-edges of its shapes: 32 K >= r + 2 cells for K = 1, 2, 3, 4, 6, 8, whole and
-ragged chunks of 16 anti-diagonals, its widest band and the first past it.
+edges of its shapes: 32 K >= r + 2 cells for K = 1, 2, 3, 4 on one warp, 120 W
++ 8 >= r + 2 on W = 2, 3, 4, 6, 9, whole and ragged chunks of anti-diagonals,
+its widest band and the first past it.
 
 Tolerance: costs carry the double-float normalisation (2^-48 of |z| <= sqrt(m)
 against differences of ~0.05 sigma and more: ~2^-40 per term at worst) and the
@@ -36,6 +37,26 @@ def test_at_the_edges_of_its_shapes(series, m, r):
         assert ix.sync_status() == dtws.DTWS_OK
     want = oracle.dtw_at(series, q, r, offs)
     np.testing.assert_allclose(got, want, rtol=1e-10, atol=1e-18 * m)
+
+
+@pytest.mark.parametrize("m,r", [(127, 126), (128, 127), (247, 246), (248, 247), (500, 246), (501, 247), (367, 366),
+                                 (700, 367), (487, 486), (990, 487), (727, 726), (801, 727), (1023, 1022),
+                                 (1025, 1023), (1100, 1024)])
+def test_several_walking_warps(series, m, r):
+    """Bands past one warp: the overlaps of two to nine warps, each at its widest
+    band and the first past it, queries no longer than the band and longer,
+    both parities of m + r (where the walks from both ends meet)."""
+    q, o = synth.noisy_copy(series, m, m + r, m + 2 * r, noise=0.1)
+    offs = np.random.default_rng(m + r).integers(0, series.size - m + 1, 5)
+    offs[:3] = [o, 0, series.size - m]
+    with dtws.Index(series) as ix:
+        got = ix.dtw_at_f64(q, r, offs)
+        idx, dist = ix.query(q, r, 2)
+        assert ix.sync_status() == dtws.DTWS_OK
+    np.testing.assert_allclose(got, oracle.dtw_at(series, q, r, offs), rtol=1e-10)
+    oi, od = oracle.search_cascade(series, q, r, 2)
+    np.testing.assert_array_equal(idx, oi)
+    np.testing.assert_allclose(dist, od, rtol=1e-6)
 
 
 @pytest.mark.parametrize("unnormalised,scale", [(0, 1.0), (1, 1.0), (1, 2.0 ** -30), (1, 2.0 ** 20)])
