@@ -209,6 +209,10 @@ bool dtw_default_shape(int m, int r, int *L, int *K, int *warps);
 bool dtw_shape_valid(int m, int r, int L, int K, int warps);
 cudaError_t launch_dtw_at_shape(const QueryBufs &b, QueryArgs a, const int64_t *offsets, int64_t count, float *out,
                                 int L, int K, int warps, cudaStream_t s);
+// Throughput shapes for many offsets (dtw_at64.cu); cudaErrorNotSupported, nothing
+// launched, where they do not apply.
+cudaError_t launch_dtw_at_f64_many(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets, int64_t count,
+                                   double *out, cudaStream_t s);
 cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                               int64_t count, double *out, cudaStream_t s);
 cudaError_t launch_lbs_at(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,

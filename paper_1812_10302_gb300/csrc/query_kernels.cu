@@ -1408,24 +1408,25 @@ cudaError_t dtw_fx_at_launch(const QueryBufs &b, const QueryArgs &a, const int64
 }
 
 // Few offsets get the fixed-point walk (latency), a cluster each: up to two
-// per SM where one warp walks, up to one cluster per two SMs where several do
-// (a CTA then fills an SM).  Past that the double-float walks, a group of warps
-// per window (throughput).  Measured for 64 / 600 windows, fixed-point (from
-// one end) against double-float: m = 512, r = 51 103 / 190 us against 210 /
-// 213; m = 1024, r = 102 210 / 599 against 598 / 609; from both ends 64 take
-// 78 and 132 us, and at m = 1024, r = 921 428 us.
+// per SM where one warp walks, up to three clusters per two SMs where several
+// do (a CTA then fills an SM: three waves).  Past that the walks for many
+// windows.  Measured for 64 windows, from both ends (from one, in
+// double-float): m = 512, r = 51 78 us (103, 210); m = 1024, r = 102 132 us
+// (210, 598); m = 1024, r = 921 428 us.
 constexpr int kFxAtPerSm = 2;
 }  // namespace
 
 cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                               int64_t count, double *out, cudaStream_t s) {
     const FxPlan p = fx_plan(a.r);
-    if (fx_used(a.m, a.r) && count > 0 && count <= (int64_t)(p.W == 1 ? kFxAtPerSm * b.num_sms : b.num_sms / 2)) {
+    if (fx_used(a.m, a.r) && count > 0 && count <= (int64_t)(p.W == 1 ? kFxAtPerSm * b.num_sms : b.num_sms + b.num_sms / 2)) {
 #define DTWS_FX_CASE(KK, WW) \
     if (p.K == KK && p.W == WW) return dtw_fx_at_launch<KK, WW>(b, a, offsets, count, out, s);
         DTWS_FX_SHAPES(DTWS_FX_CASE)
 #undef DTWS_FX_CASE
     }
+    const cudaError_t many = launch_dtw_at_f64_many(b, a, offsets, count, out, s);
+    if (many != cudaErrorNotSupported) return many;
     k_reset_cursor<<<1, 1, 0, s>>>(b.st);
     return dtw64_dispatch(b, a, offsets, count, out, count, s, FinalOut{});
 }

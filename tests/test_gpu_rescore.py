@@ -91,3 +91,26 @@ def test_a_match_and_its_exact_copies_keep_their_order():
             idx, dist = ix.query(q, 20, k)
             np.testing.assert_array_equal(idx, [4_000, 9_000, 20_000, 25_000][:k])
             assert np.all(dist == dist[0])
+
+
+@pytest.mark.parametrize("m,r", [(2, 0), (2, 1), (3, 1), (9, 8), (40, 22), (41, 23), (60, 38), (60, 39), (100, 46), (101, 47),
+                                 (101, 54), (102, 55), (200, 78), (201, 79), (200, 94), (200, 95), (300, 110), (301, 111),
+                                 (300, 158), (300, 159), (400, 222), (401, 223), (2500, 20)])
+def test_many_offsets(series, m, r):
+    """The throughput shapes (more than two offsets per SM) at their widest bands
+    and the first past them, both parities, constant and repeated windows, a
+    spike that sets the grid the values are split on."""
+    x = series.copy()
+    x[9000] += 1e4
+    q, o = synth.noisy_copy(x, m, m + r, m + 2 * r, noise=0.1)
+    some = np.random.default_rng(m + r).integers(0, x.size - m + 1, 24)
+    some[:5] = [o, 0, x.size - m, 3000, 9000 - m // 2]
+    offs = np.tile(some, 14)
+    with dtws.Index(x) as ix:
+        got = ix.dtw_at_f64(q, r, offs)
+        few = ix.dtw_at_f64(q, r, some)
+        assert ix.sync_status() == dtws.DTWS_OK
+    want = oracle.dtw_at(x, q, r, some)
+    np.testing.assert_allclose(got[:24], want, rtol=1e-10, atol=1e-18 * m)
+    np.testing.assert_array_equal(got, np.tile(got[:24], 14))
+    np.testing.assert_allclose(few, want, rtol=1e-10, atol=1e-18 * m)
