@@ -527,6 +527,187 @@ __device__ T dtw_diag(const T *__restrict__ qp, const T *__restrict__ cp, const 
     return (T)__shfl_sync(gmask, res, pe / K, L);
 }
 
+// ------------------------------------------------------------------ walk from both ends
+// dtw_diag by one warp from both ends of the matrix at once: lanes 0-15 walk
+// forward to anti-diagonal m - 1, lanes 16-31 the reversed sequences to their
+// m - 2 (the forward walk's m), in lockstep, K cells per lane; the DTW is the
+// best way of joining the two.  A walk's latency is what a search waits for
+// when few candidates are left, and half the steps with twice the cells per
+// lane take about 0.6 of the time: a step of dtw_diag is a chain of ~80 cycles
+// (exchange, minimum, multiply-add) with K = 4 cells' issue beside it.  It
+// also abandons on more: every path crosses both frontiers, so their minima
+// together bound it.  The sum is rounded in another order than dtw_diag's.
+// qp, cp, cbs, back, thr, cells: as dtw_diag; cp is overwritten (its m samples
+// carry the reversed walk's last anti-diagonals to the forward lanes).
+template <int K, int CP>
+__device__ __forceinline__ void ends_rot_c(float (&cv)[K], float fresh, int lane) {
+    constexpr int s = CP % K;
+    if constexpr (K & 1) {
+        cv[s] = fresh;
+    } else {
+        const float from_next = __shfl_down_sync(0xffffffffu, cv[s], 1, 16);
+        cv[s] = lane == 15 ? fresh : from_next;
+    }
+}
+template <int K, int QP>
+__device__ __forceinline__ void ends_rot_q(float (&qv)[K], float fresh, int lane) {
+    constexpr int s = ((K - 1 - QP) % K + K) % K;
+    if constexpr (K & 1) {
+        qv[s] = fresh;
+    } else {
+        const float from_prev = __shfl_up_sync(0xffffffffu, qv[s], 1, 16);
+        qv[s] = lane == 0 ? fresh : from_prev;
+    }
+}
+
+template <int K, bool ABANDON>
+__device__ float dtw_ends(const float *__restrict__ qp, float *__restrict__ cp, const float *cbs, float back, int m, int r,
+                          float thr, int ln, int &cells) {
+    constexpr int L = 16, U = diag_unroll(K);
+    constexpr unsigned kAll = 0xffffffffu;
+    const float INF = __int_as_float(0x7f800000);
+    const int lane = ln & 15;
+    const bool rev = ln >= 16;
+    const int sg = rev ? -1 : 1;
+    const float *q0 = qp + (rev ? m - 1 : 0), *c0 = cp + (rev ? m - 1 : 0);
+    const int p0 = (r - (r & 1)) >> 1;
+    float p1[K], p2[K], qv[K], cv[K], pen[K];
+#pragma unroll
+    for (int t = 0; t < K; ++t) {
+        p1[t] = INF;
+        p2[t] = (lane * K + t == p0) ? 0.0f : INF;
+        pen[t] = lane * K + t == r ? INF : 0.0f;
+    }
+    const int last = m - 2;
+    int a = 0;
+    {
+        const int qb = r >> 1, cb = (r & 1) ? (1 - r) >> 1 : -(r >> 1);
+#pragma unroll
+        for (int t = 0; t < K; ++t) {
+            qv[t] = q0[sg * (qb - (lane * K + t))];
+            cv[t] = c0[sg * (cb + (lane * K + t))];
+        }
+        if (r & 1) {  // a = 0 is an odd step
+            diag_step<L, K, 1, 0, 0>(qv, cv, p1, p2, pen, lane, r, kAll);
+            a = 1;
+#pragma unroll
+            for (int t = 0; t < K; ++t) qv[t] = q0[sg * (qb + 1 - (lane * K + t))];
+        }
+    }
+    int bi = (a + r) >> 1;
+    const int bj = (a - r) >> 1;
+    // the values that arrive next are one further along at each pair
+    const float *cf = c0 + sg * (bj + ((K & 1) ? (lane + 1) * K - 1 : L * K - 1));
+    const float *qf = q0 + sg * (bi - ((K & 1) ? lane * K : 0));
+    while (a + 2 * U - 1 <= last) {
+        static_for<U>([&](auto uc) {
+            constexpr int u = decltype(uc)::value;
+            cf += sg;
+            const float cn = *cf;
+            diag_step<L, K, 0, u % K, u % K>(qv, cv, p1, p2, pen, lane, r, kAll);
+            ends_rot_c<K, u % K>(cv, cn, lane);
+            qf += sg;
+            const float qn = *qf;
+            diag_step<L, K, 1, u % K, (u + 1) % K>(qv, cv, p1, p2, pen, lane, r, kAll);
+            ends_rot_q<K, u % K>(qv, qn, lane);
+        });
+        a += 2 * U;
+        bi += U;
+        if (ABANDON) {
+            // p1: anti-diagonal a-1, p2: a-2, both on rows bi - 1 - p
+            float raw = INF, low = INF;
+#pragma unroll
+            for (int t = 0; t < K; ++t) {
+                const int i = bi - 1 - (lane * K + t);
+                const float tail = (cbs && i >= 0 && i < m) ? cbs[(i + kTailG) / kTailG] : 0.0f;
+                const float v = fminf(p1[t], p2[t]);
+                raw = fminf(raw, v);
+                low = fminf(low, v + fmaxf(tail, back));
+            }
+            // (costs are not negative: their bit patterns order like their values)
+            const unsigned inf = 0x7f800000u, rb = __float_as_uint(raw);
+            const float f = __uint_as_float(__reduce_min_sync(kAll, rev ? inf : rb));
+            const float b = __uint_as_float(__reduce_min_sync(kAll, rev ? rb : inf));
+            const float w = __uint_as_float(__reduce_min_sync(kAll, rev ? inf : __float_as_uint(low)));
+            if (w > thr || f + b > thr) {
+                if (ln == 0) cells += 2 * (int)band_cells_upto(a - 1, m, r);
+                return INF;
+            }
+        }
+    }
+    // the rest, one pair at a time (phase 0: windows shift by register moves),
+    // then one step more for the forward lanes; the reversed ones keep what
+    // they had: their newest anti-diagonal moves to p2, the one before to hold
+    float hold[K];
+    for (;; a += 2) {
+        if (a > last) {
+#pragma unroll
+            for (int t = 0; t < K; ++t) hold[t] = p2[t];
+            diag_step<L, K, 0, 0, 0>(qv, cv, p1, p2, pen, lane, r, kAll);
+            break;
+        }
+        cf += sg;
+        const float cn = *cf;
+        diag_step<L, K, 0, 0, 0>(qv, cv, p1, p2, pen, lane, r, kAll);
+        const float from_next = __shfl_down_sync(kAll, cv[0], 1, L);
+#pragma unroll
+        for (int t = 0; t < K - 1; ++t) cv[t] = cv[t + 1];
+        cv[K - 1] = ((K & 1) || lane == L - 1) ? cn : from_next;
+        if (a + 1 > last) {
+#pragma unroll
+            for (int t = 0; t < K; ++t) hold[t] = p2[t];
+            diag_step<L, K, 1, 0, 0>(qv, cv, p1, p2, pen, lane, r, kAll);
+            break;
+        }
+        qf += sg;
+        const float qn = *qf;
+        diag_step<L, K, 1, 0, 0>(qv, cv, p1, p2, pen, lane, r, kAll);
+        const float from_prev = __shfl_up_sync(kAll, qv[K - 1], 1, L);
+#pragma unroll
+        for (int t = K - 1; t > 0; --t) qv[t] = qv[t - 1];
+        qv[0] = ((K & 1) || lane == 0) ? qn : from_prev;
+    }
+    // The join: the reversed walk's cell p' of an even (odd) step is the
+    // forward one's r - p' (r - 1 - p').  A path goes through anti-diagonal
+    // m - 1 and then m or, diagonally, m + 1, or from m - 2 diagonally to m.
+    const bool even = ((m - 1 + r) & 1) == 0;  // anti-diagonal m - 1 is an even step
+    __syncwarp();
+    if (rev) {
+#pragma unroll
+        for (int t = 0; t < K; ++t)
+            if (lane * K + t <= r) cp[lane * K + t] = p2[t];
+    }
+    __syncwarp();
+    float best = INF, n[K + 1];
+    if (!rev) {
+#pragma unroll
+        for (int u = 0; u <= K; ++u) {
+            const int p = lane * K + u - (even ? 1 : 0), j = (even ? r - 1 : r) - p;
+            n[u] = p >= 0 && j >= 0 ? cp[j] : INF;
+        }
+#pragma unroll
+        for (int t = 0; t < K; ++t)
+            best = fminf(best, fminf(p1[t] + fminf(n[t], n[t + 1]), p2[t] + (even ? n[t + 1] : n[t])));
+    }
+    __syncwarp();
+    if (rev) {
+#pragma unroll
+        for (int t = 0; t < K; ++t)
+            if (lane * K + t <= r) cp[lane * K + t] = hold[t];
+    }
+    __syncwarp();
+    if (!rev) {
+#pragma unroll
+        for (int t = 0; t < K; ++t) {
+            const int j = (even ? r : r - 1) - (lane * K + t);
+            if (j >= 0) best = fminf(best, p1[t] + cp[j]);
+        }
+    }
+    __syncwarp();  // (cp is read before the next window is written)
+    if (ln == 0) cells += (int)band_cells_upto(2 * m - 2, m, r);
+    return __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(best)));
+}
+
 // ------------------------------------------------------------------ multi-warp FP32 walk
 // dtw_diag with the r+1 cells of an anti-diagonal spread over W warps of one
 // group (32 W lanes, K cells each): bands up to 32 W K - 1 (2047 with four

@@ -95,6 +95,13 @@ __host__ __device__ constexpr int dtw_min_blocks(int K) {
     return (K >= 1 && K <= 2) ? 4 : (K >= 1 && K <= 4) ? 3 : (K >= 16) ? 1 : 2;
 }
 
+// Shapes whose seeds walk from both ends (dtw_ends): one warp per window, up to
+// 16 cells per lane.  The search waits for the few seeds of a top-k search one
+// walk long (ten of m = 999, r = 99: 95 us, 140 from one end).  The survivor
+// pass stays with dtw_diag: it is bound by its bounds, not by walks, and the
+// wider walk's registers spill at its three CTAs per SM.
+__host__ __device__ constexpr bool ends_applies(int L, int K) { return L == 32 && K >= 1 && K <= 8; }
+
 // The body of k_dtw for one query (the CTA's part of its candidate stream);
 // the persistent batch stage (k_dtw_pool) runs it for one query after
 // another.  In survivor mode with b.surv_mh set, the survivors' window
@@ -415,6 +422,8 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
         } else {
             if (MODE == kModeOut)
                 d = dtw_diag<float, L, K, false>(qs, cbuf, nullptr, 0.0f, m, r, thr, gmask, lane, cells);
+            else if constexpr (MODE == kModeSeed && ends_applies(L, K))
+                d = dtw_ends<2 * K, true>(qs, cbuf, cbs, back, m, r, thr, lane, cells);
             else
                 d = dtw_diag<float, L, K, true>(qs, cbuf, cbs, back, m, r, thr, gmask, lane, cells);
         }
@@ -461,7 +470,7 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
 }
 
 template <int L, int K, int MODE>
-__global__ void __launch_bounds__(256, dtw_min_blocks(K)) k_dtw(QueryBufs b, QueryArgs a, const int64_t *offsets,
+__global__ void __launch_bounds__(256, MODE == kModeSeed ? 1 : dtw_min_blocks(K)) k_dtw(QueryBufs b, QueryArgs a, const int64_t *offsets,
                                                               int64_t count_host, float *out, int staged) {
     dtw_body<L, K, MODE>(b, a, offsets, count_host, out, staged);
 }
@@ -614,6 +623,8 @@ static cudaError_t dtw_dispatch(const QueryBufs &b, const QueryArgs &a, const in
     if (!tuned && a.r > kDiagRMax && a.r <= kWideRMax)
         return dtw_wide_launch<MODE>(b, a, offsets, count, out, count_for_grid, s);
     if (!tuned && !plan_dtw<float>(a.m, a.r, tail, &p)) return cudaErrorInvalidValue;
+    // (a seed's walk is latency: two warps to a CTA, so that none shares a scheduler)
+    if (MODE == kModeSeed && p.warps > 2) p.warps = 2;
     const int blocks = dtw_blocks(p, b.num_sms, count_for_grid);
 #define DTWS_CASE(LL, KK)                                                                                     \
     if (p.L == LL && p.K == KK) {                                                                             \

@@ -45,8 +45,7 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
         float d32;
         if constexpr (W32 == 1) {
             __syncwarp();
-            d32 = dtw_diag<float, 32, K32, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, 0xffffffffu, lane,
-                                                  cells);
+            d32 = dtw_ends<2 * K32, false>(q32 + pad, c32 + pad, nullptr, 0.0f, m, r, INF, lane, cells);
         } else {
             __shared__ MwXchg xchg;
             group_bar(1, kThr);
@@ -62,6 +61,9 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
         }
         return;
     }
+    // of several answers all are walked on common terms in the final stage
+    // (k_final_fx), which would wait here for nothing
+    if (a.k > 1) return;
     const int dir = cluster_rank();
     dfloat *qd, *cd;
     fx_setup<S>(smraw, b.qh64, m, r, dir, &qd, &cd);

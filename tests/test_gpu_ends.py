@@ -1,0 +1,31 @@
+"""The walk from both ends (seeds, survivors and the FP32 pre-score on one warp
+per window) against the FP64 oracle, at the edges of its shapes (two to
+sixteen cells a lane: 32 K >= r + 1, K = 1, 2, 3, 4, 6, 8), both parities of m + r
+(where the ends meet), queries hardly longer than the band, and candidates so
+close together that few can be abandoned."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1812_10302_gb300 import dtws, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m,r", [(17, 16), (18, 16), (33, 31), (34, 32), (64, 63), (65, 63), (66, 64), (97, 95), (100, 96),
+                                 (128, 127), (129, 127), (140, 128), (193, 191), (200, 192), (256, 255), (400, 255),
+                                 (333, 40), (334, 41), (1024, 102)])
+@pytest.mark.parametrize("exact_envelope", [0, 1])
+def test_answers_at_shape_edges(m, r, exact_envelope):
+    x = synth.random_walk(6_000, m + r)
+    x[1000:5000] = np.sin(np.arange(4000) / 30.0) * 5 + 0.3 * x[1000:5000]  # many near ties
+    q, _ = synth.noisy_copy(x, m, m, r, noise=0.2)
+    with dtws.Index(x, options=dict(exact_envelope=exact_envelope)) as ix:
+        idx, dist = ix.query(q, r, 5)
+        assert ix.sync_status() == dtws.DTWS_OK
+        bi, bd = ix.query_batch([q, q[: m - 1]], [r, min(r, m - 2)], 5)
+    oi, od = oracle.search_cascade(x, q, r, 5)
+    np.testing.assert_array_equal(idx, oi)
+    np.testing.assert_allclose(dist, od, rtol=1e-6)
+    np.testing.assert_array_equal(bi[0], oi)
+    np.testing.assert_allclose(bd[0], od, rtol=1e-6)
