@@ -710,31 +710,34 @@ __device__ float dtw_ends(const float *__restrict__ qp, float *__restrict__ cp, 
 
 // ------------------------------------------------------------------ multi-warp FP32 walk
 // dtw_diag with the r+1 cells of an anti-diagonal spread over W warps of one
-// group (32 W lanes, K cells each): bands up to 32 W K - 1 (2047 with four
-// warps of 16 cells).  Inside a warp the neighbour cell arrives by shuffle;
-// across a warp boundary through shared memory: after each step every warp's
-// first and last lane publish their newest cell into the other half of a
-// double buffer and the group meets at its named barrier, so a step's reads
-// (this half) never race the next step's writes (the other half).  The
-// register windows rotate as in dtw_diag; each warp's boundary lane loads
-// its fresh value from the padded arrays instead of a neighbour warp.
+// group, K consecutive cells per lane (K odd, so that every lane loads its own
+// register windows without bank conflicts).  Neighbouring warps overlap by one
+// lane on each side: lane l of warp w holds place 30 w + l, so its first lane
+// repeats the cells of its lower neighbour's lane 30 and its last those of its
+// upper neighbour's lane 1.  An anti-diagonal needs one cell from below (even
+// steps) or above (odd steps), so an error at a warp's edge travels K cells,
+// one lane, in K pairs of steps; then the overlaps are taken anew from their
+// owners, through shared memory and one barrier of the group, together with
+// the abandon test.  (With the boundary cells published and the group meeting
+// after every step, the FP32 pre-score of a window of m = 1871, r = 191 took
+// some 400 us, and the survivor pass of a search of m = 1024, r = 921 320 us
+// instead of 248.)
+constexpr int kMwK = 17, kMwW = 9;  // most cells per lane, most warps
+__host__ __device__ constexpr int mw_cells(int W, int K) { return (30 * W + 2) * K; }
 struct MwXchg {
-    float first[2][8], last[2][8];  // [buffer][warp]: lane 0's p1[0], lane 31's p1[K-1]
-    float red[2][8];                // per-warp partial sums / minima
+    float edge[2][kMwW][2][2 * kMwK];  // [buffer][warp][lane 1, lane 30][p1, p2]
+    float red[2][kMwW];                // per-warp partial sums / minima
     float res;
 };
 
+// A step: diag_step of lane place gl; the group's first and last places end
+// the band (inside it a warp's outermost lanes take whatever wraps around).
 template <int W, int K, int ODD, int QP, int CP>
 __device__ __forceinline__ void diag_step_mw(const float (&qv)[K], const float (&cv)[K], float (&p1)[K],
-                                             float (&p2)[K], const float (&pen)[K], int gl, int lane, int w, int r,
-                                             const MwXchg &x, int buf) {
+                                             float (&p2)[K], const float (&pen)[K], int gl, int lane, int r) {
     const float INF = __int_as_float(0x7f800000);
     float nb = __shfl_sync(0xffffffffu, ODD ? p1[0] : p1[K - 1], ODD ? ((lane + 1) & 31) : ((lane - 1) & 31));
-    if (ODD) {
-        if (lane == 31) nb = (w == W - 1) ? INF : x.first[buf][w + 1];
-    } else {
-        if (lane == 0) nb = (w == 0) ? INF : x.last[buf][w - 1];
-    }
+    if (ODD ? (gl == 30 * W + 1) : (gl == 0)) nb = INF;
     float cur[K];
 #pragma unroll
     for (int t = 0; t < K; ++t) {
@@ -743,7 +746,7 @@ __device__ __forceinline__ void diag_step_mw(const float (&qv)[K], const float (
         const float d = qv[((t - QP) % K + K) % K] - cv[(t + CP) % K];
         float v = fmaf(d, d, min3f(left, up, p2[t]));
         if (ODD) {
-            if constexpr (K <= 8) v = v + pen[t];  // (as in diag_step)
+            if constexpr (K <= 9) v = v + pen[t];  // (as in diag_step)
             else if (gl * K + t == r) v = INF;
         }
         cur[t] = v;
@@ -755,59 +758,19 @@ __device__ __forceinline__ void diag_step_mw(const float (&qv)[K], const float (
     }
 }
 
-template <int W, int K>
-__device__ __forceinline__ void mw_publish(const float (&p1)[K], int lane, int w, MwXchg &x, int &buf, int bar) {
-    const int nbuf = buf ^ 1;
-    if (lane == 0) x.first[nbuf][w] = p1[0];
-    if (lane == 31) x.last[nbuf][w] = p1[K - 1];
-    group_bar(bar, 32 * W);
-    buf = nbuf;
-}
-
-template <int K, int CP>
-__device__ __forceinline__ void rot_c_mw(float (&cv)[K], const float *cp, int cbase_new, int gl, int lane) {
-    constexpr int s = CP % K;
-    const float from_next = __shfl_down_sync(0xffffffffu, cv[s], 1);
-    const float fresh = cp[cbase_new + (gl + 1) * K - 1];
-    cv[s] = lane == 31 ? fresh : from_next;
-}
-template <int K, int QP>
-__device__ __forceinline__ void rot_q_mw(float (&qv)[K], const float *qp, int qbase_new, int gl, int lane) {
-    constexpr int s = ((K - 1 - QP) % K + K) % K;
-    const float from_prev = __shfl_up_sync(0xffffffffu, qv[s], 1);
-    const float fresh = qp[qbase_new - gl * K];
-    qv[s] = lane == 0 ? fresh : from_prev;
-}
-template <int K>
-__device__ __forceinline__ void shift_c_mw(float (&cv)[K], const float *cp, int cbase_new, int gl, int lane) {
-    const float from_next = __shfl_down_sync(0xffffffffu, cv[0], 1);
-    const float fresh = cp[cbase_new + (gl + 1) * K - 1];
-#pragma unroll
-    for (int t = 0; t < K - 1; ++t) cv[t] = cv[t + 1];
-    cv[K - 1] = lane == 31 ? fresh : from_next;
-}
-template <int K>
-__device__ __forceinline__ void shift_q_mw(float (&qv)[K], const float *qp, int qbase_new, int gl, int lane) {
-    const float from_prev = __shfl_up_sync(0xffffffffu, qv[K - 1], 1);
-    const float fresh = qp[qbase_new - gl * K];
-#pragma unroll
-    for (int t = K - 1; t > 0; --t) qv[t] = qv[t - 1];
-    qv[0] = lane == 0 ? fresh : from_prev;
-}
-
 // qp, cp: element 0 of the query / the group's normalised window, padded by
 // diag_pad(r, 32*W, K) on both sides (+inf / -inf); cbs: the coarse tail
-// bound and back (as dtw_diag) or nullptr and 0.  Called by all 32 W threads of warps
-// w = 0..W-1 of the group; bar: the group's named barrier.  Every thread
-// returns the distance (+inf when abandoned); thread 0 of the group adds the
-// cells evaluated to `cells`.
+// bound and back (as dtw_diag) or nullptr and 0; r < mw_cells(W, K).  Called
+// by all 32 W threads of warps w = 0..W-1 of the group; bar: the group's named
+// barrier.  Every thread returns the distance (+inf when abandoned); thread 0
+// of the group adds the cells evaluated to `cells`.
 template <int W, int K, bool ABANDON>
 __device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restrict__ cp, const float *cbs, float back,
                              int m, int r, float thr, int w, int lane, MwXchg &x, int bar, int &cells) {
-    static_assert(W >= 2 && W <= 8, "two to eight warps");
-    constexpr int U = diag_unroll(K);
+    static_assert(W >= 2 && W <= kMwW && (K & 1) && K <= kMwK, "two to nine warps, an odd cell count");
     const float INF = __int_as_float(0x7f800000);
-    const int gl = w * 32 + lane;
+    const int gl = w * 30 + lane;
+    const bool own = (w == 0 || lane > 0) && (w == W - 1 || lane < 31);  // not an overlap
     const int p0 = (r - (r & 1)) >> 1;
     float p1[K], p2[K], qv[K], cv[K], pen[K];
 #pragma unroll
@@ -816,44 +779,47 @@ __device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restri
         p2[t] = (gl * K + t == p0) ? 0.0f : INF;
         pen[t] = (gl * K + t == r) ? INF : 0.0f;
     }
-    int buf = 1;
-    mw_publish<W, K>(p1, lane, w, x, buf, bar);  // buffer 0 := the all-inf anti-diagonal -1
+    const float *ql = qp - gl * K, *cl = cp + gl * K;  // this place's own cells
+    int buf = 0;
     const int last = 2 * m - 2;
     const int pe_even = r >> 1, pe_odd = (r - 1) >> 1;
     int a = 0;
-    if (r & 1) {
-        const int qb = (r - 1) >> 1, cb = (1 - r) >> 1;
+    {
+        const int qb = r >> 1, cb = (r & 1) ? (1 - r) >> 1 : -(r >> 1);
 #pragma unroll
         for (int t = 0; t < K; ++t) {
-            qv[t] = qp[qb - (gl * K + t)];
-            cv[t] = cp[cb + (gl * K + t)];
+            qv[t] = ql[qb - t];
+            cv[t] = cl[cb + t];
         }
-        diag_step_mw<W, K, 1, 0, 0>(qv, cv, p1, p2, pen, gl, lane, w, r, x, buf);
-        mw_publish<W, K>(p1, lane, w, x, buf, bar);
-        a = 1;
-        shift_q_mw<K>(qv, qp, qb + 1, gl, lane);
-    } else {
-        const int qb = r >> 1, cb = -(r >> 1);
+        if (r & 1) {  // a = 0 is an odd step (what wraps around is still +inf)
+            diag_step_mw<W, K, 1, 0, 0>(qv, cv, p1, p2, pen, gl, lane, r);
+            a = 1;
 #pragma unroll
-        for (int t = 0; t < K; ++t) {
-            qv[t] = qp[qb - (gl * K + t)];
-            cv[t] = cp[cb + (gl * K + t)];
+            for (int t = 0; t < K; ++t) qv[t] = ql[qb + 1 - t];
         }
     }
     int bi = (a + r) >> 1, bj = (a - r) >> 1;
-    while (a + 2 * U - 1 < last) {
-        static_for<U>([&](auto uc) {
+    while (a + 2 * K - 1 < last) {
+        static_for<K>([&](auto uc) {
             constexpr int u = decltype(uc)::value;
-            diag_step_mw<W, K, 0, u % K, u % K>(qv, cv, p1, p2, pen, gl, lane, w, r, x, buf);
-            mw_publish<W, K>(p1, lane, w, x, buf, bar);
-            rot_c_mw<K, u % K>(cv, cp, bj + u + 1, gl, lane);
-            diag_step_mw<W, K, 1, u % K, (u + 1) % K>(qv, cv, p1, p2, pen, gl, lane, w, r, x, buf);
-            mw_publish<W, K>(p1, lane, w, x, buf, bar);
-            rot_q_mw<K, u % K>(qv, qp, bi + u + 1, gl, lane);
+            const float cn = cl[bj + u + K];
+            diag_step_mw<W, K, 0, u, u>(qv, cv, p1, p2, pen, gl, lane, r);
+            cv[u] = cn;
+            const float qn = ql[bi + u + 1];
+            diag_step_mw<W, K, 1, u, (u + 1) % K>(qv, cv, p1, p2, pen, gl, lane, r);
+            qv[K - 1 - u] = qn;
         });
-        a += 2 * U;
-        bi += U;
-        bj += U;
+        a += 2 * K;
+        bi += K;
+        bj += K;
+        if (lane == 1 || lane == 30) {
+            float *e = x.edge[buf][w][lane == 30];
+#pragma unroll
+            for (int t = 0; t < K; ++t) {
+                e[t] = p1[t];
+                e[K + t] = p2[t];
+            }
+        }
         if (ABANDON) {
             const float rest = a <= last - kCorner ? back : 0.0f;  // (as in dtw_diag)
             float low = INF;
@@ -863,41 +829,59 @@ __device__ float dtw_diag_mw(const float *__restrict__ qp, const float *__restri
                 const float tail = (cbs && i >= 0 && i < m) ? cbs[(i + kTailG) / kTailG] : 0.0f;
                 low = fminf(low, fminf(p1[t], p2[t]) + fmaxf(tail, rest));
             }
+            // (costs are not negative: their bit patterns order like their values)
+            const unsigned l = __reduce_min_sync(0xffffffffu, own ? __float_as_uint(low) : 0x7f800000u);
+            if (lane == 0) x.red[buf][w] = __uint_as_float(l);
+        }
+        group_bar(bar, 32 * W);
+        if (ABANDON) {
+            float low = INF;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
-            if (lane == 0) x.red[0][w] = low;
-            group_bar(bar, 32 * W);
-#pragma unroll
-            for (int v = 0; v < W; ++v) low = fminf(low, x.red[0][v]);
+            for (int v = 0; v < W; ++v) low = fminf(low, x.red[buf][v]);
             if (low > thr) {
                 if (gl == 0) cells += (int)band_cells_upto(a - 1, m, r);
-                group_bar(bar, 32 * W);  // x.red is read before anyone writes it again
+                group_bar(bar, 32 * W);  // x is read before anyone writes it again
                 return INF;
             }
         }
+        if (!own) {
+            const float *e = lane == 0 ? x.edge[buf][w - 1][1] : x.edge[buf][w + 1][0];
+#pragma unroll
+            for (int t = 0; t < K; ++t) {
+                p1[t] = e[t];
+                p2[t] = e[K + t];
+            }
+        }
+        __syncwarp();
+        buf ^= 1;
     }
+    // the rest: fewer than K pairs, so the overlaps last
     bool at_end = false;
     for (;; a += 2, ++bi, ++bj) {
-        diag_step_mw<W, K, 0, 0, 0>(qv, cv, p1, p2, pen, gl, lane, w, r, x, buf);
-        mw_publish<W, K>(p1, lane, w, x, buf, bar);
+        const float cn = cl[bj + K];
+        diag_step_mw<W, K, 0, 0, 0>(qv, cv, p1, p2, pen, gl, lane, r);
         if (a == last) {
 #pragma unroll
             for (int t = 0; t < K; ++t)
-                if (gl * K + t == pe_even) x.res = p1[t];
+                if (own && gl * K + t == pe_even) x.res = p1[t];
             at_end = true;
         }
         if (at_end) break;
-        shift_c_mw<K>(cv, cp, bj + 1, gl, lane);
-        diag_step_mw<W, K, 1, 0, 0>(qv, cv, p1, p2, pen, gl, lane, w, r, x, buf);
-        mw_publish<W, K>(p1, lane, w, x, buf, bar);
+#pragma unroll
+        for (int t = 0; t < K - 1; ++t) cv[t] = cv[t + 1];
+        cv[K - 1] = cn;
+        const float qn = ql[bi + 1];
+        diag_step_mw<W, K, 1, 0, 0>(qv, cv, p1, p2, pen, gl, lane, r);
         if (a + 1 == last) {
 #pragma unroll
             for (int t = 0; t < K; ++t)
-                if (gl * K + t == pe_odd) x.res = p1[t];
+                if (own && gl * K + t == pe_odd) x.res = p1[t];
             at_end = true;
         }
         if (at_end) break;
-        shift_q_mw<K>(qv, qp, bi + 1, gl, lane);
+#pragma unroll
+        for (int t = K - 1; t > 0; --t) qv[t] = qv[t - 1];
+        qv[0] = qn;
     }
     group_bar(bar, 32 * W);
     const float res = x.res;

@@ -24,6 +24,12 @@ namespace dtws {
 //     whose cells overlap by one lane on each side.  In kFxUnit = 8 steps an
 //     error at a warp's edge travels four cells, one lane; then the overlap is
 //     taken anew from the neighbours (one exchange per chunk).
+//   * With six such warps and more the producers beside them take more issue
+//     slots than the walk: a second CTA per direction forms most of the costs
+//     and writes them into the walking CTA's ring (distributed shared memory).
+//     m = 1024, r = 921, whole call: 302 us, 428 with two CTAs to a cluster; at
+//     W = 2 to 4 the cluster's barrier per chunk costs more than that (m = 2048,
+//     r = 200 403 us, 305 without).
 //
 // The fixed point: with an upper bound U of the DTW (the caller's, or the
 // diagonal path's cost) no partial sum above U lies on the best path.
@@ -43,7 +49,7 @@ namespace dtws {
 // m = 1024, r = 102 (210, 412), 170 us at r = 200 (311, 513); bound by the
 // consumers' ALU issue (25 cycles per cell of a lane) past two cells per lane,
 // and on several warps by the producers' beside it.
-constexpr int kFxUnit = 8, kFxRMax = 1023, kFxClusterCtas = 2;
+constexpr int kFxUnit = 8, kFxRMax = 1023;
 // a saturated cost; the value saturated sums are set back to every kFxUnit
 // steps (kFxInf + kFxUnit * kFxCost < 2^64, so no sum wraps in between)
 constexpr unsigned long long kFxCost = 1ull << 60, kFxInf = 1ull << 61, kFxRedo = 1ull << 51;
@@ -53,6 +59,7 @@ template <int K_, int W_>
 struct Fx {
     static constexpr int K = K_, W = W_;
     static constexpr int kThreads = W == 1 ? 384 : 768, kWarps = kThreads / 32;
+    static constexpr int kCtas = W < 6 ? 2 : 4;  // of a cluster: two that walk, past W = 4 two that only form costs
     static constexpr int kSteps = W == 1 ? 16 : kFxUnit;   // anti-diagonals of a chunk
     static constexpr int kLanes = W == 1 ? 32 : 30 * W + 2;  // lanes without the overlaps
     static constexpr int kCells = K * kLanes;
@@ -154,15 +161,18 @@ __device__ __forceinline__ unsigned long long fx_round(float hi, float lo) {
 // -1e15): a cell outside [0, m)^2 comes out far above 2^59, as do sums that
 // overflow, and everything not below 2^59 becomes kFxCost.  dst: the steps'
 // ring slots.
+// far: the ring of the cluster's CTA `rank` instead of this one's (dst: this
+// one's address of the slots).
 template <typename S>
 __device__ __forceinline__ void fx_produce(const dfloat *qd, const dfloat *cd, int r, float f, int v0, int blk,
-                                           unsigned long long *dst, int lane) {
+                                           unsigned long long *dst, int lane, bool far, int rank) {
     const int p = blk * 32 + lane, a = v0 - (r & 1);
     if (S::kCells % 32 && p >= S::kCells) return;
     const int pc = p < r ? p : r;  // (past the band no cost counts, and no address either)
     const dfloat *qp = qd + (((a + r) >> 1) - pc), *cp = cd + (((a - r) >> 1) + pc);
     const int pl = p / S::K, pt = p - pl * S::K;
     unsigned long long *o = dst + ((pt >> 1) * S::kLanes + pl) * 2 + (pt & 1);
+    const unsigned oa = far ? peer_addr(o, rank) : 0u;
     const bool in0 = p <= r, in1 = p < r;  // cells of an even, of an odd step
     dfloat c = cp[0];
 #pragma unroll
@@ -176,8 +186,9 @@ __device__ __forceinline__ void fx_produce(const dfloat *qd, const dfloat *cd, i
             const float sq = __fmul_rn(h, h);
             const float er = fmaf(h + h, l, fmaf(h, h, -sq));
             const bool fine = (e ? in1 : in0) && sq < 0x1p59f;
-            const unsigned long long w = fx_round(sq, er);
-            o[(s + e) * S::kStep] = fine ? w : kFxCost;
+            const unsigned long long w = fx_round(sq, er), v = fine ? w : kFxCost;
+            if (S::kCtas > 2 && far) peer_store(oa + (s + e) * S::kStep * 8, v);
+            else o[(s + e) * S::kStep] = v;
         }
     }
 }
@@ -224,20 +235,22 @@ __device__ __forceinline__ void fx_clamp(unsigned long long (&v)[K]) {
     }
 }
 
-// The walk by the S::kThreads threads of each of a cluster's two CTAs (all
-// of them).  dir: the CTA's rank, 1 for the reversed sequences.  qd, cd:
+// The walk by the S::kThreads threads of each of a cluster's CTAs (all of
+// them).  rank: the CTA's; its lowest bit is the direction, 1 for the reversed
+// sequences; ranks 2 and 3 only form costs.  qd, cd:
 // element 0 of q_hat and of the normalised window as double-floats (reversed
-// when dir is 1), padded by fx_pad(r) elements of +1e15 and -1e15 on both
+// in direction 1), padded by fx_pad(r) elements of +1e15 and -1e15 on both
 // sides; bound: an upper bound of the DTW, 0 for the diagonal path's cost;
-// ring: S::kRing bytes, 16-byte aligned.  Every thread of both CTAs returns
+// ring: S::kRing bytes, 16-byte aligned.  Every thread of all CTAs returns
 // the distance.
 template <typename S>
 __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict__ cd, int m, int r, float bound,
-                         int dir, FxShared &sh, unsigned long long *ring) {
+                         int rank, FxShared &sh, unsigned long long *ring) {
     constexpr int K = S::K, W = S::W;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, dir = rank & 1;
+    const bool helper = rank >= 2;  // (forms costs for the ring of rank - 2)
     // the diagonal path's cost, an upper bound of the DTW (the same sum, in
-    // the same order, in every thread of both CTAs)
+    // the same order, in every thread of all CTAs)
     auto euclid = [&]() {
         float ed = 0.0f;
         for (int j = t; j < m; j += S::kThreads) {
@@ -261,24 +274,46 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
     int h = scale_of(bound);          // the scale is 2^(2h)
     // the forward walk ends on anti-diagonal m - 1, the reversed one on the
     // next (its own m - 2)
-    const int V = m - dir + (r & 1), chunks = (V + S::kSteps - 1) / S::kSteps;
+    const int V = m - dir + (r & 1);
+    // (the directions meet at every chunk where the cluster's barrier ends it:
+    // as many for both then)
+    const int chunks = ((S::kCtas > 2 ? m + (r & 1) : V) + S::kSteps - 1) / S::kSteps;
+    const bool walks = warp < W && !helper;
+    // a chunk ends where its walkers and producers meet
+    auto meet = []() {
+        if constexpr (S::kCtas > 2) cluster_bar();
+        else __syncthreads();
+    };
     const int p0 = (r - (r & 1)) >> 1;
     const int vl = W == 1 ? lane : warp * 30 + lane;
     // the lanes whose cells are this warp's own
-    const bool own = warp < W && (warp == 0 || lane > 0) && (warp == W - 1 || lane < 31);
+    const bool own = walks && (warp == 0 || lane > 0) && (warp == W - 1 || lane < 31);
     for (int pass = 0;; ++pass) {
         const float f = ldexpf(1.0f, h);
-        // a chunk's units: kFxUnit steps of one block of 32 cells each
+        // a chunk's units: kFxUnit steps of one block of 32 cells each, of the
+        // blocks that hold cells of the band; the others' costs never change
         constexpr int kBlks = (S::kCells + 31) / 32;
+        const int blks = S::kCtas == 2 ? kBlks : r / 32 + 1;  // (two CTAs: no division by a variable)
         auto produce = [&](int c, int w, int nw) {
             unsigned long long *buf = ring + (size_t)(c & 1) * S::kSteps * S::kStep;
-            for (int u = w; u < kBlks * (S::kSteps / kFxUnit); u += nw) {
-                const int blk = u % kBlks, s0 = u / kBlks * kFxUnit;
-                fx_produce<S>(qd, cd, r, f, c * S::kSteps + s0, blk, buf + s0 * S::kStep, lane);
+            for (int u = w; u < blks * (S::kSteps / kFxUnit); u += nw) {
+                const int blk = u % blks, s0 = u / blks * kFxUnit;
+                fx_produce<S>(qd, cd, r, f, c * S::kSteps + s0, blk, buf + s0 * S::kStep, lane, helper, dir);
             }
         };
-        produce(0, warp, S::kWarps);
-        __syncthreads();
+        if constexpr (S::kCtas > 2) {
+            for (int p = blks * 32 + t; p < S::kCells && !helper; p += S::kThreads) {
+                const int pl = p / K, pt = p - pl * K;
+                for (int s = 0; s < 2 * S::kSteps; ++s)
+                    ring[(size_t)s * S::kStep + ((pt >> 1) * S::kLanes + pl) * 2 + (pt & 1)] = kFxCost;
+            }
+        }
+        // the helper's warps first, then the ones that don't walk
+        const int pw = S::kCtas == 2 ? warp - W : helper ? warp : S::kWarps + warp - W;
+        constexpr int kPw = S::kCtas == 2 ? S::kWarps - W : 2 * S::kWarps - W;
+        if constexpr (S::kCtas == 2) produce(0, warp, S::kWarps);
+        else if (!walks) produce(0, pw, kPw);
+        meet();
         unsigned long long p1[K], p2[K];
 #pragma unroll
         for (int u = 0; u < K; ++u) {
@@ -290,8 +325,8 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
         }
         for (int c = 0; c < chunks; ++c) {
             const unsigned long long *buf = ring + (size_t)(c & 1) * S::kSteps * S::kStep;
-            if (warp < W) {
-                const int steps = V - c * S::kSteps < S::kSteps ? V - c * S::kSteps : S::kSteps;
+            if (walks) {
+                const int steps = V - c * S::kSteps < S::kSteps ? V - c * S::kSteps : S::kSteps;  // (0: none left)
                 if (steps == S::kSteps) {
 #pragma unroll 1
                     for (int s0 = 0; s0 < S::kSteps; s0 += kFxUnit) {
@@ -323,11 +358,11 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
                     }
                 }
             } else if (c + 1 < chunks) {
-                produce(c + 1, warp - W, S::kWarps - W);
+                produce(c + 1, pw, kPw);
             }
-            __syncthreads();
+            meet();
             if constexpr (W > 1) {
-                if ((lane == 0 && warp > 0 && warp < W) || (lane == 31 && warp < W - 1)) {
+                if (walks && ((lane == 0 && warp > 0) || (lane == 31 && warp < W - 1))) {
                     const ulonglong2 *e = lane == 0 ? sh.edge[c & 1][warp - 1][1] : sh.edge[c & 1][warp + 1][0];
                     const ulonglong2 a0 = e[0], a1 = e[1], b0 = e[2], b1 = e[3];
                     p1[0] = a0.x;
@@ -358,7 +393,7 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
             }
         }
         cluster_bar();
-        if (!dir && warp < W) {
+        if (!dir && walks) {
             const bool even = ((m - 1 + r) & 1) == 0;  // anti-diagonal m - 1 is an even step
             const unsigned a1 = peer_addr(last1, 1), a2 = peer_addr(last2, 1);
             auto at = [](unsigned a, int j) { return j >= 0 ? peer_load(a + (unsigned)j * 8) : kFxInf; };
@@ -385,7 +420,7 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
             if (lane == 0) atomicMin(&sh.res, best);
         }
         __syncthreads();
-        if (!dir && t == 0) peer_store(peer_addr(&sh.res, 1), sh.res);
+        if (rank == 0 && t > 0 && t < S::kCtas) peer_store(peer_addr(&sh.res, t), sh.res);
         cluster_bar();
         const unsigned long long res = sh.res;
         __syncthreads();  // (sh.res is read before it is written again)

@@ -95,11 +95,12 @@ __host__ __device__ constexpr int dtw_min_blocks(int K) {
     return (K >= 1 && K <= 2) ? 4 : (K >= 1 && K <= 4) ? 3 : (K >= 16) ? 1 : 2;
 }
 
-// Shapes whose seeds walk from both ends (dtw_ends): one warp per window, up to
-// 16 cells per lane.  The search waits for the few seeds of a top-k search one
-// walk long (ten of m = 999, r = 99: 95 us, 140 from one end).  The survivor
-// pass stays with dtw_diag: it is bound by its bounds, not by walks, and the
-// wider walk's registers spill at its three CTAs per SM.
+// Shapes whose seeds walk from both ends (dtw_ends): one warp per window, up
+// to 16 cells per lane.  A top-k search waits for its seeds one walk long
+// (m = 999, r = 99: the seeds' phase takes 146 us, 186 from one end; on four
+// warps, dtw_diag_mw, a walk of m = 1871, r = 191 took half as long again).  The
+// survivor pass stays with dtw_diag: it is bound by its bounds, not by walks,
+// and the wider walk's registers spill at its three CTAs per SM.
 __host__ __device__ constexpr bool ends_applies(int L, int K) { return L == 32 && K >= 1 && K <= 8; }
 
 // The body of k_dtw for one query (the CTA's part of its candidate stream);
@@ -647,7 +648,7 @@ static cudaError_t dtw_dispatch(const QueryBufs &b, const QueryArgs &a, const in
 // ------------------------------------------------------------------ wide bands
 // The FP32 DTW kernel for bands past the one-warp walks (kDiagRMax < r <=
 // 2047): a group of W = 4 warps per candidate (dtw_diag_mw, K cells per
-// lane, 128 K >= r + 1), two groups per CTA of 256 threads (one when the
+// lane, 122 K >= r + 1), two groups per CTA of 256 threads (one when the
 // copies do not fit).  The same three modes and the same per-candidate
 // steps as k_dtw (one candidate at a time per group, the pre-check of the
 // survivor mode over the group's 128 threads); group decisions come from
@@ -655,8 +656,7 @@ static cudaError_t dtw_dispatch(const QueryBufs &b, const QueryArgs &a, const in
 // its threads take the same branches.
 
 __host__ __device__ inline int wide_k(int r) {
-    const int need = (r + 1 + 32 * kWideW - 1) / (32 * kWideW);
-    return need <= 6 ? 6 : need <= 8 ? 8 : need <= 12 ? 12 : 16;
+    return r < mw_cells(kWideW, 5) ? 5 : r < mw_cells(kWideW, 9) ? 9 : r < mw_cells(kWideW, 13) ? 13 : 17;
 }
 __host__ __device__ inline size_t wide_span(int m, int r, int K) {
     return (size_t)((m + 2 * diag_pad(r, 32 * kWideW, K) + 3) & ~3);

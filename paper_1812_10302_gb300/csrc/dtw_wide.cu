@@ -35,10 +35,10 @@ cudaError_t dtw_wide_launch(const QueryBufs &b, const QueryArgs &a, const int64_
                             float *out, int64_t count_for_grid, cudaStream_t s) {
     if (a.r <= kDiagRMax || a.r > kWideRMax) return cudaErrorInvalidValue;
     switch (wide_k(a.r)) {
-    case 6: return wide_launch_k<6, MODE>(b, a, offsets, count, out, count_for_grid, s);
-    case 8: return wide_launch_k<8, MODE>(b, a, offsets, count, out, count_for_grid, s);
-    case 12: return wide_launch_k<12, MODE>(b, a, offsets, count, out, count_for_grid, s);
-    default: return wide_launch_k<16, MODE>(b, a, offsets, count, out, count_for_grid, s);
+    case 5: return wide_launch_k<5, MODE>(b, a, offsets, count, out, count_for_grid, s);
+    case 9: return wide_launch_k<9, MODE>(b, a, offsets, count, out, count_for_grid, s);
+    case 13: return wide_launch_k<13, MODE>(b, a, offsets, count, out, count_for_grid, s);
+    default: return wide_launch_k<17, MODE>(b, a, offsets, count, out, count_for_grid, s);
     }
 }
 

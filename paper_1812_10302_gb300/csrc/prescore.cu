@@ -7,16 +7,15 @@ namespace dtws {
 // Pre-score of the best Euclidean seed, run on a side stream while the
 // lower-bound scan streams: its FP32 DTW enters the result list (the survivor
 // pass skips it) and its extended-precision re-score waits for the final
-// stage.  Two clusters of two CTAs: the first walks the fixed-point re-score
+// stage.  Two clusters: the first walks the fixed-point re-score
 // (dtw_fx), the second's first CTA the FP32 DTW (one warp, or several past
 // one warp's four cells per lane).  When the scan is short the search waits
 // for this kernel, so its latency counts: at m = 1001, r = 400 the final stage
 // waits 0.17 ms for it, against 0.47 ms with the double-float walk on four
 // warps.
-__host__ __device__ constexpr int fx_f32_warps(int W) { return W == 1 ? 1 : W == 2 ? 4 : 8; }
-__host__ __device__ constexpr int fx_f32_cells(int K, int W) { return W == 1 ? K : W <= 4 ? 2 : 4; }
+__host__ __device__ constexpr int fx_f32_cells(int K, int W) { return W == 1 ? K : 5; }
 template <int K, int W>
-__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+__global__ void __cluster_dims__(Fx<K, W>::kCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
 k_prescore_fx(QueryBufs b, QueryArgs a) {
     using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -27,10 +26,10 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
     if (idx == 0xffffffffu) return;
     const int m = a.m, r = a.r, t = threadIdx.x;
     const float *xw = b.x + idx;
-    if (blockIdx.x >= kFxClusterCtas) {  // the FP32 DTW, as the survivor pass would compute it
-        constexpr int W32 = fx_f32_warps(W), K32 = fx_f32_cells(K, W), kThr = 32 * W32;
-        static_assert(kThr * K32 + 2 >= S::kCells || kThr * K32 > kFxRMax, "a cell per offset of the band");
-        if (blockIdx.x > kFxClusterCtas || t >= kThr) return;
+    if (blockIdx.x >= S::kCtas) {  // the FP32 DTW, as the survivor pass would compute it
+        constexpr int W32 = W, K32 = fx_f32_cells(K, W), kThr = 32 * W32;
+        static_assert(W == 1 ? 32 * K32 >= S::kCells : mw_cells(W32, K32) >= S::kCells, "a cell per offset of the band");
+        if (blockIdx.x > S::kCtas || t >= kThr) return;
         const int lane = t & 31, pad = diag_pad(r, kThr, K32);
         float *q32 = (float *)smraw, *c32 = q32 + pre_span(m, r, kThr, K32);
         const float INF = __int_as_float(0x7f800000);
@@ -64,12 +63,12 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
     // of several answers all are walked on common terms in the final stage
     // (k_final_fx), which would wait here for nothing
     if (a.k > 1) return;
-    const int dir = cluster_rank();
+    const int rank = cluster_rank(), dir = rank & 1;
     dfloat *qd, *cd;
     fx_setup<S>(smraw, b.qh64, m, r, dir, &qd, &cd);
     fx_window<S>(xw, m, a.raw != 0, dir, cd, sh);
-    const double d64 = dtw_fx<S>(qd, cd, m, r, 0.0f, dir, sh, (unsigned long long *)smraw);
-    if (t == 0 && dir == 0) {
+    const double d64 = dtw_fx<S>(qd, cd, m, r, 0.0f, rank, sh, (unsigned long long *)smraw);
+    if (t == 0 && rank == 0) {
         st->pre_d64 = d64;
         __threadfence();
         st->pre_done = 1;
@@ -78,12 +77,12 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
 
 template <int K, int W>
 static cudaError_t prescore_fx_launch(const QueryBufs &b, const QueryArgs &a, cudaStream_t s) {
-    const size_t fx = fx_bytes(a.m, a.r), f32 = pre_span(a.m, a.r, 32 * fx_f32_warps(W), fx_f32_cells(K, W)) * 8;
+    const size_t fx = fx_bytes(a.m, a.r), f32 = pre_span(a.m, a.r, 32 * W, fx_f32_cells(K, W)) * 8;
     const size_t smem = fx > f32 ? fx : f32;
     cudaError_t e =
         cudaFuncSetAttribute(k_prescore_fx<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_prescore_fx<K, W><<<2 * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a);
+    k_prescore_fx<K, W><<<2 * Fx<K, W>::kCtas, Fx<K, W>::kThreads, smem, s>>>(b, a);
     return cudaGetLastError();
 }
 

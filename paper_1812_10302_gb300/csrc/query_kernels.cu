@@ -1376,24 +1376,24 @@ __global__ void k_reset_cursor(QueryState *st) { st->work = 0; }
 
 // The fixed-point walk at given offsets, a cluster of two CTAs per window.
 template <int K, int W>
-__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+__global__ void __cluster_dims__(Fx<K, W>::kCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
 k_dtw_fx_at(QueryBufs b, QueryArgs a, const int64_t *offsets, int64_t count, double *out) {
     using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ FxShared sh;
     if (!b.st->valid) return;
-    const int m = a.m, t = threadIdx.x, dir = cluster_rank();
+    const int m = a.m, t = threadIdx.x, rank = cluster_rank(), dir = rank & 1;
     dfloat *qd, *cd;
     fx_setup<S>(smraw, b.qh64, m, a.r, dir, &qd, &cd);
-    for (int64_t c = blockIdx.x / kFxClusterCtas; c < count; c += gridDim.x / kFxClusterCtas) {
+    for (int64_t c = blockIdx.x / S::kCtas; c < count; c += gridDim.x / S::kCtas) {
         const int64_t o = offsets[c];
         if (o < 0 || o >= a.N) {
-            if (t == 0 && dir == 0) out[c] = __longlong_as_double(0x7ff8000000000000ll);
+            if (t == 0 && rank == 0) out[c] = __longlong_as_double(0x7ff8000000000000ll);
             continue;
         }
         fx_window<S>(b.x + o, m, a.raw != 0, dir, cd, sh);
-        const double d = dtw_fx<S>(qd, cd, m, a.r, 0.0f, dir, sh, (unsigned long long *)smraw);
-        if (t == 0 && dir == 0) out[c] = d;
+        const double d = dtw_fx<S>(qd, cd, m, a.r, 0.0f, rank, sh, (unsigned long long *)smraw);
+        if (t == 0 && rank == 0) out[c] = d;
     }
 }
 
@@ -1403,23 +1403,24 @@ cudaError_t dtw_fx_at_launch(const QueryBufs &b, const QueryArgs &a, const int64
     const size_t smem = fx_bytes(a.m, a.r);
     cudaError_t e = cudaFuncSetAttribute(k_dtw_fx_at<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_dtw_fx_at<K, W><<<(unsigned)count * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, offsets, count, out);
+    k_dtw_fx_at<K, W><<<(unsigned)count * Fx<K, W>::kCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, offsets, count, out);
     return cudaGetLastError();
 }
 
 // Few offsets get the fixed-point walk (latency), a cluster each: up to two
-// per SM where one warp walks, up to three clusters per two SMs where several
-// do (a CTA then fills an SM: three waves).  Past that the walks for many
-// windows.  Measured for 64 windows, from both ends (from one, in
-// double-float): m = 512, r = 51 78 us (103, 210); m = 1024, r = 102 132 us
-// (210, 598); m = 1024, r = 921 428 us.
+// per SM where one warp walks, up to three per two SMs where several do, one
+// per two SMs where a cluster has four CTAs (each then fills an SM: three and
+// two waves).  Past that the walks for many windows.  Measured for 64 windows,
+// from both ends (from one, in double-float): m = 512, r = 51 78 us (103, 210);
+// m = 1024, r = 102 132 us (210, 598); m = 1024, r = 921 558 us.
 constexpr int kFxAtPerSm = 2;
 }  // namespace
 
 cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int64_t *offsets,
                               int64_t count, double *out, cudaStream_t s) {
     const FxPlan p = fx_plan(a.r);
-    if (fx_used(a.m, a.r) && count > 0 && count <= (int64_t)(p.W == 1 ? kFxAtPerSm * b.num_sms : b.num_sms + b.num_sms / 2)) {
+    const int64_t few = p.W == 1 ? kFxAtPerSm * b.num_sms : p.W < 6 ? b.num_sms * 3 / 2 : b.num_sms / 2;
+    if (fx_used(a.m, a.r) && count > 0 && count <= few) {
 #define DTWS_FX_CASE(KK, WW) \
     if (p.K == KK && p.W == WW) return dtw_fx_at_launch<KK, WW>(b, a, offsets, count, out, s);
         DTWS_FX_SHAPES(DTWS_FX_CASE)
@@ -1894,7 +1895,7 @@ __global__ void k_final_sort(QueryBufs b, QueryArgs a, int64_t *out_idx, float *
 // itself.  A top-10 search re-scores ten windows here: 0.1 ms, against 0.53 ms
 // on one double-float warp each (m = 999, r = 99).
 template <int K, int W>
-__global__ void __cluster_dims__(kFxClusterCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
+__global__ void __cluster_dims__(Fx<K, W>::kCtas, 1, 1) __launch_bounds__(Fx<K, W>::kThreads, W == 1 ? 2 : 1)
 k_final_fx(QueryBufs b, QueryArgs a, FinalOut fin) {
     using S = Fx<K, W>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1905,8 +1906,8 @@ k_final_fx(QueryBufs b, QueryArgs a, FinalOut fin) {
     __shared__ int ms_n, ms_skip, last;
     __shared__ float ms_bound;
     QueryState *st = b.st;
-    const int m = a.m, t = threadIdx.x, dir = cluster_rank();
-    const int first = (int)(blockIdx.x / kFxClusterCtas), clusters = (int)(gridDim.x / kFxClusterCtas);
+    const int m = a.m, t = threadIdx.x, rank = cluster_rank(), dir = rank & 1;
+    const int first = (int)(blockIdx.x / S::kCtas), clusters = (int)(gridDim.x / S::kCtas);
     const bool valid = st->valid != 0;
     for (int j = t; j < a.list_cap; j += S::kThreads) ms_keys[j] = valid ? st->res_keys[j] : kEmptyKey;
     __syncthreads();
@@ -1940,13 +1941,13 @@ k_final_fx(QueryBufs b, QueryArgs a, FinalOut fin) {
     if (ms_skip + first < ms_n) fx_setup<S>(smraw, b.qh64, m, a.r, dir, &qd, &cd);
     for (int c = ms_skip + first; c < ms_n; c += clusters) {
         fx_window<S>(b.x + ms_idx[c], m, a.raw != 0, dir, cd, sh);
-        const double d = dtw_fx<S>(qd, cd, m, a.r, ms_bound, dir, sh, (unsigned long long *)smraw);
-        if (t == 0 && dir == 0) {
+        const double d = dtw_fx<S>(qd, cd, m, a.r, ms_bound, rank, sh, (unsigned long long *)smraw);
+        if (t == 0 && rank == 0) {
             st->margin_d64[c] = d;
             __threadfence();  // (before this CTA counts itself done)
         }
     }
-    if (dir != 0) return;
+    if (rank != 0) return;
     __syncthreads();
     if (t == 0) {
         __threadfence();
@@ -1965,7 +1966,9 @@ static cudaError_t final_fx_launch(const QueryBufs &b, const QueryArgs &a, Final
     const size_t smem = fx_bytes(a.m, a.r);
     cudaError_t e = cudaFuncSetAttribute(k_final_fx<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_final_fx<K, W><<<a.list_cap * kFxClusterCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, fin);
+    // (a CTA of several walking warps fills an SM: few more clusters than answers)
+    const int clusters = W == 1 || a.k + 8 > a.list_cap ? a.list_cap : a.k + 8;
+    k_final_fx<K, W><<<clusters * Fx<K, W>::kCtas, Fx<K, W>::kThreads, smem, s>>>(b, a, fin);
     return cudaGetLastError();
 }
 

@@ -29,3 +29,25 @@ def test_answers_at_shape_edges(m, r, exact_envelope):
     np.testing.assert_allclose(dist, od, rtol=1e-6)
     np.testing.assert_array_equal(bi[0], oi)
     np.testing.assert_allclose(bd[0], od, rtol=1e-6)
+
+
+@pytest.mark.parametrize("m,r", [(513, 512), (620, 512), (609, 608), (611, 609), (700, 610), (1097, 1096), (1100, 1097),
+                                 (1099, 1098), (1585, 1584), (1590, 1585), (2048, 2047), (2100, 2047), (1024, 921)])
+def test_overlapping_warps(m, r):
+    """The walk over four warps at the widest band of each cell count (122 K >
+    r, K = 5, 9, 13, 17) and the first past it, both parities, with and without
+    abandoning; the pre-score's shapes beside it."""
+    x = synth.random_walk(3 * m, m + r)
+    q, o = synth.noisy_copy(x, m, m, r, noise=0.2)
+    offs = np.array([o, 0, x.size - m, m // 2, m + 1])
+    with dtws.Index(x) as ix:
+        got = ix.dtw_at(q, r, offs)
+        idx, dist = ix.query(q, r, 2)
+        one, d1 = ix.query(q, r, 1)
+        assert ix.sync_status() == dtws.DTWS_OK
+    np.testing.assert_allclose(got, oracle.dtw_at(x, q, r, offs), rtol=1e-4, atol=1e-6 * m)
+    oi, od = oracle.search_cascade(x, q, r, 2)
+    np.testing.assert_array_equal(idx, oi)
+    np.testing.assert_allclose(dist, od, rtol=1e-6)
+    assert one[0] == oi[0]
+    np.testing.assert_allclose(d1[0], od[0], rtol=1e-6)
