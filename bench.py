@@ -407,12 +407,12 @@ def gpu_arm(args):
         got = n_off * cells(m, r) / (walk_ms * 1e-3)
         dtw_ms = float(phases[4])
         surv = st["dtw_cells"] / (dtw_ms * 1e-3) if dtw_ms > 0 else None
-        # the library's shape for DTW at offsets: four cells per lane on 8 or
-        # 16 lanes for bands of 9..64 cells, else the survivor pass's shape
+        # the shapes for DTW at offsets take bands of 5..256 cells (8 lanes x 7
+        # cells for 52 cells at m = 512), the survivor pass's the others
         need = r + 1
-        shape = (f"{8 if need <= 32 else 16} lanes x 4 cells per window" if 8 < need <= 64
+        shape = ("the least-cost lanes x cells for the band (csrc/dtw_at.cuh)" if 5 <= need <= 256
                  else "the survivor pass's shape")
-        dtw_roof = {"kernel": "k_dtw (the walk: dtws_dtw_at, no pruning)", "shape": shape,
+        dtw_roof = {"kernel": "k_dtw_at (the walk: dtws_dtw_at, no pruning)", "shape": shape,
                     "bound": "alu", "achieved": got,
                     "peak": peak_cells, "unit": "cells/s", "frac": got / peak_cells, "ops_per_cell": 5,
                     "peak_source": f"{sms} SMs x 128 lanes x {mhz:.0f} MHz / 5",

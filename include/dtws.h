@@ -82,7 +82,9 @@ typedef struct {
     float alpha_per_m;      /* absolute margin per query sample, default 1e-6 */
     int32_t seed_random;    /* random seed windows, default 4 (0..64) */
     int32_t seed_proposals; /* proposals of the proxy (or learned) scan,
-                               default 16 (0..64) */
+                               default 16 (0..64); with the proxy's the best
+                               window of every scanning warp is scored too
+                               (0: no scan) */
     int32_t proxy_terms;    /* evenly spaced query positions in the proxy
                                distance: 16, 8, 4 (other values round down to
                                one of them, or 2), default 16 */
@@ -104,7 +106,8 @@ typedef struct {
                                graph once and replays it for later calls with
                                the same arguments (not with the learned
                                ordering); dtws_query does the same for one
-                               query (not while timing is on).  The query
+                               query, from its second repeat (not while
+                               timing is on).  The query
                                values may change between replays. */
     int32_t exclusion_zone; /* z >= 0 (default 0): dtws_query returns the k
                                best windows of which no two lie within z
@@ -178,9 +181,10 @@ void dtws_default_options(dtws_options *opt);
  * Create a search handle over series[0..n) (FP32, host or device).  The
  * series is COPIED into library-owned device memory padded to the tile size,
  * so the caller may release its buffer once the call returns; this call
- * synchronises `stream`.  It also builds the anchored FP64 prefix sums of the
+ * synchronises `stream`.  It also builds the anchored prefix sums of the
  * series (blocks of DTWS_M_MAX samples, each summed relative to its first
- * sample) that every window statistic derives from.
+ * sample, in FP32 expansions more exact than FP64) that every window
+ * statistic derives from.
  * Errors: DTWS_EINVAL (n < 2, n > DTWS_N_MAX, null), DTWS_ENONFINITE (a NaN
  * or Inf sample), DTWS_ENOMEM, DTWS_ECUDA.  On error *out is NULL.
  */
@@ -199,8 +203,9 @@ dtws_status dtws_get_options(dtws_t h, dtws_options *opt);
  * k: 1 <= k <= min(N, DTWS_K_MAX).
  * out_idx: int64 [k], offsets ascending by (distance, offset).
  * out_dist: FP32 [k], squared banded DTW of the z-normalised query and
- *   window, re-scored in extended precision (FP64 statistics, DTW in
- *   double-float arithmetic, ~48 significant bits) and rounded to FP32.
+ *   window, re-scored in extended precision (FP64 statistics, DTW in 64-bit
+ *   fixed point, or in double-float arithmetic where that does not fit:
+ *   ~48 significant bits) and rounded to FP32.
  *   The offsets are ordered by that re-scored distance, then by offset.
  * A window (or query) whose variance is <= 1e-24*max(1, mean^2) normalises
  * to all zeros.  Per-series data for this m (window statistics) and r
@@ -208,7 +213,8 @@ dtws_status dtws_get_options(dtws_t h, dtws_options *opt);
  * With options.exclusion_zone = z > 0 the k results are more than z
  * samples apart (see dtws_options).  With options.batch_graph = 1 a call
  * whose arguments (pointers, m, r, k, options) repeat the previous one's
- * replays the captured search; the query values may differ.
+ * captures the search, and later ones replay it; the query values may differ.
+ * (A stream under capture by the caller takes a search that has run once.)
  * With options.unnormalised = 1 neither side is normalised (raw values).
  * Errors: DTWS_EINVAL synchronously (also unnormalised DTW with the learned
  * ordering or with a series beyond +-2^32); DTWS_ENONFINITE and
@@ -292,10 +298,11 @@ dtws_status dtws_series_envelope(dtws_t h, int32_t r, float *U, float *L, void *
 dtws_status dtws_dtw_at(dtws_t h, const float *Q, int32_t m, int32_t r,
                         const int64_t *offsets, int64_t count, float *out, void *stream);
 
-/* Same, in extended precision: per-window two-pass FP64 statistics (Eq. 5),
-   normalised values formed in FP64 and the DTW in double-float arithmetic
-   (~48 significant bits; plain FP64 for bands wider than 511): the re-score
-   kernel of dtws_query.  out: FP64 [count]. */
+/* Same, in extended precision: per-window two-pass statistics (Eq. 5) exact to
+   FP64, and the DTW in 64-bit fixed point for few offsets (up to two per SM
+   and bands to 1023: the re-score of dtws_query) or in double-float arithmetic
+   (~48 significant bits; plain FP64 for bands wider than 2047).
+   out: FP64 [count]. */
 dtws_status dtws_dtw_at_f64(dtws_t h, const float *Q, int32_t m, int32_t r,
                             const int64_t *offsets, int64_t count, double *out,
                             void *stream);
@@ -449,7 +456,7 @@ dtws_status dtws_trainer_destroy(dtws_trainer_t t);
  * Q FP32 [m] (raw), offsets int64 [count] (each in [0, n-m]), out FP32
  * [count]; nothing is staged.  Result: the FP32 Sakoe-Chiba-banded DTW of
  * the z-normalised query against each z-normalised window, each window's
- * mean and deviation computed two-pass in FP64, the same quantity as
+ * mean and deviation computed two-pass, exact to FP64, the same quantity as
  * dtws_dtw_at; an offset out of range, or a non-finite query, gives NaN.
  * count may be any value >= 0 (the work cursor is 64-bit); count == 0
  * returns at once.
