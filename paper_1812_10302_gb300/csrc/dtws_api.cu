@@ -675,7 +675,11 @@ QueryArgs make_args(dtws_t h, int m, int r, int k, bool raw) {
     float g = 1.17549435e-38f;
     while (g * 2.0f <= a.alpha * 0.25f) g *= 2.0f;
     a.qgrid = g;
-    a.prescore = a.r <= kDiagRMaxF32 ? 1 : 0;
+    // The best Euclidean seed is scored on the side stream.  Of several answers
+    // it is among the exact seeds already (exact_seeds): scored twice, by walks
+    // that round in different orders, its two keys can differ and the list then
+    // hold it twice.
+    a.prescore = k == 1 && a.r <= kDiagRMaxF32 ? 1 : 0;
     a.tune_l = a.tune_k = a.tune_w = 0;
     for (const auto &t : h->tune)
         if (t.m == m && t.r == a.r) {
@@ -873,6 +877,7 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
     Exec e{make_bufs(h, se, ee), s, h->side, h->ev_fork, h->ev_join, le, true};
     QueryArgs a = make_args(h, m, r, k);
     a.xz_z = xz_z;
+    if (xz_z > 0) a.prescore = a.r <= kDiagRMaxF32 ? 1 : 0;  // (no exact seeds then)
     int64_t launches = 0;
     // Repeated queries with the same arguments replay one CUDA graph of the
     // search, captured when they repeat (the caches above are resolved first, on the caller's stream;

@@ -60,8 +60,7 @@ k_prescore_fx(QueryBufs b, QueryArgs a) {
         }
         return;
     }
-    // of several answers all are walked on common terms in the final stage
-    // (k_final_fx), which would wait here for nothing
+    // (with an exclusion zone, several answers: all are re-scored at the end)
     if (a.k > 1) return;
     const int rank = cluster_rank(), dir = rank & 1;
     dfloat *qd, *cd;

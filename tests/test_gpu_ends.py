@@ -51,3 +51,20 @@ def test_overlapping_warps(m, r):
     np.testing.assert_allclose(dist, od, rtol=1e-6)
     assert one[0] == oi[0]
     np.testing.assert_allclose(d1[0], od[0], rtol=1e-6)
+
+
+@pytest.mark.parametrize("m,r", [(64, 5), (64, 20), (128, 60), (200, 142), (400, 300), (600, 560)])
+@pytest.mark.parametrize("k", [2, 5])
+def test_no_window_is_scored_twice(m, r, k):
+    """With no more windows than the exact seeds reach, every window is scored
+    once: the best Euclidean seed is one of them, and a second score, rounded
+    in another order, could put it into the list of results twice."""
+    x = synth.random_walk(m + k, m + r)
+    q, _ = synth.noisy_copy(x, m, m, r, noise=0.3)
+    with dtws.Index(x) as ix:
+        idx, dist = ix.query(q, r, k)
+        assert ix.sync_status() == dtws.DTWS_OK
+        assert ix.last_stats()["dtw_started"] <= k + 1
+    oi, od = oracle.search_cascade(x, q, r, k)
+    np.testing.assert_array_equal(idx, oi)
+    np.testing.assert_allclose(dist, od, rtol=1e-6)
