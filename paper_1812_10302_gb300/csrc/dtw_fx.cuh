@@ -249,6 +249,11 @@ __device__ double dtw_fx(const dfloat *__restrict__ qd, const dfloat *__restrict
     constexpr int K = S::K, W = S::W;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, dir = rank & 1;
     const bool helper = rank >= 2;  // (forms costs for the ring of rank - 2)
+    // A helper's first act is a store into its walker's shared memory, which
+    // may only be touched once every CTA of the cluster is known to have
+    // started.  (With two CTAs the first access comes after a chunk's meeting
+    // and the join's barrier.)
+    if constexpr (S::kCtas > 2) cluster_bar();
     // the diagonal path's cost, an upper bound of the DTW (the same sum, in
     // the same order, in every thread of all CTAs)
     auto euclid = [&]() {

@@ -59,6 +59,23 @@ def test_several_walking_warps(series, m, r):
     np.testing.assert_allclose(dist, od, rtol=1e-6)
 
 
+@pytest.mark.parametrize("m,r", [(500, 487), (620, 600), (740, 730), (1060, 1000)])
+def test_clusters_of_four_in_several_waves(series, m, r):
+    """Bands whose costs come from a second pair of CTAs (six and nine walking
+    warps), with twice as many clusters as fit the GPU: a cluster of a later
+    wave starts, CTA by CTA, as earlier ones end, and none of its CTAs touches
+    another's shared memory before all have started."""
+    q, o = synth.noisy_copy(series, m, m + r, m + 2 * r, noise=0.1)
+    offs = np.random.default_rng(m + r).integers(0, series.size - m + 1, 70)
+    offs[:3] = [o, 0, series.size - m]
+    with dtws.Index(series) as ix:
+        got = [ix.dtw_at_f64(q, r, offs) for _ in range(5)]
+        assert ix.sync_status() == dtws.DTWS_OK
+    np.testing.assert_allclose(got[0], oracle.dtw_at(series, q, r, offs), rtol=1e-10)
+    for g in got[1:]:
+        np.testing.assert_array_equal(g, got[0])
+
+
 @pytest.mark.parametrize("unnormalised,scale", [(0, 1.0), (1, 1.0), (1, 2.0 ** -30), (1, 2.0 ** 20)])
 def test_far_below_the_euclidean_distance(unnormalised, scale):
     """Shifted copies of a smooth window: warping absorbs the shift, so the DTW
