@@ -479,6 +479,13 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
     return DTWS_OK;
 }
 
+// The kept graph of a repeated query.
+void drop_query_graph(dtws_t h) {
+    if (h->qgraph_exec) cudaGraphExecDestroy(h->qgraph_exec);
+    h->qgraph_exec = nullptr;
+    h->qgraph_sig.clear();
+}
+
 void free_learn(LearnEntry &e) {
     for (void *p : {e.E, e.E2, e.Q, e.Q2, (void *)e.S, (void *)e.S2})
         if (p) cudaFree(p);
@@ -500,7 +507,8 @@ int learn_half(int m) {
     return enc_phase(m) > 0 ? (b + 3) / 4 : b / 2;
 }
 
-// Embeddings of the windows at offsets j*b for query length m (cached).
+// Embeddings of the windows at offsets j*b for query length m (cached).  The
+// kept query graph goes with an entry whose arrays are freed: it may read them.
 dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, LearnEntry **out, bool *computed) {
     *computed = false;
     for (auto &e : h->learn)
@@ -512,6 +520,7 @@ dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, Lea
     for (size_t i = 0; i < h->learn.size();)
         if (h->learn[i].version != h->enc_version) {
             CK(cudaDeviceSynchronize());
+            drop_query_graph(h);
             free_learn(h->learn[i]);
             h->learn.erase(h->learn.begin() + i);
         } else {
@@ -522,6 +531,7 @@ dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, Lea
         for (size_t i = 1; i < h->learn.size(); ++i)
             if (h->learn[i].used < h->learn[lru].used) lru = i;
         CK(cudaDeviceSynchronize());
+        drop_query_graph(h);
         free_learn(h->learn[lru]);
         h->learn.erase(h->learn.begin() + lru);
     }
@@ -886,8 +896,11 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
     const bool graph = h->opt.batch_graph && !h->opt.timing;
     std::vector<int64_t> sig;
     if (graph) {
-        sig = {(int64_t)(intptr_t)Qd, (int64_t)(intptr_t)idx_d, (int64_t)(intptr_t)dist_d,
-               (int64_t)(intptr_t)le, le ? le->version : 0};
+        sig = {(int64_t)(intptr_t)Qd, (int64_t)(intptr_t)idx_d, (int64_t)(intptr_t)dist_d, le ? le->version : 0};
+        // (the arrays, not the entry: its place in the cache says nothing about them)
+        for (const void *p : {le ? le->Q : nullptr, le ? (void *)le->S : nullptr, le ? le->Q2 : nullptr,
+                              le ? (void *)le->S2 : nullptr})
+            sig.push_back((int64_t)(intptr_t)p);
         sig_push(sig, h->opt);
         sig_push(sig, e.b);
         sig_push(sig, a);
@@ -925,9 +938,7 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
                 set_err("query graph capture: %s", cudaGetErrorString(ce));
                 return DTWS_ECUDA;
             }
-            if (h->qgraph_exec) cudaGraphExecDestroy(h->qgraph_exec);
-            h->qgraph_exec = nullptr;
-            h->qgraph_sig.clear();
+            drop_query_graph(h);
             cudaGraphExec_t ex = nullptr;
             const cudaError_t ie = cudaGraphInstantiate(&ex, g, 0);
             cudaGraphDestroy(g);
@@ -962,11 +973,8 @@ void drop_graph(dtws_t h) {
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
     h->graph_exec = nullptr;
     h->graph_sig.clear();
-    if (h->qgraph_exec) cudaGraphExecDestroy(h->qgraph_exec);
-    h->qgraph_exec = nullptr;
-    h->qgraph_sig.clear();
+    drop_query_graph(h);
 }
-
 
 // Lanes for `count` queries in flight.
 dtws_status ensure_lanes(dtws_t h, int count) {

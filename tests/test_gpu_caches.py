@@ -62,3 +62,25 @@ def test_query_seen_once_is_taken_under_capture():
         g.replay()
         torch.cuda.synchronize()
         assert (int(oi), float(od)) == want
+
+
+def test_a_kept_graph_does_not_outlive_its_embeddings():
+    """Learned ordering, two slots of embeddings: a query is captured, another
+    length takes its slot and a third one brings the first length back to the
+    same place of the cache, at other addresses.  The plain ordering's answers
+    every time."""
+    from oracle import encoder as enc
+    from paper_1812_10302_gb300 import dtws, synth
+
+    x = synth.walk_with_bursts(400_000, 61, 62, 63)
+    qs = {m: synth.noisy_copy(x, m, 64 + m, 65 + m, noise=0.2)[0] for m in (64, 128, 256)}
+    with dtws.Index(x) as ix:
+        want = {m: ix.query(q, m // 10) for m, q in qs.items()}
+    with dtws.Index(x) as ix:
+        ix.set_encoder(enc.init_params(3))
+        ix.set_options(ordering=dtws.DTWS_ORDER_LEARNED)
+        for m in (64, 128, 128, 256, 64, 128, 128, 128, 256, 256, 64, 128, 256):
+            i, d = ix.query(qs[m], m // 10)
+            assert ix.sync_status() == dtws.DTWS_OK
+            np.testing.assert_array_equal(i, want[m][0])
+            np.testing.assert_array_equal(d, want[m][1])
