@@ -60,9 +60,12 @@ struct Arena {
     }
 };
 
+// A cache entry of `kept` arrays belongs to a graph that the caller captured
+// (see get_stats): it is not reused for another length or band.
 struct StatsEntry {
     int m = 0;
     int64_t used = 0;
+    bool kept = false;
     char *block = nullptr;  // the allocation the arrays lie in
     float *mu_hi = nullptr, *mu_lo = nullptr, *inv_sigma = nullptr;
     float *smu_hi = nullptr, *sinv_sigma = nullptr;  // every kProxyStride-th window (proxy scan)
@@ -70,6 +73,7 @@ struct StatsEntry {
 struct EnvEntry {
     int r = 0;
     int64_t used = 0;
+    bool kept = false;
     char *block = nullptr;
     float *U = nullptr, *L = nullptr;
 };
@@ -82,6 +86,7 @@ struct TuneEntry {
 struct LearnEntry {
     int m = 0;
     int64_t used = 0, version = 0, rows = 0, rows2 = 0;
+    bool kept = false;
     void *E = nullptr;   // BF16 [rows][64]: windows at offsets j*b
     void *E2 = nullptr;  // BF16 [rows2][64]: windows at offsets j*b + b/2 (b >= 2)
     void *Q = nullptr, *Q2 = nullptr;    // their int8 copies for the scan
@@ -283,6 +288,15 @@ void free_env(EnvEntry &e) {
     e = EnvEntry();
 }
 
+bool stream_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
 // A stream is about to read or write the caches.
 void use_caches(dtws_t h, cudaStream_t s) {
     h->cache_mixed = h->cache_mixed || (h->cache_used && h->cache_stream != s);
@@ -332,6 +346,23 @@ cudaError_t clear_stats_tail(dtws_t h, const StatsEntry &e, cudaStream_t s) {
     return ce;
 }
 
+// The entry to reuse in a cache of `slots` entries that are not kept: the least
+// recently used one, or -1 while there are fewer.
+template <typename E>
+int reusable(const std::vector<E> &cache, int slots) {
+    int free_n = 0, lru = -1;
+    for (size_t i = 0; i < cache.size(); ++i) {
+        if (cache[i].kept) continue;
+        ++free_n;
+        if (lru < 0 || cache[i].used < cache[lru].used) lru = (int)i;
+    }
+    return free_n >= slots ? lru : -1;
+}
+
+// The window statistics of length m (cached).  What a stream under capture is
+// given is computed when the captured graph runs, not now: it goes to arrays of
+// its own (where the capture allows an allocation), under a length that no
+// other call asks for.
 dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *computed) {
     *computed = false;
     for (auto &e : h->stats)
@@ -342,10 +373,9 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
             return DTWS_OK;
         }
     StatsEntry e;
-    if ((int)h->stats.size() >= kCacheSlots) {  // the least recently used slot's arrays
-        size_t lru = 0;
-        for (size_t i = 1; i < h->stats.size(); ++i)
-            if (h->stats[i].used < h->stats[lru].used) lru = i;
+    const bool captured = stream_capturing(s);
+    const int lru = captured ? -1 : reusable(h->stats, kCacheSlots);
+    if (lru >= 0) {
         CK(settle_caches(h, s));
         e = h->stats[lru];
         h->stats.erase(h->stats.begin() + lru);
@@ -367,7 +397,8 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
             return DTWS_ECUDA;
         }
     }
-    e.m = m;
+    e.m = captured ? 0 : m;
+    e.kept = captured;
     const cudaError_t ce = launch_window_stats(h->x, h->n, m, h->pf, h->bf, h->pok, h->pscale, e.mu_hi, e.mu_lo,
                                                e.inv_sigma, e.smu_hi, e.sinv_sigma, s);
     if (ce != cudaSuccess) {  // nothing half-initialised stays in the cache
@@ -412,8 +443,14 @@ dtws_status get_ident(dtws_t h, cudaStream_t s, StatsEntry **out, bool *computed
             set_err("unnormalised statistics: %s", cudaGetErrorString(ce));
             return DTWS_ECUDA;
         }
-        h->ident = e;
         *computed = true;
+        if (stream_capturing(s)) {  // (as get_stats)
+            e.kept = true;
+            h->stats.push_back(e);
+            *out = &h->stats.back();
+            return DTWS_OK;
+        }
+        h->ident = e;
     }
     use_caches(h, s);
     *out = &h->ident;
@@ -426,6 +463,7 @@ dtws_status query_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool 
     return h->opt.unnormalised ? get_ident(h, s, out, computed) : get_stats(h, m, s, out, computed);
 }
 
+// The series' envelope for half-width r (cached; under capture as get_stats).
 dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *computed) {
     *computed = false;
     for (auto &e : h->env)
@@ -436,10 +474,9 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
             return DTWS_OK;
         }
     EnvEntry e;
-    if ((int)h->env.size() >= kCacheSlots) {  // the least recently used slot's arrays
-        size_t lru = 0;
-        for (size_t i = 1; i < h->env.size(); ++i)
-            if (h->env[i].used < h->env[lru].used) lru = i;
+    const bool captured = stream_capturing(s);
+    const int lru = captured ? -1 : reusable(h->env, kCacheSlots);
+    if (lru >= 0) {
         CK(settle_caches(h, s));
         e = h->env[lru];
         h->env.erase(h->env.begin() + lru);
@@ -463,7 +500,8 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
             return DTWS_ECUDA;
         }
     }
-    e.r = r;
+    e.r = captured ? -1 : r;
+    e.kept = captured;
     const cudaError_t ce = launch_envelope(h->x, h->n, r, e.U, e.L, s);
     if (ce != cudaSuccess) {
         free_env(e);
@@ -509,6 +547,7 @@ int learn_half(int m) {
 
 // Embeddings of the windows at offsets j*b for query length m (cached).  The
 // kept query graph goes with an entry whose arrays are freed: it may read them.
+// Under capture as get_stats.
 dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, LearnEntry **out, bool *computed) {
     *computed = false;
     for (auto &e : h->learn)
@@ -517,8 +556,9 @@ dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, Lea
             *out = &e;
             return DTWS_OK;
         }
-    for (size_t i = 0; i < h->learn.size();)
-        if (h->learn[i].version != h->enc_version) {
+    const bool captured = stream_capturing(s);
+    for (size_t i = 0; i < h->learn.size() && !captured;)
+        if (h->learn[i].version != h->enc_version && !h->learn[i].kept) {
             CK(cudaDeviceSynchronize());
             drop_query_graph(h);
             free_learn(h->learn[i]);
@@ -526,17 +566,16 @@ dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, Lea
         } else {
             ++i;
         }
-    if ((int)h->learn.size() >= kLearnSlots) {
-        size_t lru = 0;
-        for (size_t i = 1; i < h->learn.size(); ++i)
-            if (h->learn[i].used < h->learn[lru].used) lru = i;
+    const int lru = captured ? -1 : reusable(h->learn, kLearnSlots);
+    if (lru >= 0) {
         CK(cudaDeviceSynchronize());
         drop_query_graph(h);
         free_learn(h->learn[lru]);
         h->learn.erase(h->learn.begin() + lru);
     }
     LearnEntry e;
-    e.m = m;
+    e.m = captured ? 0 : m;
+    e.kept = captured;
     e.version = h->enc_version;
     e.rows = enc_rows(h, m);
     e.rows2 = enc_rows2(h, m);
@@ -847,15 +886,6 @@ dtws_status enqueue_search(dtws_t h, const Exec &e, const QueryArgs &a, const fl
     launches += 1 + 1 + 1 + 2 + 1 + nf;  // qprep, ED seeds, scan, order x2, DTW, final
     *launches_out = launches;
     return DTWS_OK;
-}
-
-bool stream_capturing(cudaStream_t s) {
-    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return c != cudaStreamCaptureStatusNone;
 }
 
 // One query on the handle's own buffers (dtws_query).
