@@ -214,7 +214,12 @@ dtws_status dtws_get_options(dtws_t h, dtws_options *opt);
  * samples apart (see dtws_options).  With options.batch_graph = 1 a call
  * whose arguments (pointers, m, r, k, options) repeat the previous one's
  * captures the search, and later ones replay it; the query values may differ.
- * (A stream under capture by the caller takes a search that has run once.)
+ * On a stream that the caller is capturing: device arrays only, and with
+ * options.batch_graph = 1 the search that ran last or the one whose graph is
+ * kept, any other is refused (DTWS_ECUDA).  The per-series data of m and r that
+ * the captured search reads then stay in the handle, beside the cached ones,
+ * until dtws_clear_cache or dtws_destroy; the captured graph must not run after
+ * either.
  * With options.unnormalised = 1 neither side is normalised (raw values).
  * Errors: DTWS_EINVAL synchronously (also unnormalised DTW with the learned
  * ordering or with a series beyond +-2^32); DTWS_ENONFINITE and

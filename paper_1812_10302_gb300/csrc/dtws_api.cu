@@ -60,8 +60,8 @@ struct Arena {
     }
 };
 
-// A cache entry of `kept` arrays belongs to a graph that the caller captured
-// (see get_stats): it is not reused for another length or band.
+// A cache entry of `kept` arrays is read by a graph that the caller captured: it
+// is not reused for another length or band while the handle and its caches last.
 struct StatsEntry {
     int m = 0;
     int64_t used = 0;
@@ -150,6 +150,8 @@ struct dtws_ctx {
     // staging of host arrays: device side, and pinned host memory for results
     void *stage = nullptr;
     size_t stage_cap = 0;
+    bool stage_kept = false;      // read by a graph that the caller captured: not freed when a larger one takes its place
+    std::vector<void *> stages;   // such ones
     void *hstage = nullptr;
     size_t hstage_cap = 0;
     int64_t reads = 0;  // results read back
@@ -225,9 +227,11 @@ bool is_device_ptr(const void *p) {
 
 dtws_status ensure_stage(dtws_t h, size_t bytes) {
     if (h->stage_cap >= bytes) return DTWS_OK;
-    if (h->stage) cudaFree(h->stage);
+    if (h->stage && h->stage_kept) h->stages.push_back(h->stage);
+    else if (h->stage) cudaFree(h->stage);
     h->stage = nullptr;
     h->stage_cap = 0;
+    h->stage_kept = false;
     size_t cap = bytes < 4096 ? 4096 : bytes;
     void *p = nullptr;
     if (g_fail_allocs > 0) {
@@ -359,21 +363,22 @@ int reusable(const std::vector<E> &cache, int slots) {
     return free_n >= slots ? lru : -1;
 }
 
-// The window statistics of length m (cached).  What a stream under capture is
-// given is computed when the captured graph runs, not now: it goes to arrays of
-// its own (where the capture allows an allocation), under a length that no
-// other call asks for.
+// The window statistics of length m (cached).  An entry that a stream under
+// capture is given is kept.  What such a stream would have to compute is computed
+// when the captured graph runs, not now: it goes to arrays of its own (where the
+// capture allows an allocation), under a length that no other call asks for.
 dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *computed) {
     *computed = false;
+    const bool captured = stream_capturing(s);
     for (auto &e : h->stats)
         if (e.m == m) {
             e.used = ++h->clock;
+            e.kept = e.kept || captured;
             use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
     StatsEntry e;
-    const bool captured = stream_capturing(s);
     const int lru = captured ? -1 : reusable(h->stats, kCacheSlots);
     if (lru >= 0) {
         CK(settle_caches(h, s));
@@ -466,15 +471,16 @@ dtws_status query_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool 
 // The series' envelope for half-width r (cached; under capture as get_stats).
 dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *computed) {
     *computed = false;
+    const bool captured = stream_capturing(s);
     for (auto &e : h->env)
         if (e.r == r) {
             e.used = ++h->clock;
+            e.kept = e.kept || captured;
             use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
     EnvEntry e;
-    const bool captured = stream_capturing(s);
     const int lru = captured ? -1 : reusable(h->env, kCacheSlots);
     if (lru >= 0) {
         CK(settle_caches(h, s));
@@ -550,13 +556,14 @@ int learn_half(int m) {
 // Under capture as get_stats.
 dtws_status get_learn(dtws_t h, int m, const StatsEntry *se, cudaStream_t s, LearnEntry **out, bool *computed) {
     *computed = false;
+    const bool captured = stream_capturing(s);
     for (auto &e : h->learn)
         if (e.m == m && e.version == h->enc_version) {
             e.used = ++h->clock;
+            e.kept = e.kept || captured;
             *out = &e;
             return DTWS_OK;
         }
-    const bool captured = stream_capturing(s);
     for (size_t i = 0; i < h->learn.size() && !captured;)
         if (h->learn[i].version != h->enc_version && !h->learn[i].kept) {
             CK(cudaDeviceSynchronize());
@@ -905,6 +912,7 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
     } else {  // an exact envelope already cached for this r is still used
         for (auto &en : h->env)
             if (en.r == rr) ee = &en;
+        if (ee && stream_capturing(s)) ee->kept = true;
     }
     record(h, 7, s);
     if ((st = ensure_workspace(h)) != DTWS_OK) return st;
@@ -934,18 +942,21 @@ dtws_status run_query(dtws_t h, const float *Qd, int m, int r, int k, int64_t *i
         sig_push(sig, h->opt);
         sig_push(sig, e.b);
         sig_push(sig, a);
-        if (h->qgraph_exec && sig == h->qgraph_sig) {
-            CK(cudaGraphLaunch(h->qgraph_exec, s));
-            launches = h->qgraph_launches;
-        } else if (sig != h->qseen_sig || stream_capturing(s)) {
-            // a query seen for the first time is launched as it is: capturing
-            // and instantiating a graph costs more than one replay saves (and
-            // a stream that is being captured by the caller cannot be forked
-            // into a capture of its own)
-            if (stream_capturing(s) && sig != h->qseen_sig) {
-                set_err("dtws_query: a stream under capture takes a query that has run once before");
+        const bool kept = h->qgraph_exec && sig == h->qgraph_sig;
+        if (stream_capturing(s)) {
+            // (the caller's capture takes neither a capture of our own nor the
+            // kept graph: the kernels themselves, of a search that has run)
+            if (!kept && sig != h->qseen_sig) {
+                set_err("dtws_query: a stream under capture takes the query that ran last, or the one whose graph is kept");
                 return DTWS_ECUDA;
             }
+            if ((st = enqueue_search(h, e, a, Qd, idx_d, dist_d, &launches)) != DTWS_OK) return st;
+        } else if (kept) {
+            CK(cudaGraphLaunch(h->qgraph_exec, s));
+            launches = h->qgraph_launches;
+        } else if (sig != h->qseen_sig) {
+            // a query seen for the first time is launched as it is: capturing
+            // and instantiating a graph costs more than one replay saves
             h->qseen_sig = sig;
             if ((st = enqueue_search(h, e, a, Qd, idx_d, dist_d, &launches)) != DTWS_OK) return st;
         } else {
@@ -1458,6 +1469,7 @@ dtws_status dtws_destroy(dtws_t h) {
                     h->bqf_block, h->pool_block};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    for (void *p : h->stages) cudaFree(p);
     if (h->hstage) cudaFreeHost(h->hstage);
     if (h->ev_ok)
         for (auto &e : h->ev) cudaEventDestroy(e);
@@ -1612,6 +1624,7 @@ dtws_status dtws_query(dtws_t h, const float *Q, int32_t m, int32_t r, int32_t k
         if ((st = run_query(h, Qd, m, r, k, idx_d, dist_d, s, z)) != DTWS_OK) return st;
     } else if (z > 0) {
         char *kp = sp + round_up(qb, 256) + round_up(ib, 256) + round_up(db, 256);
+        if (stream_capturing(s)) h->stage_kept = true;
         int64_t *kidx = (int64_t *)kp;
         float *kdist = (float *)(kp + round_up(kib, 256));
         if ((st = run_query(h, Qd, m, r, K, kidx, kdist, s)) != DTWS_OK) return st;
@@ -1720,6 +1733,9 @@ dtws_status dtws_clear_cache(dtws_t h) {
     h->stats.clear();
     h->env.clear();
     h->learn.clear();
+    for (void *p : h->stages) cudaFree(p);
+    h->stages.clear();
+    h->stage_kept = false;
     return DTWS_OK;
 }
 

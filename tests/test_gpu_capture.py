@@ -110,3 +110,96 @@ def test_a_length_first_met_under_capture(mode, options):
             assert new.take() == want
         cap.close()
         assert ix.sync_status() == dtws.DTWS_OK
+
+
+@pytest.mark.parametrize("before", [1, 2, 3])
+@pytest.mark.parametrize("options", [dict(), dict(batch_graph=0), dict(exclusion_zone=4)])
+def test_a_captured_search_outlives_the_caches_slots(before, options):
+    """A search that ran once, twice (captured by the handle) or three times
+    (replayed by it) is taken by the caller's capture; the captured graph gives
+    the same answer after more lengths, bands and larger arrays than the
+    handle's caches and its stage hold."""
+    from paper_1812_10302_gb300 import dtws
+
+    x = _series(40_000, 18)
+    s = torch.cuda.Stream()
+    one = _Call(x, 128, 3)
+    with dtws.Index(x, options=options) as ix:
+        for _ in range(before):
+            one(ix, s)
+        want = one.take()
+        cap = _Capture(s)
+        with cap:
+            one(ix, s)
+        cap.run()
+        assert one.take() == want
+        one(ix, s)
+        assert one.take() == want
+        for rep in range(2):
+            for m in (64, 96, 160, 192, 224, 256, 288, 320, 352, 384, 6000):
+                ix.query(x[100:100 + m], m // 7, stream=s)
+            cap.run()
+            assert one.take() == want
+        one(ix, s)
+        assert one.take() == want
+        cap.close()
+        assert ix.sync_status() == dtws.DTWS_OK
+
+
+def test_a_captured_learned_search_outlives_its_slots():
+    """The embeddings that a captured search reads stay too."""
+    from oracle import encoder as enc
+    from paper_1812_10302_gb300 import dtws, synth
+
+    x = synth.walk_with_bursts(300_000, 71, 72, 73)
+    s = torch.cuda.Stream()
+    one = _Call(x, 128, 4)
+    with dtws.Index(x) as ix:
+        ix.set_encoder(enc.init_params(3))
+        ix.set_options(ordering=dtws.DTWS_ORDER_LEARNED)
+        one(ix, s)
+        want = one.take()
+        cap = _Capture(s)
+        with cap:
+            one(ix, s)
+        for m in (64, 192, 256, 320, 64, 192):
+            ix.query(x[100:100 + m], m // 7, stream=s)
+        cap.run()
+        assert one.take() == want
+        ix.set_encoder(enc.init_params(4))
+        for m in (64, 192, 256, 320, 128):
+            ix.query(x[100:100 + m], m // 7, stream=s)
+        cap.run()
+        assert one.take() == want
+        cap.close()
+        assert ix.sync_status() == dtws.DTWS_OK
+
+
+def test_other_searches_are_refused_under_capture():
+    """Under capture a handle that keeps graphs takes no search but the last one
+    and the one whose graph it keeps, and is as it was afterwards."""
+    from paper_1812_10302_gb300 import dtws
+
+    x = _series(30_000, 28)
+    s = torch.cuda.Stream()
+    a, b, c = (_Call(x, m, m) for m in (100, 200, 300))
+    with dtws.Index(x) as ix:
+        want = {}
+        for call in (a, a, c, b):  # a's graph is kept, b ran last
+            call(ix, s)
+            want[call] = call.take()
+        for call, taken in ((a, True), (b, True), (c, False)):
+            cap = _Capture(s)
+            with cap:
+                if taken:
+                    call(ix, s)
+                else:
+                    with pytest.raises(dtws.DtwsError):
+                        call(ix, s)
+            if taken:
+                cap.run()
+                assert call.take() == want[call]
+            cap.close()
+        for call in (a, b, c, c, a):
+            call(ix, s)
+            assert call.take() == want[call]
