@@ -1324,9 +1324,13 @@ dtws_status run_batch(dtws_t h, const float *Qd, const int64_t *q_off, const int
             bool c3;
             StatsEntry *se;
             bool c1;
-            // the learned embeddings are scaled by 1/sigma from the handle's statistics of m
-            if ((st = get_stats(h, m, l.stream, &se, &c1)) != DTWS_OK) return fail(st);
-            if ((st = get_learn(h, m, se, l.stream, &le, &c3)) != DTWS_OK) return fail(st);
+            // The learned embeddings are scaled by 1/sigma from the handle's
+            // statistics of m.  Whichever query met m first, every lane takes them
+            // in the order of `root`, which computes them.
+            if ((st = get_stats(h, m, root, &se, &c1)) != DTWS_OK) return fail(st);
+            if ((st = get_learn(h, m, se, root, &le, &c3)) != DTWS_OK) return fail(st);
+            CKB(cudaEventRecord(h->batch_fork, root));
+            CKB(cudaStreamWaitEvent(l.stream, h->batch_fork, 0));
         }
         Exec e{qb[q], l.stream, l.side, l.ev_fork, l.ev_join, le, false, 1, deferq[q] ? &h->pool : nullptr};
         int64_t n_l = 0;

@@ -229,3 +229,22 @@ def test_seeding_by_proposal_count():
     for name in ("proxy", "trained", "untrained"):
         assert hits[(16, name)] >= 29
     assert hits[(16, "trained")] >= hits[(16, "untrained")]
+
+
+def test_batch_lanes_share_embeddings(params):
+    """Queries of few lengths over four lanes on a handle that has no embeddings
+    yet: most lanes take what another query's turn computed, three lengths
+    over two slots."""
+    x = synth.walk_with_bursts(1_500_000, 81, 82, 83)
+    for ms in ([128] * 8, [256, 64, 512, 256, 64, 512, 512, 64]):
+        qs = [synth.noisy_copy(x, m, 90 + i, 95 + i)[0] for i, m in enumerate(ms)]
+        rs = [m // 10 for m in ms]
+        with dtws.Index(x) as ix:
+            want = ix.query_batch(qs, rs, k=3)
+            ix.set_encoder(params)
+            ix.set_options(ordering=dtws.DTWS_ORDER_LEARNED)
+            for _ in range(3):
+                got = ix.query_batch(qs, rs, k=3)
+                assert ix.sync_status() == dtws.DTWS_OK
+                np.testing.assert_array_equal(got[0], want[0])
+                np.testing.assert_array_equal(got[1], want[1])
