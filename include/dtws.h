@@ -27,7 +27,10 @@
  * wait that ran out) are recorded in the handle and returned by
  * dtws_sync_status().
  *
- * Threading: a handle may be used from one host thread at a time.
+ * Threading: a handle may be used from one host thread at a time.  Its calls may
+ * come on different streams: the work of a call starts after the work of the
+ * handle's call before it.  (A graph that the caller captured from a call is the
+ * caller's to order against the handle's other calls.)
  */
 #ifndef DTWS_H
 #define DTWS_H

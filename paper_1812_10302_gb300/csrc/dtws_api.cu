@@ -134,10 +134,10 @@ struct dtws_ctx {
     StatsEntry ident;                    // unnormalised DTW: mean 0, 1/sigma 1 for every window
     std::vector<EnvEntry> env;
     int64_t clock = 0;
-    // the stream whose order every queued reader of the caches is in (several
-    // since the last device-wide wait: a slot that is reused waits for all)
-    cudaStream_t cache_stream = nullptr;
-    bool cache_used = false, cache_mixed = false;
+    // the end of the last call's work and the stream it is on (see InOrder)
+    cudaEvent_t turn = nullptr;
+    unsigned long long turn_stream = 0;
+    bool turn_taken = false;
     char *work_block = nullptr, *cand_block = nullptr;
     QueryState *st = nullptr;
     int *status = nullptr;
@@ -301,20 +301,30 @@ bool stream_capturing(cudaStream_t s) {
     return c != cudaStreamCaptureStatusNone;
 }
 
-// A stream is about to read or write the caches.
-void use_caches(dtws_t h, cudaStream_t s) {
-    h->cache_mixed = h->cache_mixed || (h->cache_used && h->cache_stream != s);
-    h->cache_used = true;
-    h->cache_stream = s;
-}
-// A cache slot's arrays are about to be rewritten in the order of `s`: no
-// kernel queued elsewhere may still read them.
-cudaError_t settle_caches(dtws_t h, cudaStream_t s) {
-    if (!h->cache_used || (!h->cache_mixed && h->cache_stream == s)) return cudaSuccess;
-    const cudaError_t e = cudaDeviceSynchronize();
-    h->cache_used = h->cache_mixed = false;
-    return e;
-}
+// Calls on one handle share its workspace and its caches: the work of a call
+// starts after the work of the call before it, whichever stream that was on.
+// (Two searches at once would read each other's lists, and the CTAs of one
+// cluster could then disagree on how many windows they have to walk.)  Streams
+// are told apart by their ids: a destroyed stream's handle can come back, and
+// the per-thread default streams share one.  A stream under capture is left
+// alone: what runs there later is for the caller to order.
+struct InOrder {
+    dtws_t h;
+    cudaStream_t s;
+    bool on = false;
+    cudaError_t begun = cudaSuccess;
+    InOrder(dtws_t h, cudaStream_t s) : h(h), s(s) {
+        if (!h || stream_capturing(s)) return;
+        unsigned long long id = 0;
+        begun = cudaStreamGetId(s, &id);
+        if (begun == cudaSuccess && h->turn_taken && id != h->turn_stream) begun = cudaStreamWaitEvent(s, h->turn, 0);
+        on = begun == cudaSuccess;
+        h->turn_stream = id;
+    }
+    ~InOrder() {
+        if (on) h->turn_taken = cudaEventRecord(h->turn, s) == cudaSuccess;
+    }
+};
 
 // Window statistics arrays that serve every m (room for the windows of m = 2):
 // a slot of another length is reused as it is.  Past the windows of the
@@ -374,14 +384,12 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
         if (e.m == m) {
             e.used = ++h->clock;
             e.kept = e.kept || captured;
-            use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
     StatsEntry e;
     const int lru = captured ? -1 : reusable(h->stats, kCacheSlots);
-    if (lru >= 0) {
-        CK(settle_caches(h, s));
+    if (lru >= 0) {  // (its readers come before in the order of s: see InOrder)
         e = h->stats[lru];
         h->stats.erase(h->stats.begin() + lru);
     } else {
@@ -413,7 +421,6 @@ dtws_status get_stats(dtws_t h, int m, cudaStream_t s, StatsEntry **out, bool *c
         return DTWS_ECUDA;
     }
     e.used = ++h->clock;
-    use_caches(h, s);
     h->stats.push_back(e);
     *out = &h->stats.back();
     *computed = true;
@@ -457,7 +464,6 @@ dtws_status get_ident(dtws_t h, cudaStream_t s, StatsEntry **out, bool *computed
         }
         h->ident = e;
     }
-    use_caches(h, s);
     *out = &h->ident;
     return DTWS_OK;
 }
@@ -476,14 +482,12 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
         if (e.r == r) {
             e.used = ++h->clock;
             e.kept = e.kept || captured;
-            use_caches(h, s);
             *out = &e;
             return DTWS_OK;
         }
     EnvEntry e;
     const int lru = captured ? -1 : reusable(h->env, kCacheSlots);
     if (lru >= 0) {
-        CK(settle_caches(h, s));
         e = h->env[lru];
         h->env.erase(h->env.begin() + lru);
     } else {
@@ -516,7 +520,6 @@ dtws_status get_env(dtws_t h, int r, cudaStream_t s, EnvEntry **out, bool *compu
         return DTWS_ECUDA;
     }
     e.used = ++h->clock;
-    use_caches(h, s);
     h->env.push_back(e);
     *out = &h->env.back();
     *computed = true;
@@ -1170,7 +1173,6 @@ dtws_status run_batch(dtws_t h, const float *Qd, const int64_t *q_off, const int
         sum_m += m_arr[q];
         sum_N += h->n - m_arr[q] + 1;
     }
-    use_caches(h, s);  // (the lanes fork from s and join into it)
     if ((st = ensure_lanes(h, nl)) != DTWS_OK) return st;
     long long pool_want = std::min<long long>(1ll << 27, std::max<long long>(1, sum_N));
     if (h->pool_limit >= 0) pool_want = h->pool_limit;
@@ -1477,6 +1479,7 @@ dtws_status dtws_destroy(dtws_t h) {
     if (h->hstage) cudaFreeHost(h->hstage);
     if (h->ev_ok)
         for (auto &e : h->ev) cudaEventDestroy(e);
+    if (h->turn) cudaEventDestroy(h->turn);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->side) cudaStreamDestroy(h->side);
@@ -1554,6 +1557,7 @@ dtws_status dtws_create(const float *series, int64_t n, void *stream, dtws_t *ou
         return fail(DTWS_ENONFINITE);
     }
     CKF(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
+    CKF(cudaEventCreateWithFlags(&h->turn, cudaEventDisableTiming));
     CKF(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     CKF(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
     for (auto &e : h->ev)
@@ -1610,6 +1614,8 @@ dtws_status dtws_query(dtws_t h, const float *Q, int32_t m, int32_t r, int32_t k
         else K = (int)(want < N ? want : N);
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     const bool qdev = is_device_ptr(Q), idev = is_device_ptr(out_idx), ddev = is_device_ptr(out_dist);
     const size_t qb = (size_t)m * 4, ib = (size_t)k * 8, db = (size_t)k * 4;
     const size_t kib = (size_t)K * 8, kdb = (size_t)K * 4;  // the K-list (exclusion zone only)
@@ -1655,6 +1661,8 @@ dtws_status dtws_query_batch(dtws_t h, const float *Q_cat, const int64_t *q_off,
         if (st != DTWS_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     const bool qdev = is_device_ptr(Q_cat), idev = is_device_ptr(out_idx), ddev = is_device_ptr(out_dist);
     const size_t qb = (size_t)q_off[nq] * 4, ib = (size_t)nq * k * 8, db = (size_t)nq * k * 4;
     dtws_status st = ensure_stage(h, 256 + round_up(qb, 256) + round_up(ib, 256) + round_up(db, 256));
@@ -1755,6 +1763,8 @@ dtws_status dtws_debug_lock_selftest(dtws_t h, int64_t wait_ns, void *stream) {
     b.wait_ns = wait_ns;
     QueryArgs a = make_args(h, 2, 0, 1);
     a.xz_z = 1;
+    const InOrder turn(h, (cudaStream_t)stream);
+    CK(turn.begun);
     CK(launch_lock_selftest(b, a, (cudaStream_t)stream));
     return DTWS_OK;
 }
@@ -1780,6 +1790,8 @@ dtws_status dtws_autotune(dtws_t h, const int32_t *m_arr, const int32_t *r_arr, 
             return DTWS_EINVAL;
         }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     dtws_status st;
     if ((st = ensure_workspace(h)) != DTWS_OK) return st;
     CK(cudaStreamSynchronize(s));
@@ -1889,6 +1901,8 @@ dtws_status dtws_set_encoder(dtws_t h, const float *params, int32_t count, void 
         return DTWS_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     if (!h->enc_blob) {
         uint8_t *blob = nullptr;
         if (dalloc(&blob, kEncBlobBytes) != cudaSuccess) {
@@ -1920,6 +1934,8 @@ dtws_status dtws_learned_embeddings(dtws_t h, int32_t m, float *out, int64_t row
         return DTWS_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     StatsEntry *se;
     LearnEntry *le;
     bool c1, c2;
@@ -1949,6 +1965,8 @@ dtws_status dtws_window_stats(dtws_t h, int32_t m, float *mu_hi, float *mu_lo, f
         return DTWS_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     StatsEntry *se;
     bool c;
     dtws_status st = get_stats(h, m, s, &se, &c);
@@ -1968,6 +1986,8 @@ dtws_status dtws_series_envelope(dtws_t h, int32_t r, float *U, float *L, void *
         return DTWS_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     EnvEntry *ee;
     bool c;
     dtws_status st = get_env(h, r, s, &ee, &c);
@@ -2023,6 +2043,8 @@ dtws_status dtws_dtw_at(dtws_t h, const float *Q, int32_t m, int32_t r, const in
                         int64_t count, float *out, void *stream) {
     if (!out) return DTWS_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     QueryBufs b;
     QueryArgs a;
     const int64_t *off_d;
@@ -2044,6 +2066,8 @@ dtws_status dtws_dtw_at_f64(dtws_t h, const float *Q, int32_t m, int32_t r, cons
                             int64_t count, double *out, void *stream) {
     if (!out) return DTWS_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     QueryBufs b;
     QueryArgs a;
     const int64_t *off_d;
@@ -2065,6 +2089,8 @@ dtws_status dtws_lower_bounds_at(dtws_t h, const float *Q, int32_t m, int32_t r,
                                  int64_t count, float *kim, float *keogh_q, float *keogh_s, void *stream) {
     if (!kim || !keogh_q || !keogh_s) return DTWS_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
+    const InOrder turn(h, s);
+    CK(turn.begun);
     QueryBufs b;
     QueryArgs a;
     const int64_t *off_d;
