@@ -21,7 +21,7 @@ namespace {
 //   * odd cell counts, whose lanes load their own register windows (dtw_diag),
 //     and a spare cell, so that the neighbour exchange may wrap;
 //   * window values come raw from L1 and are normalised by the lane that takes
-//     them, one per pair of steps (18 operations): staged copies of 8 bytes a
+//     them, one per pair of steps (19 operations): staged copies of 8 bytes a
 //     sample left 8 warps on an SM, which issued in 64 % of the cycles;
 //   * the register windows move by copies (2 K per pair of steps): rotated in
 //     place over K unrolled pairs, as dtw_diag's, the loop outgrew the
@@ -38,12 +38,29 @@ namespace {
 __host__ __device__ constexpr int r64_threads(int K) { return K <= 5 ? 512 : K <= 7 ? 384 : 256; }
 
 // A window's normalisation: its mean in three parts (it may be many sigma, and
-// its error is every value's), 1/sigma in two.
+// its error is every value's), 1/sigma in two.  Samples and mean are taken
+// times the power of two f that brings 1/sigma into [1, 2), whatever the
+// series' units: at sigma = 1e36 the low part of 1/sigma itself is subnormal
+// (2e-9 of it), and the difference of two samples of either sign overflows.
 struct R64Norm {
-    float m1, m2, m3, ih, il;
+    float f, m1, m2, m3, ih, il;
 };
+// (The exponents are added as integers: FP64 issues at 1/64 of FP32's rate here,
+// and ldexp and ilogb took 1 % of a walk.  A mean of FP32 samples is zero or a
+// normal FP64 value, and so is it times 2^-126 .. 2^40.)
+__device__ __forceinline__ double times_pow2(double v, int e) {
+    return v == 0.0 ? v : __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
+}
+__device__ __forceinline__ R64Norm r64_scaled(double mu, double inv) {
+    // inv's exponent; 0 for no sigma, where every value is 0 (2^-126 is the least
+    // that is normal in FP32: 1/sigma >= 2^-128 is then 2^-2 or more)
+    const int e = inv > 0.0 ? max((__double2hiint(inv) >> 20) - 1023, -126) : 0;
+    const double sm = times_pow2(mu, e);
+    const dfloat m = df_from(sm), v = df_from(times_pow2(inv, -e));
+    return R64Norm{__int_as_float((e + 127) << 23), m.hi, m.lo, (float)(sm - (double)m.hi - (double)m.lo), v.hi, v.lo};
+}
 __device__ __forceinline__ dfloat r64_norm(const R64Norm &n, float x) {
-    const dfloat s = df_two_sum(x, -n.m1), u = df_two_sum(s.hi, -n.m2);
+    const dfloat s = df_two_sum(__fmul_rn(x, n.f), -n.m1), u = df_two_sum(s.hi, -n.m2);
     const dfloat d = df_fast_two_sum(u.hi, __fadd_rn(s.lo, u.lo) - n.m3);
     const float p = __fmul_rn(d.hi, n.ih);
     return df_fast_two_sum(p, fmaf(d.hi, n.il, fmaf(d.lo, n.ih, fmaf(d.hi, n.ih, -p))));
@@ -174,9 +191,7 @@ k_dtw64_many(QueryBufs b, QueryArgs a, const int64_t *__restrict__ offsets, int6
         double mu, var;
         mean_and_variance(xw, m, lane, L, gsum, mu, var);
         const double inv = var <= 1e-24 * (mu * mu > 1.0 ? mu * mu : 1.0) ? 0.0 : 1.0 / sqrt(var);
-        const dfloat mf = df_from(mu), vf = df_from(inv);
-        const R64Norm norm{mf.hi, mf.lo, (float)(mu - (double)mf.hi - (double)mf.lo), vf.hi, vf.lo};
-        const double d = r64_walk<L, K>(qs, xw, m, r, norm, gmask, lane);
+        const double d = r64_walk<L, K>(qs, xw, m, r, r64_scaled(mu, inv), gmask, lane);
         if (lane == 0) out[c] = d;
     }
 }

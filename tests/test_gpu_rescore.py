@@ -131,3 +131,32 @@ def test_many_offsets(series, m, r):
     np.testing.assert_allclose(got[:24], want, rtol=1e-10, atol=1e-18 * m)
     np.testing.assert_array_equal(got, np.tile(got[:24], 14))
     np.testing.assert_allclose(few, want, rtol=1e-10, atol=1e-18 * m)
+
+
+@pytest.mark.parametrize("m,r", [(60, 23), (200, 78), (400, 222)])
+@pytest.mark.parametrize("power", [-60, -27, 100, 118, None])
+def test_many_offsets_in_any_units(series, m, r, power):
+    """The throughput shapes on a series times a power of two (None: the largest
+    that FP32 holds, both signs among the samples of a window): normalisation
+    takes the units off exactly, so the distances are those of the plain series,
+    as those of few offsets are.  (Below 2^-27 no window's variance may fall
+    under the zero-variance rule's 1e-24: constant windows are left out.)"""
+    x = (series - np.float32(7.25)).astype(np.float32)
+    x[::2] *= -1.0
+    s = 127 - int(np.floor(np.log2(np.abs(x).max()))) if power is None else power
+    q, o = synth.noisy_copy(x, m, m + r, m + 2 * r, noise=0.1)
+    some = np.random.default_rng(m + r).integers(4000, x.size - m + 1, 24)
+    some[:3] = [o, 0, x.size - m]
+    xs, qs = np.ldexp(x, s), np.ldexp(q, s)
+    assert np.isfinite(xs).all() and np.isfinite(qs).all()
+    with dtws.Index(xs) as ix:
+        many = ix.dtw_at_f64(qs, r, np.tile(some, 14))
+        few = ix.dtw_at_f64(qs, r, some)
+        assert ix.sync_status() == dtws.DTWS_OK
+    want = oracle.dtw_at(x, q, r, some)
+    if power == -60:  # sigma ~ 1e-17: every window counts as constant, the query too
+        np.testing.assert_array_equal(many, np.zeros(many.size))
+        np.testing.assert_array_equal(few, np.zeros(few.size))
+        return
+    np.testing.assert_allclose(few, want, rtol=1e-10)
+    np.testing.assert_allclose(many, np.tile(want, 14), rtol=1e-10)
