@@ -80,6 +80,12 @@ struct QueryBufs {
 // k-th entry, which changes by one 64-bit store, from one valid bound to a
 // smaller valid one.  With `append` the window also joins the candidate
 // buffer (DTWS_EOVERFLOW when full).
+// Bound by the lock: at a loose bound every group of the survivor pass has an
+// offer.  So an offer that changes nothing (most lie in a bucket that has a
+// better window) asks for no lock, who waits asks again at doubling intervals
+// -- ten thousand groups 64 ns apart kept the holder's own accesses waiting --
+// and the holder reads the list eight entries at a time.  1e6 windows of m =
+// 128, k = z = 64: 1934 -> 18.5 ms; 1e7 of m = 256, k = 40, z = 200: 279 -> 11.
 static __device__ __noinline__ void xz_offer(const QueryBufs &b, const QueryArgs &a, unsigned long long key, bool append) {
     QueryState *st = b.st;
     if (append) {
@@ -87,50 +93,57 @@ static __device__ __noinline__ void xz_offer(const QueryBufs &b, const QueryArgs
         if (i < b.xz_cap) b.xz_buf[i] = key;
         else atomicOr(b.status, kStOverflow);
     }
+    constexpr int kB = 8;  // entries read at a time
+    static_assert(kKMax % kB == 0, "whole steps");
     const int k = a.k;
-    const unsigned W = (unsigned)(2 * a.xz_z + 1);
-    const unsigned bk = key_idx(key) / W;
-    unsigned long long *Lp = st->xz_keys[bk & 1u];
-    if (key >= *((volatile unsigned long long *)&Lp[k - 1])) return;  // changes nothing
+    const unsigned W = (unsigned)(2 * a.xz_z + 1), bk = key_idx(key) / W, lo = bk * W;  // the bucket: [lo, lo + W)
+    volatile unsigned long long *Lp = st->xz_keys[bk & 1u];
+    // k better keys, or a better one of the same bucket: an entry gives way only
+    // to better ones, so one that is seen in passing, while the list is
+    // rewritten, settles it as well
+    auto changes_nothing = [&]() {
+        if (key >= Lp[k - 1]) return true;
+        bool better = false;
+        for (int j0 = 0; j0 < k; j0 += kB) {
+            unsigned long long t[kB];
+#pragma unroll
+            for (int u = 0; u < kB; ++u) t[u] = Lp[j0 + u];
+#pragma unroll
+            for (int u = 0; u < kB; ++u) better |= t[u] <= key && key_idx(t[u]) - lo < W;
+        }
+        return better;
+    };
+    if (changes_nothing()) return;
     int *lock = &st->xz_lock[bk & 1u];
     const long long t0 = global_ns();
-    while (atomicCAS(lock, 0, 1) != 0) {
+    for (unsigned ns = 64; atomicCAS(lock, 0, 1) != 0; ns = ns < 16384 ? 2 * ns : ns) {
         if (global_ns() - t0 > b.wait_ns) {
             atomicOr(b.status, kStTimeout);
             return;
         }
-        __nanosleep(64);
+        __nanosleep(ns);
+        if (changes_nothing()) return;
     }
     __threadfence();
     unsigned long long v[kKMax];
-    int n = 0, same = -1;
-    for (int j = 0; j < k; ++j) {
-        v[j] = *((volatile unsigned long long *)&Lp[j]);
-        if (v[j] != kEmptyKey) {
-            ++n;
-            if (key_idx(v[j]) / W == bk) same = j;
+    int pos = 0, out = k - 1;  // the entry that the key comes before, the one that leaves: its bucket's, else the last
+    for (int j0 = 0; j0 < k; j0 += kB) {
+        unsigned long long t[kB];
+#pragma unroll
+        for (int u = 0; u < kB; ++u) t[u] = Lp[j0 + u];
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+            v[j0 + u] = t[u];
+            pos += t[u] < key;
+            if (j0 + u < k && t[u] != kEmptyKey && key_idx(t[u]) - lo < W) out = j0 + u;
         }
     }
-    bool changed = false;
-    if (same >= 0) {
-        if (key < v[same]) {  // the bucket's entry improves: drop it, insert below
-            for (int j = same; j + 1 < k; ++j) v[j] = v[j + 1];
-            v[k - 1] = kEmptyKey;
-            changed = true;
+    if (key < v[out]) {  // (so pos <= out)
+        for (int j = pos; j <= out && j < k - 1; ++j) Lp[j] = j == pos ? key : v[j - 1];
+        if (out == k - 1) {
+            __threadfence();
+            Lp[k - 1] = pos == k - 1 ? key : v[k - 2];
         }
-    } else {
-        changed = key < v[k - 1];
-    }
-    if (changed) {
-        int pos = k - 1;
-        while (pos > 0 && v[pos - 1] > key) {
-            v[pos] = v[pos - 1];
-            --pos;
-        }
-        v[pos] = key;
-        for (int j = 0; j < k - 1; ++j) Lp[j] = v[j];
-        __threadfence();
-        *((volatile unsigned long long *)&Lp[k - 1]) = v[k - 1];
     }
     __threadfence();
     atomicExch(lock, 0);
