@@ -929,13 +929,19 @@ __global__ void __launch_bounds__(kEdWarps * 32) k_seed_ed(QueryBufs b, QueryArg
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, key, o);
         key = v < key ? v : key;
     }
+    // With an exclusion zone the first threshold needs k windows of each parity
+    // of its buckets: where the blocks are few (a short series) every warp's
+    // best is offered.  (2e5 windows, k = 20: 25 blocks fill neither parity's
+    // list, and all the windows then survive the scan.)
+    const bool by_warp = a.xz_z > 0 && gridDim.x < 4u * (unsigned)a.k;
+    if (by_warp && lane == 0 && key != kEmptyKey) xz_offer(b, a, key, false);
     if (lane == 0) wkey[warp] = key;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int u = 1; u < kEdWarps; ++u) key = wkey[u] < key ? wkey[u] : key;
         if (key != kEmptyKey) {
             list_insert(st->ed_keys, exact_seeds(a) ? 2 : a.k, key);
-            if (a.xz_z > 0) xz_offer(b, a, key, false);
+            if (a.xz_z > 0 && !by_warp) xz_offer(b, a, key, false);
         }
     }
 }

@@ -44,3 +44,17 @@ def test_lists_of_every_length(k, z, kind):
             assert ix.sync_status() == dtws.DTWS_OK
             np.testing.assert_array_equal(idx, oi)
             np.testing.assert_allclose(dist, od, rtol=1e-4, atol=1e-6 * m)
+
+
+@pytest.mark.parametrize("n,m,k,z", [(200_000, 128, 20, 200), (30_000, 64, 6, 100)])
+def test_a_short_series_has_a_first_bound(n, m, k, z):
+    """The seeds of a short series hold k windows far enough apart, so that the
+    scan has a bound: without one every window passes it."""
+    x = synth.random_walk(n, n + m)
+    q, _ = synth.noisy_copy(x, m, m, k, noise=0.2)
+    with dtws.Index(x, options=dict(exclusion_zone=z)) as ix:
+        idx, dist = ix.query(q, m // 10, k)
+        assert ix.sync_status() == dtws.DTWS_OK
+        assert ix.last_stats()["pass_keogh_q"] < 0.9 * (n - m + 1)
+    assert np.all(np.diff(np.sort(idx)) > z)
+    np.testing.assert_allclose(dist, oracle.dtw_at(x, q, m // 10, idx), rtol=1e-4, atol=1e-6 * m)
