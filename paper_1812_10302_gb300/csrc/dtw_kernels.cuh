@@ -95,6 +95,30 @@ __host__ __device__ constexpr int dtw_min_blocks(int K) {
     return (K >= 1 && K <= 2) ? 4 : (K >= 1 && K <= 4) ? 3 : (K >= 16) ? 1 : 2;
 }
 
+// The query's ordered terms as the survivors' pre-check takes them: Eq. 10 over
+// all of them, the largest |q_hat| first (rank_terms), Eq. 8 over the ones past
+// the scan's kScanTerms.  What a term of Eq. 10 adds grows with |q_hat|, and
+// neighbouring positions one after another read the same sectors of the
+// series' envelope: 2e7 windows that a loose query of m = 128, r = 6 leaves
+// took 25.8 ms in the scan's order (spread over the query), 14.6 in this one;
+// of m = 256, r = 25 46.4 and 43.1.
+struct PreTerms {
+    int pos[kTerms], pos8[kTerms - kScanTerms];
+    float q[kTerms], u8[kTerms - kScanTerms], l8[kTerms - kScanTerms];
+};
+// By all the block's threads, which meet afterwards.
+__device__ __forceinline__ void load_terms(const QueryBufs &b, int m, PreTerms &s) {
+    for (int t = threadIdx.x; t < terms_of(m); t += blockDim.x) {
+        s.pos[t] = (int)b.st->e10_pos[t];
+        s.q[t] = b.st->e10_q[t];
+        if (t >= kScanTerms) {
+            s.pos8[t - kScanTerms] = (int)b.ord[t];
+            s.u8[t - kScanTerms] = b.sU[t];
+            s.l8[t - kScanTerms] = b.sL[t];
+        }
+    }
+}
+
 // Shapes whose seeds walk from both ends (dtw_ends): one warp per window, up
 // to 16 cells per lane.  A top-k search waits for its seeds one walk long
 // (m = 999, r = 99: the seeds' phase takes 146 us, 186 from one end; on four
@@ -138,22 +162,14 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                                        (lay.tail ? lay.tail_bytes() : 0))
                            : nullptr;
     // survivor pass: the seeds' offsets (already evaluated by the seed pass)
-    // and the query's ordered terms (positions) with q_hat and the
-    // query envelope there (the pre-check reads them for every candidate)
+    // and the query's ordered terms (the pre-check reads them for every candidate)
     __shared__ unsigned seeds_s[kSeedMax];
     __shared__ int n_seeds_s;
-    __shared__ int ord_s[128];
-    __shared__ float sq_s[128], su_s[128], sl_s[128];
+    __shared__ PreTerms terms;
     if (MODE == kModeSurv) {
         if (threadIdx.x == 0) n_seeds_s = st->n_seeds;
         for (int t = threadIdx.x; t < st->n_seeds; t += blockDim.x) seeds_s[t] = st->seed_off[t];
-        for (int t = threadIdx.x; t < 128; t += blockDim.x) {
-            const bool in = t < terms_of(m);
-            ord_s[t] = in ? (int)b.ord[t] : 0;
-            sq_s[t] = in ? b.sq[t] : 0.0f;
-            su_s[t] = in ? b.sU[t] : 0.0f;
-            sl_s[t] = in ? b.sL[t] : 0.0f;
-        }
+        load_terms(b, m, terms);
     }
     __syncthreads();
     int *cursor = MODE == kModeSurv ? &st->work2 : &st->work;
@@ -239,39 +255,37 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
                     pc.t0 = id;
                     pc.r = r;
                     const float *xp = b.x + id;
-                    const int budget = terms_of(m);
+                    const int T = terms_of(m);
                     float acc = 0.0f, acc8 = lbv;
                     // 8 terms per step: their loads are issued together, the
                     // abandon test runs once per step
                     constexpr int kB = 8;
-                    for (int j0 = 0; j0 < budget; j0 += kB) {
-                        float xv[kB], uv[kB], lv[kB];
-                        const bool eq8 = j0 >= kScanTerms;
+                    for (int j0 = 0; j0 < T && pass; j0 += kB) {
+                        float uv[kB], lv[kB];
+#pragma unroll
+                        for (int t = 0; t < kB; ++t) env_at(pc, terms.pos[min(j0 + t, T - 1)], uv[t], lv[t]);
 #pragma unroll
                         for (int t = 0; t < kB; ++t) {
-                            const int j = j0 + t < budget ? j0 + t : budget - 1;
-                            const int pos = ord_s[j];
-                            if (eq8) xv[t] = xp[pos];
-                            env_at(pc, pos, uv[t], lv[t]);
-                        }
-#pragma unroll
-                        for (int t = 0; t < kB; ++t) {
-                            if (j0 + t >= budget) break;
-                            const int j = j0 + t;
+                            if (j0 + t >= T) break;
                             const float u = fmaf(uv[t] - pmh, pis, -pls), l = fmaf(lv[t] - pmh, pis, -pls);
-                            const float q = sq_s[j];
+                            const float q = terms.q[j0 + t];
                             const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
                             acc = fmaf(dq, dq, acc);
-                            if (eq8) {
-                                const float cv = fmaf(xv[t] - pmh, pis, -pls);
-                                const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                                acc8 = fmaf(e, e, acc8);
-                            }
                         }
-                        if (acc > th || acc8 > th) {
-                            pass = false;
-                            break;
+                        pass = !(acc > th);
+                    }
+                    for (int j0 = 0; j0 < T - kScanTerms && pass; j0 += kB) {
+                        float xv[kB];
+#pragma unroll
+                        for (int t = 0; t < kB; ++t) xv[t] = xp[terms.pos8[min(j0 + t, T - kScanTerms - 1)]];
+#pragma unroll
+                        for (int t = 0; t < kB; ++t) {
+                            if (j0 + t >= T - kScanTerms) break;
+                            const float cv = fmaf(xv[t] - pmh, pis, -pls);
+                            const float e = fmaxf(cv - terms.u8[j0 + t], 0.0f) + fmaxf(terms.l8[j0 + t] - cv, 0.0f);
+                            acc8 = fmaf(e, e, acc8);
                         }
+                        pass = !(acc8 > th);
                     }
                 }
                 my_idx = id;
@@ -360,24 +374,22 @@ __device__ __forceinline__ void dtw_body(const QueryBufs &b, const QueryArgs &a,
             // same exit)
             float acc = 0.0f, acc8 = lb;
             bool pruned = false;
-            const int budget = terms_of(m);
-            for (int c0 = 0; c0 < budget; c0 += L) {
+            const int T = terms_of(m);
+            for (int c0 = 0; c0 < T; c0 += L) {
                 const int j = c0 + lane;
-                const bool eq8 = c0 >= kScanTerms;
+                const bool eq8 = c0 < T - kScanTerms;
                 float v = 0.0f, v8 = 0.0f;
-                if (j < budget) {
-                    const int pos = ord_s[j];
-                    const float x = eq8 ? xw[pos] : 0.0f;
+                if (eq8 && j < T - kScanTerms) {
+                    const float cv = fmaf(xw[terms.pos8[j]] - mh, is, -ls);
+                    const float e = fmaxf(cv - terms.u8[j], 0.0f) + fmaxf(terms.l8[j] - cv, 0.0f);
+                    v8 = e * e;
+                }
+                if (j < T) {
                     float U, Lo;
-                    env_at(tc, pos, U, Lo);
-                    const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
+                    env_at(tc, terms.pos[j], U, Lo);
+                    const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = terms.q[j];
                     const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
                     v = dq * dq;
-                    if (eq8) {
-                        const float cv = fmaf(x - mh, is, -ls);
-                        const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                        v8 = e * e;
-                    }
                 }
 #pragma unroll
                 for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask, v, o, L);
@@ -668,8 +680,7 @@ __host__ __device__ inline size_t wide_tail(int m) { return (size_t)((tail_entri
 // which are in lb), then the corners.  True: the window is out.
 constexpr int kWideTries = 8;  // candidates a warp looks at before the group meets
 __device__ __forceinline__ bool wide_prune(const QueryBufs &b, const float *qs, unsigned idx, float lb, float thr, int m,
-                                           int r, int lane, const int *ord_s, const float *sq_s, const float *su_s,
-                                           const float *sl_s, bool has_env, float *back) {
+                                           int r, int lane, const PreTerms &terms, bool has_env, float *back) {
     const float mh = b.mu_hi[idx], is = b.inv_sigma[idx], ls = b.mu_lo[idx] * is;
     const float *xw = b.x + idx;
     if (corner_applies(m) && corner_bound(qs, xw, mh, is, ls, m, r, lane, back) > thr) return true;
@@ -683,23 +694,23 @@ __device__ __forceinline__ bool wide_prune(const QueryBufs &b, const float *qs, 
     tc.n = b.n;
     tc.t0 = idx;
     tc.r = r;
+    const int T = terms_of(m);
     float acc = 0.0f, acc8 = lb;
-    for (int c0 = 0; c0 < terms_of(m); c0 += 32) {
+    for (int c0 = 0; c0 < T; c0 += 32) {
         const int j = c0 + lane;
-        const bool eq8 = c0 >= kScanTerms;
+        const bool eq8 = c0 < T - kScanTerms;
         float v = 0.0f, v8 = 0.0f;
-        if (j < terms_of(m)) {
-            const int pos = ord_s[j];
+        if (eq8 && j < T - kScanTerms) {
+            const float cv = fmaf(xw[terms.pos8[j]] - mh, is, -ls);
+            const float e = fmaxf(cv - terms.u8[j], 0.0f) + fmaxf(terms.l8[j] - cv, 0.0f);
+            v8 = e * e;
+        }
+        if (j < T) {
             float U, Lo;
-            env_at(tc, pos, U, Lo);
-            const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = sq_s[j];
+            env_at(tc, terms.pos[j], U, Lo);
+            const float u = fmaf(U - mh, is, -ls), l = fmaf(Lo - mh, is, -ls), q = terms.q[j];
             const float dq = fmaxf(q - u, 0.0f) + fmaxf(l - q, 0.0f);
             v = dq * dq;
-            if (eq8) {
-                const float cv = fmaf(xw[pos] - mh, is, -ls);
-                const float e = fmaxf(cv - su_s[j], 0.0f) + fmaxf(sl_s[j] - cv, 0.0f);
-                v8 = e * e;
-            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -726,8 +737,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
     __shared__ bool dry_s[GMAX][W];
     __shared__ unsigned seeds_s[kSeedMax];
     __shared__ int n_seeds_s;
-    __shared__ int ord_s[128];
-    __shared__ float sq_s[128], su_s[128], sl_s[128];
+    __shared__ PreTerms terms;
     QueryState *st = b.st;
     if (!st->valid) return;
     const int m = a.m, r = a.r;
@@ -748,13 +758,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
     if (MODE == kModeSurv) {
         if (threadIdx.x == 0) n_seeds_s = st->n_seeds;
         for (int i = threadIdx.x; i < st->n_seeds; i += blockDim.x) seeds_s[i] = st->seed_off[i];
-        for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-            const bool in = i < terms_of(m);
-            ord_s[i] = in ? (int)b.ord[i] : 0;
-            sq_s[i] = in ? b.sq[i] : 0.0f;
-            su_s[i] = in ? b.sU[i] : 0.0f;
-            sl_s[i] = in ? b.sL[i] : 0.0f;
-        }
+        load_terms(b, m, terms);
     }
     __syncthreads();
     if (g >= G) return;
@@ -802,7 +806,7 @@ __global__ void __launch_bounds__(256, 2) k_dtw_mw(QueryBufs b, QueryArgs a, con
                     bool seen = id == pre;  // scored already: by the seed pass or on the side stream
                     for (int i = lane; i < n_seeds_s; i += 32) seen |= seeds_s[i] == id;
                     if (__any_sync(0xffffffffu, seen)) continue;
-                    if (wide_prune(b, qs, id, lb, th, m, r, lane, ord_s, sq_s, su_s, sl_s, has_env, &fback)) continue;
+                    if (wide_prune(b, qs, id, lb, th, m, r, lane, terms, has_env, &fback)) continue;
                     found = id;
                     break;
                 }

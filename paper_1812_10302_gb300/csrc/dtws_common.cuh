@@ -127,6 +127,10 @@ struct QueryState {
     // CTAs of the proxy scan and of the survivor histogram that have
     // finished: the last one of each takes the step that needs all of them
     unsigned int prop_done, bin_done, final_done;
+    // the query's ordered terms, the largest |q_hat| first (Eq. 10 of the
+    // survivors' pre-check)
+    float e10_q[kTerms];
+    unsigned short e10_pos[kTerms];
     // (last: the words above that the scans' atomics meet on stay where they were)
     unsigned long long warp_best[kCtaSlots * kScanConsumers];  // each proxy-scan warp's best window
 };

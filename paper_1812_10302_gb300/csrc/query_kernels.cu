@@ -846,11 +846,41 @@ __global__ void __launch_bounds__(1024) k_seed_gather(QueryBufs b, QueryArgs a, 
 // occupies one slot.
 __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z);
 constexpr int kEdWarps = 16;  // warps of a block
+
+// The ordered terms by |q_hat|, largest first (ties in the scan's order), into
+// the query's state: four lanes count each term's betters.  One block of
+// k_seed_ed, whose others take longer, so that nothing waits for it (at the
+// start of every survivor CTA it took 2.5 us of a search of 66).
+__device__ __forceinline__ void rank_terms(const QueryBufs &b, int m) {
+    static_assert(4 * kTerms == kEdWarps * 32 && kTerms % 16 == 0, "four threads a term");
+    __shared__ float mag[kTerms];
+    const int T = terms_of(m), t = threadIdx.x >> 2, part = threadIdx.x & 3;
+    if (threadIdx.x < kTerms) mag[threadIdx.x] = threadIdx.x < T ? fabsf(b.sq[threadIdx.x]) : -1.0f;
+    __syncthreads();
+    const float v = mag[t];
+    int rank = 0;
+#pragma unroll 8
+    for (int i = 0; i < kTerms / 4; ++i) {
+        const int j = 4 * i + part;
+        rank += mag[j] > v || (mag[j] == v && j < t);
+    }
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if (part == 0 && t < T) {
+        b.st->e10_q[rank] = b.sq[t];
+        b.st->e10_pos[rank] = b.ord[t];
+    }
+}
+
 __global__ void __launch_bounds__(kEdWarps * 32) k_seed_ed(QueryBufs b, QueryArgs a, int slots, int n_random,
                                                            unsigned long long rng) {
     __shared__ unsigned long long wkey[kEdWarps];
     QueryState *st = b.st;
     if (!st->valid) return;
+    if (blockIdx.x == gridDim.x - 1) {
+        rank_terms(b, a.m);
+        return;
+    }
     constexpr int kW = 2 * kProxyHalf + 1;
     const int lane = lane_id(), warp = threadIdx.x >> 5, w = blockIdx.x * kEdWarps + warp;
     long long first = -1;  // the warp's windows: first .. first + nw - 1
@@ -933,7 +963,7 @@ __global__ void __launch_bounds__(kEdWarps * 32) k_seed_ed(QueryBufs b, QueryArg
     // of its buckets: where the blocks are few (a short series) every warp's
     // best is offered.  (2e5 windows, k = 20: 25 blocks fill neither parity's
     // list, and all the windows then survive the scan.)
-    const bool by_warp = a.xz_z > 0 && gridDim.x < 4u * (unsigned)a.k;
+    const bool by_warp = a.xz_z > 0 && gridDim.x - 1 < 4u * (unsigned)a.k;
     if (by_warp && lane == 0 && key != kEmptyKey) xz_offer(b, a, key, false);
     if (lane == 0) wkey[warp] = key;
     __syncthreads();
@@ -991,7 +1021,7 @@ cudaError_t launch_seed_ed(const QueryBufs &b, const QueryArgs &a, int ctas, int
     int warps = slots > 0 ? slots + n_random : max_seeds;
     if (warps < 1) warps = 1;
     if (slots <= 0 && warps > kEdMax) warps = kEdMax;
-    k_seed_ed<<<(warps + kEdWarps - 1) / kEdWarps, kEdWarps * 32, 0, s>>>(b, a, slots, n_random, rng);
+    k_seed_ed<<<(warps + kEdWarps - 1) / kEdWarps + 1, kEdWarps * 32, 0, s>>>(b, a, slots, n_random, rng);
     return cudaGetLastError();
 }
 
