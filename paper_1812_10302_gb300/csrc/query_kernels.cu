@@ -1478,7 +1478,7 @@ cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int6
 // normalised with the window's statistics: looser than the window-clipped
 // envelope, still admissible), is evaluated for each survivor by the DTW
 // kernel, whose tail bound consists of exactly its per-row terms.
-static_assert(kScanTerms == 64 && kScanTerms <= kTerms, "two of the scan's terms per lane in registers");
+static_assert(kScanTerms == 64 && kScanTerms <= kTerms, "two of the scan's terms per lane");
 constexpr int kLaneRow = 4;     // passers in a row of 32 from which each lane first takes kLaneFirst terms
 constexpr int kLaneFirst = 8;
 constexpr int kLaneEqMin = 16;  // windows left after them from which the lanes go on
@@ -1506,15 +1506,17 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// The ordered query terms the scan takes: in shared memory for the lane-wise
-// form, and each lane's own first two (terms lane and 32 + lane) in registers
-// for the warp-wise one.  nt of them; past nt an envelope that every value
-// lies in.
+// The ordered query terms the scan takes, in shared memory: nt of them; past
+// nt an envelope that every value lies in.  (A lane's own two terms of the
+// warp-wise form stay there too until a row needs them: held in registers across
+// the tile loop, with every row's LB_KimFL and two counters, they made the scan
+// spill at its 40 registers: 32 bytes out and 40 in per thread.  1e8 windows,
+// whole search, a query with a close match: m = 512 392 -> 333 us, m = 128 381 ->
+// 335, m = 1024 588 -> 517.)
 struct EqTerms {
-    const int *o;
-    const float *u, *l;
-    int nt, o0, o1;
-    float u0, l0, u1, l1;
+    int o[kScanTerms];
+    float u[kScanTerms], l[kScanTerms];
+    int nt;
 };
 
 // Each warp scans 32 windows at a time with LB_KimFL (one window per lane);
@@ -1523,9 +1525,8 @@ struct EqTerms {
 // envelope (Eq. 8) at the first kScanTerms ordered positions.  The sum is
 // a lower bound: LB_KimFL is the cost of the path's first and last cells, in
 // columns 0 and m-1, the terms bound the cells of other columns.  Survivors
-// are appended as (bound, offset) by one warp-aggregated atomic; their number
-// is returned.  A row with several passers first gives each lane kLaneFirst
-// terms of its own window; what is left is taken one window at a time, 32
+// are appended as (bound, offset) by one warp-aggregated atomic.  A row with
+// several passers first gives each lane kLaneFirst terms of its own window; what is left is taken one window at a time, 32
 // terms per step, where a single term above what is left of thr already
 // prunes (a vote), or lane by lane to the end where most of the row is left
 // (a loose bound).  No thread waits on another warp's survivors.
@@ -1536,18 +1537,21 @@ struct EqTerms {
 // the scan more than it saved: the random loads of the series envelope stall
 // the warps that feed the ring.  128 terms instead of 64: scan +90 us,
 // survivor pass -37 us.)
-__device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, QueryState *st, const EqTerms &e,
-                                            float thr, unsigned bal, int wrow, int lane, float kim, int64_t i0) {
-    const int w = wrow + lane;
+// sa, xa: shared-memory addresses of the lane's window's mean (1/sigma TW floats
+// on) and first sample; first: the row's first window.
+template <int TW>
+__device__ __forceinline__ void lb_row_keogh(float *cand_lb, unsigned *cand_idx, int *n_cand, const EqTerms &e, float thr,
+                                             unsigned bal, unsigned sa, unsigned xa, float kim, unsigned first) {
+    const int lane = lane_id();
     unsigned keep = 0;  // windows of this row that survive Eq. 8
     float my_lb = kim;  // the lane's window: its bound so far
     if (__popc(bal) >= kLaneRow) {
-        const float mh = t.mh[w], is = t.is[w], sd = shift_bound(mh, is);
+        const float mh = lds_at<0>(sa), is = lds_at<TW * 4>(sa), sd = shift_bound(mh, is);
         bool alive = (bal >> lane) & 1u;
         float s2 = kim;
 #pragma unroll
         for (int j = 0; j < kLaneFirst; ++j)
-            s2 += keogh_term((t.xs[w + e.o[j]] - mh) * is, e.u[j] + sd, e.l[j] - sd);
+            s2 += keogh_term((lds_at<0>(xa + 4u * (unsigned)e.o[j]) - mh) * is, e.u[j] + sd, e.l[j] - sd);
         alive = alive && !(s2 > thr);
         bal = __ballot_sync(0xffffffffu, alive);
         if (__popc(bal) >= kLaneEqMin) {
@@ -1556,7 +1560,7 @@ __device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, Q
                 if (alive) {
 #pragma unroll
                     for (int v = 0; v < kLaneFirst; ++v)
-                        s2 += keogh_term((t.xs[w + e.o[j0 + v]] - mh) * is, e.u[j0 + v] + sd, e.l[j0 + v] - sd);
+                        s2 += keogh_term((lds_at<0>(xa + 4u * (unsigned)e.o[j0 + v]) - mh) * is, e.u[j0 + v] + sd, e.l[j0 + v] - sd);
                     alive = !(s2 > thr);
                 }
             }
@@ -1565,19 +1569,20 @@ __device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, Q
             bal = 0;
         }
     }
+    const int o0 = e.o[lane], o1 = e.o[32 + lane];
+    const float u0 = e.u[lane], l0 = e.l[lane], u1 = e.u[32 + lane], l1 = e.l[32 + lane];
     while (bal) {
         const int src = __ffs(bal) - 1;
         bal &= bal - 1;
-        const int ws = wrow + src;
-        const float smh = t.mh[ws], sis = t.is[ws], ssd = shift_bound(smh, sis);
+        const unsigned off = 4u * (unsigned)(src - lane);  // (modulo 2^32)
+        const float smh = lds_at<0>(sa + off), sis = lds_at<TW * 4>(sa + off), ssd = shift_bound(smh, sis);
         const float left = thr - __shfl_sync(0xffffffffu, kim, src);
-        const float *xw = t.xs + ws;
         // a window that survives these steps (the neighbourhood of a match)
         // goes to the DTW stage with the partial sum, itself a lower bound,
         // rather than holding this warp for the full sum
-        const float t0 = keogh_term((xw[e.o0] - smh) * sis, e.u0 + ssd, e.l0 - ssd);
+        const float t0 = keogh_term((lds_at<0>(xa + off + 4u * (unsigned)o0) - smh) * sis, u0 + ssd, l0 - ssd);
         if (__any_sync(0xffffffffu, t0 > left)) continue;
-        const float t1 = keogh_term((xw[e.o1] - smh) * sis, e.u1 + ssd, e.l1 - ssd);
+        const float t1 = keogh_term((lds_at<0>(xa + off + 4u * (unsigned)o1) - smh) * sis, u1 + ssd, l1 - ssd);
         if (__any_sync(0xffffffffu, t0 + t1 > left)) continue;
         const float s2 = warp_sum(t0 + t1);
         if (s2 > left) continue;
@@ -1587,15 +1592,14 @@ __device__ __forceinline__ int lb_row_keogh(const Tile &t, const QueryBufs &b, Q
     // one append per row of 32 windows: a warp-aggregated atomic
     if (keep) {
         int base = 0;
-        if (lane == 0) base = atomicAdd(&st->n_cand, __popc(keep));
+        if (lane == 0) base = atomicAdd(n_cand, __popc(keep));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (keep & (1u << lane)) {
             const int pos = base + __popc(keep & ((1u << lane) - 1u));
-            b.cand_lb[pos] = my_lb;
-            b.cand_idx[pos] = (unsigned)(i0 + w);
+            cand_lb[pos] = my_lb;
+            cand_idx[pos] = first + (unsigned)lane;
         }
     }
-    return __popc(keep);
 }
 
 template <int TW>
@@ -1610,17 +1614,18 @@ __global__ void __launch_bounds__(kScanThreads, 5) k_lb_scan(QueryBufs b, QueryA
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     constexpr int kPerWarp = TW / kScanConsumers;
     // the ordered query terms the scan uses, in shared memory
-    __shared__ int o_s[kScanTerms];
-    __shared__ float u_s[kScanTerms], l_s[kScanTerms];
+    __shared__ EqTerms eq;
     const int nt = terms_of(m) < kScanTerms ? terms_of(m) : kScanTerms;
     for (int j = threadIdx.x; j < kScanTerms; j += blockDim.x) {
-        o_s[j] = j < nt ? (int)b.ord[j] : 0;
-        u_s[j] = j < nt ? b.sU[j] : DINF;
-        l_s[j] = j < nt ? b.sL[j] : -DINF;
+        eq.o[j] = j < nt ? (int)b.ord[j] : 0;
+        eq.u[j] = j < nt ? b.sU[j] : DINF;
+        eq.l[j] = j < nt ? b.sL[j] : -DINF;
+        eq.nt = nt;
     }
     __syncthreads();
-    const EqTerms eq{o_s, u_s, l_s, nt, o_s[lane], o_s[32 + lane], u_s[lane], l_s[lane], u_s[32 + lane], l_s[32 + lane]};
-    unsigned c1 = 0, c2 = 0;  // (per lane: at most the windows its warp scans)
+    __shared__ unsigned kim_passes;  // (at most the windows that the CTA scans)
+    if (threadIdx.x == 0) kim_passes = 0;
+    __syncthreads();
     const int64_t ntiles = (a.N + TW - 1) / TW;
     tile_pipeline<LbLayout<TW>>(smraw, b, m, ntiles, &st->tile_ctr[1], stages, [&](const Tile &t, int64_t i0) {
         // 32-bit shared addresses of this lane's first window (row 0); the
@@ -1631,54 +1636,49 @@ __global__ void __launch_bounds__(kScanThreads, 5) k_lb_scan(QueryBufs b, QueryA
         // windows of this tile that exist: w < rem
         const int rem = a.N - i0 < TW ? (int)(a.N - i0) : TW;
         constexpr int kRows = kPerWarp / 32;
+        // LB_KimFL of the window whose statistics and first sample lie RO bytes
+        // past the lane's
+        auto kim_of = [&](auto ro, unsigned at) {
+            constexpr int RO = decltype(ro)::value;
+            const float mh = lds_at<RO>(sa + at), is = lds_at<RO + TW * 4>(sa + at);
+            const float sd = shift_bound(mh, is);
+            const float d0 = fmaxf(fabsf(fmaf(mh - lds_at<RO>(xa + at), is, qf)) - sd, 0.0f);
+            const float d1 = fmaxf(fabsf(fmaf(mh - lds_at<RO>(xl + at), is, ql)) - sd, 0.0f);
+            return fmaf(d0, d0, d1 * d1);
+        };
         // LB_KimFL for every row first (unrolled, constant offsets), then the
-        // rare part for the rows where some window passed (one copy of it)
+        // rare part for the rows where some window passed (one copy of it,
+        // which forms the row's bound again rather than keep every row's)
         unsigned bals[kRows];
-        float kims[kRows];
         static_for<kRows>([&](auto uc) {
             constexpr int u = decltype(uc)::value;
-            constexpr int RO = u * 32 * 4;
             bool pass = false;
-            float kim = 0.0f;
-            if ((int)w0 + u * 32 < rem) {
-                const float mh = lds_at<RO>(sa), is = lds_at<RO + TW * 4>(sa);
-                const float sd = shift_bound(mh, is);
-                const float d0 = fmaxf(fabsf(fmaf(mh - lds_at<RO>(xa), is, qf)) - sd, 0.0f);
-                const float d1 = fmaxf(fabsf(fmaf(mh - lds_at<RO>(xl), is, ql)) - sd, 0.0f);
-                kim = fmaf(d0, d0, d1 * d1);
-                pass = !(kim > thr);
-            }
+            if ((int)w0 + u * 32 < rem) pass = !(kim_of(std::integral_constant<int, u * 32 * 4>{}, 0u) > thr);
             bals[u] = __ballot_sync(0xffffffffu, pass);
-            kims[u] = kim;
         });
         unsigned any = 0;
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            c1 += (unsigned)__popc(bals[u]);
-            any |= bals[u];
-        }
+        for (int u = 0; u < kRows; ++u) any |= bals[u];
         if (any) {
 #pragma unroll 1
             for (int u = 0; u < kRows; ++u) {
-                // (the row's ballot and bound picked by constant indices, so
-                // the arrays stay in registers)
+                // (the row's ballot picked by constant indices, so that the
+                // array stays in registers)
                 unsigned bu = 0;
-                float ku = 0.0f;
                 static_for<kRows>([&](auto vc) {
                     constexpr int v = decltype(vc)::value;
                     bu = u == v ? bals[v] : bu;
-                    ku = u == v ? kims[v] : ku;
                 });
                 if (!bu) continue;
-                const int w = (int)w0 + u * 32;
-                c2 += lb_row_keogh(t, b, st, eq, thr, bu, w - lane, lane, ku, i0);
+                if (lane == 0) atomicAdd(&kim_passes, (unsigned)__popc(bu));
+                const float ku = kim_of(std::integral_constant<int, 0>{}, (unsigned)u * 128u);
+                lb_row_keogh<TW>(b.cand_lb, b.cand_idx, &st->n_cand, eq, thr, bu, sa + (unsigned)u * 128u,
+                                 xa + (unsigned)u * 128u, ku, (unsigned)i0 + w0 + (unsigned)(u * 32 - lane));
             }
         }
     });
-    if (lane == 0) {
-        if (c1) atomicAdd(&st->ctr[kCtrKim], (unsigned long long)c1);
-        if (c2) atomicAdd(&st->ctr[kCtrKeoghQ], (unsigned long long)c2);
-    }
+    __syncthreads();
+    if (threadIdx.x == 0 && kim_passes) atomicAdd(&st->ctr[kCtrKim], (unsigned long long)kim_passes);
 }
 
 template <int TW>
@@ -1763,7 +1763,10 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_hist(QueryBufs b) {
     const int base = carry + inc - v;
     st->bin_off[2 * t] = base;
     st->bin_off[2 * t + 1] = base + v0;
-    if (t == 0) st->work2 = 0;
+    if (t == 0) {
+        st->work2 = 0;
+        st->ctr[kCtrKeoghQ] = (unsigned long long)st->n_cand;
+    }
 }
 
 // Each CTA takes a contiguous chunk of the survivors, counts its bins in
