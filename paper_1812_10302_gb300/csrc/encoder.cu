@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kSeqGroups * kSeqThreads) k_seq_forward(const 
     stage_weights(sm, blob, false);
     zero_smem(sm + SeqSmem::SHARED, kSeqGroups * SeqSmem::GROUP);
     __syncthreads();
-    for (int r = blockIdx.x * kSeqGroups + grp; r < rows; r += gridDim.x * kSeqGroups) {
+    for (int r = blockIdx.x + grp * gridDim.x; r < rows; r += gridDim.x * kSeqGroups) {
         float *us = reinterpret_cast<float *>(gm + SeqSmem::U);
         const float *ur = r < split ? u + (size_t)r * 64 : u2 + (size_t)(r - split) * 64;
         if (t < 64) us[t] = t < NU ? ur[t] : 0.0f;
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kSeqGroups * kSeqThreads) k_seq_backward(const
     static_assert(SeqSmem::G - SeqSmem::H4 >= 64 * LDX * 2, "a layer's h fits");
     float *de = reinterpret_cast<float *>(gm + SeqSmem::E);
     float *dg = reinterpret_cast<float *>(gm + SeqSmem::G);
-    for (int r = blockIdx.x * kSeqGroups + grp; r < rows; r += gridDim.x * kSeqGroups) {
+    for (int r = blockIdx.x + grp * gridDim.x; r < rows; r += gridDim.x * kSeqGroups) {
         uint8_t *w = ws + (size_t)r * SeqWs::BYTES;
         const bf16 *hg = reinterpret_cast<const bf16 *>(w + SeqWs::ACT);
         bf16 *dz = reinterpret_cast<bf16 *>(w + SeqWs::DZ);
@@ -983,7 +983,8 @@ cudaError_t launch_enc_prep(const float *X, const int64_t *off, int rows, int m,
 cudaError_t launch_enc_forward(const uint8_t *blob, const float *u, const float *u2, int split, int rows, float *e,
                                uint8_t *ws, int num_sms, cudaStream_t s) {
     const int smem = enc::SeqSmem::bytes(enc::kSeqGroups), threads = enc::kSeqGroups * enc::kSeqThreads;
-    const int ctas = (rows + enc::kSeqGroups - 1) / enc::kSeqGroups, grid = ctas < num_sms ? ctas : num_sms;
+    // a sequence per CTA first, then per group: a small batch uses every SM
+    const int grid = rows < num_sms ? rows : num_sms;
     cudaError_t err;
     if (ws) {
         if ((err = set_smem((const void *)enc::k_seq_forward<true>, smem)) != cudaSuccess) return err;
@@ -1002,7 +1003,7 @@ cudaError_t launch_enc_backward(const uint8_t *blob, const float *y, int B, int 
     const int smem = enc::SeqSmem::bytes(enc::kSeqGroups);
     cudaError_t err = set_smem((const void *)enc::k_seq_backward, smem);
     if (err != cudaSuccess) return err;
-    const int ctas = (rows + enc::kSeqGroups - 1) / enc::kSeqGroups, grid = ctas < num_sms ? ctas : num_sms;
+    const int grid = rows < num_sms ? rows : num_sms;  // (as the forward pass)
     enc::k_seq_backward<<<grid, enc::kSeqGroups * enc::kSeqThreads, smem, s>>>(blob, rows, ws);
     // Two CTAs per SM over the four layers, each with dozens of sequences: every
     // CTA ends with 28 KB of atomic sums (with eight per SM those took 80 of

@@ -54,3 +54,13 @@ def test_gradient_does_not_depend_on_the_order_of_the_batch(triples, batch):
     dl, dg = dtws.enc_loss_grad(*(torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (p, uq, uc, y)))
     assert abs(dl - loss) <= 2e-5 * loss
     assert np.linalg.norm(dg - grad) <= 2e-5 * np.linalg.norm(grad)
+
+
+@pytest.mark.parametrize("rows", [151, 152, 153, 303, 305, 1521])
+def test_sequences_around_the_number_of_sms(triples, rows):
+    """Sequences go to the SMs first, then to the groups of each: none is left
+    out where their number passes the SMs' (152)."""
+    p, u = triples[0], triples[1][:rows]
+    e = dtws.enc_forward(p, u)
+    some = np.unique(np.linspace(0, rows - 1, 40).astype(int))
+    np.testing.assert_array_equal(e[some], np.concatenate([dtws.enc_forward(p, u[i:i + 1]) for i in some]))
