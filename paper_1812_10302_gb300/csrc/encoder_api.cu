@@ -6,6 +6,7 @@
 
 #include "dtws.h"
 #include "dtws_internal.h"
+#include "pointers.h"
 
 using namespace dtws;
 
@@ -45,15 +46,6 @@ cudaError_t pack_params(const float *params, float *pbuf, uint8_t *blob, cudaStr
     cudaError_t e = cudaMemcpyAsync(pbuf, params, (size_t)kEncParams * 4, cudaMemcpyDefault, s);
     if (e != cudaSuccess) return e;
     return launch_enc_pack(pbuf, nullptr, nullptr, nullptr, blob, false, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, s);
-}
-
-bool on_device(const void *p) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
 bool finite_all(const float *v, int64_t n) {
@@ -130,10 +122,10 @@ dtws_status dtws_enc_loss_grad(const float *params, const float *uq, const float
     const int sms = num_sms();
     // The batch is worked through in parts (30 KB of activations per sequence:
     // 210 MB instead of 610 at 10,000 triples); one allocation holds everything
-    // (seven, of that size, took 0.9 ms per call).  Inputs already on the
+    // (seven, of that size, took 0.9 ms per call).  Inputs already on this
     // device are read where they are.
     const int part = batch < enc_chunk_pairs(sms) ? batch : enc_chunk_pairs(sms);
-    const bool qdev = on_device(uq), cdev = on_device(uc), ydev = on_device(y);
+    const bool qdev = readable_in_place(uq), cdev = readable_in_place(uc), ydev = readable_in_place(y);
     size_t bytes = 0;
     auto take = [&](size_t n) {
         const size_t at = bytes;
