@@ -103,6 +103,7 @@ struct Lane {
     char *block = nullptr;  // the allocation its arrays lie in
     float *cand_lb = nullptr, *sort_lb = nullptr;
     unsigned *cand_idx = nullptr, *sort_idx = nullptr;
+    unsigned long long *warp_best = nullptr;
     StatsEntry stats;  // slot that serves every m (in the lane's block)
     cudaStream_t stream = nullptr, side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_done = nullptr;
@@ -140,6 +141,7 @@ struct dtws_ctx {
     bool turn_taken = false;
     char *work_block = nullptr, *cand_block = nullptr;
     QueryState *st = nullptr;
+    unsigned long long *warp_best = nullptr;
     int *status = nullptr;
     float *qh32 = nullptr, *Uq = nullptr, *Lq = nullptr, *sq = nullptr, *sU = nullptr, *sL = nullptr;
     double *qh64 = nullptr;
@@ -636,10 +638,12 @@ dtws_status ensure_workspace(dtws_t h) {
     Arena a;
     const size_t st = a.take<QueryState>(1), qh32 = a.take<float>(kMMax), Uq = a.take<float>(kMMax),
                  Lq = a.take<float>(kMMax), sq = a.take<float>(kMMax), sU = a.take<float>(kMMax),
-                 sL = a.take<float>(kMMax), qh64 = a.take<double>(kMMax), ord = a.take<unsigned short>(kMMax);
+                 sL = a.take<float>(kMMax), qh64 = a.take<double>(kMMax), ord = a.take<unsigned short>(kMMax),
+                 wb = a.take<unsigned long long>(kScanSlots);
     CK(a.alloc());
     h->work_block = a.base;
     h->st = a.at<QueryState>(st);
+    h->warp_best = a.at<unsigned long long>(wb);
     h->qh32 = a.at<float>(qh32);
     h->Uq = a.at<float>(Uq);
     h->Lq = a.at<float>(Lq);
@@ -670,6 +674,7 @@ QueryBufs make_bufs(dtws_t h, const StatsEntry *se, const EnvEntry *ee) {
     QueryBufs b;
     memset(&b, 0, sizeof b);  // padding included: the bytes enter graph signatures
     b.st = h->st;
+    b.warp_best = h->warp_best;
     b.x = h->x;
     b.x_sub = h->x_sub;
     b.mu_hi = se ? se->mu_hi : nullptr;
@@ -1030,7 +1035,7 @@ dtws_status ensure_lanes(dtws_t h, int count) {
         const int64_t cap = h->n;
         Arena a;
         const size_t cl = a.take<float>(cap), sl = a.take<float>(cap), ci = a.take<unsigned>(cap),
-                     si = a.take<unsigned>(cap);
+                     si = a.take<unsigned>(cap), wb = a.take<unsigned long long>(kScanSlots);
         const StatsLayout sl_ = take_stats(a, stats_cap(h));
         cudaError_t e = a.alloc();
         auto al = [&](cudaError_t r) {
@@ -1042,6 +1047,7 @@ dtws_status ensure_lanes(dtws_t h, int count) {
             l.sort_lb = a.at<float>(sl);
             l.cand_idx = a.at<unsigned>(ci);
             l.sort_idx = a.at<unsigned>(si);
+            l.warp_best = a.at<unsigned long long>(wb);
             place_stats(&l.stats, a, sl_);
         }
         al(cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking));
@@ -1068,6 +1074,7 @@ dtws_status ensure_lanes(dtws_t h, int count) {
 
 QueryBufs lane_bufs(dtws_t h, const Lane &l, const EnvEntry *ee) {
     QueryBufs b = make_bufs(h, &l.stats, ee);  // (the caller sets the query's own state and buffers)
+    b.warp_best = l.warp_best;
     b.cand_lb = l.cand_lb;
     b.sort_lb = l.sort_lb;
     b.cand_idx = l.cand_idx;

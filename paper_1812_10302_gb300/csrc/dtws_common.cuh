@@ -35,6 +35,7 @@ constexpr int kSeedMax = 128;       // random seeds + proxy proposals
 constexpr int kPropMax = 64;
 constexpr int kCtaSlots = 1024;     // per-CTA best windows of one proposal scan (at most this many CTAs)
 constexpr int kScanConsumers = 8;   // consumer warps of a scan's CTA
+constexpr int kScanSlots = kCtaSlots * kScanConsumers;
 constexpr int kProxyStride = 4;     // the proxy scan looks at every fourth window
 // Euclidean seeds around each proxy proposal: offsets within +-kProxyHalf.
 // A match off the proxy's grid is never scored by the proxy itself; on a
@@ -131,9 +132,9 @@ struct QueryState {
     // survivors' pre-check)
     float e10_q[kTerms];
     unsigned short e10_pos[kTerms];
-    // (last: the words above that the scans' atomics meet on stay where they were)
-    unsigned long long warp_best[kCtaSlots * kScanConsumers];  // each proxy-scan warp's best window
 };
+
+static_assert(sizeof(QueryState) <= 64 * 1024, "a batch holds one per query");
 
 // Scalars of one query, passed by value to every kernel.
 struct QueryArgs {

@@ -57,6 +57,9 @@ struct QueryBufs {
     int *status;
     long long wait_ns;
     int num_sms;
+    // each proxy-scan warp's best window (kScanSlots keys): read between that
+    // scan and the next launch only, so one per lane, not per query
+    unsigned long long *warp_best;
     // survivor pass of the persistent batch stage: the survivors' window
     // statistics (mean high part, 1/sigma, mean low part * 1/sigma), indexed
     // like sort_idx; null elsewhere

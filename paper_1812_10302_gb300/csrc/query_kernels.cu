@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kScanThreads) k_seed_scan(QueryBufs b, QueryAr
     if (lane_id() == 0) {
         wbest[threadIdx.x >> 5] = best;
         if ((threadIdx.x >> 5) < kScanConsumers)
-            b.st->warp_best[blockIdx.x * kScanConsumers + (threadIdx.x >> 5)] = best;
+            b.warp_best[blockIdx.x * kScanConsumers + (threadIdx.x >> 5)] = best;
     }
     __shared__ int last, wcnt[kScanConsumers + 2], total;
     // (every copy into the stages has landed unless a wait ran out)
@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(kEdWarps * 32) k_seed_ed(QueryBufs b, QueryArg
     int nw = 0;
     if (slots > 0) {
         if (w < slots) {
-            const unsigned long long key = st->warp_best[w];
+            const unsigned long long key = b.warp_best[w];
             if (key != kEmptyKey) {
                 const long long c = key_idx(key), lo = c - kProxyHalf > 0 ? c - kProxyHalf : 0;
                 const long long hi = c + kProxyHalf < a.N - 1 ? c + kProxyHalf : a.N - 1;
