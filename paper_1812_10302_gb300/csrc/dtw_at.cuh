@@ -26,6 +26,7 @@ namespace dtws {
     X(2, 4) X(2, 5) X(2, 7) X(4, 3) X(4, 4) X(4, 5) X(4, 6) X(4, 7) X(4, 8) X(8, 3) X(8, 4) X(8, 5) X(8, 6) X(8, 7) X(8, 8) X(16, 3) \
         X(16, 4) X(16, 5) X(16, 6) X(16, 7) X(16, 8) X(32, 3) X(32, 4) X(32, 5) X(32, 6) X(32, 7) X(32, 8)
 constexpr int kAtThreads = 256;
+constexpr size_t kAtSmemMax = (size_t)224 * 1024;  // of an SM, and of a CTA at most
 // resident CTAs the register bound is set for
 __host__ __device__ constexpr int at_min_blocks(int K) { return K <= 3 ? 4 : 3; }
 
@@ -57,9 +58,9 @@ inline bool at_plan(int m, int r, AtPlan *best) {
         const size_t span = at_span(m, r, LL, KK) * 4, per = (size_t)(32 / LL) * span;                 \
         const int blocks = at_min_blocks(KK);                                                          \
         int warps = kAtThreads / 32;                                                                   \
-        while (warps > 1 && span + (size_t)warps * per > (size_t)224 * 1024 / blocks) --warps;         \
+        while (warps > 1 && span + (size_t)warps * per > kAtSmemMax / blocks) --warps;                 \
         const size_t total = span + (size_t)warps * per;                                               \
-        int on_sm = (int)((size_t)224 * 1024 / total);                                                 \
+        int on_sm = (int)(kAtSmemMax / total); /* (0: no warp's copies fit) */                         \
         if (on_sm > blocks) on_sm = blocks;                                                            \
         const int w = on_sm * warps;                                                                   \
         const double score = w > 0 ? LL * (7 * KK + ((KK & 1) ? 6 : 10)) * (w + 5.0) / w : 0.0;                         \

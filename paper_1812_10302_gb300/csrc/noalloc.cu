@@ -33,12 +33,15 @@ namespace {
 constexpr int kNoAllocCursor = DTWS_NOALLOC_M_MAX;      // 64-bit slot after q_hat (8-byte aligned)
 constexpr int kNoAllocFloats = DTWS_NOALLOC_M_MAX + 64;  // q_hat, cursor, padding
 
-// The largest launch this entry point makes is one warp (a group of 32
-// lanes) at m = DTWS_NOALLOC_M_MAX and r = m - 1: the normalised query
-// (4 m bytes) plus one ring of 2r + 2 floats (8 m bytes).  It must fit the
-// 227 KB a CTA may opt into on this part; the run-time check below also
-// compares it with the device's own limit.
+// Shared memory of the launches this entry point makes.  Bands of 5 to 256
+// cells: a padded query and 32 / L padded windows per warp, as many warps as
+// kAtSmemMax holds (dtw_at.cuh).  Other bands, one warp at least (a group of 32
+// lanes) at m = DTWS_NOALLOC_M_MAX and r = m - 1: the normalised query (4 m
+// bytes) plus one ring of 2r + 2 floats (8 m bytes).  Both must fit the 227 KB
+// a CTA may opt into on this part; the run-time checks below also compare them
+// with the device's own limit.
 static_assert(12 * DTWS_NOALLOC_M_MAX <= 227 * 1024, "scratch query length too long for one warp's shared memory");
+static_assert(dtws::kAtSmemMax <= 227 * 1024, "more shared memory than a CTA may have");
 
 }  // namespace
 
@@ -279,9 +282,11 @@ extern "C" dtws_status dtws_dtw_at_noalloc(const float *series, int64_t n, const
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    {  // one warp's shared memory must fit the device's per-block limit
-        int optin = 0;
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    int optin = 0;  // the device's limit per block
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    AtPlan p{};
+    const bool many = at_plan(m, rr, &p) && (optin <= 0 || p.smem <= (size_t)optin);
+    if (!many) {
         const size_t need = noalloc_smem(m, rr, lanes_for(rr), 1);
         if (optin > 0 && need > (size_t)optin) {
             set_error_detail("dtws_dtw_at_noalloc: m=%d, r=%d need %zu bytes of shared memory per warp, "
@@ -292,8 +297,7 @@ extern "C" dtws_status dtws_dtw_at_noalloc(const float *series, int64_t n, const
     cudaStream_t s = (cudaStream_t)stream;
     k_noalloc_prep<<<1, kPrepThreads, 0, s>>>(Q, m, scratch);
     cudaError_t e = cudaGetLastError();
-    AtPlan p{};
-    if (e == cudaSuccess && at_plan(m, rr, &p)) {
+    if (e == cudaSuccess && many) {
         e = cudaErrorInvalidValue;
 #define DTWS_CASE(LL, KK) \
     if (p.L == LL && p.K == KK) e = launch_noalloc_at<LL, KK>(series, n, m, rr, offsets, count, out, scratch, p, sms, s);
