@@ -21,10 +21,11 @@ namespace dtws {
 // (Two windows per lane in packed FP32 pairs, 9 K + 17 instructions for both,
 // were no faster: the packed operations stall the dispatch, 55 % issue, and
 // two windows per group halve the warps that fit.)
-// Shapes: X(L, K).
-#define DTWS_AT_SHAPES(X)                                                                                        \
-    X(2, 4) X(2, 5) X(2, 7) X(4, 3) X(4, 4) X(4, 5) X(4, 6) X(4, 7) X(4, 8) X(8, 3) X(8, 4) X(8, 5) X(8, 6) X(8, 7) X(8, 8) X(16, 3) \
-        X(16, 4) X(16, 5) X(16, 6) X(16, 7) X(16, 8) X(32, 3) X(32, 4) X(32, 5) X(32, 6) X(32, 7) X(32, 8)
+// Shapes: X(L, K): those that at_plan takes for some length up to 8192 and
+// some band (never 8 or 16 lanes of 6 cells: it was tried for all of them).
+#define DTWS_AT_SHAPES(X)                                                                                 \
+    X(2, 4) X(2, 5) X(2, 7) X(4, 3) X(4, 4) X(4, 5) X(4, 6) X(4, 7) X(4, 8) X(8, 3) X(8, 4) X(8, 5) X(8, 7) \
+    X(8, 8) X(16, 3) X(16, 4) X(16, 5) X(16, 7) X(16, 8) X(32, 3) X(32, 4) X(32, 5) X(32, 6) X(32, 7) X(32, 8)
 constexpr int kAtThreads = 256;
 constexpr size_t kAtSmemMax = (size_t)224 * 1024;  // of an SM, and of a CTA at most
 // resident CTAs the register bound is set for
