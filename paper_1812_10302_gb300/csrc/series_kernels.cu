@@ -10,6 +10,7 @@
 #include <cmath>
 
 #include "dtws_internal.h"
+#include "fp_pair.cuh"
 #include "fp_sum.cuh"
 
 namespace dtws {
@@ -106,39 +107,6 @@ cudaError_t launch_fill(float *p, int64_t count, float v, int num_sms, cudaStrea
 }
 
 // ------------------------------------------------------------------ FP32 pairs
-// Unevaluated sums hi + lo of two floats with error-free transformations
-// (Knuth's TwoSum, Dekker's Fast2Sum, the FMA product error).
-struct f2 {
-    float hi, lo;
-};
-__device__ __forceinline__ f2 two_sum(float a, float b) {
-    const float s = a + b, bb = s - a;
-    return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ f2 fast_two_sum(float a, float b) {
-    const float s = a + b;
-    return {s, b - (s - a)};
-}
-__device__ __forceinline__ f2 f2_add(f2 x, f2 y) {
-    f2 s = two_sum(x.hi, y.hi);
-    const f2 t = two_sum(x.lo, y.lo);
-    s.lo += t.hi;
-    s = fast_two_sum(s.hi, s.lo);
-    s.lo += t.lo;
-    return fast_two_sum(s.hi, s.lo);
-}
-__device__ __forceinline__ f2 f2_neg(f2 x) { return {-x.hi, -x.lo}; }
-__device__ __forceinline__ f2 f2_mul(f2 x, f2 y) {
-    const float p = x.hi * y.hi;
-    float e = fmaf(x.hi, y.hi, -p);
-    e = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, e));
-    return fast_two_sum(p, e);
-}
-__device__ __forceinline__ f2 f2_mul_f(f2 x, float f) {
-    const float p = x.hi * f;
-    const float e = fmaf(x.lo, f, fmaf(x.hi, f, -p));
-    return fast_two_sum(p, e);
-}
 __device__ __forceinline__ f2 ld2(const float *h, const float *l, int64_t t) { return {h[t], l[t]}; }
 
 // ------------------------------------------------------------------ prefix
@@ -318,13 +286,10 @@ cudaError_t launch_prefix(const float *x, int64_t n, float *pf, float *bf, int *
 // The window is evaluated two-pass from its samples instead when
 //   * a block it touches is not ok (see k_prefix), or
 //   * the subtraction cancelled, var <= 1e-6 * S2/m, or
-//   * var is below the bound the sums' rounding implies.  Each stored prefix
-//     is within 2^-48 of its magnitude, and the difference of two keeps their
-//     low parts to 2^-49 of the larger; so with P, E the prefixes at the
-//     window's ends S1 is off by less than 1.5 2^-48 (|P1| + |E1|), S2 by
-//     1.5 2^-48 (P2 + E2), and the pair operations on them by less than
-//     2^-48 12 S2 of m var; var then holds 2^-26 relative accuracy only if
-//     m*var >= 2^-22 (1.5 (P2 + E2) + 12 S2 + 3|S1/m| (|P1| + |E1|)).  (A
+//   * var is below the bound the sums' rounding implies.  With e1, e2 the bounds
+//     of f2_diff, S1 is off by no more than 2^-48 e1, S2 by 2^-48 e2, and the
+//     pair operations on them by less than 2^-48 12 S2 of m var; var then holds
+//     2^-26 relative accuracy only if m*var >= 2^-22 (e2 + 12 S2 + 2|S1/m| e1).  (A
 //     window over two blocks takes the totals M2 of its blocks' squares and
 //     the shift terms instead: 3 M2 + 4|S1/m| sqrt(B M2).  That bound for
 //     every window sent one in a hundred of a random walk's at m = 64 to the
@@ -356,12 +321,6 @@ __device__ __forceinline__ float2 load_at(const float *p) {
     const float2 a = *reinterpret_cast<const float2 *>(p);
     return S == 0 ? a : make_float2(a.y, p[2]);
 }
-// x - y, the low parts' difference rounded.
-__device__ __forceinline__ f2 f2_diff(f2 x, f2 y) {
-    const f2 s = two_sum(x.hi, -y.hi);
-    return fast_two_sum(s.hi, s.lo + (x.lo - y.lo));
-}
-
 // The two-pass evaluation (near-constant windows, or blocks whose values the
 // FP32 pairs cannot carry), by the window's thread: such windows come in runs,
 // and sums in FP32 expansions (fp_sum.cuh) run at full rate where FP64 sums,
@@ -425,10 +384,9 @@ k_window_stats(StatsIn in, float *__restrict__ mu_hi, float *__restrict__ mu_lo,
                     E1 = ld2(t1h, t1l, b0);
                     E2 = ld2(t2h, t2l, b0);
                 }
-                S1 = f2_diff(E1, P1);
-                S2 = f2_diff(E2, P2);
-                err2 = fmaf(12.0f, S2.hi, 1.5f * (P2.hi + E2.hi));
-                err1 = 1.5f * (fabsf(P1.hi) + fabsf(E1.hi));
+                S1 = f2_diff(E1, P1, err1);
+                S2 = f2_diff(E2, P2, err2);
+                err2 = fmaf(12.0f, S2.hi, err2);
             } else {
                 const int64_t b1 = b0 + 1 < in.nb ? b0 + 1 : b0;  // (past N: unused)
                 const int64_t end1 = (b1 + 1) * kBlockB;
