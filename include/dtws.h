@@ -249,8 +249,9 @@ dtws_status dtws_sync_status(dtws_t h, void *stream);
 /* Counters of the last query (synchronises the handle's work). */
 dtws_status dtws_last_stats(dtws_t h, dtws_query_stats *out);
 
-/* Drop the cached per-m window statistics and per-r series envelopes; the
-   next query recomputes what it needs. */
+/* Drop the cached per-m window statistics and embeddings and per-r series
+   envelopes, those of captured searches among them (see dtws_query); the next
+   query recomputes what it needs. */
 dtws_status dtws_clear_cache(dtws_t h);
 
 const char *dtws_strerror(dtws_status s);
@@ -309,7 +310,10 @@ dtws_status dtws_dtw_at(dtws_t h, const float *Q, int32_t m, int32_t r,
 /* Same, in extended precision: per-window two-pass statistics (Eq. 5) exact to
    FP64, and the DTW in 64-bit fixed point for few offsets (up to two per SM
    and bands to 1023: the re-score of dtws_query) or in double-float arithmetic
-   (~48 significant bits; plain FP64 for bands wider than 2047).
+   (~48 significant bits; plain FP64 for bands wider than 2047).  The walk is
+   chosen by count, m and r, so that a window's last bits may differ between
+   calls with few and with many offsets (by the double-float walk's error,
+   ~1e-14 relative on average).
    out: FP64 [count]. */
 dtws_status dtws_dtw_at_f64(dtws_t h, const float *Q, int32_t m, int32_t r,
                             const int64_t *offsets, int64_t count, double *out,

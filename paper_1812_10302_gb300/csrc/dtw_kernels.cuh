@@ -19,7 +19,7 @@
 namespace dtws {
 
 // the multi-warp FP32 kernel for bands past one warp (k_dtw_mw below): four
-// warps per candidate, up to 16 cells per lane
+// warps per candidate, up to 17 cells per lane
 constexpr int kWideW = 4;
 constexpr int kWideRMax = 32 * kWideW * 16 - 1;  // 2047
 

@@ -50,7 +50,7 @@ struct QueryBufs {
     float *qh32;                 // normalised query, FP32 [m]
     double *qh64;                // normalised query, FP64 [m]
     float *Uq, *Lq;              // query envelope [m]
-    unsigned short *ord;         // query positions by |q_hat| descending [m]
+    unsigned short *ord;         // the query's ordered terms: positions [terms_of(m)] (k_qprep)
     float *sq, *sU, *sL;         // q_hat, Uq, Lq in that order [m]
     float *cand_lb, *sort_lb;    // survivors [cap]
     unsigned int *cand_idx, *sort_idx;

@@ -1471,8 +1471,8 @@ cudaError_t launch_dtw_at_f64(const QueryBufs &b, const QueryArgs &a, const int6
 // ------------------------------------------------------------------ LB scan
 // Cascade over tiles of windows (Sec. 2.2, Eqs. 6-8, prune when a bound
 // exceeds thr): LB_KimFL (Eq. 7, squared) for every window, then LB_Keogh of
-// the window against the query envelope (Eq. 8), terms in |q_hat|-descending
-// order with early abandon.  Survivors (lb = max of the two, offset) are
+// the window against the query envelope (Eq. 8) at the first kScanTerms ordered
+// terms, added to it, with early abandon.  Survivors (the sum, offset) are
 // appended to the global survivor list.  The third bound, LB_Keogh of the
 // query against the window's envelope (Eq. 10, from the series-wide envelope
 // normalised with the window's statistics: looser than the window-clipped
@@ -1526,13 +1526,15 @@ struct EqTerms {
 // a lower bound: LB_KimFL is the cost of the path's first and last cells, in
 // columns 0 and m-1, the terms bound the cells of other columns.  Survivors
 // are appended as (bound, offset) by one warp-aggregated atomic.  A row with
-// several passers first gives each lane kLaneFirst terms of its own window; what is left is taken one window at a time, 32
-// terms per step, where a single term above what is left of thr already
-// prunes (a vote), or lane by lane to the end where most of the row is left
-// (a loose bound).  No thread waits on another warp's survivors.
-// Measured (1e8 windows, m = 512, five queries, 0.2 to 5.8e6 past LB_KimFL):
-// 231 to 384 us, 0.29 ms on average; one 32-term shuffle sum per window in
-// |q_hat| order 233 to 641 us, 0.44 ms.
+// several passers first gives each lane kLaneFirst terms of its own window;
+// what is left is taken one window at a time, 32 terms per step, where a single
+// term above what is left of thr already prunes (a vote), or lane by lane to the
+// end where most of the row is left (a loose bound).  No thread waits on
+// another warp's survivors.
+// Measured (1e8 windows, m = 512, five queries, 0.2 to 5.8e6 past LB_KimFL,
+// spilling as EqTerms' comment says): 231 to 384
+// us, 0.29 ms on average; one 32-term shuffle sum per window in |q_hat| order
+// 233 to 641 us, 0.44 ms.
 // (Eq. 10's first 32 terms here as well, for each window past Eq. 8, slowed
 // the scan more than it saved: the random loads of the series envelope stall
 // the warps that feed the ring.  128 terms instead of 64: scan +90 us,
