@@ -709,11 +709,12 @@ __device__ __forceinline__ bool wide_prune(const QueryBufs &b, const float *qs, 
     float acc = 0.0f, acc8 = lb;
     for (int c0 = 0; c0 < T; c0 += 32) {
         const int j = c0 + lane;
-        const bool eq8 = c0 < T - kScanTerms;
+        const bool eq8 = c0 >= kScanTerms;
         float v = 0.0f, v8 = 0.0f;
-        if (eq8 && j < T - kScanTerms) {
-            const float cv = fmaf(xw[terms.pos8[j]] - mh, is, -ls);
-            const float e = fmaxf(cv - terms.u8[j], 0.0f) + fmaxf(terms.l8[j] - cv, 0.0f);
+        if (eq8 && j < T) {
+            const int j8 = j - kScanTerms;
+            const float cv = fmaf(xw[terms.pos8[j8]] - mh, is, -ls);
+            const float e = fmaxf(cv - terms.u8[j8], 0.0f) + fmaxf(terms.l8[j8] - cv, 0.0f);
             v8 = e * e;
         }
         if (j < T) {
