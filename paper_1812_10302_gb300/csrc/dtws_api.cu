@@ -831,7 +831,8 @@ dtws_status enqueue_search(dtws_t h, const Exec &e, const QueryArgs &a, const fl
         return DTWS_OK;
     }
     // a wide exclusion zone needs k seeds in separate buckets of each parity
-    // for a first threshold: all the proposals the list holds
+    // for a first threshold: all the proposals that the learned scan's list
+    // holds (the proxy scan's warps offer their best windows whatever P is)
     const int P = (a.xz_z > 0 && h->opt.seed_proposals > 0) ? kPropMax : h->opt.seed_proposals;
     const int R = h->opt.seed_random;
     int64_t launches = 0;
