@@ -236,7 +236,9 @@ dtws_status dtws_query(dtws_t h, const float *Q, int32_t m, int32_t r, int32_t k
  * queries back to back; q_off (HOST int64 [nq+1]) gives query q as
  * Q_cat[q_off[q] .. q_off[q+1]); m_arr and r_arr are HOST int32 [nq] with
  * m_arr[q] == q_off[q+1]-q_off[q].  out_idx / out_dist are [nq*k]
- * row-major.  Same per-query semantics and limits as dtws_query().
+ * row-major.  Same per-query semantics and limits as dtws_query(), but not on
+ * a stream that the caller is capturing (the call's tables on the host do not
+ * outlive it).
  */
 dtws_status dtws_query_batch(dtws_t h, const float *Q_cat, const int64_t *q_off,
                              const int32_t *m_arr, const int32_t *r_arr, int32_t nq,
